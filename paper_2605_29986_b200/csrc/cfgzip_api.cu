@@ -217,6 +217,9 @@ bool aligned32(const void* p, int64_t row_stride_elems, int elem_size) {
     return (reinterpret_cast<uintptr_t>(p) & 31u) == 0 && ((row_stride_elems * elem_size) & 31) == 0;
 }
 
+// (rows of a buffer that does not even start on an element are left to the element-wise kernels)
+bool aligned_elems(const void* p, int elem_size) { return (reinterpret_cast<uintptr_t>(p) & uintptr_t(elem_size - 1)) == 0; }
+
 bool aligned16(const void* p, int64_t row_stride_elems, int elem_size) {
     return (reinterpret_cast<uintptr_t>(p) & 15u) == 0 && ((row_stride_elems * elem_size) & 15) == 0;
 }
@@ -235,6 +238,8 @@ struct DensePlan {
     int hold_warps = 0;
     int ctas_per_sm = 1; // blocks per SM the launch was sized for
     int opl = 1;         // pipelined kernel: octets per lane and row (2: bf16 chunks of 512 tokens)
+    bool shifted = false;  // pipelined kernel: rows that start anywhere
+    int chunk_octets = 32; // pipelined kernel: vectors per row and work item
     int fold = 0;        // pipelined kernel: results written by the last block of each group (no finalize launch)
     int fold_off = 0;    // fold: offset of the block's shared (row, warp) states, 0 = warps publish to the scratch directly
     int slots = 0;       // states per row in the global scratch
@@ -296,16 +301,19 @@ DensePlan plan_dense(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, 
 
 // Launch shape of the pipelined fused kernel. A block takes per_split octets (any number, not only
 // whole 32-octet chunks) of one row group, so that the blocks of a step fill the SMs evenly.
-DensePlan plan_pipe_opl(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, int elem_size, bool cm_bulk_ok, int opl) {
+DensePlan plan_pipe_opl(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, int elem_size, bool cm_bulk_ok, int opl,
+                        bool shifted) {
     DensePlan d;
     d.opl = opl;
+    d.shifted = shifted;  // rows off the 16-byte grid: each row's vectors start at its own first boundary
+    d.chunk_octets = shifted ? PipeChunk<1, kSrcShifted>::kOctets : 32 * opl;
     d.table_words = (ps.maxKW + 1) * 32;
     d.use_plan_kernel = mixed;
     d.n_groups_ub = mixed ? ceil_div(B, kGroupRows) + ps.n_live_same_v : ceil_div(B, kGroupRows);
     if (!ps.all_c16 || !ctx->pipeline) return d;
     if (mixed && (B > ctx->reserved_rows || d.n_groups_ub > ctx->max_groups)) return d;
-    const int chunk_octets = 32 * opl;
-    const int stage_bytes = 8 * chunk_octets * 8 * elem_size + chunk_octets * 16;
+    const int chunk_octets = d.chunk_octets;
+    const int stage_bytes = 32 * opl * (8 * 8 * elem_size + 16);
     const size_t cap = size_t(ctx->smem_optin) - 2048;  // room for the kernel's static shared memory
     // two octets per lane: the variant is compiled for at most 12 warps (its stages are twice as large and it needs
     // more registers per thread)
@@ -359,7 +367,7 @@ DensePlan plan_pipe_opl(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixe
     d.depth = depth;
     d.stage_stride = stride;
     const int fit = std::max(1, int((cap + 1024) / (smem + 1024)));
-    d.ctas_per_sm = opl == 2 ? 1 : std::min(ctx->ctas_per_sm, fit);
+    d.ctas_per_sm = opl == 2 || shifted ? 1 : std::min(ctx->ctas_per_sm, fit);
     const int target = ctx->sm_count * d.ctas_per_sm * ctx->waves;
     const int n_oct = 4 * ps.VW;
     // blocks of groups that turn out not to exist leave at once, so size the split for the fewest
@@ -381,7 +389,7 @@ DensePlan plan_pipe_opl(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixe
     d.threads = d.WT * WR * 32;
     for (;;) {
         d.S = ceil_div(n_oct, per);
-        if (size_t(d.n_groups_ub) * kGroupRows * (size_t(d.S) * d.WT + 1) <= kPartialSlots) break;
+        if (size_t(d.n_groups_ub) * kGroupRows * (size_t(d.S) * d.WT + 2) <= kPartialSlots) break;
         if (per >= n_oct) return d;
         per *= 2;
     }
@@ -415,10 +423,11 @@ DensePlan plan_pipe_opl(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixe
 // Launch shape of the pipelined fused kernel. bf16 rows may be streamed with one octet (16 bytes) or two octets
 // (32 bytes) per lane and row; two octets halve the per-row bookkeeping but double a work item, so they are taken
 // only when every warp of the launch still gets several items.
-DensePlan plan_pipe(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, int elem_size, bool cm_bulk_ok) {
-    const DensePlan one = plan_pipe_opl(ctx, ps, B, mixed, elem_size, cm_bulk_ok, 1);
-    if (elem_size != 2 || ctx->lane_octets == 1) return one;
-    const DensePlan two = plan_pipe_opl(ctx, ps, B, mixed, elem_size, cm_bulk_ok, 2);
+DensePlan plan_pipe(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, int elem_size, bool cm_bulk_ok,
+                    bool shifted = false) {
+    const DensePlan one = plan_pipe_opl(ctx, ps, B, mixed, elem_size, cm_bulk_ok, 1, shifted);
+    if (elem_size != 2 || ctx->lane_octets == 1 || shifted) return one;
+    const DensePlan two = plan_pipe_opl(ctx, ps, B, mixed, elem_size, cm_bulk_ok, 2, false);
     if (!two.ok) return one;
     if (!one.ok || ctx->lane_octets == 2) return two;
     if (ctx->lane_octets == 0) return one;
@@ -486,7 +495,8 @@ void fill_groups(cfgzip_ctx* ctx, StepArgs& a, const DensePlan& d) {
     a.slots = d.slots;
     a.fold = d.fold;
     a.fold_off = d.fold_off;
-    a.chunk_tokens = 256 * d.opl;
+    a.chunk_tokens = 8 * d.chunk_octets;
+    a.shifted = d.shifted ? 1 : 0;
     // Only a programmatic launch runs ahead of the kernel in front, and only from about 48 MB of logits on does asking
     // ahead pay (measured: B = 256 -3.6 %, qwen-size -2.3 %, B = 512 -1.6 %; shorter steps lose, B = 32 +7 %: the
     // requests compete with the loads of the kernel in front, whose end the step waits for).
@@ -538,7 +548,7 @@ int launch_pipe(cfgzip_ctx* ctx, const StepArgs& a, const DensePlan& d, dim3 gri
     CUtensorMap tmap;
     std::memset(&tmap, 0, sizeof tmap);
     bool tiled = false;
-    if (!d.use_plan_kernel && ctx->tensor_map && ctx->encode_tiled && a.V >= 256 &&
+    if (!d.use_plan_kernel && !d.shifted && ctx->tensor_map && ctx->encode_tiled && a.V >= 256 &&
         a.row_stride * (DT == kBF16 ? 2 : 4) < (int64_t(1) << 32) && a.vm_stride * 4 < (int64_t(1) << 32)) {
         const cuuint64_t dims[2] = {cuuint64_t(a.V), cuuint64_t(a.B)};
         const cuuint64_t strides[1] = {cuuint64_t(a.row_stride) * (DT == kBF16 ? 2 : 4)};
@@ -552,10 +562,13 @@ int launch_pipe(cfgzip_ctx* ctx, const StepArgs& a, const DensePlan& d, dim3 gri
     void (*kern)(StepArgs, CUtensorMap);
     const bool tempered = a.u != nullptr;  // only a sampling step has a temperature
     constexpr int kTwo = DT == kBF16 ? 2 : 1;  // f32 lanes always take one octet (32 bytes)
-#define CFGZIP_PIPE_VARIANT(OPL, LBT, MINB)                                                                         \
-    (tempered ? (tiled ? k_step_dense_pipe<DT, OPL, true, LBT, MINB, true> : k_step_dense_pipe<DT, OPL, false, LBT, MINB, true>) \
-              : (tiled ? k_step_dense_pipe<DT, OPL, true, LBT, MINB, false> : k_step_dense_pipe<DT, OPL, false, LBT, MINB, false>))
-    if (d.opl == 2 && kTwo == 2 && d.threads <= 384)
+#define CFGZIP_PIPE_SRC(OPL, SRC, LBT, MINB) \
+    (tempered ? k_step_dense_pipe<DT, OPL, SRC, LBT, MINB, true> : k_step_dense_pipe<DT, OPL, SRC, LBT, MINB, false>)
+#define CFGZIP_PIPE_VARIANT(OPL, LBT, MINB) \
+    (tiled ? CFGZIP_PIPE_SRC(OPL, kSrcTiled, LBT, MINB) : CFGZIP_PIPE_SRC(OPL, kSrcRows, LBT, MINB))
+    if (d.shifted)  // (no variant with more blocks per SM: the rows' own pointers need the registers)
+        kern = CFGZIP_PIPE_SRC(1, kSrcShifted, 512, 1);
+    else if (d.opl == 2 && kTwo == 2 && d.threads <= 384)
         kern = CFGZIP_PIPE_VARIANT(kTwo, 384, 1);
     else if (d.opl != 1)
         return CFGZIP_E_ARG;  // the planner never asks for this
@@ -566,6 +579,7 @@ int launch_pipe(cfgzip_ctx* ctx, const StepArgs& a, const DensePlan& d, dim3 gri
     else
         kern = CFGZIP_PIPE_VARIANT(1, 512, 1);
 #undef CFGZIP_PIPE_VARIANT
+#undef CFGZIP_PIPE_SRC
     if ((rc = ensure_smem(kern, d.smem)) != CFGZIP_OK) return rc;
     return launch(ctx, kern, grid, block, d.smem, st, a, tmap);
 }
@@ -574,10 +588,7 @@ template <int DT>
 int launch_fused(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, int mode, bool aligned, float* logp_full,
                  cudaStream_t st) {
     int rc;
-    if (!aligned) {
-        // rows off the 16-byte grid: the per-row kernel with element-wise accesses
-        rc = launch(ctx, k_step_generic<DT, true>, dim3(unsigned(a.B)), dim3(256), 0, st, a);
-    } else if (mode == CFGZIP_SPARSE) {
+    if (aligned && mode == CFGZIP_SPARSE) {
         int S, per_split;
         if (plan_sparse(ctx, ps, a.B, true, &S, &per_split)) {
             a.S = S;
@@ -591,8 +602,9 @@ int launch_fused(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, in
         }
     } else {
         const bool cm_bulk_ok = (reinterpret_cast<uintptr_t>(a.class_mask) & 15u) == 0 && (a.cm_stride & 3) == 0;
-        DensePlan d = plan_pipe(ctx, ps, a.B, mixed, DT == kBF16 ? 2 : 4, cm_bulk_ok);
-        if (!d.ok) d = plan_dense(ctx, ps, a.B, mixed, 4 * ps.VW, 32, true);
+        DensePlan d = plan_pipe(ctx, ps, a.B, mixed, DT == kBF16 ? 2 : 4, cm_bulk_ok, !aligned);
+        if (d.shifted && !aligned_elems(a.logits, DT == kBF16 ? 2 : 4)) d.ok = false;
+        if (!d.ok && aligned) d = plan_dense(ctx, ps, a.B, mixed, 4 * ps.VW, 32, true);
         if (d.ok) {
             if (d.use_plan_kernel && (rc = run_plan_kernel(ctx, a.row_part, a.B, a.V, d, st)) != CFGZIP_OK) return rc;
             // Automatic mode on a long step: the class-list kernel runs first, keeps the row batches (the 8 rows the
@@ -601,7 +613,7 @@ int launch_fused(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, in
             // Short steps are dense outright (the extra launch would cost more than the class lists can save).
             int sp_S = 0, sp_per = 0;
             const int permille = ctx->auto_permille >= 0 ? ctx->auto_permille : (DT == kBF16 ? 10 : 40);
-            const bool choose = mode == CFGZIP_AUTO && d.depth > 0 && permille > 0 && ctx->d_row_mode != nullptr &&
+            const bool choose = mode == CFGZIP_AUTO && d.depth > 0 && aligned && permille > 0 && ctx->d_row_mode != nullptr &&
                                 a.B <= ctx->reserved_rows && ctx->auto_min_bytes >= 0 &&
                                 int64_t(a.B) * a.V * (DT == kBF16 ? 2 : 4) >= ctx->auto_min_bytes &&
                                 plan_sparse(ctx, ps, a.B, true, &sp_S, &sp_per);
@@ -677,26 +689,24 @@ int launch_filtered(cfgzip_ctx* ctx, const StepArgs& a, unsigned rows_grid, int 
 }
 
 // A sampling step: the streaming kernel leaves the states of a row in token order, the sampling kernel
-// (one block per row) draws the token. Rows off the 16-byte grid, and shapes the pipelined kernel does not
-// take, go through the per-row kernel, whose single state per row stands for the whole row.
+// (one block per row) draws the token. Shapes the pipelined kernel does not take go through the per-row kernel, whose
+// single state per row stands for the whole row.
 template <int DT>
 int launch_sample(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, bool aligned, int top_k, float top_p,
                   cudaStream_t st) {
     const bool filtered = top_k > 0 || top_p < 1.f;  // the draw is restricted to the most probable tokens
     int rc;
-    DensePlan d;
-    if (aligned) {
-        const bool cm_bulk_ok = (reinterpret_cast<uintptr_t>(a.class_mask) & 15u) == 0 && (a.cm_stride & 3) == 0;
-        d = plan_pipe(ctx, ps, a.B, mixed, DT == kBF16 ? 2 : 4, cm_bulk_ok);
-    }
-    if (d.ok && d.depth) {
+    const bool cm_bulk_ok = (reinterpret_cast<uintptr_t>(a.class_mask) & 15u) == 0 && (a.cm_stride & 3) == 0;
+    DensePlan d = plan_pipe(ctx, ps, a.B, mixed, DT == kBF16 ? 2 : 4, cm_bulk_ok, !aligned);
+    if (d.ok && d.depth && !(d.shifted && !aligned_elems(a.logits, DT == kBF16 ? 2 : 4))) {
         if (d.use_plan_kernel && (rc = run_plan_kernel(ctx, a.row_part, a.B, a.V, d, st)) != CFGZIP_OK) return rc;
         // a sampling step keeps one state per warp slot in token order and a kernel of its own for the draw
         if (d.fold_off) d.smem -= size_t(kGroupRows) * (d.WT + 1) * sizeof(Partial);
         d.fold = d.fold_off = 0;
-        d.slots = d.S * d.WT + 1;
+        d.slots = d.S * d.WT + 1 + (d.shifted ? 1 : 0);
         fill_groups(ctx, a, d);
-        const int n_chunks = ceil_div(ps.V >> 3, 32 * d.opl);
+        a.head_state = d.shifted ? 1 : 0;
+        const int n_chunks = ceil_div(ps.V >> 3, d.chunk_octets);
         a.run_chunks = std::max(1, ceil_div(n_chunks, d.S * d.WT));
         a.tail_state = 1;
         const dim3 grid(unsigned(d.n_groups_ub) * unsigned(d.S)), block{unsigned(d.threads)};

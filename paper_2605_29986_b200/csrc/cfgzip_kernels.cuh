@@ -61,6 +61,9 @@ struct StepArgs {
     int32_t masks_per_row;      // > 0: several class masks per logits row (register dense kernel only): row r of the masks,
                                 // vocab masks and results belongs to logits row r / masks_per_row, and the logits are not modified
     int32_t tail_state;         // sampling kernel: the last state of a row stands for the octets past the last whole vector
+    int32_t head_state;         // sampling kernel: the first state of a row stands for the tokens in front of its first vector
+                                // (rows off the vector grid)
+    int32_t shifted;            // rows start anywhere: the vectors of a row begin at row_head tokens, not at token 0
     float scale;                // log2(e) / temperature: the sums are of exp(z / T); log2(e) in a greedy step
     float inv_t;                // 1 / temperature
     const float* u;             // sampling step: dev [B] uniform numbers in [0, 1), else null
@@ -69,6 +72,15 @@ struct StepArgs {
     unsigned int* tickets;
     int32_t* status;            // [0] empty rows, [1] bad tokens, [2] bad rows, [3] copies that never arrived
 };
+
+// Tokens in front of the first vector boundary of a row that may start anywhere (16 bytes for bf16, 32 for f32: an
+// octet is one vector either way), and how many whole vectors follow.
+template <int DT>
+__device__ __forceinline__ int row_head(const char* rowp, int V) {
+    constexpr unsigned ES = DT == kBF16 ? 2 : 4, kVec = 8 * ES;
+    const unsigned past = unsigned(reinterpret_cast<uintptr_t>(rowp)) & (kVec - 1u);
+    return min(V, int(((kVec - past) & (kVec - 1u)) / ES));
+}
 
 // The logits row behind row r of the masks and results (they differ when a logits row has several masks).
 __device__ __forceinline__ int64_t logits_row(const StepArgs& a, int r) { return a.masks_per_row > 0 ? r / a.masks_per_row : r; }
@@ -386,13 +398,79 @@ __device__ __forceinline__ void publish_tail_octets(const StepArgs& a, const Par
     const Partial p = dense_tail_octets<DT>(a, P, s_row[lane], tail_first, tail_end, scale);
     if (s_row[lane] >= 0) row_slots(a, g, lane)[a.slots - 1] = p;
 }
-// The same into any array of states: row slot r's state goes to base[r * stride + slot].
-template <int DT>
-__device__ __forceinline__ void publish_tail_octets_to(const StepArgs& a, const PartDev& P, const int* s_row, int lane,
-                                                       int tail_first, int tail_end, float scale, Partial* base, int stride,
-                                                       int slot) {
-    const Partial p = dense_tail_octets<DT>(a, P, s_row[lane], tail_first, tail_end, scale);
-    if (s_row[lane] >= 0) base[lane * stride + slot] = p;
+// Order-preserving map between floats and signed integers (for the integer warp reductions).
+__device__ __forceinline__ int float_order_key(float x) {
+    const int i = __float_as_int(x);
+    return i >= 0 ? i : i ^ 0x7FFFFFFF;
+}
+__device__ __forceinline__ float float_from_order_key(int k) { return __int_as_float(k >= 0 ? k : k ^ 0x7FFFFFFF); }
+
+// What the vectors of a row leave over: the tokens in front of the first vector (rows off the vector grid), those past
+// the last one, and the vocab-mask octets from the last whole octet on (ragged end, padding of the last word). The
+// rows of the group are dealt over its blocks and their warps, each warp takes its rows one at a time with a lane per
+// token (lanes 0..7 the first octet, lanes 8..23 the 16 tokens from the last whole octet on), allow bits from the class
+// table: two round trips to memory for a row, where one lane walking the tokens took two per token.
+// to_head / to_tail(row slot): where the states go (the same place: one state for both).
+template <int DT, bool SHIFT, typename H, typename T>
+__device__ __forceinline__ void publish_edges(const StepArgs& a, const PartDev& P, const uint32_t* table, const int* s_row,
+                                              int nrow, int split, int warp, int lane, float scale, bool apart, H&& to_head,
+                                              T&& to_tail) {
+    constexpr int ES = DT == kBF16 ? 2 : 4;
+    const int n_full = a.V >> 3, n_octets = 4 * a.VW;
+    const bool in_head = lane < 8;
+    const int t = in_head ? lane : 8 * (n_full - 1) + lane - 8;
+    const bool have = lane < 24 && t >= 0 && t < a.V;
+    const int n_warps = blockDim.x >> 5;
+    if (!SHIFT && n_full == n_octets) {  // the vectors cover the vocabulary: nothing is left over
+        for (int j = split + a.S * warp; j < nrow; j += a.S * n_warps)
+            if (lane == 0) *to_tail(j) = partial_empty();
+        return;
+    }
+    uint32_t word = 0u;
+    bool asked = false;
+    for (int j = split + a.S * warp; j < nrow; j += a.S * n_warps) {
+        if (!asked && have) word = table[P.c16[t]];
+        asked = true;
+        const int row = s_row[j];
+        char* rowp = reinterpret_cast<char*>(a.logits) + int64_t(row) * a.row_stride * ES;
+        const int head = SHIFT ? row_head<DT>(rowp, a.V) : 0;
+        const int tail = head + ((a.V - head) & ~7);  // first token past the last whole vector
+        const bool mine = have && (in_head ? t < head : t >= tail);
+        const bool allowed = (word >> j) & 1u;
+        const uint32_t allow = __ballot_sync(0xFFFFFFFFu, allowed && !in_head);
+        if (a.vocab_mask && lane < n_octets - n_full)
+            reinterpret_cast<uint8_t*>(a.vocab_mask)[int64_t(row) * a.vm_stride * 4 + n_full + lane] =
+                lane == 0 ? uint8_t(allow >> 16) : uint8_t(0);
+        float z = -INFINITY;
+        if (mine) {
+            if (allowed) z = load_elem<DT>(rowp, t);
+            else store_neg_inf<DT>(rowp, t);
+        }
+        auto reduce = [&](bool part, int first) {  // the state of the lanes of one side; `first`: its octet position
+            const float m = float_from_order_key(__reduce_max_sync(0xFFFFFFFFu, float_order_key(part ? z : -INFINITY)));
+            float e = part && m > kRefFloor ? ex2f((z - m) * scale) : 0.f;
+#pragma unroll
+            for (int d = 16; d >= 1; d >>= 1) e += __shfl_xor_sync(0xFFFFFFFFu, e, d);
+            return Partial{m, e, m > -INFINITY ? first : kNoPos, 0};
+        };
+        const Partial pt = reduce(mine && !in_head, (a.V - head) >> 3);
+        if (!SHIFT) {
+            if (lane == 0) *to_tail(j) = pt;
+        } else {
+            const Partial ph = reduce(mine && in_head, 0);
+            if (lane == 0) {
+                if (apart) {
+                    *to_head(j) = ph;
+                    *to_tail(j) = pt;
+                } else {
+                    float m = ph.m, sum = ph.s;
+                    int pos = ph.pos;
+                    partial_merge(m, sum, pos, pt.m, pt.s, pt.pos, scale);
+                    *to_tail(j) = Partial{m, sum, pos, 0};
+                }
+            }
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------------------
@@ -535,13 +613,6 @@ __device__ __forceinline__ void dense_octet_row(Octet<DT>& oc, char* rowp, uint8
     if (vmp) vmp[o] = uint8_t(byte);
     acc.add_octet(f, o);
 }
-
-// Order-preserving map between floats and signed integers (for the integer warp reductions).
-__device__ __forceinline__ int float_order_key(float x) {
-    const int i = __float_as_int(x);
-    return i >= 0 ? i : i ^ 0x7FFFFFFF;
-}
-__device__ __forceinline__ float float_from_order_key(int k) { return __int_as_float(k >= 0 ? k : k ^ 0x7FFFFFFF); }
 
 // Reduce the 8 row states of a warp over its 32 lanes and publish them in the warp's slot of each row.
 // The state of row slot r goes to base[r * stride + slot] (global scratch, or the block's shared array).
@@ -703,6 +774,18 @@ struct PipeGeom {
     static constexpr int kStageBytes = kBatchRows * kRowBytes + kChunkOctets * 16;  // + class ids of the chunk
 };
 
+// How the logits of a work item reach shared memory: one bulk copy per row, one tiled 2-D copy for 8 consecutive rows,
+// or one bulk copy per row from that row's own first vector boundary on (rows that start anywhere).
+enum : int { kSrcRows = 0, kSrcTiled = 1, kSrcShifted = 2 };
+
+// Octets of a chunk. Where the rows start anywhere, vector o of a row holds the tokens 8 o + head .. 8 o + head + 7, so
+// its allow bits come from the token octets o and o + 1: a chunk is then the 31 vectors whose bits the 32 octets of
+// class ids in a stage give (lane l takes the second half of its bits from lane l + 1).
+template <int OPL, int SRC>
+struct PipeChunk {
+    static constexpr int kOctets = SRC == kSrcShifted ? 31 : 32 * OPL;
+};
+
 // Where the rows of a batch live. With consecutive rows (CONSEC) the address of row i is one
 // wide multiply-add from the batch's base; otherwise each row has its own base pointer.
 struct BatchAddr {
@@ -716,69 +799,106 @@ struct BatchAddr {
 // this lane's OPL octets of row i lie at src + i * srow + lane_off. n_act: how many of the lane's octets are whole
 // vectors of the row (OPL everywhere except at the end of the vocabulary).
 // FULL: all 8 rows live and every lane's octets inside the whole-vector range (no per-row tests).
-template <int DT, int OPL, bool FULL, bool CONSEC>
+// kSrcShifted: n_ids octets of class ids are in the stage; heads: row_head of the 8 rows, four bits each; the vocab-mask
+// byte of token octet o is written by the same lane as vector o of the rows. V: tokens.
+template <int DT, int OPL, bool FULL, int SRC>
 __device__ __forceinline__ void pipe_consume_item(const char* src, uint32_t lane_off, uint32_t srow, const uint32_t* T, int rb,
                                                   int live, int n_act, int o, int lane, const BatchAddr& ba,
                                                   char* const (&rowp)[kBatchRows], uint8_t* const (&vmp)[kBatchRows],
-                                                  RowAcc (&acc)[kBatchRows], float scale, bool wide) {
+                                                  RowAcc (&acc)[kBatchRows], float scale, bool wide, int n_ids, uint32_t heads,
+                                                  int V) {
     using G = PipeGeom<DT, OPL>;
-    uint32_t lo[OPL], hi[OPL];
-#pragma unroll
-    for (int q = 0; q < OPL; ++q) {
-        const bool act = FULL || q < n_act;
+    constexpr bool CONSEC = SRC == kSrcTiled;
+    if constexpr (SRC == kSrcShifted) {
+        uint32_t lo, hi;
         uint4 cv = make_uint4(0, 0, 0, 0);
-        if (act) cv = *reinterpret_cast<const uint4*>(src + kBatchRows * G::kRowBytes + (lane * OPL + q) * 16);
-        octet_allow_bits(cv, T, rb, act, lo[q], hi[q]);
-    }
-    const bool both = FULL || n_act == OPL;
+        const bool have = FULL || lane < n_ids;
+        if (have) cv = *reinterpret_cast<const uint4*>(src + kBatchRows * G::kRowBytes + lane * 16);
+        octet_allow_bits(cv, T, rb, have, lo, hi);
+        const uint32_t lo2 = __shfl_down_sync(0xFFFFFFFFu, lo, 1), hi2 = __shfl_down_sync(0xFFFFFFFFu, hi, 1);
+        if (lane == 31) return;  // its bits served lane 30
 #pragma unroll
-    for (int i = 0; i < kBatchRows; ++i) {
-        if (FULL || (i < live && n_act > 0)) {
-            Octet<DT> oc[OPL];
-            float f[8 * OPL];
-            uint32_t bytes = 0;
-#pragma unroll
-            for (int q = 0; q < OPL; ++q) {
-                const uint32_t byte = ((i < 4 ? lo[q] : hi[q]) >> (8 * (i & 3))) & 0xFFu;  // 0 for an octet past the range
-                if (FULL || q < n_act)
-                    oc[q].load_shared_at(src + i * srow + lane_off + q * G::kOctetBytes);
-                else
-                    oc[q].fill_neg_inf();
-                oc[q].mask(byte, f + 8 * q);
-                bytes |= byte << (8 * q);
+        for (int i = 0; i < kBatchRows; ++i) {
+            if (FULL || i < live) {
+                const uint32_t byte = ((i < 4 ? lo : hi) >> (8 * (i & 3))) & 0xFFu;
+                if (vmp[i] && (FULL || 8 * o + 8 <= V)) st_global_u8(vmp[i] + o, byte);
+                const int head = int((heads >> (4 * i)) & 15u);
+                if (FULL || 8 * o + head + 8 <= V) {
+                    const uint32_t next = ((i < 4 ? lo2 : hi2) >> (8 * (i & 3))) & 0xFFu;
+                    Octet<DT> oc;
+                    float f[8];
+                    oc.load_shared_at(src + i * G::kRowBytes + lane_off);
+                    oc.mask(((byte | (next << 8)) >> head) & 0xFFu, f);
+                    oc.store_at(rowp[i] + size_t(o) * G::kOctetBytes, true);  // f32 vectors sit on 32-byte boundaries here
+                    acc[i].add_octet(f, o, scale);
+                }
             }
-            char* zp = CONSEC ? ptr_mad(ba.item_base, i, ba.row_bytes) : rowp[i] + size_t(o) * G::kOctetBytes;
-            char* vp = CONSEC ? (ba.vm_item ? ptr_mad(reinterpret_cast<char*>(ba.vm_item), i, ba.vm_bytes) : nullptr)
-                              : (vmp[i] ? reinterpret_cast<char*>(vmp[i]) + o : nullptr);
-            if (OPL == 1) {
-                oc[0].store_at(zp, wide);
-                if (vp) st_global_u8(vp, bytes);
-            } else {
-                if (both && wide) {
-                    st_stream32(zp, oc[0].raw(), oc[OPL - 1].raw());
+        }
+    } else {
+        uint32_t lo[OPL], hi[OPL];
+#pragma unroll
+        for (int q = 0; q < OPL; ++q) {
+            const bool act = FULL || q < n_act;
+            uint4 cv = make_uint4(0, 0, 0, 0);
+            if (act) cv = *reinterpret_cast<const uint4*>(src + kBatchRows * G::kRowBytes + (lane * OPL + q) * 16);
+            octet_allow_bits(cv, T, rb, act, lo[q], hi[q]);
+        }
+        const bool both = FULL || n_act == OPL;
+#pragma unroll
+        for (int i = 0; i < kBatchRows; ++i) {
+            if (FULL || (i < live && n_act > 0)) {
+                Octet<DT> oc[OPL];
+                float f[8 * OPL];
+                uint32_t bytes = 0;
+#pragma unroll
+                for (int q = 0; q < OPL; ++q) {
+                    const uint32_t byte = ((i < 4 ? lo[q] : hi[q]) >> (8 * (i & 3))) & 0xFFu;  // 0 for an octet past the range
+                    if (FULL || q < n_act)
+                        oc[q].load_shared_at(src + i * srow + lane_off + q * G::kOctetBytes);
+                    else
+                        oc[q].fill_neg_inf();
+                    oc[q].mask(byte, f + 8 * q);
+                    bytes |= byte << (8 * q);
+                }
+                char* zp = CONSEC ? ptr_mad(ba.item_base, i, ba.row_bytes) : rowp[i] + size_t(o) * G::kOctetBytes;
+                char* vp = CONSEC ? (ba.vm_item ? ptr_mad(reinterpret_cast<char*>(ba.vm_item), i, ba.vm_bytes) : nullptr)
+                                  : (vmp[i] ? reinterpret_cast<char*>(vmp[i]) + o : nullptr);
+                if (OPL == 1) {
+                    oc[0].store_at(zp, wide);
+                    if (vp) st_global_u8(vp, bytes);
                 } else {
-                    oc[0].store_at(zp);
-                    if (both) oc[OPL - 1].store_at(zp + G::kOctetBytes);
+                    if (both && wide) {
+                        st_stream32(zp, oc[0].raw(), oc[OPL - 1].raw());
+                    } else {
+                        oc[0].store_at(zp);
+                        if (both) oc[OPL - 1].store_at(zp + G::kOctetBytes);
+                    }
+                    if (vp) {
+                        if (both) st_global_u16(vp, bytes); else st_global_u8(vp, bytes & 0xFFu);
+                    }
                 }
-                if (vp) {
-                    if (both) st_global_u16(vp, bytes); else st_global_u8(vp, bytes & 0xFFu);
-                }
+                acc[i].template add_values<8 * OPL>(f, o, scale);
             }
-            acc[i].template add_values<8 * OPL>(f, o, scale);
         }
     }
 }
 
-// TMAP: the 8 rows of a batch are consecutive rows of the logits matrix and arrive as tiled 2-D copies
+// SRC: kSrcTiled: the 8 rows of a batch are consecutive rows of the logits matrix and arrive as tiled 2-D copies
 // through `tmap` (box = 256 elements x 8 rows: one per chunk, two for a chunk of 512 bf16 tokens);
-// otherwise one bulk copy per row. OPL: octets per lane and row (see PipeGeom).
+// otherwise one bulk copy per row. kSrcShifted: rows that start anywhere (an odd vocabulary packed end to end); their
+// vectors start row_head tokens in, the tokens left over on both sides go through publish_edges. (One token per thread
+// and one block per row took 223 us for 48 rows of 100003 bf16 logits.) OPL: octets per lane and row (see PipeGeom).
 // LBT / MINB: launch bounds (threads per block, blocks per SM) the variant is compiled for; they set
 // the register budget: (512, 1) 128 registers, (384, 1) 168, (320, 2) 96, (256, 3) 80. TEMPERED: the sums
 // are of exp(z / T) with the step's temperature (sampling steps); otherwise T = 1 is compiled in.
-template <int DT, int OPL, bool TMAP, int LBT, int MINB, bool TEMPERED>
+template <int DT, int OPL, int SRC, int LBT, int MINB, bool TEMPERED>
 __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_constant__ StepArgs a,
                                                          const __grid_constant__ CUtensorMap tmap) {
     using G = PipeGeom<DT, OPL>;
+    constexpr bool TMAP = SRC == kSrcTiled, SHIFT = SRC == kSrcShifted;
+    constexpr int kChunkOctets = PipeChunk<OPL, SRC>::kOctets;
+    __shared__ char* s_vec[SHIFT ? kGroupRows : 1];  // first vector of every row of the group
+    __shared__ int s_nvec[SHIFT ? kGroupRows : 1];   // and the number of its whole vectors
     extern __shared__ __align__(128) uint32_t smem[];
     uint32_t* T = smem;
     int* s_row = reinterpret_cast<int*>(T + a.table_words);
@@ -810,6 +930,12 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
         if (TMAP) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap) : "memory");
     }
     const int part = group_rows_setup(a, g, s_row, tid);
+    if (SHIFT && tid < kGroupRows) {  // (the threads that have just set s_row)
+        char* rowp = reinterpret_cast<char*>(a.logits) + int64_t(max(s_row[tid], 0)) * a.row_stride * (DT == kBF16 ? 2 : 4);
+        const int head = row_head<DT>(rowp, a.V);
+        s_vec[tid] = rowp + head * (DT == kBF16 ? 2 : 4);
+        s_nvec[tid] = (a.V - head) >> 3;
+    }
     __syncthreads();
     const PartDev P = a.group_part ? a.parts[part] : a.p0;
     const int nrow = __popc(__ballot_sync(0xFFFFFFFFu, s_row[lane] >= 0));
@@ -832,7 +958,7 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
     // The number of chunks is rarely a multiple of the number of warp slots, so some slots get one chunk more than
     // the others; the deal starts at a different slot for every row batch (rot_chunks further on), which spreads the
     // extra chunks evenly over the warps and the blocks instead of giving the first ones one more in every row batch.
-    const int n_chunks = (n_full + G::kChunkOctets - 1) / G::kChunkOctets;
+    const int n_chunks = (n_full + kChunkOctets - 1) / kChunkOctets;
     const int stride_chunks = TEMPERED ? 1 : a.S * a.WT;  // round-robin: warps that share a row batch of the group
     auto first_chunk_of = [&](int rb) {  // this warp's first chunk of row batch rb
         if (TEMPERED) return (split * a.WT + wt) * a.run_chunks;
@@ -880,10 +1006,24 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
             return;
         }
         slot_info[p_slot] = (p_rb << 24) | chunk;
-        const int o0 = chunk * G::kChunkOctets;
+        const int o0 = chunk * kChunkOctets;
         char* dst = my_ring + size_t(p_slot) * G::kStageBytes;
-        const uint32_t nvec = uint32_t(min(n_full - o0, G::kChunkOctets));  // >= 1: chunk < n_chunks
-        if (TMAP) {
+        const uint32_t nvec = uint32_t(min(n_full - o0, kChunkOctets));  // >= 1: chunk < n_chunks
+        uint32_t n_ids = nvec;
+        if (SHIFT) {
+            n_ids = uint32_t(min(n_octets - o0, 32));  // one octet more than vectors (the class ids are padded to n_octets)
+            const int live = min(kBatchRows, nrow - p_rb * kBatchRows);
+            uint32_t total = n_ids * 16u;
+            for (int i = 0; i < live; ++i)
+                total += uint32_t(max(0, min(s_nvec[p_rb * kBatchRows + i] - o0, kChunkOctets))) * G::kOctetBytes;
+            mbar_expect_tx(bar + p_slot, total);
+            for (int i = 0; i < live; ++i) {
+                const int n = min(s_nvec[p_rb * kBatchRows + i] - o0, kChunkOctets);
+                if (n > 0)
+                    bulk_g2s(dst + i * G::kRowBytes, s_vec[p_rb * kBatchRows + i] + size_t(o0) * G::kOctetBytes,
+                             uint32_t(n) * G::kOctetBytes, bar + p_slot);
+            }
+        } else if (TMAP) {
             // a box holds 32 octets of the 8 rows; the second box of a two-octet chunk is fetched only if the chunk
             // reaches into it (its lanes are idle otherwise); parts of a box past V or past the last row are filled in
             const int nbox = (OPL == 2 && nvec > 32u) ? 2 : 1;
@@ -901,7 +1041,7 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
                          row_bytes, bar + p_slot);
             }
         }
-        bulk_g2s(dst + kBatchRows * G::kRowBytes, reinterpret_cast<const char*>(P.c16) + size_t(o0) * 16, nvec * 16u, bar + p_slot);
+        bulk_g2s(dst + kBatchRows * G::kRowBytes, reinterpret_cast<const char*>(P.c16) + size_t(o0) * 16, n_ids * 16u, bar + p_slot);
         ++p_issued;
         if (++p_slot == depth) p_slot = 0;
     };
@@ -919,9 +1059,14 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
         const int live0 = min(kBatchRows, nrow - wr * kBatchRows);
         int chunk = first_chunk_of(wr);
         for (int d = 0; d < a.prefetch_items && chunk < chunk_end; ++d, chunk += TEMPERED ? 1 : stride_chunks) {
-            const int o0 = chunk * G::kChunkOctets;
-            const uint32_t nvec = uint32_t(min(n_full - o0, G::kChunkOctets));
-            if (TMAP) {
+            const int o0 = chunk * kChunkOctets;
+            const uint32_t nvec = uint32_t(min(n_full - o0, kChunkOctets));
+            if (SHIFT) {
+                for (int i = 0; i < live0; ++i) {
+                    const int n = min(s_nvec[wr * kBatchRows + i] - o0, kChunkOctets);
+                    if (n > 0) bulk_prefetch(s_vec[wr * kBatchRows + i] + size_t(o0) * G::kOctetBytes, uint32_t(n) * G::kOctetBytes);
+                }
+            } else if (TMAP) {
                 tma_prefetch_2d(&tmap, o0 * 8, row0);
                 if (OPL == 2 && nvec > 32u) tma_prefetch_2d(&tmap, o0 * 8 + 256, row0);
             } else {
@@ -990,7 +1135,11 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
     Partial* const s_state = (!TEMPERED && a.fold_off) ? reinterpret_cast<Partial*>(reinterpret_cast<char*>(smem) + a.fold_off) : nullptr;
     Partial* const pub_base = s_state ? s_state : row_slots(a, g, 0);
     const int pub_stride = s_state ? a.WT + 1 : a.slots;
-    const int my_slot = s_state ? wt : split * a.WT + wt;
+    const int my_slot = s_state ? wt : split * a.WT + wt + (SHIFT ? a.head_state : 0);
+    // What the vectors leave over, while the first copies are on their way
+    publish_edges<DT, SHIFT>(
+        a, P, T, s_row, nrow, split, warp, lane, scale, SHIFT && a.head_state != 0, [&](int j) { return row_slots(a, g, j); },
+        [&](int j) { return pub_base + j * pub_stride + (s_state ? a.WT : a.slots - 1); });
     // where this lane's octets of a row sit inside a stage: two tiled copies leave two boxes of 8 rows x 32 octets
     // behind one another, anything else whole rows of the chunk
     const uint32_t lane_off = (TMAP && OPL == 2) ? uint32_t(lane >> 4) * G::kBoxBytes + uint32_t(lane & 15) * 2u * G::kOctetBytes
@@ -1005,7 +1154,9 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
     char* base0 = nullptr;
     uint8_t* vm0 = nullptr;
     int live = 0;
+    uint32_t heads = 0u;  // SHIFT: tokens in front of the first vector of the batch's rows, four bits each
     auto open_batch = [&](int rb) {  // fresh row states and row addresses for row batch rb
+        if (SHIFT) heads = 0u;
 #pragma unroll
         for (int i = 0; i < kBatchRows; ++i) {
             acc[i].init();
@@ -1015,6 +1166,11 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
                 const int row = s_row[min(rb * kBatchRows + i, kGroupRows - 1)];
                 rowp[i] = reinterpret_cast<char*>(a.logits) + int64_t(max(row, 0)) * a.row_stride * ES;
                 vmp[i] = vm8 ? vm8 + int64_t(max(row, 0)) * a.vm_stride * 4 : nullptr;
+                if (SHIFT) {
+                    const int head = row_head<DT>(rowp[i], a.V);
+                    rowp[i] += head * ES;
+                    heads |= uint32_t(head) << (4 * i);
+                }
             }
         }
         live = min(kBatchRows, nrow - rb * kBatchRows);
@@ -1028,7 +1184,7 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
     while (cur_rb * kBatchRows < nrow) {
         const int info = slot_info[slot];
         if (info < 0) break;
-        const int rb = info >> 24, o0 = (info & 0xFFFFFF) * G::kChunkOctets;
+        const int rb = info >> 24, o0 = (info & 0xFFFFFF) * kChunkOctets;
         while (cur_rb < rb) {  // the previous row batch of this warp is complete (possibly without any chunk)
             warp_rows_publish_to(acc, live, cur_rb, lane, scale, pub_base, pub_stride, my_slot);
             cur_rb += WR;
@@ -1045,12 +1201,13 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
         const int o = o0 + lane * OPL;
         ba.item_base = base0 + size_t(o) * G::kOctetBytes;
         ba.vm_item = vm0 ? vm0 + o : nullptr;
-        if (live == kBatchRows && o0 + G::kChunkOctets <= n_full)
-            pipe_consume_item<DT, OPL, true, TMAP>(src, lane_off, srow, T, rb, live, OPL, o, lane, ba, rowp, vmp, acc, scale,
-                                                   a.wide != 0);
+        // (the vectors of a row that starts anywhere end at most one octet before the last whole octet)
+        if (live == kBatchRows && o0 + kChunkOctets <= (SHIFT ? n_full - 1 : n_full))
+            pipe_consume_item<DT, OPL, true, SRC>(src, lane_off, srow, T, rb, live, OPL, o, lane, ba, rowp, vmp, acc, scale,
+                                                  a.wide != 0, 32, heads, a.V);
         else
-            pipe_consume_item<DT, OPL, false, TMAP>(src, lane_off, srow, T, rb, live, max(0, min(OPL, n_full - o)), o, lane, ba,
-                                                    rowp, vmp, acc, scale, a.wide != 0);
+            pipe_consume_item<DT, OPL, false, SRC>(src, lane_off, srow, T, rb, live, max(0, min(OPL, n_full - o)), o, lane, ba,
+                                                   rowp, vmp, acc, scale, a.wide != 0, min(n_octets - o0, 32), heads, a.V);
         ++consumed;
         if (++slot == depth) { slot = 0; phase ^= 1u; }
         __syncwarp();  // every lane has its data out of the slot before it is refilled
@@ -1072,16 +1229,13 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
             if (++slot == depth) { slot = 0; phase ^= 1u; }
         }
     }
-    // the block that reaches the end of the vocabulary takes the octets past the last whole vector
-    if (warp == 0 && split == 0)
-        publish_tail_octets_to<DT>(a, P, s_row, lane, n_full, n_octets, scale, pub_base, pub_stride, s_state ? a.WT : a.slots - 1);
     if (!fold && !s_state) return;
     __shared__ int s_last;
     if (s_state) {
         // first the block's own states: one per row and block goes out instead of one per row and warp
         __syncthreads();
         for (int j = warp; j < nrow; j += n_warps) {
-            const int n_mine = a.WT + (split == 0 ? 1 : 0);  // only the block that owns the end of the vocabulary has a tail state
+            const int n_mine = a.WT + (j % a.S == split ? 1 : 0);  // the state of what the vectors left over
             float m = -INFINITY, s = 0.f;
             int pos = kNoPos;
             if (lane < n_mine) {
@@ -1597,20 +1751,25 @@ __global__ void __launch_bounds__(kSampleThreads) k_sample_rows(const __grid_con
     float base = s_base;
 
     // the tokens the chosen state stands for
-    const int n_full8 = (a.V >> 3) << 3;
-    int t_lo, t_hi;
-    if (a.tail_state && pick == n_states - 1) {
-        t_lo = n_full8;
-        t_hi = a.V;
-    } else {
-        const long long lim = a.tail_state ? n_full8 : a.V;
-        t_lo = int(min(static_cast<long long>(pick) * a.run_chunks * a.chunk_tokens, lim));
-        t_hi = int(min(static_cast<long long>(pick + 1) * a.run_chunks * a.chunk_tokens, lim));
-    }
     constexpr int ES = DT == kBF16 ? 2 : 4;
     const char* rowp = reinterpret_cast<const char*>(a.logits) + int64_t(row) * a.row_stride * ES;
+    const int head = a.shifted ? row_head<DT>(rowp, a.V) : 0;
+    const int vec_end = head + ((a.V - head) & ~7);  // first token past the last whole vector
+    int t_lo, t_hi;
+    if (a.tail_state && pick == n_states - 1) {
+        t_lo = vec_end;
+        t_hi = a.V;
+    } else if (a.head_state && pick == 0) {
+        t_lo = 0;
+        t_hi = head;
+    } else {
+        const long long lim = a.tail_state ? vec_end : a.V, run_tokens = static_cast<long long>(a.run_chunks) * a.chunk_tokens;
+        const long long first = head + (pick - a.head_state) * run_tokens;
+        t_lo = int(min(first, lim));
+        t_hi = int(min(first + run_tokens, lim));
+    }
     auto load8 = [&](int t0, float (&e)[8]) {
-        if (aligned && t0 + 8 <= t_hi) {  // t_lo is a multiple of 8 tokens: 16-byte (bf16) / 32-byte (f32) vectors
+        if (aligned && t0 + 8 <= t_hi) {  // t_lo is on a vector boundary: 16-byte (bf16) / 32-byte (f32) vectors
             if (DT == kBF16) {
                 const uint4 v = __ldcg(reinterpret_cast<const uint4*>(rowp + size_t(t0) * 2));
                 e[0] = __uint_as_float(v.x << 16); e[1] = __uint_as_float(v.x & 0xFFFF0000u);
@@ -1783,10 +1942,10 @@ __device__ __forceinline__ unsigned long long block_exclusive_scan_u64(unsigned 
     return before + inc - v;
 }
 
-// Eight consecutive logits of a row from token t0 on (-inf past `end`), as floats.
+// Eight consecutive logits of a row from token t0 on (-inf in front of token 0 and past `end`), as floats.
 template <int DT>
 __device__ __forceinline__ void load_eight(const char* rowp, int t0, int end, bool aligned, float (&e)[8]) {
-    if (aligned && t0 + 8 <= end) {
+    if (aligned && t0 >= 0 && t0 + 8 <= end) {
         if (DT == kBF16) {
             const uint4 v = __ldcg(reinterpret_cast<const uint4*>(rowp + size_t(t0) * 2));
             e[0] = __uint_as_float(v.x << 16); e[1] = __uint_as_float(v.x & 0xFFFF0000u);
@@ -1801,16 +1960,16 @@ __device__ __forceinline__ void load_eight(const char* rowp, int t0, int end, bo
         }
     } else {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) e[q] = t0 + q < end ? ldcg_elem<DT>(rowp, t0 + q) : -INFINITY;
+        for (int q = 0; q < 8; ++q) e[q] = t0 + q >= 0 && t0 + q < end ? ldcg_elem<DT>(rowp, t0 + q) : -INFINITY;
     }
 }
 
 // Visit every token of a row, the block's threads side by side (8 consecutive tokens per thread and round, four
 // rounds in flight together).
 template <int DT, typename F>
-__device__ __forceinline__ void row_visit(const char* rowp, int V, bool aligned, F&& f) {
+__device__ __forceinline__ void row_visit(const char* rowp, int lead, int V, bool aligned, F&& f) {
     constexpr int kInFlight = 4;
-    for (int t0 = threadIdx.x * 8; t0 < V; t0 += kFiltThreads * 8 * kInFlight) {
+    for (int t0 = int(threadIdx.x) * 8 - lead; t0 < V; t0 += kFiltThreads * 8 * kInFlight) {
         float e[kInFlight][8];
 #pragma unroll
         for (int r = 0; r < kInFlight; ++r) load_eight<DT>(rowp, t0 + r * kFiltThreads * 8, V, aligned, e[r]);
@@ -2090,6 +2249,9 @@ __global__ void __launch_bounds__(kFiltThreads) k_sample_filtered(const __grid_c
     }
     constexpr int ES = DT == kBF16 ? 2 : 4;
     const char* rowp = reinterpret_cast<const char*>(a.logits) + int64_t(row) * a.row_stride * ES;
+    // Rows are gone over eight tokens at a time from token -lead on, so that the eight are one vector of the row: a row
+    // that starts anywhere has `head` tokens in front of its first vector.
+    const int head = a.shifted ? row_head<DT>(rowp, a.V) : 0, lead = (8 - head) & 7;
     const float scale = a.scale;
     const uint32_t key_max = logit_key<DT>(M);
     // The candidates are the tokens at or above M - 41 / scale (below M - 40 / scale the fixed-point weight is zero;
@@ -2105,8 +2267,8 @@ __global__ void __launch_bounds__(kFiltThreads) k_sample_filtered(const __grid_c
     int attempt = 0;
     {
         const uint32_t list_key0 = peer_shared(l_key, 0u), list_id0 = peer_shared(l_id, 0u);
-        const int share = ((a.V + int(n_peers) - 1) / int(n_peers) + 7) & ~7;
-        const int t_begin = min(int(crank) * share, a.V), t_end = min(t_begin + share, a.V);
+        const int share = ((a.V + lead + int(n_peers) - 1) / int(n_peers) + 7) & ~7;
+        const int t_begin = min(int(crank) * share - lead, a.V), t_end = min(t_begin + share, a.V);
         constexpr int kInFlight = 4;
         float units = 41.f;
         cluster_barrier();  // the first block's counters are cleared before anybody adds to them
@@ -2351,7 +2513,7 @@ __global__ void __launch_bounds__(kFiltThreads) k_sample_filtered(const __grid_c
     m = 0xFFFFFFFFu;
     auto above = [&](uint32_t lo) {  // (count, weight) of the tokens with key >= lo
         CountMass v{0u, 0ull};
-        row_visit<DT>(rowp, a.V, aligned != 0, [&](int, float z) {
+        row_visit<DT>(rowp, lead, a.V, aligned != 0, [&](int, float z) {
             if (logit_key<DT>(z) >= lo) {
                 v.n += 1u;
                 v.w += fixed_weight(z, M, scale);
@@ -2404,8 +2566,8 @@ __global__ void __launch_bounds__(kFiltThreads) k_sample_filtered(const __grid_c
     // Draw in token order. Every thread owns one contiguous segment of the row: first the ties per segment (their
     // rank decides which of them are kept), then the kept weight per segment, then the one thread whose segment
     // holds the crossing walks it once more.
-    const int seg = ((a.V + kFiltThreads - 1) / kFiltThreads + 7) & ~7;
-    const int t_lo = min(tid * seg, a.V), t_hi = min(t_lo + seg, a.V);
+    const int seg = ((a.V + lead + kFiltThreads - 1) / kFiltThreads + 7) & ~7;
+    const int t_lo = min(tid * seg - lead, a.V), t_hi = min(t_lo + seg, a.V);
     auto seg_visit = [&](auto&& f) {
         for (int t0 = t_lo; t0 < t_hi; t0 += 32) {
             float e[4][8];

@@ -1,0 +1,97 @@
+"""Rows that do not start on a vector boundary (an odd vocabulary packed end to end, a view into a larger buffer): the
+streaming kernel's shifted variant and the sampling kernels behind it, against the CPU oracle."""
+import numpy as np
+import pytest
+import torch
+
+import synth
+from synth import rng
+from paper_2605_29986_b200 import binding as cz
+from _gpu_util import Ctx, compare_step, dev, dtype_code, host, oracle_step, run_fused
+from test_gpu_sample import check_sample, run_sample
+from test_gpu_sample_filtered import check_filtered, run_filtered
+
+pytestmark = pytest.mark.gpu
+
+
+def inputs(V, K, B, dtype, tag, stride=None, p=0.3, sigma=2.0):
+    part = synth.zipf_partition(V, K, seed=tag)
+    cm = synth.class_mask_bernoulli(K, B, p, rng.stream_key(rng.SEED_BASE, 901, tag, V))
+    z = synth.logits_normal(B, stride or V, sigma, dtype, (902, tag, V))
+    return part, cm, z
+
+
+# one octet and less, the edges of a chunk of 31 vectors, tails of every length, rows enough for several groups
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("V,B", [(1, 3), (7, 9), (9, 8), (17, 33), (247, 8), (249, 40), (255, 17), (257, 31), (505, 8),
+                                 (10001, 70), (20002, 1), (20003, 5), (20005, 32), (20007, 65), (70009, 33)])
+def test_greedy(V, B, dtype):
+    K = max(1, min(300, V // 2))
+    part, cm, z = inputs(V, K, B, dtype, 1)
+    with Ctx([part]) as ctx:
+        compare_step(run_fused(ctx, None, cm, z, V), oracle_step([part], None, cm, z, V), V, "V=%d B=%d" % (V, B))
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("offset", [1, 3, 6, 7])
+def test_view_into_a_buffer(offset, dtype):
+    V, K, B, stride = 3001, 90, 11, 3010
+    part, cm, z = inputs(V, K, B, dtype, 2, stride)
+    want = oracle_step([part], None, cm, z, V)
+    flat = np.zeros(offset + B * stride + 8, dtype=z.dtype)
+    flat[offset:offset + B * stride] = z.reshape(-1)
+    with Ctx([part]) as ctx:
+        d, d_cm, es = dev(flat), dev(cm), z.dtype.itemsize
+        VW = (V + 31) // 32
+        d_vm, d_am = torch.zeros((B, VW), dtype=torch.int32, device="cuda"), torch.zeros(B, dtype=torch.int32, device="cuda")
+        d_rep, d_lse, d_lpa = torch.zeros_like(d_am), torch.zeros(B, device="cuda"), torch.zeros(B, device="cuda")
+        cz.cfgzip_masked_logsoftmax_argmax(ctx.h, ctx.ids[0], None, d_cm, cm.shape[1], d.data_ptr() + offset * es, dtype_code(z),
+                                           stride, B, d_vm, VW, d_am, d_rep, d_lpa, d_lse)
+        torch.cuda.synchronize()
+        back = host(d, z.dtype)
+        rows = back[offset:offset + B * stride].reshape(B, stride)
+        compare_step(dict(logits=rows, vocab_mask=host(d_vm, np.uint32), argmax=d_am.cpu().numpy(), rep=d_rep.cpu().numpy(),
+                          lse=d_lse.cpu().numpy(), logp_argmax=d_lpa.cpu().numpy()), want, V)
+        assert np.array_equal(rows[:, V:], z[:, V:]) and not back[:offset].any() and not back[offset + B * stride:].any()
+
+
+def test_ties_and_maxima_at_the_edges():
+    V, K, B = 2005, 40, 16
+    part, cm, z = inputs(V, K, B, "f32", 3)
+    cm[:] = 0xFFFFFFFF
+    for b in range(B):  # equal maxima in front of, inside and behind the vectors of the row
+        z[b, [(b % 9), 8 * b + 5, V - 1 - (b % 7)]] = 50.0
+    with Ctx([part]) as ctx:
+        compare_step(run_fused(ctx, None, cm, z, V), oracle_step([part], None, cm, z, V), V)
+
+
+def test_mixed_partitions():
+    V, B = 9001, 77
+    parts = [synth.zipf_partition(V, k, seed=i) for i, k in enumerate((50, 333, 700))]
+    row_part = (np.arange(B) * 7 % 3).astype(np.int32)
+    cm = synth.class_mask_bernoulli(700, B, 0.2, rng.stream_key(rng.SEED_BASE, 903))
+    z = synth.logits_normal(B, V, 2.0, "bf16", (904,))
+    with Ctx(parts) as ctx:
+        compare_step(run_fused(ctx, row_part, cm, z, V), oracle_step(parts, row_part, cm, z, V), V)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("V,B", [(7, 4), (249, 9), (5003, 33), (40001, 40)])
+def test_sampling(V, B, dtype):
+    part, cm, z = inputs(V, max(1, min(200, V // 3)), B, dtype, 5)
+    for n, fill in enumerate((0.0, 0.37, 0.999999)):
+        u = np.full(B, fill, dtype=np.float32) if n != 1 else np.linspace(0, 0.99, B, dtype=np.float32)
+        with Ctx([part]) as ctx:
+            got = run_sample(ctx, None, cm, z, V, u, 1.25)
+            check_sample(got, [part], None, cm, z, V, u, 1.25, "V=%d" % V)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("V,B,inv_t,top_k,top_p", [(7, 4, 1.0, 3, 0.9), (249, 9, 5.0, 20, 1.0), (5003, 33, 1.0, 0, 0.9),
+                                                   (40001, 40, 1.0, 0, 0.95), (40001, 80, 5.0, 50, 0.9)])
+def test_filtered_sampling(V, B, inv_t, top_k, top_p, dtype):
+    part, cm, z = inputs(V, max(1, min(200, V // 3)), B, dtype, 6)
+    u = np.linspace(0, 0.99, B, dtype=np.float32)
+    with Ctx([part]) as ctx:
+        got = run_filtered(ctx, None, cm, z, V, u, inv_t, top_k, top_p)
+        check_filtered(got, [part], None, cm, z, V, u, inv_t, top_k, top_p, "V=%d" % V)
