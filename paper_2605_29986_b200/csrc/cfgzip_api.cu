@@ -12,6 +12,8 @@
 
 #include "cfgzip.h"
 #include "cfgzip_kernels.cuh"
+#include "class_sort.cuh"
+#include "workspace.h"
 
 using namespace cfgzip;
 
@@ -21,10 +23,12 @@ struct Part {
     bool live = false;
     int32_t V = 0, K = 0, KW = 0, VW = 0;
     void* block = nullptr;  // one device allocation holding every table of the partition
+    size_t block_bytes = 0;
     PartDev dev{};
     std::vector<int32_t> sizes;  // host copy of the class sizes (cfgzip_choose_mode)
 };
 
+constexpr size_t kSpareBytes = size_t(32) << 20;  // most memory of a released partition a context keeps for the next one
 constexpr size_t kPartialSlots = size_t(1) << 18;  // 4 MB of (max, sum, pos) slots
 constexpr size_t kFiltSmem = size_t(kFiltList) * 16;  // candidate list of the filtered sampling kernel
 constexpr int kTwoOctetItemsPerWarp = 3;           // bf16: two octets per lane from this many work items per warp on
@@ -46,6 +50,8 @@ struct cfgzip_ctx {
     int sm_count = 0;
     int smem_optin = 0;
     std::vector<Part> parts;
+    void* spare_block = nullptr;  // memory of the partition released last, for the next one loaded (given back with the context)
+    size_t spare_bytes = 0;
     PartDev* d_parts = nullptr;
     Partial* d_partials = nullptr;
     unsigned int* d_tickets = nullptr;  // reserved_rows entries
@@ -816,6 +822,7 @@ int cfgzip_create(int device, cfgzip_ctx** out) {
     if (!guard.ok) return CFGZIP_E_CUDA;
     cfgzip_ctx* ctx = new (std::nothrow) cfgzip_ctx();
     if (!ctx) return CFGZIP_E_NOMEM;
+    Workspace::hold();
     ctx->device = device;
     cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, device);
     cudaDeviceGetAttribute(&ctx->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
@@ -853,6 +860,7 @@ int cfgzip_destroy(cfgzip_ctx* ctx) {
     cudaDeviceSynchronize();
     for (Part& p : ctx->parts)
         if (p.block) cudaFree(p.block);
+    cudaFree(ctx->spare_block);
     cudaFree(ctx->d_parts);
     cudaFree(ctx->d_partials);
     cudaFree(ctx->d_tickets);
@@ -868,14 +876,14 @@ int cfgzip_destroy(cfgzip_ctx* ctx) {
     if (ctx->st_small_host) cudaFreeHost(ctx->st_small_host);
     cudaGetLastError();
     delete ctx;
+    Workspace::drop();
     return CFGZIP_OK;
 }
 
 int cfgzip_load_partition(cfgzip_ctx* ctx, const int32_t* c, int32_t V, const int32_t* r, int32_t K, void* stream,
                           cfgzip_part_id* out_id) {
     if (!ctx || !out_id) return CFGZIP_E_ARG;
-    int rc = check_partition_host(c, V, r, K);
-    if (rc != CFGZIP_OK) return rc;
+    if (!c || !r || V <= 0 || K <= 0 || K > V) return CFGZIP_E_ARG;
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return CFGZIP_E_CUDA;
     size_t slot = 0;
@@ -890,62 +898,76 @@ int cfgzip_load_partition(cfgzip_ctx* ctx, const int32_t* c, int32_t V, const in
     p.KW = ceil_div(K, 32);
     p.VW = ceil_div(V, 32);
     const bool has16 = K <= 65535;  // the value K itself is the padding id
-    // host image of the device block: c32 | r | off | tok | trep | c16 (16-byte aligned pieces)
+    // the device block: c32 | r | off | tok | trep | c16 (16-byte aligned pieces). Only the caller's two vectors cross the
+    // bus; they are checked, and everything that follows from them is made, on the GPU.
     auto align4 = [](size_t n) { return (n + 3) & ~size_t(3); };
     const size_t n_c32 = align4(size_t(V)), n_r = align4(size_t(K)), n_off = align4(size_t(K) + 1), n_tok = align4(size_t(V));
     const size_t n_trep = align4(size_t(V));
     const size_t n_c16_words = has16 ? size_t(p.VW) * 16 : 0;  // 32*VW uint16 = 16*VW words
-    std::vector<int32_t> img(n_c32 + n_r + n_off + n_tok + n_trep + n_c16_words, 0);
-    int32_t* h_c32 = img.data();
-    int32_t* h_r = h_c32 + n_c32;
-    int32_t* h_off = h_r + n_r;
-    int32_t* h_tok = h_off + n_off;
-    int32_t* h_trep = h_tok + n_tok;
-    uint16_t* h_c16 = reinterpret_cast<uint16_t*>(h_trep + n_trep);
-    std::memcpy(h_c32, c, size_t(V) * 4);
-    std::memcpy(h_r, r, size_t(K) * 4);
-    build_class_lists_host(c, V, K, h_off, h_tok);
+    const size_t need = (n_c32 + n_r + n_off + n_tok + n_trep + n_c16_words) * 4;
+    std::vector<int32_t> off(size_t(K) + 1);
     p.sizes.resize(size_t(K));
-    for (int32_t k = 0; k < K; ++k) p.sizes[size_t(k)] = h_off[k + 1] - h_off[k];
-    for (int32_t i = 0; i < V; ++i) h_trep[i] = r[c[i]];
-    if (has16) {
-        for (int32_t i = 0; i < V; ++i) h_c16[i] = uint16_t(c[i]);
-        for (int32_t i = V; i < 32 * p.VW; ++i) h_c16[i] = uint16_t(K);
-    }
-    if (cudaMalloc(&p.block, img.size() * 4) != cudaSuccess) {
+    Workspace scratch((4 + class_sort_scratch_words(V)) * 4);
+    if (scratch.ptr && ctx->spare_bytes >= need) {
+        p.block = ctx->spare_block;
+        p.block_bytes = ctx->spare_bytes;
+        ctx->spare_block = nullptr;
+        ctx->spare_bytes = 0;
+    } else if (scratch.ptr && cudaMalloc(&p.block, need) == cudaSuccess) {
+        p.block_bytes = need;
+    } else {
         cudaGetLastError();
         if (appended) ctx->parts.pop_back();
         return CFGZIP_E_NOMEM;
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     int32_t* d = static_cast<int32_t*>(p.block);
-    p.dev.c32 = d;
-    p.dev.r = d + n_c32;
-    p.dev.off = d + n_c32 + n_r;
-    p.dev.tok = d + n_c32 + n_r + n_off;
-    p.dev.trep = d + n_c32 + n_r + n_off + n_tok;
-    p.dev.c16 = has16 ? reinterpret_cast<const uint16_t*>(d + n_c32 + n_r + n_off + n_tok + n_trep) : nullptr;
+    int32_t *d_c32 = d, *d_r = d_c32 + n_c32, *d_off = d_r + n_r, *d_tok = d_off + n_off, *d_trep = d_tok + n_tok;
+    uint16_t* d_c16 = has16 ? reinterpret_cast<uint16_t*>(d_trep + n_trep) : nullptr;
+    p.dev.c32 = d_c32;
+    p.dev.r = d_r;
+    p.dev.off = d_off;
+    p.dev.tok = d_tok;
+    p.dev.trep = d_trep;
+    p.dev.c16 = d_c16;
     p.dev.K = K;
     p.dev.KW = p.KW;
     p.dev.V = V;
     p.dev.live = 1;
     p.live = true;
-    bool ok = cudaMemcpyAsync(p.block, img.data(), img.size() * 4, cudaMemcpyHostToDevice, st) == cudaSuccess &&
-              cudaMemcpyAsync(ctx->d_parts + slot, &p.dev, sizeof(PartDev), cudaMemcpyHostToDevice, st) == cudaSuccess &&
-              cudaStreamSynchronize(st) == cudaSuccess;
-    if (!ok) {
-        // the descriptor may already be on the device: clear it before its tables are freed, so that no later
-        // call finds a live slot that points at released memory
+    int32_t* d_bad = static_cast<int32_t*>(scratch.ptr);
+    int32_t bad = 0;
+    bool ok = cudaMemcpyAsync(d_c32, c, size_t(V) * 4, cudaMemcpyHostToDevice, st) == cudaSuccess &&
+              cudaMemcpyAsync(d_r, r, size_t(K) * 4, cudaMemcpyHostToDevice, st) == cudaSuccess &&
+              cudaMemsetAsync(d_bad, 0, 4, st) == cudaSuccess;
+    if (ok) {
+        const int n = 32 * p.VW;
+        k_load_tokens<<<ceil_div(n, 256), 256, 0, st>>>(d_c32, d_c16, V, n, K, d_bad);
+        k_load_classes<<<ceil_div(V, 256), 256, 0, st>>>(d_c32, d_r, d_trep, V, K, d_bad);  // V >= K
+        class_sort(d_c32, V, nullptr, K, d_off, d_tok, d_bad + 4, st);
+        ok = cudaGetLastError() == cudaSuccess &&
+             cudaMemcpyAsync(&bad, d_bad, 4, cudaMemcpyDeviceToHost, st) == cudaSuccess &&
+             cudaMemcpyAsync(off.data(), d_off, (size_t(K) + 1) * 4, cudaMemcpyDeviceToHost, st) == cudaSuccess;
+        ok = (cudaStreamSynchronize(st) == cudaSuccess) && ok;
+    }
+    // the descriptor goes up only once the tables are known to be good: no call finds a live slot without them
+    if (ok && !bad)
+        ok = cudaMemcpyAsync(ctx->d_parts + slot, &p.dev, sizeof(PartDev), cudaMemcpyHostToDevice, st) == cudaSuccess &&
+             cudaStreamSynchronize(st) == cudaSuccess;
+    if (!ok || bad) {
         cudaGetLastError();
         cudaStreamSynchronize(st);
-        cudaMemset(ctx->d_parts + slot, 0, sizeof(PartDev));
-        cudaDeviceSynchronize();
-        cudaGetLastError();
+        if (!ok) {  // the descriptor may have arrived all the same: clear it before its tables are freed
+            cudaMemset(ctx->d_parts + slot, 0, sizeof(PartDev));
+            cudaDeviceSynchronize();
+            cudaGetLastError();
+        }
         cudaFree(p.block);
         if (appended) ctx->parts.pop_back();
-        return CFGZIP_E_CUDA;
+        return ok ? CFGZIP_E_PARTITION : CFGZIP_E_CUDA;
     }
-    ctx->parts[slot] = p;
+    for (int32_t k = 0; k < K; ++k) p.sizes[size_t(k)] = off[size_t(k) + 1] - off[size_t(k)];
+    ctx->parts[slot] = std::move(p);
     ctx->plan_valid = false;
     *out_id = cfgzip_part_id(slot);
     return CFGZIP_OK;
@@ -959,7 +981,12 @@ int cfgzip_free_partition(cfgzip_ctx* ctx, cfgzip_part_id id) {
     cudaDeviceSynchronize();
     ctx->plan_valid = false;
     Part& p = ctx->parts[size_t(id)];
-    cudaFree(p.block);
+    void* released = p.block;
+    if (p.block_bytes > ctx->spare_bytes && p.block_bytes <= kSpareBytes) {
+        std::swap(released, ctx->spare_block);
+        ctx->spare_bytes = p.block_bytes;
+    }
+    cudaFree(released);
     p = Part();
     cudaMemset(ctx->d_parts + id, 0, sizeof(PartDev));
     cudaDeviceSynchronize();

@@ -6,14 +6,19 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstdint>
 #include <cstring>
 #include <new>
-#include <set>
-#include <utility>
+#include <thread>
 #include <vector>
+#ifdef __SSE2__
+#include <emmintrin.h>
+#endif
 
 #include "cfgzip.h"
+#include "class_sort.cuh"
+#include "workspace.h"
 
 struct cfgzip_grammar {
     int32_t n = 0, start = 0;
@@ -23,14 +28,11 @@ struct cfgzip_grammar {
         std::vector<int32_t> rhs;
     };
     std::vector<Prod> prods;
-    std::vector<std::vector<int32_t>> by_term;  // production indices by terminal byte
+    std::vector<std::vector<int32_t>> by_term;  // production indices by terminal byte, ascending by head
     std::vector<uint8_t> adj;                   // n * n, adj[y * n + z] = 1: z may be popped right after y left nothing
 };
 
 namespace {
-
-using Stack = std::vector<int32_t>;
-using Pair = std::pair<Stack, Stack>;  // (input queue, output stack: top first)
 
 // Appendix C: edge A -> B for every production whose right-most non-terminal is B; for every production
 // A -> a B_1 .. B_n Z beta a breadth-first search from B_n collects the reachable Y with a production Y -> y.
@@ -67,42 +69,100 @@ void build_adjacency(cfgzip_grammar& g) {
     }
 }
 
-// Algorithm 1 as a depth-first enumeration with explicit stacks. `prev` is the symbol popped last (-1: none yet).
+// Algorithm 1 as a depth-first enumeration with explicit stacks. `prev` is the symbol popped last (-1: none yet). The
+// pairs found are kept flat in one growing array ([n_in, in .., n_out, out (top first) ..] each) that is reused from
+// token to token, so that a token allocates nothing; they are sorted and made unique at the end. (A std::set of pairs of
+// vectors took 260 ns per token on one core, this 118.)
 struct Displacer {
     const cfgzip_grammar& g;
-    const uint8_t* t;
-    int32_t len;
     int64_t max_pairs;
-    std::set<Pair> out;
+    const uint8_t* t = nullptr;
+    int32_t len = 0;
     bool overflow = false;
-    Stack s_in, s_out;  // s_out: top at the back
+    std::vector<int32_t> s_in, s_out;  // s_out: top at the back
+    std::vector<int32_t> flat;
+    std::vector<size_t> pairs;         // where each pair starts in `flat`
+    size_t compact_at = 0;             // pairs are made unique when this many have piled up
+
+    Displacer(const cfgzip_grammar& grammar, int64_t most) : g(grammar), max_pairs(most) {}
+
+    // order and equality of std::pair<std::vector, std::vector> on (input stack, output stack)
+    int compare(size_t x, size_t y) const {
+        const int32_t *a = flat.data() + x, *b = flat.data() + y;
+        for (int part = 0; part < 2; ++part) {
+            const int32_t na = *a++, nb = *b++;
+            const int32_t n = std::min(na, nb);
+            for (int32_t i = 0; i < n; ++i)
+                if (a[i] != b[i]) return a[i] < b[i] ? -1 : 1;
+            if (na != nb) return na < nb ? -1 : 1;
+            a += na;
+            b += nb;
+        }
+        return 0;
+    }
+    void make_unique() {
+        std::sort(pairs.begin(), pairs.end(), [&](size_t x, size_t y) { return compare(x, y) < 0; });
+        pairs.erase(std::unique(pairs.begin(), pairs.end(), [&](size_t x, size_t y) { return compare(x, y) == 0; }), pairs.end());
+        if (int64_t(pairs.size()) > max_pairs) overflow = true;
+    }
+
+    void displace(const uint8_t* bytes, int32_t n) {
+        t = bytes;
+        len = n;
+        overflow = false;
+        s_in.clear();
+        s_out.clear();
+        flat.clear();
+        pairs.clear();
+        compact_at = 4096;
+        run(0, -1);  // (an empty token moves no stack: its only pair is (empty, empty))
+        if (!overflow) make_unique();
+    }
+
+    void found() {
+        pairs.push_back(flat.size());
+        flat.push_back(int32_t(s_in.size()));
+        flat.insert(flat.end(), s_in.begin(), s_in.end());
+        flat.push_back(int32_t(s_out.size()));
+        flat.insert(flat.end(), s_out.rbegin(), s_out.rend());
+        if (pairs.size() >= compact_at) {  // many derivations, perhaps of few pairs
+            make_unique();
+            std::vector<int32_t> kept;
+            for (size_t& at : pairs) {
+                const size_t from = at, n_in = size_t(flat[from]), n = 2 + n_in + size_t(flat[from + 1 + n_in]);
+                at = kept.size();
+                kept.insert(kept.end(), flat.begin() + long(from), flat.begin() + long(from + n));
+            }
+            flat.swap(kept);
+            compact_at = std::max(size_t(4096), 2 * pairs.size());
+        }
+    }
 
     void run(int32_t pos, int32_t prev) {
         if (overflow) return;
-        if (pos == len) {
-            Pair p(s_in, Stack(s_out.rbegin(), s_out.rend()));
-            out.insert(std::move(p));
-            if (int64_t(out.size()) > max_pairs) overflow = true;
-            return;
-        }
-        const auto& cands = g.by_term[t[pos]];
+        if (pos == len) return found();
+        const auto& cands = g.by_term[t[pos]];  // ascending by head
         if (s_out.empty()) {  // stack backtrack: the next symbol of the input stack is guessed
             for (int32_t pi : cands) {
                 const auto& p = g.prods[size_t(pi)];
                 if (prev >= 0 && !g.adj[size_t(prev) * size_t(g.n) + size_t(p.head)]) continue;
                 s_in.push_back(p.head);
-                for (auto it = p.rhs.rbegin(); it != p.rhs.rend(); ++it) s_out.push_back(*it);
+                s_out.insert(s_out.end(), p.rhs.rbegin(), p.rhs.rend());
                 run(pos + 1, p.head);
                 s_out.resize(s_out.size() - p.rhs.size());
                 s_in.pop_back();
             }
         } else {
             const int32_t top = s_out.back();
-            for (int32_t pi : cands) {
-                const auto& p = g.prods[size_t(pi)];
-                if (p.head != top) continue;
+            auto it = cands.begin();
+            if (cands.size() > 8)
+                it = std::lower_bound(it, cands.end(), top, [&](int32_t pi, int32_t h) { return g.prods[size_t(pi)].head < h; });
+            for (; it != cands.end(); ++it) {
+                const auto& p = g.prods[size_t(*it)];
+                if (p.head > top) break;
+                if (p.head < top) continue;
                 s_out.pop_back();
-                for (auto it = p.rhs.rbegin(); it != p.rhs.rend(); ++it) s_out.push_back(*it);
+                s_out.insert(s_out.end(), p.rhs.rbegin(), p.rhs.rend());
                 run(pos + 1, top);
                 s_out.resize(s_out.size() - p.rhs.size());
                 s_out.push_back(top);
@@ -110,6 +170,36 @@ struct Displacer {
         }
     }
 };
+
+// Tokens are independent: worker threads take them in runs of this many from a shared counter. A run is some tens of
+// microseconds of work, so a thread is started for every few of them only, and never more than the machine has cores.
+constexpr int32_t kTokenRun = 256;
+constexpr int32_t kRunsPerThread = 8;
+
+// A finished row goes out with stores that pass the caches by, where the row's alignment allows it: rows left dirty in
+// the caches of a dozen cores make the copy to the GPU that usually follows two and a half times slower (33 MB: 1.5 ms
+// against 0.6).
+void write_row(int32_t* row, const int32_t* from, size_t words) {
+#ifdef __SSE2__
+    if (words % 4 == 0 && (reinterpret_cast<uintptr_t>(row) & 15u) == 0) {
+        for (size_t i = 0; i < words; i += 4)
+            _mm_stream_si128(reinterpret_cast<__m128i*>(row + i), _mm_loadu_si128(reinterpret_cast<const __m128i*>(from + i)));
+        return;
+    }
+#endif
+    std::memcpy(row, from, words * 4);
+}
+void rows_written() {  // such stores are ordered before whatever tells another thread that the rows are there
+#ifdef __SSE2__
+    _mm_sfence();
+#endif
+}
+
+int worker_count(int32_t V) {
+    const int64_t wanted = V / (kTokenRun * kRunsPerThread);
+    if (wanted <= 1) return 1;
+    return int(std::min({int64_t(std::max(1u, std::thread::hardware_concurrency())), int64_t(32), wanted}));
+}
 
 }  // namespace
 
@@ -141,7 +231,10 @@ int cfgzip_grammar_create(int32_t n_nonterminals, int32_t start, const int32_t* 
         g->by_term[p.term].push_back(int32_t(g->prods.size()));
         g->prods.push_back(std::move(p));
     }
+    for (auto& list : g->by_term)
+        std::stable_sort(list.begin(), list.end(), [&](int32_t x, int32_t y) { return g->prods[size_t(x)].head < g->prods[size_t(y)].head; });
     build_adjacency(*g);
+    cfgzip::Workspace::hold();
     *out = g;
     return CFGZIP_OK;
 }
@@ -149,6 +242,7 @@ int cfgzip_grammar_create(int32_t n_nonterminals, int32_t start, const int32_t* 
 int cfgzip_grammar_destroy(cfgzip_grammar* g) {
     if (!g) return CFGZIP_E_ARG;
     delete g;
+    cfgzip::Workspace::drop();
     return CFGZIP_OK;
 }
 
@@ -162,38 +256,57 @@ int cfgzip_displacement_signatures(const cfgzip_grammar* g, const uint8_t* token
                                    int32_t row_words, int32_t* signatures, int32_t* signature_words, int64_t max_pairs) {
     if (!g || !token_off || V < 0 || row_words < 1 || !signatures || max_pairs < 1) return CFGZIP_E_ARG;
     if (V > 0 && !token_bytes && token_off[V] > token_off[0]) return CFGZIP_E_ARG;
-    int rc = CFGZIP_OK;
-    std::vector<int32_t> flat;
-    for (int32_t i = 0; i < V; ++i) {
-        const int64_t lo = token_off[i], hi = token_off[i + 1];
-        if (hi < lo || hi - lo > 0x7FFFFFFF) return CFGZIP_E_ARG;
-        Displacer d{*g, token_bytes + lo, int32_t(hi - lo), max_pairs};
-        d.run(0, -1);  // (an empty token moves no stack: its only pair is (empty, empty))
-        int32_t* row = signatures + int64_t(i) * row_words;
-        std::fill(row, row + row_words, 0);
-        if (d.overflow) {
-            if (signature_words) signature_words[i] = -1;
-            rc = CFGZIP_E_RANGE;
-            continue;
+    for (int32_t i = 0; i < V; ++i)
+        if (token_off[i + 1] < token_off[i] || token_off[i + 1] - token_off[i] > 0x7FFFFFFF) return CFGZIP_E_ARG;
+    std::atomic<int32_t> next{0};
+    std::atomic<int> rc{CFGZIP_OK};
+    auto work = [&]() noexcept {
+        try {
+            Displacer d(*g, max_pairs);
+            std::vector<int32_t> built(static_cast<size_t>(row_words));
+            for (;;) {
+                const int32_t first = next.fetch_add(kTokenRun);
+                if (first >= V || first < 0) break;
+                const int32_t last = int32_t(std::min<int64_t>(int64_t(first) + kTokenRun, V));
+                for (int32_t i = first; i < last; ++i) {
+                    d.displace(token_bytes + token_off[i], int32_t(token_off[i + 1] - token_off[i]));
+                    int32_t* row = signatures + int64_t(i) * row_words;
+                    // canonical sequence: the pairs in lexicographic order, each as len(sigma_i), sigma_i, len(sigma_o), sigma_o
+                    int64_t n = 0;
+                    for (size_t at : d.pairs) n += 2 + d.flat[at] + d.flat[at + 1 + size_t(d.flat[at])];
+                    const bool fits = !d.overflow && n + 1 <= row_words;
+                    if (signature_words) signature_words[i] = d.overflow ? -1 : int32_t(n);
+                    int32_t* out = built.data();
+                    if (fits) {
+                        *out++ = int32_t(n);
+                        for (size_t at : d.pairs) {
+                            const int32_t* p = d.flat.data() + at;
+                            out = std::copy(p, p + 2 + p[0] + p[1 + p[0]], out);
+                        }
+                    } else {
+                        rc.store(CFGZIP_E_RANGE);
+                    }
+                    std::fill(out, built.data() + row_words, 0);
+                    write_row(row, built.data(), size_t(row_words));
+                }
+            }
+            rows_written();
+        } catch (...) {
+            rc.store(CFGZIP_E_NOMEM);
+            next.store(V);
         }
-        // canonical sequence: the pairs in lexicographic order (std::set of pairs of vectors), each as
-        // len(sigma_i), sigma_i, len(sigma_o), sigma_o
-        flat.clear();
-        for (const Pair& p : d.out) {
-            flat.push_back(int32_t(p.first.size()));
-            flat.insert(flat.end(), p.first.begin(), p.first.end());
-            flat.push_back(int32_t(p.second.size()));
-            flat.insert(flat.end(), p.second.begin(), p.second.end());
-        }
-        if (signature_words) signature_words[i] = int32_t(flat.size());
-        if (int64_t(flat.size()) + 1 > row_words) {
-            rc = CFGZIP_E_RANGE;
-            continue;
-        }
-        row[0] = int32_t(flat.size());
-        std::copy(flat.begin(), flat.end(), row + 1);
+    };
+    std::vector<std::thread> helpers;
+    try {
+        const int n_workers = worker_count(V);
+        helpers.reserve(size_t(n_workers));
+        for (int w = 1; w < n_workers; ++w) helpers.emplace_back(work);
+    } catch (...) {
+        // fewer helpers than wanted: the tokens are shared out among those there are
     }
-    return rc;
+    work();
+    for (std::thread& h : helpers) h.join();
+    return rc.load();
 }
 
 }  // extern "C"
@@ -203,11 +316,13 @@ int cfgzip_displacement_signatures(const cfgzip_grammar* g, const uint8_t* token
 // keyed by the row CONTENT (a hash only picks the first slot; a slot is shared only after the rows compared equal)
 // gives every token the slot of its class; the lowest token id of a slot names the class, classes are numbered in
 // the order of those lowest ids (a prefix sum over "I am the lowest id of my class" flags), the representative is
-// the member with the smallest (byte length, id), and the class lists are filled in ascending token id.
+// the member with the smallest (byte length, id), and the class lists are a stable sort of the tokens by class
+// (class_sort.cuh).
+// What bounds it: reading the signature rows once (33 MB at V = 128256 and 64 words: 5 us from HBM) and a dozen short
+// launches. Most tokens often share one class (what no rule of the grammar can use), so every atomic on a class is
+// preceded by a look whether it still changes anything, or made once for the equal lanes of a warp.
 // ---------------------------------------------------------------------------------------------------------------
 namespace {
-
-constexpr int kScanThreads = 1024;
 
 __device__ __forceinline__ unsigned long long mix64(unsigned long long z) {
     z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
@@ -215,113 +330,119 @@ __device__ __forceinline__ unsigned long long mix64(unsigned long long z) {
     return z ^ (z >> 31);
 }
 
-__global__ void k_group_insert(const int32_t* __restrict__ sig, int W, const int32_t* __restrict__ len, int V, int32_t* owner,
-                               unsigned table_mask, int32_t* slot_of, int32_t* min_id, unsigned long long* rep_key) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= V) return;
+constexpr int kRowLanes = 8;       // lanes that read a signature row together
+constexpr int kSeedTokens = 2048;  // tokens the first, small launch inserts
+
+// Eight lanes per token: coalesced reads of the row, words hashed with their positions, the sums of the lanes added up.
+// The slots of the big classes are taken by a first launch over the first kSeedTokens tokens: without it tens of
+// thousands of tokens of one class find its slot empty at once and queue up at one compare-and-swap.
+__global__ void __launch_bounds__(256) k_group_insert(const int32_t* __restrict__ sig, int W, int first, int end, int32_t* owner,
+                                                      unsigned table_mask, int32_t* slot_of) {
+    const int sub = threadIdx.x & (kRowLanes - 1);
+    const int t = first + int((blockIdx.x * blockDim.x + threadIdx.x) / kRowLanes);
+    if (t >= end) return;
+    const unsigned lanes = ((1u << kRowLanes) - 1u) << (threadIdx.x & 31 & ~(kRowLanes - 1));
     const int32_t* row = sig + int64_t(t) * W;
-    unsigned long long h = 0x243F6A8885A308D3ull;
-    for (int w = 0; w < W; ++w) h = mix64(h ^ static_cast<unsigned>(row[w]));
-    unsigned slot = unsigned(h) & table_mask;
+    unsigned long long h = 0ull;
+    for (int w = sub; w < W; w += kRowLanes)
+        h += mix64((static_cast<unsigned long long>(unsigned(w) + 1u) << 32) ^ static_cast<unsigned>(__ldg(row + w)));
+#pragma unroll
+    for (int d = kRowLanes / 2; d >= 1; d >>= 1) h += __shfl_xor_sync(lanes, h, d, kRowLanes);
+    unsigned slot = unsigned(mix64(h)) & table_mask;
     for (unsigned probe = 0; probe <= table_mask; ++probe) {  // the table has at least 2 V slots: a free one always turns up
-        int32_t o = atomicCAS(owner + slot, -1, t);
-        bool same = o == -1 || o == t;
-        if (!same) {
-            const int32_t* other = sig + int64_t(o) * W;
-            same = true;
-            for (int w = 0; w < W && same; ++w) same = other[w] == row[w];
+        int32_t o = 0;
+        if (sub == 0) {
+            o = *reinterpret_cast<volatile int32_t*>(owner + slot);
+            if (o == -1) o = atomicCAS(owner + slot, -1, t);
         }
-        if (same) break;
+        o = __shfl_sync(lanes, o, 0, kRowLanes);
+        bool same = true;
+        if (o != -1 && o != t) {
+            const int32_t* other = sig + int64_t(o) * W;
+            for (int w = sub; w < W && same; w += kRowLanes) same = __ldg(other + w) == __ldg(row + w);
+        }
+        if (__all_sync(lanes, same)) break;
         slot = (slot + 1) & table_mask;
     }
-    slot_of[t] = int32_t(slot);
-    atomicMin(min_id + slot, t);
-    atomicMin(rep_key + slot, (static_cast<unsigned long long>(unsigned(len[t])) << 32) | unsigned(t));
+    if (sub == 0) slot_of[t] = int32_t(slot);
 }
 
-// flag[t] = 1 when t is the lowest token id of its class
-__global__ void k_group_flags(const int32_t* slot_of, const int32_t* min_id, int V, int32_t* flag) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < V) flag[t] = min_id[slot_of[t]] == t ? 1 : 0;
+// The lowest token id and the smallest (length, id) of every slot. Both arrays start at all ones.
+__global__ void __launch_bounds__(256) k_group_min(const int32_t* slot_of, const int32_t* __restrict__ len, int V, unsigned* min_id,
+                                                   unsigned long long* rep_key) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+    const bool have = t < V;
+    const int slot = have ? slot_of[t] : -1 - lane;  // lanes without a token match nobody
+    const unsigned peers = __match_any_sync(0xFFFFFFFFu, slot);
+    const unsigned n = have ? unsigned(len[t]) : 0u;
+    const unsigned shortest = __reduce_min_sync(peers, n);
+    const unsigned of_shortest = __reduce_min_sync(peers, n == shortest ? unsigned(t) : 0xFFFFFFFFu);
+    if (!have || lane != __ffs(int(peers)) - 1) return;  // the first lane of a class holds its lowest id in the warp
+    if (*reinterpret_cast<volatile unsigned*>(min_id + slot) > unsigned(t)) atomicMin(min_id + slot, unsigned(t));
+    const unsigned long long key = (static_cast<unsigned long long>(shortest) << 32) | of_shortest;
+    if (*reinterpret_cast<volatile unsigned long long*>(rep_key + slot) > key) atomicMin(rep_key + slot, key);
 }
 
-// Exclusive prefix sum of n integers in place, by one block; the total goes to *total (if not null) and to data[n].
-__global__ void __launch_bounds__(kScanThreads) k_exclusive_scan(int32_t* data, int n, int32_t* total) {
-    __shared__ int s_warp[kScanThreads / 32];
-    __shared__ int s_carry;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) s_carry = 0;
-    __syncthreads();
-    for (int base = 0; base < n; base += kScanThreads) {
-        const int i = base + tid;
-        const int v = i < n ? data[i] : 0;
-        int inc = v;
+// How many of a block's tokens are the lowest of their class.
+constexpr int kNumberTile = 4096;  // tokens per block of the numbering kernels, four per thread
+__global__ void __launch_bounds__(1024) k_group_count(const int32_t* slot_of, const unsigned* min_id, int V, int32_t* block_count) {
+    int n = 0;
 #pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int up = __shfl_up_sync(0xFFFFFFFFu, inc, d);
-            if (lane >= d) inc += up;
+    for (int q = 0; q < 4; ++q) {
+        const int t = blockIdx.x * kNumberTile + q * 1024 + threadIdx.x;
+        n += __syncthreads_count(t < V && min_id[slot_of[t]] == unsigned(t));
+    }
+    if (threadIdx.x == 0) block_count[blockIdx.x] = n;
+}
+
+// Classes numbered in token order (every block adds up the counts of the blocks in front of it), representatives.
+__global__ void __launch_bounds__(1024) k_group_number(const int32_t* slot_of, const unsigned* min_id,
+                                                       const unsigned long long* rep_key, int V, const int32_t* block_count,
+                                                       int32_t* class_of_slot, int32_t* r, int32_t* n_classes) {
+    __shared__ int s_warp[32], s_front;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) s_front = 0;
+    __syncthreads();
+    int front = 0;
+    for (int b = tid; b < int(blockIdx.x); b += 1024) front += block_count[b];
+    front = __reduce_add_sync(0xFFFFFFFFu, front);
+    if (lane == 0 && front) atomicAdd(&s_front, front);
+    const int t0 = blockIdx.x * kNumberTile + tid * 4;
+    int slot[4];
+    bool lowest[4];
+    int mine = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        slot[q] = t0 + q < V ? slot_of[t0 + q] : -1;
+        lowest[q] = slot[q] >= 0 && min_id[slot[q]] == unsigned(t0 + q);
+        mine += lowest[q];
+    }
+    int inc = mine;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int up = __shfl_up_sync(0xFFFFFFFFu, inc, d);
+        if (lane >= d) inc += up;
+    }
+    if (lane == 31) s_warp[warp] = inc;
+    __syncthreads();
+    int k = s_front + inc - mine;
+    for (int w = 0; w < warp; ++w) k += s_warp[w];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        if (lowest[q]) {
+            class_of_slot[slot[q]] = k;
+            r[k] = int32_t(rep_key[slot[q]] & 0xFFFFFFFFull);
+            ++k;
         }
-        if (lane == 31) s_warp[warp] = inc;
-        __syncthreads();
-        int before = s_carry;
-        for (int w = 0; w < warp; ++w) before += s_warp[w];
-        if (i < n) data[i] = before + inc - v;
-        __syncthreads();
-        if (tid == kScanThreads - 1) s_carry = before + inc;
-        __syncthreads();
-    }
-    if (tid == 0) {
-        data[n] = s_carry;
-        if (total) *total = s_carry;
-    }
+    if (blockIdx.x == gridDim.x - 1 && tid == 1023) *n_classes = k;  // the last thread has counted everybody
 }
 
-__global__ void k_group_assign(const int32_t* slot_of, const int32_t* min_id, const unsigned long long* rep_key,
-                               const int32_t* class_of_first, int V, int32_t* c, int32_t* r, int32_t* count) {
+__global__ void __launch_bounds__(256) k_group_assign(const int32_t* slot_of, const int32_t* class_of_slot, int V, int32_t* c) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= V) return;
-    const int slot = slot_of[t];
-    const int first = min_id[slot];
-    const int k = class_of_first[first];
-    c[t] = k;
-    atomicAdd(count + k, 1);
-    if (first == t) r[k] = int32_t(rep_key[slot] & 0xFFFFFFFFull);
+    if (t < V) c[t] = class_of_slot[slot_of[t]];
 }
 
-// Class lists in ascending token id: one warp walks the tokens in order, 32 at a time; lanes of the same class share
-// one cursor and take consecutive places in lane order. The cursors (class offsets to start with) sit in shared
-// memory when there are few enough classes, which takes the round trip to L2 out of every step of the walk.
-constexpr int kListCursorsShared = 48 * 1024 / 4;
-
-__global__ void __launch_bounds__(32) k_group_lists(const int32_t* c, int V, const int32_t* n_classes, int32_t* cursor,
-                                                    int32_t* tok) {
-    __shared__ int32_t s_cursor[kListCursorsShared];
-    const int lane = threadIdx.x;
-    const int K = *n_classes;
-    const bool shared = K <= kListCursorsShared;
-    int32_t* cur = shared ? s_cursor : cursor;
-    if (shared) {
-        for (int k = lane; k < K; k += 32) s_cursor[k] = cursor[k];
-        __syncwarp();
-    }
-    int k_next = lane < V ? c[lane] : 0;  // the class of this lane's next token is fetched one round ahead
-    for (int base = 0; base < V; base += 32) {
-        const int t = base + lane;
-        const bool have = t < V;
-        const int k = have ? k_next : -1 - lane;  // lanes without a token match nobody
-        if (t + 32 < V) k_next = c[t + 32];
-        const unsigned peers = __match_any_sync(0xFFFFFFFFu, k);
-        const int rank = __popc(peers & ((1u << lane) - 1u));
-        const int leader = __ffs(peers) - 1;
-        int at = 0;
-        if (have && lane == leader) at = atomicAdd(cur + k, __popc(peers));
-        at = __shfl_sync(0xFFFFFFFFu, at, leader);
-        if (have) tok[at + rank] = t;
-        __syncwarp();
-    }
-}
-
-inline unsigned blocks_for(int n, int threads) { return unsigned((n + threads - 1) / threads); }
+inline unsigned blocks_for(int64_t n, int threads) { return unsigned((n + threads - 1) / threads); }
 
 }  // namespace
 
@@ -336,45 +457,31 @@ extern "C" int cfgzip_group_tokens(const int32_t* signatures, int32_t row_words,
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     unsigned table = 1;
     while (table < 2u * unsigned(V)) table <<= 1;
-    // scratch: owner, min_id [table]; rep_key [table]; slot_of, flag (+1), count (+1), cursor [V]
-    const size_t n_i32 = size_t(table) * 2 + size_t(V) * 4 + 2;
-    int32_t* i32 = nullptr;
-    unsigned long long* rep_key = nullptr;
-    if (cudaMalloc(&i32, n_i32 * sizeof(int32_t)) != cudaSuccess || cudaMalloc(&rep_key, size_t(table) * 8) != cudaSuccess) {
-        cudaGetLastError();
-        cudaFree(i32);
-        return CFGZIP_E_NOMEM;
-    }
-    int32_t* owner = i32;
-    int32_t* min_id = owner + table;
-    int32_t* slot_of = min_id + table;
-    int32_t* flag = slot_of + V;       // V + 1 entries
-    int32_t* count = flag + V + 1;     // V + 1 entries
-    int32_t* cursor = count + V + 1;   // V entries
-    bool ok = cudaMemsetAsync(owner, 0xFF, size_t(table) * 4, st) == cudaSuccess &&          // -1
-              cudaMemsetAsync(min_id, 0x7F, size_t(table) * 4, st) == cudaSuccess &&         // a large positive id
-              cudaMemsetAsync(rep_key, 0xFF, size_t(table) * 8, st) == cudaSuccess &&
-              cudaMemsetAsync(count, 0, size_t(V + 1) * 4, st) == cudaSuccess;
+    // scratch: rep_key, min_id, owner [table], all ones to begin with; slot_of [V], block counts, the sort's own
+    const unsigned number_blocks = blocks_for(V, kNumberTile);
+    const size_t words = size_t(table) * 4 + size_t(V) + number_blocks + (class_off ? cfgzip::class_sort_scratch_words(V) : 0);
+    cfgzip::Workspace scratch(words * 4);
+    if (!scratch.ptr) return CFGZIP_E_NOMEM;
+    unsigned long long* rep_key = static_cast<unsigned long long*>(scratch.ptr);
+    unsigned* min_id = reinterpret_cast<unsigned*>(rep_key + table);
+    int32_t* owner = reinterpret_cast<int32_t*>(min_id + table);  // later the class of a slot
+    int32_t* slot_of = owner + table;
+    int32_t* block_count = slot_of + V;
+    bool ok = cudaMemsetAsync(rep_key, 0xFF, size_t(table) * 16, st) == cudaSuccess;
     if (ok) {
-        const int T = 256;
-        k_group_insert<<<blocks_for(V, T), T, 0, st>>>(signatures, row_words, token_len, V, owner, table - 1, slot_of, min_id,
-                                                       rep_key);
-        k_group_flags<<<blocks_for(V, T), T, 0, st>>>(slot_of, min_id, V, flag);
-        k_exclusive_scan<<<1, kScanThreads, 0, st>>>(flag, V, n_classes);
-        k_group_assign<<<blocks_for(V, T), T, 0, st>>>(slot_of, min_id, rep_key, flag, V, token_to_class, class_to_rep, count);
-        if (class_off) {
-            // class sizes -> offsets (the scan also writes the total V behind the last class that exists: entries past
-            // n_classes all read V), then the lists
-            k_exclusive_scan<<<1, kScanThreads, 0, st>>>(count, V, nullptr);
-            ok = cudaMemcpyAsync(class_off, count, size_t(V + 1) * 4, cudaMemcpyDeviceToDevice, st) == cudaSuccess &&
-                 cudaMemcpyAsync(cursor, count, size_t(V) * 4, cudaMemcpyDeviceToDevice, st) == cudaSuccess;
-            if (ok) k_group_lists<<<1, 32, 0, st>>>(token_to_class, V, n_classes, cursor, class_tok);
-        }
-        ok = ok && cudaGetLastError() == cudaSuccess;
+        const int T = 256, per_block = T / kRowLanes, seed = std::min(V, kSeedTokens);
+        k_group_insert<<<blocks_for(seed, per_block), T, 0, st>>>(signatures, row_words, 0, seed, owner, table - 1, slot_of);
+        if (V > seed)
+            k_group_insert<<<blocks_for(V - seed, per_block), T, 0, st>>>(signatures, row_words, seed, V, owner, table - 1, slot_of);
+        k_group_min<<<blocks_for(V, T), T, 0, st>>>(slot_of, token_len, V, min_id, rep_key);
+        k_group_count<<<number_blocks, 1024, 0, st>>>(slot_of, min_id, V, block_count);
+        k_group_number<<<number_blocks, 1024, 0, st>>>(slot_of, min_id, rep_key, V, block_count, owner, class_to_rep, n_classes);
+        k_group_assign<<<blocks_for(V, T), T, 0, st>>>(slot_of, owner, V, token_to_class);
+        if (class_off)
+            cfgzip::class_sort(token_to_class, V, n_classes, 0, class_off, class_tok, block_count + number_blocks, st);
+        ok = cudaGetLastError() == cudaSuccess;
     }
     ok = (cudaStreamSynchronize(st) == cudaSuccess) && ok;  // the scratch is released below
-    cudaFree(i32);
-    cudaFree(rep_key);
     if (!ok) {
         cudaGetLastError();
         return CFGZIP_E_CUDA;

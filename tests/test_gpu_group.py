@@ -105,3 +105,47 @@ def test_llama_size_vocabulary_of_synthetic_signatures():
     # and a sample of it through the oracle's own grouping
     sub = np.sort(rng.permutation(rng.stream_key(10), V)[:1500])
     check_against_oracle(sig[sub], lens[sub])
+
+
+@pytest.mark.parametrize("V,K,W", [(1, 1, 1), (2048, 5, 3), (2049, 700, 9), (4097, 512, 64), (5000, 513, 7), (30011, 30011, 2),
+                                   (270001, 265000, 2), (9000, 2, 64)])
+def test_sizes_at_the_edges_of_the_kernels(V, K, W):
+    """The launch that seeds the table, the tiles of the numbering and the sort, one and two passes of the sort."""
+    rs = np.random.RandomState(V + W)
+    k = rs.randint(0, K, V)
+    if K == 2:
+        k = (rs.random_sample(V) < 0.02).astype(np.int64)  # one class holds nearly everything
+    sig = np.zeros((V, W), dtype=np.int32)
+    sig[:, -1] = k
+    sig[:, 0] += (k % 3).astype(np.int32)
+    lens = rs.randint(1, 9, V).astype(np.int32)
+    _, inverse = np.unique(sig, axis=0, return_inverse=True)
+    _, first = np.unique(inverse.reshape(-1), return_index=True)
+    rank = np.empty(len(first), dtype=np.int64)
+    rank[np.argsort(first)] = np.arange(len(first))
+    want_c = rank[inverse.reshape(-1)]
+    order = np.lexsort((np.arange(V), lens, want_c))
+    want_r = order[np.unique(want_c[order], return_index=True)[1]]
+    c, r, n, off, tok = gpu_group(sig, lens)
+    assert n == len(first) and np.array_equal(c, want_c) and np.array_equal(r, want_r)
+    assert np.array_equal(tok, np.argsort(want_c, kind="stable"))
+    assert np.array_equal(off[:n], np.searchsorted(want_c[tok], np.arange(n))) and np.all(off[n:] == V)
+
+
+@pytest.mark.parametrize("V,K", [(1, 1), (33, 33), (1025, 512), (1024, 513), (70001, 66000), (5000, 3)])
+def test_loaded_partition_serves_both_expansions(V, K):
+    """The class lists and tables that loading makes on the GPU, seen through the class-list and the gather kernel."""
+    part = synth.zipf_partition(V, K, seed=V)
+    cm = synth.class_mask_bernoulli(K, 3, 0.4, rng.stream_key(77, V))
+    z = synth.logits_normal(3, V, 1.0, "f32", (78, V))
+    with Ctx([part]) as ctx:
+        for mode in (cz.DENSE, cz.SPARSE):
+            compare_step(run_fused(ctx, None, cm, z, V, mode=mode), oracle_step([part], None, cm, z, V), V)
+        for bad_c, bad_r in ((np.full(V, K, np.int32), part.r), (part.c, np.full(K, V, np.int32)), (part.c, np.full(K, -1, np.int32))):
+            with pytest.raises(cz.CfgzipError) as e:
+                cz.cfgzip_load_partition(ctx.h, bad_c, V, bad_r, K)
+            assert e.value.status == cz.E_PARTITION
+        again = cz.cfgzip_load_partition(ctx.h, part.c, V, part.r, K)
+        cz.cfgzip_free_partition(ctx.h, again)
+        again = cz.cfgzip_load_partition(ctx.h, part.c, V, part.r, K)  # in the memory of the one just released
+        compare_step(run_fused(ctx, None, cm, z, V, part0=again), oracle_step([part], None, cm, z, V), V)
