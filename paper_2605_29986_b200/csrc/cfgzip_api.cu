@@ -30,7 +30,6 @@ struct Part {
 
 constexpr size_t kSpareBytes = size_t(32) << 20;  // most memory of a released partition a context keeps for the next one
 constexpr size_t kPartialSlots = size_t(1) << 18;  // 4 MB of (max, sum, pos) slots
-constexpr size_t kFiltSmem = size_t(kFiltList) * 16;  // candidate list of the filtered sampling kernel
 constexpr int kTwoOctetItemsPerWarp = 3;           // bf16: two octets per lane from this many work items per warp on
 constexpr int kDefaultRows = 16384;
 
@@ -677,20 +676,23 @@ int launch_fused(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, in
 }
 
 // The draw of a sampling step with top-k / top-p. One block per row leaves most of the device idle on a short batch,
-// so 4 or 2 blocks (a thread-block cluster) share a row while that many blocks still fit the device in one wave.
+// so 8, 4 or 2 blocks (a thread-block cluster) share a row while that many still fit the device in one wave, two of the
+// kernel's blocks to an SM.
 template <int DT>
 int launch_filtered(cfgzip_ctx* ctx, const StepArgs& a, unsigned rows_grid, int aligned, int top_k, float top_p,
                     cudaStream_t st) {
     int rc;
-    if ((rc = ensure_smem(k_sample_filtered<DT>, kFiltSmem)) != CFGZIP_OK) return rc;
-    const unsigned sms = unsigned(std::max(ctx->sm_count, 1));
-    const unsigned per_row = rows_grid * 4 <= sms ? 4u : (rows_grid * 2 <= sms ? 2u : 1u);
+    if ((rc = ensure_smem(k_sample_filtered<DT>, sizeof(FiltShared))) != CFGZIP_OK) return rc;
+    const unsigned fit = 2u * unsigned(std::max(ctx->sm_count, 1));
+    unsigned per_row = kFiltPeers;
+    while (per_row > 1 && unsigned(a.B) * per_row > fit) per_row /= 2;
     ctx->cluster_now = int(per_row);
-    rc = launch(ctx, k_sample_filtered<DT>, dim3(rows_grid * per_row), dim3(kFiltThreads), kFiltSmem, st, a, aligned, top_k,
-                top_p);
+    rc = launch(ctx, k_sample_filtered<DT>, dim3(rows_grid * per_row), dim3(kFiltThreads), sizeof(FiltShared), st, a, aligned,
+                top_k, top_p);
     ctx->cluster_now = 1;
     if (rc != CFGZIP_OK && per_row > 1)  // a device that cannot place such a cluster: one block per row
-        rc = launch(ctx, k_sample_filtered<DT>, dim3(rows_grid), dim3(kFiltThreads), kFiltSmem, st, a, aligned, top_k, top_p);
+        rc = launch(ctx, k_sample_filtered<DT>, dim3(rows_grid), dim3(kFiltThreads), sizeof(FiltShared), st, a, aligned, top_k,
+                    top_p);
     return rc;
 }
 

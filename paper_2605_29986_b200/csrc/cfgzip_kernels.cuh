@@ -5,7 +5,6 @@
 #pragma once
 
 #include <cuda.h>
-#include <type_traits>
 
 #include "cfgzip_device.cuh"
 
@@ -1848,27 +1847,36 @@ __global__ void __launch_bounds__(kSampleThreads) k_sample_rows(const __grid_con
 }
 
 // ---------------------------------------------------------------------------------------
-// Second kernel of a sampling step with top-k / top-p: one block per row keeps, of the row's allowed tokens in the
+// Second kernel of a sampling step with top-k / top-p: keeps, of the row's allowed tokens in the
 // order (value, largest first; equal values by token id, lowest first), the first top_k (0 = all) and of those the
 // shortest beginning whose weight reaches top_p times the weight of what top_k kept (>= 1: all), then draws among
 // the kept tokens by inverse CDF in token order with the row's uniform number.
-// The kept set is { key > tau } plus the first m tokens, in token order, with key == tau, where key is an
-// order-preserving integer image of the logit; tau is the largest key with enough tokens (top-k) or enough weight
-// (top-p) at or above it. Weights are 40-bit fixed-point integers (exp((z - M) / T) * 2^40), so every sum is
-// exact whatever the order of the addends: the result is deterministic. The tokens whose weight is not zero in that
-// format are first collected in shared memory (up to kFiltList of them). When they all fit, which is the rule at the
-// temperatures used for constrained decoding, nothing goes back to the row (a token of weight zero can change neither
-// a cumulative weight nor the draw): tau, the last tie that is kept and the drawn token each come out of a radix
-// search over the list, ten bits per round (list_select). Otherwise tau is found by bisection with passes over the row.
+// Weights are 40-bit fixed-point integers (exp((z - M) / T) * 2^40), so every sum is exact whatever the order of the
+// addends: the result is deterministic. A token whose weight is zero in that format can change neither a cumulative
+// weight nor the draw.
+//
+// Two ways through, both exact:
+//   short  The streaming kernel has published the largest logit of every run of tokens. The k-th largest of those is a bar
+//          that at least k tokens reach, and, the runs being many, not many more (k = 50: some 60 to 100 tokens). For top-p
+//          alone the bar is where the run maxima by themselves already weigh enough. One pass over the row collects the
+//          tokens at or above the bar, a thread each, and every thread sums over all of them.
+//   long   Otherwise (a flat distribution, a large k): the kept set is { key > tau } plus the first m tokens, in token order,
+//          with key == tau, where key is an order-preserving integer image of the logit. tau comes out of a radix search
+//          over the row itself, twelve bits a pass (bf16: two passes, f32: three; count and weight of 4096 buckets in shared
+//          memory), the draw out of one more pass that leaves the kept weight of every chunk of 256 tokens.
+// Bound: latency of a chain of block-wide steps. Collecting every token that carries weight first took 78 us of the step for
+// 64 rows of 151936 bf16 logits at T = 0.7 (15000 such tokens a row), and some 30 passes over the row where they did not fit.
 // ---------------------------------------------------------------------------------------
-constexpr int kFiltThreads = 1024;
-constexpr int kFiltList = 12288;  // entries of the candidate list (16 bytes each, dynamic shared memory)
-constexpr int kFiltAttempts = 5;  // passes over the row with the bar for the list raised each time it overflows
-constexpr int kFiltPeers = 4;     // most blocks that share a row
+constexpr int kFiltThreads = 512;   // two blocks per SM: one row's serial steps overlap another row's passes
+constexpr int kFiltWarps = kFiltThreads / 32;
+constexpr int kFiltPeers = 8;       // most blocks that share a row
+constexpr int kFiltList = kFiltThreads;  // tokens of the short way, one per thread
+constexpr int kFiltBits = 12, kFiltBuckets = 1 << kFiltBits;
+constexpr int kFiltChunks = 1024;   // chunks of the draw's pass
 constexpr float kFixOne = 1099511627776.f;  // 2^40
 
 // Order-preserving integer image of a logit and its inverse. bf16 logits only use the upper half of the float's
-// bits, so their keys are 16 bits wide and a bisection over them takes half the steps.
+// bits, so their keys are 16 bits wide.
 template <int DT>
 __device__ __forceinline__ uint32_t logit_key(float z) {
     z = z == 0.f ? 0.f : z;  // -0.0 and +0.0 are the same value
@@ -1889,57 +1897,58 @@ struct CountMass {
     unsigned int n;
     unsigned long long w;
 };
-
-// Sum of one (count, weight) pair per thread over the block; everybody gets the total. s_n / s_w: two sets of one
-// entry per warp, used in turn (`turn` flips with every call), so that one barrier per call is enough: a warp can only
-// write a set again after every warp has passed the barrier of the call in between, i.e. has read this one.
-__device__ __forceinline__ CountMass block_sum(CountMass v, unsigned int* s_n, unsigned long long* s_w, int& turn) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int d = 16; d >= 1; d >>= 1) {
-        v.n += __shfl_xor_sync(0xFFFFFFFFu, v.n, d);
-        v.w += __shfl_xor_sync(0xFFFFFFFFu, v.w, d);
-    }
-    constexpr int kWarps = kFiltThreads / 32;
-    unsigned int* n = s_n + turn * kWarps;
-    unsigned long long* w = s_w + turn * kWarps;
-    turn ^= 1;
-    if (lane == 0) {
-        n[warp] = v.n;
-        w[warp] = v.w;
-    }
-    __syncthreads();
-    CountMass t{0u, 0ull};
-#pragma unroll
-    for (int i = 0; i < kWarps; ++i) {
-        t.n += n[i];
-        t.w += w[i];
-    }
-    return t;
+__device__ __forceinline__ void operator+=(CountMass& a, const CountMass& b) {
+    a.n += b.n;
+    a.w += b.w;
 }
 
-// Exclusive prefix sum of one 64-bit value per thread in thread order; total to everybody.
-__device__ __forceinline__ unsigned long long block_exclusive_scan_u64(unsigned long long v, unsigned long long* s_w,
-                                                                       unsigned long long& total) {
+// Shared memory of a block.
+struct FiltShared {
+    union {
+        struct {  // count and weight of the buckets; weights as two 32-bit halves, which keeps every atomic a native one
+            unsigned int n[kFiltBuckets], lo[kFiltBuckets], hi[kFiltBuckets];
+        } hist;
+        uint4 list[kFiltList];  // short way: key (or raw logit), token id, weight
+        struct {                // the draw's pass: kept weight above tau and number of ties of every chunk
+            unsigned long long above[kFiltChunks];
+            unsigned int ties[kFiltChunks];
+        } chunk;
+    };
+    unsigned long long pick[8];  // result of a search, written into every block of the cluster by the first
+    unsigned long long scan_w[2][kFiltWarps];
+    unsigned int scan_n[2][kFiltWarps];
+    unsigned long long peer_w[kFiltPeers];
+    float warp_max[kFiltWarps];
+    unsigned int list_n;
+    unsigned long long kept_w, topk_w;
+};
+
+// Exclusive prefix of one (count, weight) pair per thread in thread order; total to everybody. The two sets of partial sums
+// are used in turn (`turn` flips with every call), so that one barrier per call is enough.
+__device__ __forceinline__ CountMass filt_scan(CountMass v, FiltShared& sh, int& turn, CountMass& total) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned long long inc = v;
+    CountMass inc = v;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
-        const unsigned long long up = __shfl_up_sync(0xFFFFFFFFu, inc, d);
-        if (lane >= d) inc += up;
+        const unsigned int un = __shfl_up_sync(0xFFFFFFFFu, inc.n, d);
+        const unsigned long long uw = __shfl_up_sync(0xFFFFFFFFu, inc.w, d);
+        if (lane >= d) inc += CountMass{un, uw};
+    }
+    if (lane == 31) {
+        sh.scan_n[turn][warp] = inc.n;
+        sh.scan_w[turn][warp] = inc.w;
     }
     __syncthreads();
-    if (lane == 31) s_w[warp] = inc;
-    __syncthreads();
-    unsigned long long before = 0ull, all = 0ull;
+    CountMass before{0u, 0ull};
+    total = CountMass{0u, 0ull};
 #pragma unroll
-    for (int w = 0; w < kFiltThreads / 32; ++w) {
-        const unsigned long long t = s_w[w];
-        if (w < warp) before += t;
-        all += t;
+    for (int i = 0; i < kFiltWarps; ++i) {
+        const CountMass t{sh.scan_n[turn][i], sh.scan_w[turn][i]};
+        if (i < warp) before += t;
+        total += t;
     }
-    total = all;
-    return before + inc - v;
+    turn ^= 1;
+    return CountMass{before.n + inc.n - v.n, before.w + inc.w - v.w};
 }
 
 // Eight consecutive logits of a row from token t0 on (-inf in front of token 0 and past `end`), as floats.
@@ -1963,25 +1972,11 @@ __device__ __forceinline__ void load_eight(const char* rowp, int t0, int end, bo
         for (int q = 0; q < 8; ++q) e[q] = t0 + q >= 0 && t0 + q < end ? ldcg_elem<DT>(rowp, t0 + q) : -INFINITY;
     }
 }
-
-// Visit every token of a row, the block's threads side by side (8 consecutive tokens per thread and round, four
-// rounds in flight together).
-template <int DT, typename F>
-__device__ __forceinline__ void row_visit(const char* rowp, int lead, int V, bool aligned, F&& f) {
-    constexpr int kInFlight = 4;
-    for (int t0 = int(threadIdx.x) * 8 - lead; t0 < V; t0 += kFiltThreads * 8 * kInFlight) {
-        float e[kInFlight][8];
-#pragma unroll
-        for (int r = 0; r < kInFlight; ++r) load_eight<DT>(rowp, t0 + r * kFiltThreads * 8, V, aligned, e[r]);
-#pragma unroll
-        for (int r = 0; r < kInFlight; ++r)
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-                if (e[r][q] > kRefFloor) f(t0 + r * kFiltThreads * 8 + q, e[r][q]);  // masked logits are -inf
-    }
+__device__ __forceinline__ float max_eight(const float (&e)[8]) {
+    return fmax3(fmax3(e[0], e[1], e[2]), fmax3(e[3], e[4], e[5]), fmaxf(e[6], e[7]));
 }
 
-// ---- thread-block cluster: rank, barrier, reads of a peer block's shared memory -----------------
+// ---- thread-block cluster: rank, barrier, accesses to a peer block's shared memory -----------------
 __device__ __forceinline__ uint32_t cluster_rank() {
     uint32_t r;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -1996,6 +1991,9 @@ __device__ __forceinline__ uint32_t cluster_blocks() {
 __device__ __forceinline__ void cluster_barrier() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// the same in two halves
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ uint32_t peer_shared(const void* mine, uint32_t rank) {
     uint32_t r;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(mine)), "r"(rank));
@@ -2011,6 +2009,11 @@ __device__ __forceinline__ uint32_t ld_peer_u32(uint32_t addr) {
     asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
     return v;
 }
+__device__ __forceinline__ uint4 ld_peer_v4(uint32_t addr) {
+    uint4 v;
+    asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+    return v;
+}
 __device__ __forceinline__ void st_peer_u64(uint32_t addr, unsigned long long v) {
     asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
 }
@@ -2018,188 +2021,106 @@ __device__ __forceinline__ void st_peer_u32(uint32_t addr, uint32_t v) {
     asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
-// ---- searches over the candidate list: every thread of the block walks the list (a walk is a chain of dependent
-// shared-memory accesses per entry, so more threads shorten it), the first kSelThreads threads sum over the buckets
-// (barriers and sums across 8 warps cost a fraction of those across 32)
-constexpr int kSelThreads = 256;
-constexpr int kSelBuckets = 1024;  // ten bits of the value per round; kSelBuckets / kSelThreads buckets per thread
-__device__ __forceinline__ void sel_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kSelThreads) : "memory"); }
-
-// Exclusive prefix of one (count, weight) pair per thread in thread order over those threads; total to everybody.
-// s_n / s_w: two sets of one entry per warp, used in turn as in block_sum.
-__device__ __forceinline__ CountMass sel_exclusive_scan(CountMass v, unsigned int* s_n, unsigned long long* s_w, int& turn,
-                                                        CountMass& total) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    CountMass inc = v;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const unsigned int un = __shfl_up_sync(0xFFFFFFFFu, inc.n, d);
-        const unsigned long long uw = __shfl_up_sync(0xFFFFFFFFu, inc.w, d);
-        if (lane >= d) {
-            inc.n += un;
-            inc.w += uw;
-        }
+__device__ __forceinline__ void hist_clear(FiltShared& sh) {
+    uint4* h = reinterpret_cast<uint4*>(&sh.hist);
+#pragma unroll 4
+    for (int i = threadIdx.x; i < int(sizeof(sh.hist) / 16); i += kFiltThreads) h[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+__device__ __forceinline__ void hist_add(FiltShared& sh, uint32_t bucket, unsigned long long w) {
+    atomicAdd(&sh.hist.n[bucket], 1u);
+    const uint32_t lo = static_cast<uint32_t>(w);
+    uint32_t hi = static_cast<uint32_t>(w >> 32);
+    if (lo) {
+        const uint32_t old = atomicAdd(&sh.hist.lo[bucket], lo);
+        hi += (old + lo) < old ? 1u : 0u;  // the carry out of the lower half
     }
-    constexpr int kWarps = kSelThreads / 32;
-    unsigned int* n = s_n + turn * kWarps;
-    unsigned long long* w = s_w + turn * kWarps;
-    turn ^= 1;
-    if (lane == 31) {
-        n[warp] = inc.n;
-        w[warp] = inc.w;
-    }
-    sel_sync();
-    CountMass before{0u, 0ull}, all{0u, 0ull};
-#pragma unroll
-    for (int i = 0; i < kWarps; ++i) {
-        const unsigned int tn = n[i];
-        const unsigned long long tw = w[i];
-        if (i < warp) {
-            before.n += tn;
-            before.w += tw;
-        }
-        all.n += tn;
-        all.w += tw;
-    }
-    total = all;
-    return CountMass{before.n + inc.n - v.n, before.w + inc.w - v.w};
+    if (hi) atomicAdd(&sh.hist.hi[bucket], hi);
 }
 
-// Result of a search: the value found, (count, weight) of the entries below it and of the entries at it, the
-// threshold that was used and (count, weight) of all entries that took part.
+// Result of a bucket search: the bucket, (count, weight) in front of it and in it, of everything, the threshold; found: some
+// bucket holds the threshold.
 struct Picked {
-    uint32_t x;
+    uint32_t bucket;
+    bool found;
     CountMass before, at, all;
-    unsigned long long thr;
 };
 
-// Smallest value x such that the entries of the list with value <= x together count (BY_WEIGHT: weigh) more than thr,
-// where thr = thr_of(count and weight of all entries) is fixed once the first histogram is summed (so a threshold
-// that depends on the total weight costs no pass of its own). xg(i, x, gn, gw) gives entry i's value (below 2^bits),
-// count and weight (both 0: the entry takes no part); the caller guarantees that all entries together exceed thr.
-// Ten bits of the value per round, highest first: a histogram of the round's digit over the entries that agree with
-// the digits found so far, a prefix sum over the buckets, and the one bucket in which the running sum passes thr is
-// the next digit. Weights are added as two 32-bit halves (the carry out of the lower half is seen in the value the
-// atomic returns), which keeps every atomic a native one. Called by all threads of the block.
-template <bool BY_WEIGHT, typename T, typename F>
-__device__ __forceinline__ Picked list_select(unsigned int n_list, int bits, T&& thr_of, F&& xg, unsigned int* h_n,
-                                              unsigned int* h_lo, unsigned int* h_hi, unsigned long long* s_pick,
-                                              unsigned int* s_n, unsigned long long* s_w, int& turn) {
+// The bucket in which the running count (by_weight: weight), on top of `carry`, passes thr_of(total of all buckets): the first
+// b with carry + sum(0 .. b) > thr. Summed over the histograms of n_peers blocks from first_peer on; left in sh.pick as well
+// ([0] bucket or all ones, [1] [2] in front of it, [3] [4] in it, [5] [6] of everything, [7] the threshold). Called by all threads of one block.
+template <typename T>
+__device__ __forceinline__ Picked hist_pick(FiltShared& sh, uint32_t first_peer, uint32_t n_peers, CountMass carry, bool by_weight, int& turn, T&& thr_of) {
+    constexpr int kPer = kFiltBuckets / kFiltThreads;  // 8 consecutive buckets per thread
+    static_assert(kPer == 8, "two 16-byte reads per array");
     const int tid = threadIdx.x;
-    const int rounds = bits <= 10 ? 1 : (bits + 9) / 10;
-    constexpr int kPer = kSelBuckets / kSelThreads;
-    static_assert(kPer == 4 && kSelBuckets == kFiltThreads, "one bucket per thread to clear, four per summing thread");
-    unsigned long long prefix = 0ull, thr = 0ull;
-    CountMass carry{0u, 0ull}, at{0u, 0ull};  // carry: the entries below the digits found so far
-    for (int rd = rounds - 1; rd >= 0; --rd) {
-        const int shift = rd * 10;
-        unsigned long long* pick = s_pick + 5 * (rd & 1);
-        h_n[tid] = 0u;
-        h_lo[tid] = 0u;
-        h_hi[tid] = 0u;
-        __syncthreads();
-        if (tid == 0) {  // (what stands if no bucket qualifies: cannot happen under the caller's guarantee)
-            pick[0] = 0ull;
-            pick[1] = carry.n;
-            pick[2] = carry.w;
-            pick[3] = 0ull;
-            pick[4] = 0ull;
-        }
-        for (unsigned int i = tid; i < n_list; i += kFiltThreads) {
-            uint32_t x;
-            unsigned int gn;
-            unsigned long long gw;
-            xg(i, x, gn, gw);
-            if ((gn != 0u || gw != 0ull) && (static_cast<unsigned long long>(x) >> (shift + 10)) == prefix) {
-                const uint32_t b = (x >> shift) & (kSelBuckets - 1);
-                if (gn) atomicAdd(&h_n[b], gn);
-                if (gw) {
-                    const uint32_t lo = static_cast<uint32_t>(gw);
-                    uint32_t hi = static_cast<uint32_t>(gw >> 32);
-                    if (lo) {
-                        const uint32_t old = atomicAdd(&h_lo[b], lo);
-                        hi += (old + lo) < old ? 1u : 0u;
-                    }
-                    if (hi) atomicAdd(&h_hi[b], hi);
-                }
-            }
-        }
-        __syncthreads();
-        if (tid < kSelThreads) {
-            const uint4 vn = reinterpret_cast<const uint4*>(h_n)[tid];
-            const uint4 vl = reinterpret_cast<const uint4*>(h_lo)[tid];
-            const uint4 vh = reinterpret_cast<const uint4*>(h_hi)[tid];
-            const CountMass h[kPer] = {{vn.x, (static_cast<unsigned long long>(vh.x) << 32) | vl.x},
-                                       {vn.y, (static_cast<unsigned long long>(vh.y) << 32) | vl.y},
-                                       {vn.z, (static_cast<unsigned long long>(vh.z) << 32) | vl.z},
-                                       {vn.w, (static_cast<unsigned long long>(vh.w) << 32) | vl.w}};
-            CountMass mine{0u, 0ull}, total;
+    unsigned int n[kPer];
+    unsigned long long w[kPer];
 #pragma unroll
-            for (int b = 0; b < kPer; ++b) {
-                mine.n += h[b].n;
-                mine.w += h[b].w;
-            }
-            CountMass run = sel_exclusive_scan(mine, s_n, s_w, turn, total);
-            if (rd == rounds - 1) {  // the first round sees every entry
-                thr = thr_of(total);
-                if (tid == 0) {
-                    s_pick[10] = thr;
-                    s_pick[11] = total.n;
-                    s_pick[12] = total.w;
-                }
-            }
-            run.n += carry.n;
-            run.w += carry.w;
-#pragma unroll
-            for (int b = 0; b < kPer; ++b) {
-                const unsigned long long below = BY_WEIGHT ? run.w : static_cast<unsigned long long>(run.n);
-                const unsigned long long here = BY_WEIGHT ? h[b].w : static_cast<unsigned long long>(h[b].n);
-                if (below <= thr && thr < below + here) {
-                    pick[0] = static_cast<unsigned long long>(tid * kPer + b);
-                    pick[1] = run.n;
-                    pick[2] = run.w;
-                    pick[3] = h[b].n;
-                    pick[4] = h[b].w;
-                }
-                run.n += h[b].n;
-                run.w += h[b].w;
-            }
-        }
-        __syncthreads();
-        prefix = (prefix << 10) | pick[0];
-        carry = CountMass{static_cast<unsigned int>(pick[1]), pick[2]};
-        at = CountMass{static_cast<unsigned int>(pick[3]), pick[4]};
+    for (int b = 0; b < kPer; ++b) {
+        n[b] = 0u;
+        w[b] = 0ull;
     }
-    return Picked{static_cast<uint32_t>(prefix), carry, at, CountMass{static_cast<unsigned int>(s_pick[11]), s_pick[12]}, s_pick[10]};
+    for (uint32_t p = first_peer; p < first_peer + n_peers; ++p) {
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            const int at = tid * kPer + half * 4;
+            const uint4 vn = ld_peer_v4(peer_shared(sh.hist.n + at, p)), vl = ld_peer_v4(peer_shared(sh.hist.lo + at, p)),
+                        vh = ld_peer_v4(peer_shared(sh.hist.hi + at, p));
+            const unsigned int nn[4] = {vn.x, vn.y, vn.z, vn.w}, ll[4] = {vl.x, vl.y, vl.z, vl.w}, hh[4] = {vh.x, vh.y, vh.z, vh.w};
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                n[half * 4 + b] += nn[b];
+                w[half * 4 + b] += (static_cast<unsigned long long>(hh[b]) << 32) | ll[b];
+            }
+        }
+    }
+    CountMass mine{0u, 0ull}, total;
+#pragma unroll
+    for (int b = 0; b < kPer; ++b) mine += CountMass{n[b], w[b]};
+    if (tid == 0) sh.pick[0] = ~0ull;
+    CountMass run = filt_scan(mine, sh, turn, total);  // (its barrier also orders the line above before the writes below)
+    const unsigned long long thr = thr_of(total);
+    if (tid == 0) {
+        sh.pick[5] = total.n;
+        sh.pick[6] = total.w;
+        sh.pick[7] = thr;
+    }
+    run += carry;
+#pragma unroll
+    for (int b = 0; b < kPer; ++b) {
+        const unsigned long long below = by_weight ? run.w : run.n, here = by_weight ? w[b] : n[b];
+        if (below <= thr && thr < below + here) {
+            sh.pick[0] = static_cast<unsigned long long>(tid * kPer + b);
+            sh.pick[1] = run.n;
+            sh.pick[2] = run.w;
+            sh.pick[3] = n[b];
+            sh.pick[4] = w[b];
+        }
+        run += CountMass{n[b], w[b]};
+    }
+    __syncthreads();
+    return Picked{static_cast<uint32_t>(sh.pick[0]), sh.pick[0] != ~0ull, CountMass{static_cast<unsigned int>(sh.pick[1]), sh.pick[2]},
+                  CountMass{static_cast<unsigned int>(sh.pick[3]), sh.pick[4]}, total};
 }
 
-// One row per cluster of blocks (1, 2 or 4 of them: a short batch has fewer rows than the device has
-// multiprocessors). Every block looks for the candidates in its share of the row and writes them, through the
-// cluster's shared memory, into the list of the cluster's first block, which carries on alone.
+// top_p's share of a weight, rounded up; at least one unit so that one token is kept
+__device__ __forceinline__ unsigned long long filt_target(unsigned long long S, float top_p) {
+    const unsigned long long t = static_cast<unsigned long long>(ceil(static_cast<double>(S) * static_cast<double>(top_p)));
+    return t < 1ull ? 1ull : (t > S ? S : t);
+}
+// u times the kept weight, rounded down: the first token whose cumulative weight exceeds it is drawn
+__device__ __forceinline__ unsigned long long filt_threshold(unsigned long long S_kept, float u) {
+    const unsigned long long t = static_cast<unsigned long long>(static_cast<double>(u) * static_cast<double>(S_kept));
+    return t >= S_kept ? S_kept - 1ull : t;
+}
+
+// One row per cluster of blocks (1 to 8 of them: a short batch has fewer rows than the device has multiprocessors).
+// Every block goes over its share of the row; what they find meets in the shared memory of the cluster's first block.
 template <int DT>
-__global__ void __launch_bounds__(kFiltThreads) k_sample_filtered(const __grid_constant__ StepArgs a, int aligned, int top_k,
-                                                                  float top_p) {
-    extern __shared__ __align__(16) unsigned long long filt_smem[];
-    unsigned long long* const l_w = filt_smem;                                  // kFiltList weights
-    uint32_t* const l_key = reinterpret_cast<uint32_t*>(filt_smem + kFiltList);  // kFiltList keys
-    int* const l_id = reinterpret_cast<int*>(l_key + kFiltList);                 // kFiltList token ids
-    __shared__ unsigned int s_n[2 * kFiltThreads / 32];
-    __shared__ unsigned long long s_w[2 * kFiltThreads / 32];
-    __shared__ unsigned long long s_scan[kFiltThreads / 32];
-    __shared__ unsigned int s_sel_n[2 * kSelThreads / 32];  // the searches' own sets (only some threads sum there, so
-    __shared__ unsigned long long s_sel_w[2 * kSelThreads / 32];  // their turn must not be that of the block's sums)
-    int turn_sel = 0;
-    __shared__ __align__(16) unsigned int s_hn[kSelBuckets], s_hlo[kSelBuckets], s_hhi[kSelBuckets];
-    __shared__ unsigned long long s_pick[16];
-    __shared__ unsigned long long s_top_w[kSelThreads];  // the entries with key >= tau when there are few of them
-    __shared__ uint32_t s_top_key[kSelThreads];
-    __shared__ int s_top_id[kSelThreads];
-    __shared__ unsigned int s_top_n;
-    __shared__ float s_max[kFiltThreads / 32];
-    int turn = 0;
-    __shared__ unsigned int s_list_n[kFiltAttempts];  // candidates counted in each pass over the row
-    __shared__ unsigned int s_low_n[kFiltPeers];      // per block of the cluster: the tokens with weight that stayed
-    __shared__ unsigned long long s_low_w[kFiltPeers];  // below the bar of the last pass, and their weight
+__global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __grid_constant__ StepArgs a, int aligned, int top_k,
+                                                                     float top_p) {
+    extern __shared__ __align__(16) unsigned char filt_smem[];
+    FiltShared& sh = *reinterpret_cast<FiltShared*>(filt_smem);
     pdl_prologue();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t n_peers = cluster_blocks(), crank = cluster_rank();
@@ -2223,17 +2144,32 @@ __global__ void __launch_bounds__(kFiltThreads) k_sample_filtered(const __grid_c
         if (part < 0 || part >= a.n_parts || !a.parts[part].live || a.parts[part].V != a.V) return;  // counted by the step kernel
         P = a.parts[part];
     }
-    // the row maximum from the states the streaming kernel published
+    const float scale = a.scale;
+    // the run states the streaming kernel published: the row maximum, and the maxima and sums of up to four runs per
+    // thread for the bar of the short way (leaving runs out only lowers the bar)
     const Partial* src = row_slots(a, g, j);
+    const float u = __ldg(a.u + row);  // needed late
+    constexpr int kKeep = 4;
+    float run_m[kKeep], run_s[kKeep];
     float M = -INFINITY;
-    for (int k = tid; k < a.slots; k += kFiltThreads) M = fmaxf(M, __ldcg(&src[k].m));
+#pragma unroll
+    for (int q = 0; q < kKeep; ++q) {
+        const int k = tid + q * kFiltThreads;
+        int4 raw = make_int4(__float_as_int(-INFINITY), 0, 0, 0);
+        if (k < a.slots) raw = __ldcg(reinterpret_cast<const int4*>(src + k));
+        run_m[q] = __int_as_float(raw.x);
+        run_s[q] = __int_as_float(raw.y);
+        M = fmaxf(M, run_m[q]);
+    }
+    for (int k = tid + kKeep * kFiltThreads; k < a.slots; k += kFiltThreads) M = fmaxf(M, __ldcg(&src[k].m));
 #pragma unroll
     for (int d = 16; d >= 1; d >>= 1) M = fmaxf(M, __shfl_xor_sync(0xFFFFFFFFu, M, d));
-    if (lane == 0) s_max[warp] = M;
-    if (tid < kFiltAttempts) s_list_n[tid] = 0u;
+    if (lane == 0) sh.warp_max[warp] = M;
+    if (tid == 0) sh.list_n = 0u;
+    hist_clear(sh);
     __syncthreads();
 #pragma unroll
-    for (int w = 0; w < kFiltThreads / 32; ++w) M = fmaxf(M, s_max[w]);
+    for (int w = 0; w < kFiltWarps; ++w) M = fmaxf(M, sh.warp_max[w]);
     if (!(M > kRefFloor)) {
         // nothing allowed, or only -inf allowed: the lowest allowed token (if any) and -inf logs
         if (warp == 0 && crank == 0) {
@@ -2247,383 +2183,361 @@ __global__ void __launch_bounds__(kFiltThreads) k_sample_filtered(const __grid_c
         }
         return;
     }
+    auto write_draw = [&](int token, float zt, unsigned long long S_kept) {
+        const float l = logf(static_cast<float>(S_kept) * (1.f / kFixOne));
+        a.argmax[row] = token;
+        if (a.rep) a.rep[row] = __ldg(P.trep + token);
+        if (a.lse) a.lse[row] = fmaf(M, a.inv_t, l);
+        if (a.logp_argmax) a.logp_argmax[row] = (zt - M) * a.inv_t - l;
+    };
     constexpr int ES = DT == kBF16 ? 2 : 4;
     const char* rowp = reinterpret_cast<const char*>(a.logits) + int64_t(row) * a.row_stride * ES;
     // Rows are gone over eight tokens at a time from token -lead on, so that the eight are one vector of the row: a row
-    // that starts anywhere has `head` tokens in front of its first vector.
+    // that starts anywhere has `head` tokens in front of its first vector. A chunk is 256 tokens (more only where that
+    // would be more than kFiltChunks of them); every block of the cluster takes a run of chunks.
     const int head = a.shifted ? row_head<DT>(rowp, a.V) : 0, lead = (8 - head) & 7;
-    const float scale = a.scale;
+    const int pieces = (a.V + lead + 256 * kFiltChunks - 1) / (256 * kFiltChunks), chunk = 256 * pieces;
+    const int n_chunks = (a.V + lead + chunk - 1) / chunk, per_block = (n_chunks + int(n_peers) - 1) / int(n_peers);
+    const int c_begin = min(int(crank) * per_block, n_chunks), c_end = min(c_begin + per_block, n_chunks);
+    // A token takes part when its logit is at or above M - 41 / scale (below M - 40 / scale the fixed-point weight is zero;
+    // the extra unit covers the rounding of the threshold itself).
     const uint32_t key_max = logit_key<DT>(M);
-    // The candidates are the tokens at or above M - 41 / scale (below M - 40 / scale the fixed-point weight is zero;
-    // the extra unit covers the rounding of the threshold itself). The candidates of every block go straight into the
-    // list of the cluster's first block (places are reserved in its counter, a warp at a time). A comparison of
-    // floats decides (z_cut is the lowest logit whose key reaches key_list), and a round of eight logits is skipped as
-    // soon as its maximum falls short. When the list overflows (a flat row, or a mask that allows most of the
-    // vocabulary) the row is gone over again with the bar half as far below M; what carries weight below the bar is
-    // then only counted and summed (low): enough as long as top-k and top-p end inside the list.
-    const float z_zero = key_logit<DT>(logit_key<DT>(M - 41.f / scale));
-    uint32_t key_list = 0u;
-    unsigned int n_list = 0u;
-    int attempt = 0;
-    {
-        const uint32_t list_key0 = peer_shared(l_key, 0u), list_id0 = peer_shared(l_id, 0u);
-        const int share = ((a.V + lead + int(n_peers) - 1) / int(n_peers) + 7) & ~7;
-        const int t_begin = min(int(crank) * share - lead, a.V), t_end = min(t_begin + share, a.V);
+    const float z_zero = fmaxf(key_logit<DT>(logit_key<DT>(M - 41.f / scale)), kRefFloor);
+    const int bits = 32 - __clz(int(key_max - logit_key<DT>(z_zero)));  // of key_max - key
+    const int first_lo = max(0, bits - kFiltBits);
+    auto offset_of = [&](float z) { return key_max - logit_key<DT>(z); };
+    int turn = 0;
+    // Visit the share eight tokens at a time, four rounds of loads in flight; f gets the first token and its eight logits.
+    auto visit = [&](float at_least, auto&& f) {
         constexpr int kInFlight = 4;
-        float units = 41.f;
-        cluster_barrier();  // the first block's counters are cleared before anybody adds to them
-        for (;; ++attempt, units *= 0.5f) {
-            key_list = logit_key<DT>(M - units / scale);
-            const float z_cut = key_logit<DT>(key_list);
-            const uint32_t list_n0 = peer_shared(&s_list_n[attempt], 0u);
-            CountMass low{0u, 0ull};
-            // (the loop bound is the same for the lanes of a warp: they reserve their places in the list together)
-            for (int tw = t_begin + warp * 256; tw < t_end; tw += kFiltThreads * 8 * kInFlight) {
-                const int t0 = tw + lane * 8;
-                float e[kInFlight][8];
+        const int t_end = min(c_end * chunk - lead, a.V);
+        for (int t0 = c_begin * chunk - lead + tid * 8; t0 < t_end; t0 += kFiltThreads * 8 * kInFlight) {
+            float e[kInFlight][8];
 #pragma unroll
-                for (int r = 0; r < kInFlight; ++r) load_eight<DT>(rowp, t0 + r * kFiltThreads * 8, t_end, aligned != 0, e[r]);
-                uint32_t cand = 0u;  // bit 8 r + q: logit q of round r is a candidate
+            for (int r = 0; r < kInFlight; ++r) load_eight<DT>(rowp, t0 + r * kFiltThreads * 8, t_end, aligned != 0, e[r]);
 #pragma unroll
-                for (int r = 0; r < kInFlight; ++r) {
-                    const float top = fmax3(fmax3(e[r][0], e[r][1], e[r][2]), fmax3(e[r][3], e[r][4], e[r][5]), fmaxf(e[r][6], e[r][7]));
-                    if (top >= z_cut) {
+            for (int r = 0; r < kInFlight; ++r)
+                if (max_eight(e[r]) >= at_least) f(t0 + r * kFiltThreads * 8, e[r]);
+        }
+    };
+
+    // ---- the short way
+    bool brief = top_k <= kFiltList / 2;
+    if (brief) {
+        float sum = 0.f;
 #pragma unroll
-                        for (int q = 0; q < 8; ++q) cand |= e[r][q] >= z_cut ? 1u << (8 * r + q) : 0u;
-                    }
-                    if (attempt > 0 && top >= z_zero) {
-#pragma unroll
-                        for (int q = 0; q < 8; ++q)
-                            if (e[r][q] >= z_zero && e[r][q] < z_cut) {
-                                low.n += 1u;
-                                low.w += fixed_weight(e[r][q], M, scale);
-                            }
-                    }
+        for (int q = 0; q < kKeep; ++q)
+            if (run_m[q] >= z_zero) {
+                const unsigned long long w = top_k > 0 ? 0ull : fixed_weight(run_m[q], M, scale);
+                hist_add(sh, offset_of(run_m[q]) >> first_lo, w);
+                sum += run_s[q] * ex2f((run_m[q] - M) * scale);
+            }
+        // (for top-p the weight of all tokens is not known exactly yet: the run sums give it to about 1e-5, the bar allows 1e-3)
+        __syncthreads();
+        unsigned long long goal = static_cast<unsigned long long>(max(top_k, 1)) - 1ull;
+        if (top_k == 0) {
+            CountMass all;
+            filt_scan(CountMass{0u, __float2ull_rz(sum * kFixOne)}, sh, turn, all);
+            goal = static_cast<unsigned long long>(static_cast<double>(all.w) * top_p * 1.001);
+        }
+        const Picked bar = hist_pick(sh, crank, 1u, CountMass{0u, 0ull}, top_k == 0, turn, [&](CountMass) { return goal; });
+        brief = bar.found || top_k > 0;  // (fewer runs with a token than top_k: collect every token)
+        if (brief) {
+            const unsigned long long lowest =
+                bar.found ? ((static_cast<unsigned long long>(bar.bucket) + 1ull) << first_lo) - 1ull : ~0ull;
+            const float z_bar = lowest < offset_of(z_zero) ? key_logit<DT>(key_max - uint32_t(lowest)) : z_zero;
+            const uint32_t list0 = peer_shared(sh.list, 0u), list_n0 = peer_shared(&sh.list_n, 0u);
+            unsigned long long mine = 0ull;
+            cluster_barrier();  // the first block is done with its buckets, which the list shares the space of
+            auto push = [&](int t, float z) {
+                const unsigned int at = add_peer_u32(list_n0, 1u);
+                if (at < kFiltList) {
+                    st_peer_u32(list0 + at * 16u, __float_as_uint(z));
+                    st_peer_u32(list0 + at * 16u + 4u, uint32_t(t));
                 }
-                const int cnt = __popc(cand);
-                int inc = cnt;
-#pragma unroll
-                for (int d = 1; d < 32; d <<= 1) {
-                    const int up = __shfl_up_sync(0xFFFFFFFFu, inc, d);
-                    if (lane >= d) inc += up;
-                }
-                const int warp_cnt = __shfl_sync(0xFFFFFFFFu, inc, 31);
-                if (warp_cnt == 0) continue;
-                unsigned int base = 0u;
-                if (lane == 31) base = add_peer_u32(list_n0, unsigned(warp_cnt));
-                base = __shfl_sync(0xFFFFFFFFu, base, 31);
-                unsigned int at = base + unsigned(inc - cnt);
-#pragma unroll
-                for (int r = 0; r < kInFlight; ++r)
+            };
+            if (top_k > 0) {
+                visit(z_bar, [&](int t0, const float (&e)[8]) {
 #pragma unroll
                     for (int q = 0; q < 8; ++q)
-                        if ((cand >> (8 * r + q)) & 1u) {
-                            if (at < kFiltList) {  // (key and weight follow below, for the listed logits only)
-                                st_peer_u32(list_key0 + at * 4u, __float_as_uint(e[r][q]));
-                                st_peer_u32(list_id0 + at * 4u, uint32_t(t0 + r * kFiltThreads * 8 + q));
-                            }
-                            ++at;
+                        if (e[q] >= z_bar) push(t0 + q, e[q]);
+                });
+            } else {
+                visit(z_zero, [&](int t0, const float (&e)[8]) {
+#pragma unroll
+                    for (int q = 0; q < 8; ++q)
+                        if (e[q] >= z_zero) {
+                            mine += fixed_weight(e[q], M, scale);
+                            if (e[q] >= z_bar) push(t0 + q, e[q]);
                         }
+                });
+                CountMass all;
+                filt_scan(CountMass{0u, mine}, sh, turn, all);
+                if (tid == 0) st_peer_u64(peer_shared(&sh.peer_w[crank], 0u), all.w);
             }
-            if (attempt > 0) {
-                const CountMass mine = block_sum(low, s_n, s_w, turn);
-                if (tid == 0) {
-                    st_peer_u32(peer_shared(&s_low_n[crank], 0u), mine.n);
-                    st_peer_u64(peer_shared(&s_low_w[crank], 0u), mine.w);
+            cluster_barrier();  // every block's tokens have arrived
+            const unsigned int n = ld_peer_u32(list_n0);  // (the same in every block of the cluster)
+            if (n <= unsigned(kFiltList)) {
+                cluster_arrive();  // this thread has read the first block's count
+                if (crank != 0u) {
+                    cluster_wait();
+                    return;
                 }
+                // A thread per token: its place in the order and the weight in front of it, then its place in token order.
+                const bool have = unsigned(tid) < n;
+                uint4 me = make_uint4(0u, 0u, 0u, 0u);
+                unsigned long long my_w = 0ull;
+                float my_z = 0.f;
+                if (have) {
+                    me = sh.list[tid];
+                    my_z = __uint_as_float(me.x);
+                    my_w = fixed_weight(my_z, M, scale);
+                    me.x = logit_key<DT>(my_z);
+                    sh.list[tid] = make_uint4(me.x, me.y, uint32_t(my_w), uint32_t(my_w >> 32));
+                }
+                __syncthreads();
+                CountMass front{0u, 0ull};
+                const unsigned int last = (top_k > 0 ? min(unsigned(top_k), n) : n) - 1u;
+                if (have) {
+                    for (unsigned int k = 0; k < n; ++k) {
+                        const uint4 o = sh.list[k];
+                        if (o.x > me.x || (o.x == me.x && o.y < me.y))
+                            front += CountMass{1u, (static_cast<unsigned long long>(o.w) << 32) | o.z};
+                    }
+                    if (front.n == last) sh.topk_w = front.w + my_w;
+                }
+                __syncthreads();
+                unsigned long long S = sh.topk_w;
+                if (top_k == 0) {
+                    S = 0ull;
+                    for (uint32_t p = 0; p < n_peers; ++p) S += sh.peer_w[p];
+                }
+                const unsigned long long target = top_p < 1.f ? filt_target(S, top_p) : ~0ull;
+                const bool kept = have && front.n <= last && front.w < target;
+                if (kept && (front.n == last || front.w + my_w >= target)) sh.kept_w = front.w + my_w;
+                if (have && !kept) sh.list[tid] = make_uint4(me.x, me.y, 0u, 0u);
+                __syncthreads();
+                cluster_wait();  // (long since complete: no block may leave while another reads its shared memory)
+                if (!kept) return;
+                const unsigned long long S_kept = sh.kept_w, thr = filt_threshold(S_kept, u);
+                unsigned long long cum = 0ull;
+                for (unsigned int k = 0; k < n; ++k) {
+                    const uint4 o = sh.list[k];
+                    cum += o.y <= me.y ? (static_cast<unsigned long long>(o.w) << 32) | o.z : 0ull;
+                }
+                if (my_w > 0ull && cum - my_w <= thr && thr < cum) write_draw(int(me.y), key_logit<DT>(me.x), S_kept);
+                return;
             }
-            cluster_barrier();  // every block's candidates have arrived
-            n_list = ld_peer_u32(list_n0);
-            if (n_list <= kFiltList || attempt == kFiltAttempts - 1) break;  // (the same in every block of the cluster)
         }
     }
-    if (crank != 0u) return;  // (the first block touches no other block's memory from here on)
-    for (unsigned int i = tid; i < min(n_list, unsigned(kFiltList)); i += kFiltThreads) {
-        const float z = __uint_as_float(l_key[i]);
-        l_key[i] = logit_key<DT>(z);
-        l_w[i] = fixed_weight(z, M, scale);
-    }
-    __syncthreads();
-    const bool list_whole = n_list <= kFiltList;
-    CountMass low{0u, 0ull};  // what carries weight and is not in the list
-    if (attempt > 0)
-        for (uint32_t p = 0; p < n_peers; ++p) {
-            low.n += s_low_n[p];
-            low.w += s_low_w[p];
-        }
 
-    // kept: { key > tau } and the first m tokens, in token order, with key == tau; S their weight
-    uint32_t tau = 0u;
-    unsigned int m = 0xFFFFFFFFu;
-
-    if (list_whole) do {
-        // ---- everything from the list (it holds the tokens that carry weight, or the heaviest of them, in no
-        // particular order); leaves for the passes over the row below when top-k or top-p reach past the list
-        auto select = [&](auto kind, int bits, auto&& thr_of, auto&& xg) {
-            return list_select<decltype(kind)::value>(n_list, bits, thr_of, xg, s_hn, s_hlo, s_hhi, s_pick, s_sel_n, s_sel_w, turn_sel);
-        };
-        const std::integral_constant<bool, false> by_count;
-        const std::integral_constant<bool, true> by_weight;
-        // keys from the top: x = key_max - key, below 2^key_bits
-        const int key_bits = 32 - __clz(key_max - key_list);
-        auto from_top = [&](unsigned int i, uint32_t& x, unsigned int& gn, unsigned long long& gw) {
-            x = key_max - l_key[i];
-            gn = 1u;
-            gw = l_w[i];
-        };
-        // the target of top-p: that share of the weight kept so far, rounded up; at least one unit so that one token is kept
-        auto target_of = [&](unsigned long long S) {
-            const unsigned long long t = static_cast<unsigned long long>(ceil(static_cast<double>(S) * static_cast<double>(top_p)));
-            return t < 1ull ? 1ull : (t > S ? S : t);
-        };
-        unsigned long long S = 0ull;        // weight of what is kept so far (once something has been cut)
-        unsigned long long w_above = 0ull;  // weight of the tokens with key > tau
-        unsigned int n_above = 0u;          // their number
-        unsigned int n_ties = 0u;           // tokens with key == tau
-        unsigned long long w_tie = 0ull;    // weight of each of them
-        bool cut = false;
-        // (a top_k beyond everything that carries weight only adds tokens of weight zero: nothing to do)
-        if (top_k > 0 && unsigned(top_k) >= n_list && unsigned(top_k) - n_list < low.n) break;  // ends below the list
-        if (top_k > 0 && unsigned(top_k) < n_list) {
-            // the largest key with at least top_k entries at or above it
-            const Picked pk = select(by_count, key_bits, [&](CountMass) { return static_cast<unsigned long long>(top_k) - 1ull; },
-                                     from_top);
-            tau = key_max - pk.x;
-            m = unsigned(top_k) - pk.before.n;
-            n_ties = pk.at.n;
-            w_tie = fixed_weight(key_logit<DT>(tau), M, scale);
-            w_above = pk.before.w;
-            n_above = pk.before.n;
-            S = w_above + static_cast<unsigned long long>(m) * w_tie;
-            cut = true;
-        }
-        if (top_p < 1.f) {
-            const unsigned long long target = cut ? target_of(S) : 0ull;
-            if (!cut || w_above >= target) {
-                // the largest key whose entries, with those above it, reach the target (without a cut so far the target
-                // follows from the weight of the whole list, which the search sums on its way)
-                const Picked pk = select(by_weight, key_bits,
-                                         [&](CountMass all) { return (cut ? target : target_of(all.w + low.w)) - 1ull; }, from_top);
-                const unsigned long long tgt = pk.thr + 1ull;
-                if (pk.all.w < tgt) break;  // the list does not hold the target (only possible with tokens left below it)
-                tau = key_max - pk.x;
-                w_tie = fixed_weight(key_logit<DT>(tau), M, scale);
-                w_above = pk.before.w;
-                n_above = pk.before.n;
-                n_ties = pk.at.n;
-                unsigned int need = n_ties;  // all the ties unless fewer reach the target
-                if (w_tie > 0ull) {
-                    const unsigned long long q = (tgt - w_above + w_tie - 1ull) / w_tie;
-                    if (q < need) need = unsigned(q);
-                }
-                m = need < 1u ? 1u : need;
-                cut = true;
-            } else if (w_tie > 0ull) {
-                // the target is reached among the ties at tau itself
-                const unsigned long long q = (target - w_above + w_tie - 1ull) / w_tie;
-                if (q < m) m = unsigned(q < 1ull ? 1ull : q);
-            }
-        }
-        // The ties that are kept are those with the m lowest ids; the drawn token is the lowest id t with
-        // (kept weight at ids <= t) > floor(u * kept weight). All ties weigh the same, so the kept weight needs no pass.
-        if (!cut && low.n > 0u) break;  // nothing is cut away: the draw is over the whole row
-        const float u = __ldg(a.u + row);
-        auto threshold_of = [&](unsigned long long S_kept) {  // (S_kept > 0: the row maximum is always kept)
-            const unsigned long long t = static_cast<unsigned long long>(static_cast<double>(u) * static_cast<double>(S_kept));
-            return t >= S_kept ? S_kept - 1ull : t;
-        };
-        if (cut && n_above + n_ties <= unsigned(kSelThreads)) {
-            // Few tokens at or above tau (the rule with top-k, and with top-p on a peaked distribution): one per thread,
-            // and every thread sums over all of them: the ties below its id for its rank, the kept weight up to its id
-            // for its place in the cumulative distribution.
-            const unsigned long long S_kept = w_above + static_cast<unsigned long long>(min(m, n_ties)) * w_tie;
-            const unsigned long long thr = threshold_of(S_kept);
-            const unsigned int n_top = n_above + n_ties;
-            if (tid == 0) s_top_n = 0u;
-            __syncthreads();
-            for (unsigned int i = tid; i < n_list; i += kFiltThreads)
-                if (l_key[i] >= tau) {
-                    const unsigned int at = atomicAdd(&s_top_n, 1u);
-                    s_top_key[at] = l_key[i];
-                    s_top_id[at] = l_id[i];
-                    s_top_w[at] = l_w[i];
-                }
-            __syncthreads();
-            if (tid >= kSelThreads) return;
-            const bool have = unsigned(tid) < n_top;
-            const int my_id = have ? s_top_id[tid] : a.V;
-            const uint32_t my_key = have ? s_top_key[tid] : 0u;
-            unsigned long long my_w = have ? s_top_w[tid] : 0ull;
-            if (m < n_ties) {
-                unsigned int rank = 0u;
-                for (unsigned int k = 0; k < n_top; ++k) rank += (s_top_key[k] == tau && s_top_id[k] < my_id) ? 1u : 0u;
-                if (have && my_key == tau && rank >= m) {
-                    my_w = 0ull;
-                    s_top_w[tid] = 0ull;  // (read by the others only after the barrier below)
-                }
-            }
-            sel_sync();
-            unsigned long long cum = 0ull;
-            for (unsigned int k = 0; k < n_top; ++k) cum += s_top_id[k] <= my_id ? s_top_w[k] : 0ull;
-            if (my_w > 0ull && cum - my_w <= thr && thr < cum) {  // the one thread that holds the drawn token
-                const float l = logf(static_cast<float>(S_kept) * (1.f / kFixOne));
-                const float zt = key_logit<DT>(my_key);
-                a.argmax[row] = my_id;
-                if (a.rep) a.rep[row] = __ldg(P.trep + my_id);
-                if (a.lse) a.lse[row] = fmaf(M, a.inv_t, l);
-                if (a.logp_argmax) a.logp_argmax[row] = (zt - M) * a.inv_t - l;
-            }
-            return;
-        }
-        const int id_bits = 32 - __clz(max(a.V - 1, 1));
-        int id_cut = a.V;  // the kept ties are those with ids up to id_cut
-        if (cut && m < n_ties)
-            id_cut = int(select(by_count, id_bits, [&](CountMass) { return static_cast<unsigned long long>(m) - 1ull; },
-                                [&](unsigned int i, uint32_t& x, unsigned int& gn, unsigned long long& gw) {
-                                    x = uint32_t(l_id[i]);
-                                    gn = l_key[i] == tau ? 1u : 0u;
-                                    gw = 0ull;
-                                })
-                             .x);
-        // (the kept weight is the weight of everything that takes part in the search for the token)
-        const Picked drawn = select(by_weight, id_bits, [&](CountMass all) { return threshold_of(all.w); },
-                                    [&](unsigned int i, uint32_t& x, unsigned int& gn, unsigned long long& gw) {
-                                        const uint32_t key = l_key[i];
-                                        const int id = l_id[i];
-                                        x = uint32_t(id);
-                                        gn = 0u;
-                                        gw = (!cut || key > tau || (key == tau && id <= id_cut)) ? l_w[i] : 0ull;
-                                    });
-        const int token = int(drawn.x);
-        const float l = logf(static_cast<float>(drawn.all.w) * (1.f / kFixOne));
-        for (unsigned int i = tid; i < n_list; i += kFiltThreads)
-            if (l_id[i] == token) {  // the one thread that holds the drawn token writes the row's results
-                const float zt = key_logit<DT>(l_key[i]);
-                a.argmax[row] = token;
-                if (a.rep) a.rep[row] = __ldg(P.trep + token);
-                if (a.lse) a.lse[row] = fmaf(M, a.inv_t, l);
-                if (a.logp_argmax) a.logp_argmax[row] = (zt - M) * a.inv_t - l;
-            }
-        return;
-    } while (false);
-
-    // ---- the list does not reach (a flat distribution): counts and weights come from passes over the row, tau by
-    // bisection on the key
-    tau = 0u;
-    m = 0xFFFFFFFFu;
-    auto above = [&](uint32_t lo) {  // (count, weight) of the tokens with key >= lo
-        CountMass v{0u, 0ull};
-        row_visit<DT>(rowp, lead, a.V, aligned != 0, [&](int, float z) {
-            if (logit_key<DT>(z) >= lo) {
-                v.n += 1u;
-                v.w += fixed_weight(z, M, scale);
-            }
-        });
-        return block_sum(v, s_n, s_w, turn);
+    // ---- the long way: tau and m
+    // The largest key whose tokens, with those above it, together count (by_weight: weigh) more than thr_of(everything).
+    struct Cut {
+        bool found;
+        uint32_t key;
+        CountMass above, ties, all;
+        unsigned long long thr;
     };
-    const CountMass all = above(0u);
-    unsigned long long S = all.w;
-    if (top_k > 0 && unsigned(top_k) < all.n) {
-        uint32_t lo = 0u, hi = key_max;  // count(>= lo) >= top_k holds
-        while (lo < hi) {
-            const uint32_t mid = lo + (hi - lo + 1u) / 2u;
-            if (above(mid).n >= unsigned(top_k)) lo = mid; else hi = mid - 1u;
-        }
-        tau = lo;
-        const CountMass gt = tau == key_max ? CountMass{0u, 0ull} : above(tau + 1u);
-        m = unsigned(top_k) - gt.n;
-        S = gt.w + static_cast<unsigned long long>(m) * fixed_weight(key_logit<DT>(tau), M, scale);
-    }
-    if (top_p < 1.f) {
-        unsigned long long target = static_cast<unsigned long long>(ceil(static_cast<double>(S) * static_cast<double>(top_p)));
-        target = target < 1ull ? 1ull : (target > S ? S : target);
-        const CountMass gt_tau = tau >= key_max ? CountMass{0u, 0ull} : above(tau + 1u);
-        if (gt_tau.w >= target) {
-            uint32_t lo = tau + 1u, hi = key_max;  // weight(>= lo) >= target holds
-            while (lo < hi) {
-                const uint32_t mid = lo + (hi - lo + 1u) / 2u;
-                if (above(mid).w >= target) lo = mid; else hi = mid - 1u;
-            }
-            const CountMass ge = above(lo);
-            const CountMass gt = lo == key_max ? CountMass{0u, 0ull} : above(lo + 1u);
-            const unsigned long long w_tie = fixed_weight(key_logit<DT>(lo), M, scale);
-            unsigned int need = ge.n - gt.n;
-            if (w_tie > 0ull) {
-                const unsigned long long q = (target - gt.w + w_tie - 1ull) / w_tie;
-                if (q < need) need = unsigned(q);
-            }
-            tau = lo;
-            m = need < 1u ? 1u : need;
-        } else {
-            const unsigned long long w_tie = fixed_weight(key_logit<DT>(tau), M, scale);
-            if (w_tie > 0ull) {
-                const unsigned long long q = (target - gt_tau.w + w_tie - 1ull) / w_tie;
-                if (q < m) m = unsigned(q < 1ull ? 1ull : q);
-            }
-        }
-    }
-
-    // Draw in token order. Every thread owns one contiguous segment of the row: first the ties per segment (their
-    // rank decides which of them are kept), then the kept weight per segment, then the one thread whose segment
-    // holds the crossing walks it once more.
-    const int seg = ((a.V + lead + kFiltThreads - 1) / kFiltThreads + 7) & ~7;
-    const int t_lo = min(tid * seg - lead, a.V), t_hi = min(t_lo + seg, a.V);
-    auto seg_visit = [&](auto&& f) {
-        for (int t0 = t_lo; t0 < t_hi; t0 += 32) {
-            float e[4][8];
-#pragma unroll
-            for (int r = 0; r < 4; ++r) load_eight<DT>(rowp, t0 + 8 * r, t_hi, aligned != 0, e[r]);
-#pragma unroll
-            for (int r = 0; r < 4; ++r)
+    auto search = [&](bool by_weight, auto&& thr_of) {
+        Cut cut{};
+        unsigned long long prefix = 0ull;
+        int hi = bits;
+        bool first = true;
+        do {
+            const int lo = first ? first_lo : max(0, hi - kFiltBits);
+            __syncthreads();
+            hist_clear(sh);
+            __syncthreads();
+            visit(z_zero, [&](int, const float (&e)[8]) {
 #pragma unroll
                 for (int q = 0; q < 8; ++q)
-                    if (e[r][q] > kRefFloor) f(t0 + 8 * r + q, e[r][q]);
-        }
+                    if (e[q] >= z_zero) {
+                        const unsigned long long x = offset_of(e[q]);
+                        if ((x >> hi) == prefix)
+                            hist_add(sh, uint32_t(x >> lo) & ((1u << (hi - lo)) - 1u), fixed_weight(e[q], M, scale));
+                    }
+            });
+            cluster_barrier();
+            if (crank == 0u) {
+                hist_pick(sh, 0u, n_peers, cut.above, by_weight, turn, [&](CountMass all) { return first ? thr_of(all) : cut.thr; });
+                for (int i = tid; i < 8 * int(n_peers - 1u); i += kFiltThreads)
+                    st_peer_u64(peer_shared(&sh.pick[i & 7], 1u + uint32_t(i >> 3)), sh.pick[i & 7]);
+            }
+            cluster_barrier();
+            if (first) {
+                cut.thr = sh.pick[7];
+                cut.all = CountMass{static_cast<unsigned int>(sh.pick[5]), sh.pick[6]};
+                cut.found = sh.pick[0] != ~0ull;
+                if (!cut.found) return cut;
+            }
+            prefix = (prefix << (hi - lo)) | sh.pick[0];
+            cut.above = CountMass{static_cast<unsigned int>(sh.pick[1]), sh.pick[2]};
+            cut.ties = CountMass{static_cast<unsigned int>(sh.pick[3]), sh.pick[4]};
+            hi = lo;
+            first = false;
+        } while (hi > 0);
+        cut.key = key_max - uint32_t(prefix);
+        return cut;
     };
-    unsigned long long my_ties = 0ull;
-    seg_visit([&](int, float z) { my_ties += logit_key<DT>(z) == tau ? 1ull : 0ull; });
-    unsigned long long total_ties;
-    const unsigned long long tie_base = block_exclusive_scan_u64(my_ties, s_scan, total_ties);
-    unsigned long long my_w = 0ull, ties_seen = tie_base;
-    seg_visit([&](int, float z) {
-        const uint32_t key = logit_key<DT>(z);
-        if (key > tau || (key == tau && ties_seen++ < m)) my_w += fixed_weight(z, M, scale);
-    });
-    unsigned long long S_drawn;
-    const unsigned long long w_base = block_exclusive_scan_u64(my_w, s_scan, S_drawn);
-    // u * S rounded down: the first token whose cumulative weight exceeds it is drawn
-    const float u = __ldg(a.u + row);
-    unsigned long long thr = static_cast<unsigned long long>(static_cast<double>(u) * static_cast<double>(S_drawn));
-    if (S_drawn > 0ull && thr >= S_drawn) thr = S_drawn - 1ull;
-    if (S_drawn == 0ull) {  // cannot happen while the row maximum is kept; reported as an empty row
-        if (tid == 0) {
-            a.argmax[row] = -1;
-            if (a.rep) a.rep[row] = -1;
-            if (a.lse) a.lse[row] = -INFINITY;
-            if (a.logp_argmax) a.logp_argmax[row] = -INFINITY;
+    uint32_t tau = 0u;
+    unsigned int m = 0xFFFFFFFFu, n_ties = 0u;
+    unsigned long long w_tie = 0ull, w_above = 0ull, S = 0ull;
+    bool cut = false;
+    auto take = [&](const Cut& c) {
+        tau = c.key;
+        w_tie = fixed_weight(key_logit<DT>(tau), M, scale);
+        w_above = c.above.w;
+        n_ties = c.ties.n;
+        cut = true;
+    };
+    auto ties_for = [&](unsigned long long target, unsigned int most) {  // how many ties reach the target, at least one
+        if (w_tie == 0ull) return most;
+        const unsigned long long q = (target - w_above + w_tie - 1ull) / w_tie;
+        return q < most ? unsigned(q < 1ull ? 1ull : q) : max(most, 1u);
+    };
+    if (top_k > 0) {
+        const Cut c = search(false, [&](CountMass) { return static_cast<unsigned long long>(top_k) - 1ull; });
+        if (c.found) {  // (a top_k beyond everything that carries weight cuts nothing away)
+            take(c);
+            m = unsigned(top_k) - c.above.n;
+            S = w_above + static_cast<unsigned long long>(m) * w_tie;
         }
-        return;
     }
-    if (my_w > 0ull && w_base <= thr && thr < w_base + my_w) {
-        unsigned long long cum = w_base;
-        int token = -1;
-        float zt = 0.f;
-        ties_seen = tie_base;
-        seg_visit([&](int t, float z) {
-            const uint32_t key = logit_key<DT>(z);
-            if (key > tau || (key == tau && ties_seen++ < m)) {
-                cum += fixed_weight(z, M, scale);
-                if (token < 0 && cum > thr) {
-                    token = t;
-                    zt = z;
+    if (top_p < 1.f) {
+        const unsigned long long target = cut ? filt_target(S, top_p) : 0ull;
+        if (!cut || w_above >= target) {
+            const Cut c = search(true, [&](CountMass all) { return (cut ? target : filt_target(all.w, top_p)) - 1ull; });
+            if (c.found) {
+                take(c);
+                m = ties_for(c.thr + 1ull, n_ties);
+            }
+        } else {  // the target is reached among the ties at tau itself
+            m = ties_for(target, m);
+        }
+    }
+
+    // ---- the draw, in token order: the weight above tau and the number of ties of every chunk, a warp per chunk
+    {
+        __syncthreads();
+        const uint32_t above0 = peer_shared(sh.chunk.above, 0u), ties0 = peer_shared(sh.chunk.ties, 0u);
+        constexpr int kInFlight = 4;
+        for (int c0 = c_begin + warp; c0 < c_end; c0 += kFiltWarps * kInFlight) {
+            CountMass v[kInFlight];
+#pragma unroll
+            for (int r = 0; r < kInFlight; ++r) v[r] = CountMass{0u, 0ull};
+            for (int piece = 0; piece < pieces; ++piece) {
+                float e[kInFlight][8];
+#pragma unroll
+                for (int r = 0; r < kInFlight; ++r) {
+                    const int c = c0 + r * kFiltWarps;
+                    load_eight<DT>(rowp, c * chunk + piece * 256 + lane * 8 - lead, c < c_end ? a.V : 0, aligned != 0, e[r]);
+                }
+#pragma unroll
+                for (int r = 0; r < kInFlight; ++r)
+                    if (max_eight(e[r]) >= z_zero)
+#pragma unroll
+                        for (int q = 0; q < 8; ++q)
+                            if (e[r][q] >= z_zero) {
+                                const uint32_t key = logit_key<DT>(e[r][q]);
+                                if (key > tau) v[r].w += fixed_weight(e[r][q], M, scale);
+                                else if (key == tau) v[r].n += 1u;
+                            }
+            }
+#pragma unroll
+            for (int r = 0; r < kInFlight; ++r) {
+                const int c = c0 + r * kFiltWarps;
+                v[r].n = __reduce_add_sync(0xFFFFFFFFu, v[r].n);
+#pragma unroll
+                for (int d = 16; d >= 1; d >>= 1) v[r].w += __shfl_xor_sync(0xFFFFFFFFu, v[r].w, d);
+                if (lane == 0 && c < c_end) {
+                    st_peer_u64(above0 + uint32_t(c) * 8u, v[r].w);
+                    st_peer_u32(ties0 + uint32_t(c) * 4u, v[r].n);
                 }
             }
-        });
-        const float l = logf(static_cast<float>(S_drawn) * (1.f / kFixOne));
-        a.argmax[row] = token;
-        if (a.rep) a.rep[row] = token >= 0 ? __ldg(P.trep + token) : -1;
-        if (a.lse) a.lse[row] = fmaf(M, a.inv_t, l);
-        if (a.logp_argmax) a.logp_argmax[row] = (zt - M) * a.inv_t - l;
+        }
+        cluster_barrier();
+    }
+    if (crank != 0u) return;
+    constexpr int kPer = kFiltChunks / kFiltThreads;
+    unsigned int ties[kPer];
+    unsigned long long above[kPer];
+    CountMass mine{0u, 0ull}, total;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        const int c = tid * kPer + i;
+        ties[i] = c < n_chunks ? sh.chunk.ties[c] : 0u;
+        above[i] = c < n_chunks ? sh.chunk.above[c] : 0ull;
+        mine.n += ties[i];
+    }
+    auto kept_ties = [&](unsigned int before, unsigned int here) { return min(here, m > before ? m - before : 0u); };
+    unsigned int tie_base = filt_scan(mine, sh, turn, total).n;
+    {
+        unsigned int before = tie_base;
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            mine.w += above[i] + static_cast<unsigned long long>(kept_ties(before, ties[i])) * w_tie;
+            before += ties[i];
+        }
+    }
+    mine.n = 0u;
+    unsigned long long run = filt_scan(mine, sh, turn, total).w;
+    const unsigned long long S_kept = total.w, thr = filt_threshold(S_kept, u);
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        const unsigned long long w = above[i] + static_cast<unsigned long long>(kept_ties(tie_base, ties[i])) * w_tie;
+        if (run <= thr && thr < run + w) {  // the one chunk that holds the draw
+            sh.pick[0] = static_cast<unsigned long long>(tid * kPer + i);
+            sh.pick[1] = run;
+            sh.pick[2] = tie_base;
+        }
+        run += w;
+        tie_base += ties[i];
+    }
+    __syncthreads();
+    if (warp != 0) return;
+    run = sh.pick[1];
+    unsigned int tie_run = unsigned(sh.pick[2]);
+    for (int piece = 0; piece < pieces; ++piece) {
+        const int t0 = int(sh.pick[0]) * chunk + piece * 256 + lane * 8 - lead;
+        float e[8];
+        load_eight<DT>(rowp, t0, a.V, aligned != 0, e);
+        unsigned int t_mine = 0u;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) t_mine += e[q] >= z_zero && logit_key<DT>(e[q]) == tau ? 1u : 0u;
+        unsigned int t_inc = t_mine;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const unsigned int up = __shfl_up_sync(0xFFFFFFFFu, t_inc, d);
+            if (lane >= d) t_inc += up;
+        }
+        unsigned int seen = tie_run + t_inc - t_mine;
+        unsigned long long w[8], w_mine = 0ull;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            w[q] = 0ull;
+            if (e[q] >= z_zero) {
+                const uint32_t key = logit_key<DT>(e[q]);
+                if (key > tau || (key == tau && seen++ < m)) w[q] = fixed_weight(e[q], M, scale);
+            }
+            w_mine += w[q];
+        }
+        unsigned long long inc = w_mine;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const unsigned long long up = __shfl_up_sync(0xFFFFFFFFu, inc, d);
+            if (lane >= d) inc += up;
+        }
+        unsigned long long cum = run + inc - w_mine;
+        if (cum <= thr && thr < cum + w_mine)
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                if (cum <= thr && thr < cum + w[q]) write_draw(t0 + q, e[q], S_kept);
+                cum += w[q];
+            }
+        run += __shfl_sync(0xFFFFFFFFu, inc, 31);
+        tie_run += __shfl_sync(0xFFFFFFFFu, t_inc, 31);
+        if (thr < run) return;
     }
 }
 
