@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "cfgzip.h"
+#include "cfgzip_filtered.cuh"
 #include "cfgzip_kernels.cuh"
 #include "class_sort.cuh"
 #include "workspace.h"
@@ -679,20 +680,19 @@ int launch_fused(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, in
 // so 8, 4 or 2 blocks (a thread-block cluster) share a row while that many still fit the device in one wave, two of the
 // kernel's blocks to an SM.
 template <int DT>
-int launch_filtered(cfgzip_ctx* ctx, const StepArgs& a, unsigned rows_grid, int aligned, int top_k, float top_p,
-                    cudaStream_t st) {
+int launch_filtered(cfgzip_ctx* ctx, const StepArgs& a, unsigned rows_grid, int top_k, float top_p, cudaStream_t st) {
     int rc;
     if ((rc = ensure_smem(k_sample_filtered<DT>, sizeof(FiltShared))) != CFGZIP_OK) return rc;
     const unsigned fit = 2u * unsigned(std::max(ctx->sm_count, 1));
     unsigned per_row = kFiltPeers;
     while (per_row > 1 && unsigned(a.B) * per_row > fit) per_row /= 2;
     ctx->cluster_now = int(per_row);
-    rc = launch(ctx, k_sample_filtered<DT>, dim3(rows_grid * per_row), dim3(kFiltThreads), sizeof(FiltShared), st, a, aligned,
-                top_k, top_p);
+    rc = launch(ctx, k_sample_filtered<DT>, dim3(rows_grid * per_row), dim3(kFiltThreads), sizeof(FiltShared), st, a,
+                filt_geom(a.V, int(per_row)), top_k, top_p);
     ctx->cluster_now = 1;
     if (rc != CFGZIP_OK && per_row > 1)  // a device that cannot place such a cluster: one block per row
-        rc = launch(ctx, k_sample_filtered<DT>, dim3(rows_grid), dim3(kFiltThreads), sizeof(FiltShared), st, a, aligned, top_k,
-                    top_p);
+        rc = launch(ctx, k_sample_filtered<DT>, dim3(rows_grid), dim3(kFiltThreads), sizeof(FiltShared), st, a, filt_geom(a.V, 1),
+                    top_k, top_p);
     return rc;
 }
 
@@ -720,7 +720,7 @@ int launch_sample(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, b
         const dim3 grid(unsigned(d.n_groups_ub) * unsigned(d.S)), block{unsigned(d.threads)};
         if ((rc = launch_pipe<DT>(ctx, a, d, grid, block, st)) != CFGZIP_OK) return rc;
         const unsigned rows_grid = unsigned(d.n_groups_ub) * kGroupRows;
-        if (filtered) return launch_filtered<DT>(ctx, a, rows_grid, 1, top_k, top_p, st);
+        if (filtered) return launch_filtered<DT>(ctx, a, rows_grid, top_k, top_p, st);
         const size_t pad = row_blocks_pad(ctx, rows_grid, a.B);
         if (pad && (rc = ensure_smem(k_sample_rows<DT>, pad)) != CFGZIP_OK) return rc;
         return launch(ctx, k_sample_rows<DT>, dim3(rows_grid), dim3(kSampleThreads), pad, st, a, 1);
@@ -736,7 +736,7 @@ int launch_sample(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, b
     a.p0 = ctx->parts[size_t(a.part0)].dev;
     if ((rc = launch(ctx, k_step_generic<DT, true>, dim3(unsigned(a.B)), dim3(256), 0, st, a)) != CFGZIP_OK) return rc;
     if (filtered)
-        return launch_filtered<DT>(ctx, a, unsigned(ceil_div(a.B, kGroupRows)) * kGroupRows, aligned ? 1 : 0, top_k, top_p, st);
+        return launch_filtered<DT>(ctx, a, unsigned(ceil_div(a.B, kGroupRows)) * kGroupRows, top_k, top_p, st);
     return launch(ctx, k_sample_rows<DT>, dim3(unsigned(ceil_div(a.B, kGroupRows)) * kGroupRows), dim3(kSampleThreads), 0, st,
                   a, aligned ? 1 : 0);
 }

@@ -1847,701 +1847,6 @@ __global__ void __launch_bounds__(kSampleThreads) k_sample_rows(const __grid_con
 }
 
 // ---------------------------------------------------------------------------------------
-// Second kernel of a sampling step with top-k / top-p: keeps, of the row's allowed tokens in the
-// order (value, largest first; equal values by token id, lowest first), the first top_k (0 = all) and of those the
-// shortest beginning whose weight reaches top_p times the weight of what top_k kept (>= 1: all), then draws among
-// the kept tokens by inverse CDF in token order with the row's uniform number.
-// Weights are 40-bit fixed-point integers (exp((z - M) / T) * 2^40), so every sum is exact whatever the order of the
-// addends: the result is deterministic. A token whose weight is zero in that format can change neither a cumulative
-// weight nor the draw.
-//
-// Two ways through, both exact:
-//   short  The streaming kernel has published the largest logit of every run of tokens. The k-th largest of those is a bar
-//          that at least k tokens reach, and, the runs being many, not many more (k = 50: some 60 to 100 tokens). For top-p
-//          alone the bar is where the run maxima by themselves already weigh enough. One pass over the row collects the
-//          tokens at or above the bar, a thread each, and every thread sums over all of them.
-//   long   Otherwise (a flat distribution, a large k): the kept set is { key > tau } plus the first m tokens, in token order,
-//          with key == tau, where key is an order-preserving integer image of the logit. tau comes out of a radix search
-//          over the row itself, twelve bits a pass (bf16: two passes, f32: three; count and weight of 4096 buckets in shared
-//          memory), the draw out of one more pass that leaves the kept weight of every chunk of 256 tokens.
-// Bound: latency of a chain of block-wide steps. Collecting every token that carries weight first took 78 us of the step for
-// 64 rows of 151936 bf16 logits at T = 0.7 (15000 such tokens a row), and some 30 passes over the row where they did not fit.
-// ---------------------------------------------------------------------------------------
-constexpr int kFiltThreads = 512;   // two blocks per SM: one row's serial steps overlap another row's passes
-constexpr int kFiltWarps = kFiltThreads / 32;
-constexpr int kFiltPeers = 8;       // most blocks that share a row
-constexpr int kFiltList = kFiltThreads;  // tokens of the short way, one per thread
-constexpr int kFiltBits = 12, kFiltBuckets = 1 << kFiltBits;
-constexpr int kFiltChunks = 1024;   // chunks of the draw's pass
-constexpr float kFixOne = 1099511627776.f;  // 2^40
-
-// Order-preserving integer image of a logit and its inverse. bf16 logits only use the upper half of the float's
-// bits, so their keys are 16 bits wide.
-template <int DT>
-__device__ __forceinline__ uint32_t logit_key(float z) {
-    z = z == 0.f ? 0.f : z;  // -0.0 and +0.0 are the same value
-    const uint32_t b = __float_as_uint(z);
-    const uint32_t k = (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-    return DT == kBF16 ? k >> 16 : k;
-}
-template <int DT>
-__device__ __forceinline__ float key_logit(uint32_t k) {
-    if (DT == kBF16) k = (k << 16) | ((k & 0x8000u) ? 0u : 0xFFFFu);  // the lower half of a negative value's key is all ones
-    return __uint_as_float((k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k);
-}
-__device__ __forceinline__ unsigned long long fixed_weight(float z, float M, float scale) {
-    return __float2ull_rz(ex2f((z - M) * scale) * kFixOne);
-}
-
-struct CountMass {
-    unsigned int n;
-    unsigned long long w;
-};
-__device__ __forceinline__ void operator+=(CountMass& a, const CountMass& b) {
-    a.n += b.n;
-    a.w += b.w;
-}
-
-// Shared memory of a block.
-struct FiltShared {
-    union {
-        struct {  // count and weight of the buckets; weights as two 32-bit halves, which keeps every atomic a native one
-            unsigned int n[kFiltBuckets], lo[kFiltBuckets], hi[kFiltBuckets];
-        } hist;
-        uint4 list[kFiltList];  // short way: key (or raw logit), token id, weight
-        struct {                // the draw's pass: kept weight above tau and number of ties of every chunk
-            unsigned long long above[kFiltChunks];
-            unsigned int ties[kFiltChunks];
-        } chunk;
-    };
-    unsigned long long pick[8];  // result of a search, written into every block of the cluster by the first
-    unsigned long long scan_w[2][kFiltWarps];
-    unsigned int scan_n[2][kFiltWarps];
-    unsigned long long peer_w[kFiltPeers];
-    float warp_max[kFiltWarps];
-    unsigned int list_n;
-    unsigned long long kept_w, topk_w;
-};
-
-// Exclusive prefix of one (count, weight) pair per thread in thread order; total to everybody. The two sets of partial sums
-// are used in turn (`turn` flips with every call), so that one barrier per call is enough.
-__device__ __forceinline__ CountMass filt_scan(CountMass v, FiltShared& sh, int& turn, CountMass& total) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    CountMass inc = v;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const unsigned int un = __shfl_up_sync(0xFFFFFFFFu, inc.n, d);
-        const unsigned long long uw = __shfl_up_sync(0xFFFFFFFFu, inc.w, d);
-        if (lane >= d) inc += CountMass{un, uw};
-    }
-    if (lane == 31) {
-        sh.scan_n[turn][warp] = inc.n;
-        sh.scan_w[turn][warp] = inc.w;
-    }
-    __syncthreads();
-    CountMass before{0u, 0ull};
-    total = CountMass{0u, 0ull};
-#pragma unroll
-    for (int i = 0; i < kFiltWarps; ++i) {
-        const CountMass t{sh.scan_n[turn][i], sh.scan_w[turn][i]};
-        if (i < warp) before += t;
-        total += t;
-    }
-    turn ^= 1;
-    return CountMass{before.n + inc.n - v.n, before.w + inc.w - v.w};
-}
-
-// Eight consecutive logits of a row from token t0 on (-inf in front of token 0 and past `end`), as floats.
-template <int DT>
-__device__ __forceinline__ void load_eight(const char* rowp, int t0, int end, bool aligned, float (&e)[8]) {
-    if (aligned && t0 >= 0 && t0 + 8 <= end) {
-        if (DT == kBF16) {
-            const uint4 v = __ldcg(reinterpret_cast<const uint4*>(rowp + size_t(t0) * 2));
-            e[0] = __uint_as_float(v.x << 16); e[1] = __uint_as_float(v.x & 0xFFFF0000u);
-            e[2] = __uint_as_float(v.y << 16); e[3] = __uint_as_float(v.y & 0xFFFF0000u);
-            e[4] = __uint_as_float(v.z << 16); e[5] = __uint_as_float(v.z & 0xFFFF0000u);
-            e[6] = __uint_as_float(v.w << 16); e[7] = __uint_as_float(v.w & 0xFFFF0000u);
-        } else {
-            const float4 v0 = __ldcg(reinterpret_cast<const float4*>(rowp + size_t(t0) * 4));
-            const float4 v1 = __ldcg(reinterpret_cast<const float4*>(rowp + size_t(t0) * 4 + 16));
-            e[0] = v0.x; e[1] = v0.y; e[2] = v0.z; e[3] = v0.w;
-            e[4] = v1.x; e[5] = v1.y; e[6] = v1.z; e[7] = v1.w;
-        }
-    } else {
-#pragma unroll
-        for (int q = 0; q < 8; ++q) e[q] = t0 + q >= 0 && t0 + q < end ? ldcg_elem<DT>(rowp, t0 + q) : -INFINITY;
-    }
-}
-__device__ __forceinline__ float max_eight(const float (&e)[8]) {
-    return fmax3(fmax3(e[0], e[1], e[2]), fmax3(e[3], e[4], e[5]), fmaxf(e[6], e[7]));
-}
-
-// ---- thread-block cluster: rank, barrier, accesses to a peer block's shared memory -----------------
-__device__ __forceinline__ uint32_t cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ uint32_t cluster_blocks() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-    return r;
-}
-// every thread of every block of the cluster (a hardware barrier like the block's own: no flag is polled)
-__device__ __forceinline__ void cluster_barrier() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// the same in two halves
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ uint32_t peer_shared(const void* mine, uint32_t rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(mine)), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ unsigned int add_peer_u32(uint32_t addr, unsigned int v) {
-    unsigned int old;
-    asm volatile("atom.shared::cluster.add.u32 %0, [%1], %2;" : "=r"(old) : "r"(addr), "r"(v) : "memory");
-    return old;
-}
-__device__ __forceinline__ uint32_t ld_peer_u32(uint32_t addr) {
-    uint32_t v;
-    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
-    return v;
-}
-__device__ __forceinline__ uint4 ld_peer_v4(uint32_t addr) {
-    uint4 v;
-    asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_peer_u64(uint32_t addr, unsigned long long v) {
-    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
-}
-__device__ __forceinline__ void st_peer_u32(uint32_t addr, uint32_t v) {
-    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
-}
-
-__device__ __forceinline__ void hist_clear(FiltShared& sh) {
-    uint4* h = reinterpret_cast<uint4*>(&sh.hist);
-#pragma unroll 4
-    for (int i = threadIdx.x; i < int(sizeof(sh.hist) / 16); i += kFiltThreads) h[i] = make_uint4(0u, 0u, 0u, 0u);
-}
-__device__ __forceinline__ void hist_add(FiltShared& sh, uint32_t bucket, unsigned long long w) {
-    atomicAdd(&sh.hist.n[bucket], 1u);
-    const uint32_t lo = static_cast<uint32_t>(w);
-    uint32_t hi = static_cast<uint32_t>(w >> 32);
-    if (lo) {
-        const uint32_t old = atomicAdd(&sh.hist.lo[bucket], lo);
-        hi += (old + lo) < old ? 1u : 0u;  // the carry out of the lower half
-    }
-    if (hi) atomicAdd(&sh.hist.hi[bucket], hi);
-}
-
-// Result of a bucket search: the bucket, (count, weight) in front of it and in it, of everything, the threshold; found: some
-// bucket holds the threshold.
-struct Picked {
-    uint32_t bucket;
-    bool found;
-    CountMass before, at, all;
-};
-
-// The bucket in which the running count (by_weight: weight), on top of `carry`, passes thr_of(total of all buckets): the first
-// b with carry + sum(0 .. b) > thr. Summed over the histograms of n_peers blocks from first_peer on; left in sh.pick as well
-// ([0] bucket or all ones, [1] [2] in front of it, [3] [4] in it, [5] [6] of everything, [7] the threshold). Called by all threads of one block.
-template <typename T>
-__device__ __forceinline__ Picked hist_pick(FiltShared& sh, uint32_t first_peer, uint32_t n_peers, CountMass carry, bool by_weight, int& turn, T&& thr_of) {
-    constexpr int kPer = kFiltBuckets / kFiltThreads;  // 8 consecutive buckets per thread
-    static_assert(kPer == 8, "two 16-byte reads per array");
-    const int tid = threadIdx.x;
-    unsigned int n[kPer];
-    unsigned long long w[kPer];
-#pragma unroll
-    for (int b = 0; b < kPer; ++b) {
-        n[b] = 0u;
-        w[b] = 0ull;
-    }
-    for (uint32_t p = first_peer; p < first_peer + n_peers; ++p) {
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-            const int at = tid * kPer + half * 4;
-            const uint4 vn = ld_peer_v4(peer_shared(sh.hist.n + at, p)), vl = ld_peer_v4(peer_shared(sh.hist.lo + at, p)),
-                        vh = ld_peer_v4(peer_shared(sh.hist.hi + at, p));
-            const unsigned int nn[4] = {vn.x, vn.y, vn.z, vn.w}, ll[4] = {vl.x, vl.y, vl.z, vl.w}, hh[4] = {vh.x, vh.y, vh.z, vh.w};
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                n[half * 4 + b] += nn[b];
-                w[half * 4 + b] += (static_cast<unsigned long long>(hh[b]) << 32) | ll[b];
-            }
-        }
-    }
-    CountMass mine{0u, 0ull}, total;
-#pragma unroll
-    for (int b = 0; b < kPer; ++b) mine += CountMass{n[b], w[b]};
-    if (tid == 0) sh.pick[0] = ~0ull;
-    CountMass run = filt_scan(mine, sh, turn, total);  // (its barrier also orders the line above before the writes below)
-    const unsigned long long thr = thr_of(total);
-    if (tid == 0) {
-        sh.pick[5] = total.n;
-        sh.pick[6] = total.w;
-        sh.pick[7] = thr;
-    }
-    run += carry;
-#pragma unroll
-    for (int b = 0; b < kPer; ++b) {
-        const unsigned long long below = by_weight ? run.w : run.n, here = by_weight ? w[b] : n[b];
-        if (below <= thr && thr < below + here) {
-            sh.pick[0] = static_cast<unsigned long long>(tid * kPer + b);
-            sh.pick[1] = run.n;
-            sh.pick[2] = run.w;
-            sh.pick[3] = n[b];
-            sh.pick[4] = w[b];
-        }
-        run += CountMass{n[b], w[b]};
-    }
-    __syncthreads();
-    return Picked{static_cast<uint32_t>(sh.pick[0]), sh.pick[0] != ~0ull, CountMass{static_cast<unsigned int>(sh.pick[1]), sh.pick[2]},
-                  CountMass{static_cast<unsigned int>(sh.pick[3]), sh.pick[4]}, total};
-}
-
-// top_p's share of a weight, rounded up; at least one unit so that one token is kept
-__device__ __forceinline__ unsigned long long filt_target(unsigned long long S, float top_p) {
-    const unsigned long long t = static_cast<unsigned long long>(ceil(static_cast<double>(S) * static_cast<double>(top_p)));
-    return t < 1ull ? 1ull : (t > S ? S : t);
-}
-// u times the kept weight, rounded down: the first token whose cumulative weight exceeds it is drawn
-__device__ __forceinline__ unsigned long long filt_threshold(unsigned long long S_kept, float u) {
-    const unsigned long long t = static_cast<unsigned long long>(static_cast<double>(u) * static_cast<double>(S_kept));
-    return t >= S_kept ? S_kept - 1ull : t;
-}
-
-// One row per cluster of blocks (1 to 8 of them: a short batch has fewer rows than the device has multiprocessors).
-// Every block goes over its share of the row; what they find meets in the shared memory of the cluster's first block.
-template <int DT>
-__global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __grid_constant__ StepArgs a, int aligned, int top_k,
-                                                                     float top_p) {
-    extern __shared__ __align__(16) unsigned char filt_smem[];
-    FiltShared& sh = *reinterpret_cast<FiltShared*>(filt_smem);
-    pdl_prologue();
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const uint32_t n_peers = cluster_blocks(), crank = cluster_rank();
-    const int slot = blockIdx.x / n_peers;  // the blocks of a cluster are neighbours along x
-    const int g = slot / kGroupRows, j = slot - g * kGroupRows;
-    // (every way out before the cluster's barriers depends on the row alone, so the blocks of a cluster take it together)
-    if (a.n_groups && g >= __ldg(a.n_groups)) return;
-    int row;
-    if (a.group_rows) {
-        row = a.group_rows[g * kGroupRows + j];
-    } else {
-        row = g * kGroupRows + j;
-        if (row >= a.B) row = -1;
-    }
-    if (row < 0) return;
-    PartDev P = a.p0;
-    if (a.group_part) {
-        P = a.parts[a.group_part[g]];
-    } else if (a.row_part) {
-        const int part = a.row_part[row];
-        if (part < 0 || part >= a.n_parts || !a.parts[part].live || a.parts[part].V != a.V) return;  // counted by the step kernel
-        P = a.parts[part];
-    }
-    const float scale = a.scale;
-    // the run states the streaming kernel published: the row maximum, and the maxima and sums of up to four runs per
-    // thread for the bar of the short way (leaving runs out only lowers the bar)
-    const Partial* src = row_slots(a, g, j);
-    const float u = __ldg(a.u + row);  // needed late
-    constexpr int kKeep = 4;
-    float run_m[kKeep], run_s[kKeep];
-    float M = -INFINITY;
-#pragma unroll
-    for (int q = 0; q < kKeep; ++q) {
-        const int k = tid + q * kFiltThreads;
-        int4 raw = make_int4(__float_as_int(-INFINITY), 0, 0, 0);
-        if (k < a.slots) raw = __ldcg(reinterpret_cast<const int4*>(src + k));
-        run_m[q] = __int_as_float(raw.x);
-        run_s[q] = __int_as_float(raw.y);
-        M = fmaxf(M, run_m[q]);
-    }
-    for (int k = tid + kKeep * kFiltThreads; k < a.slots; k += kFiltThreads) M = fmaxf(M, __ldcg(&src[k].m));
-#pragma unroll
-    for (int d = 16; d >= 1; d >>= 1) M = fmaxf(M, __shfl_xor_sync(0xFFFFFFFFu, M, d));
-    if (lane == 0) sh.warp_max[warp] = M;
-    if (tid == 0) sh.list_n = 0u;
-    hist_clear(sh);
-    __syncthreads();
-#pragma unroll
-    for (int w = 0; w < kFiltWarps; ++w) M = fmaxf(M, sh.warp_max[w]);
-    if (!(M > kRefFloor)) {
-        // nothing allowed, or only -inf allowed: the lowest allowed token (if any) and -inf logs
-        if (warp == 0 && crank == 0) {
-            unsigned long long cand = first_allowed_share(a, P, row, lane, 32);
-#pragma unroll
-            for (int d = 16; d >= 1; d >>= 1) {
-                const unsigned long long other = __shfl_xor_sync(0xFFFFFFFFu, cand, d);
-                cand = other < cand ? other : cand;
-            }
-            if (lane == 0) write_row_outputs(a, row, -INFINITY, 0.f, cand);
-        }
-        return;
-    }
-    auto write_draw = [&](int token, float zt, unsigned long long S_kept) {
-        const float l = logf(static_cast<float>(S_kept) * (1.f / kFixOne));
-        a.argmax[row] = token;
-        if (a.rep) a.rep[row] = __ldg(P.trep + token);
-        if (a.lse) a.lse[row] = fmaf(M, a.inv_t, l);
-        if (a.logp_argmax) a.logp_argmax[row] = (zt - M) * a.inv_t - l;
-    };
-    constexpr int ES = DT == kBF16 ? 2 : 4;
-    const char* rowp = reinterpret_cast<const char*>(a.logits) + int64_t(row) * a.row_stride * ES;
-    // Rows are gone over eight tokens at a time from token -lead on, so that the eight are one vector of the row: a row
-    // that starts anywhere has `head` tokens in front of its first vector. A chunk is 256 tokens (more only where that
-    // would be more than kFiltChunks of them); every block of the cluster takes a run of chunks.
-    const int head = a.shifted ? row_head<DT>(rowp, a.V) : 0, lead = (8 - head) & 7;
-    const int pieces = (a.V + lead + 256 * kFiltChunks - 1) / (256 * kFiltChunks), chunk = 256 * pieces;
-    const int n_chunks = (a.V + lead + chunk - 1) / chunk, per_block = (n_chunks + int(n_peers) - 1) / int(n_peers);
-    const int c_begin = min(int(crank) * per_block, n_chunks), c_end = min(c_begin + per_block, n_chunks);
-    // A token takes part when its logit is at or above M - 41 / scale (below M - 40 / scale the fixed-point weight is zero;
-    // the extra unit covers the rounding of the threshold itself).
-    const uint32_t key_max = logit_key<DT>(M);
-    const float z_zero = fmaxf(key_logit<DT>(logit_key<DT>(M - 41.f / scale)), kRefFloor);
-    const int bits = 32 - __clz(int(key_max - logit_key<DT>(z_zero)));  // of key_max - key
-    const int first_lo = max(0, bits - kFiltBits);
-    auto offset_of = [&](float z) { return key_max - logit_key<DT>(z); };
-    int turn = 0;
-    // Visit the share eight tokens at a time, four rounds of loads in flight; f gets the first token and its eight logits.
-    auto visit = [&](float at_least, auto&& f) {
-        constexpr int kInFlight = 4;
-        const int t_end = min(c_end * chunk - lead, a.V);
-        for (int t0 = c_begin * chunk - lead + tid * 8; t0 < t_end; t0 += kFiltThreads * 8 * kInFlight) {
-            float e[kInFlight][8];
-#pragma unroll
-            for (int r = 0; r < kInFlight; ++r) load_eight<DT>(rowp, t0 + r * kFiltThreads * 8, t_end, aligned != 0, e[r]);
-#pragma unroll
-            for (int r = 0; r < kInFlight; ++r)
-                if (max_eight(e[r]) >= at_least) f(t0 + r * kFiltThreads * 8, e[r]);
-        }
-    };
-
-    // ---- the short way
-    bool brief = top_k <= kFiltList / 2;
-    if (brief) {
-        float sum = 0.f;
-#pragma unroll
-        for (int q = 0; q < kKeep; ++q)
-            if (run_m[q] >= z_zero) {
-                const unsigned long long w = top_k > 0 ? 0ull : fixed_weight(run_m[q], M, scale);
-                hist_add(sh, offset_of(run_m[q]) >> first_lo, w);
-                sum += run_s[q] * ex2f((run_m[q] - M) * scale);
-            }
-        // (for top-p the weight of all tokens is not known exactly yet: the run sums give it to about 1e-5, the bar allows 1e-3)
-        __syncthreads();
-        unsigned long long goal = static_cast<unsigned long long>(max(top_k, 1)) - 1ull;
-        if (top_k == 0) {
-            CountMass all;
-            filt_scan(CountMass{0u, __float2ull_rz(sum * kFixOne)}, sh, turn, all);
-            goal = static_cast<unsigned long long>(static_cast<double>(all.w) * top_p * 1.001);
-        }
-        const Picked bar = hist_pick(sh, crank, 1u, CountMass{0u, 0ull}, top_k == 0, turn, [&](CountMass) { return goal; });
-        brief = bar.found || top_k > 0;  // (fewer runs with a token than top_k: collect every token)
-        if (brief) {
-            const unsigned long long lowest =
-                bar.found ? ((static_cast<unsigned long long>(bar.bucket) + 1ull) << first_lo) - 1ull : ~0ull;
-            const float z_bar = lowest < offset_of(z_zero) ? key_logit<DT>(key_max - uint32_t(lowest)) : z_zero;
-            const uint32_t list0 = peer_shared(sh.list, 0u), list_n0 = peer_shared(&sh.list_n, 0u);
-            unsigned long long mine = 0ull;
-            cluster_barrier();  // the first block is done with its buckets, which the list shares the space of
-            auto push = [&](int t, float z) {
-                const unsigned int at = add_peer_u32(list_n0, 1u);
-                if (at < kFiltList) {
-                    st_peer_u32(list0 + at * 16u, __float_as_uint(z));
-                    st_peer_u32(list0 + at * 16u + 4u, uint32_t(t));
-                }
-            };
-            if (top_k > 0) {
-                visit(z_bar, [&](int t0, const float (&e)[8]) {
-#pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        if (e[q] >= z_bar) push(t0 + q, e[q]);
-                });
-            } else {
-                visit(z_zero, [&](int t0, const float (&e)[8]) {
-#pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        if (e[q] >= z_zero) {
-                            mine += fixed_weight(e[q], M, scale);
-                            if (e[q] >= z_bar) push(t0 + q, e[q]);
-                        }
-                });
-                CountMass all;
-                filt_scan(CountMass{0u, mine}, sh, turn, all);
-                if (tid == 0) st_peer_u64(peer_shared(&sh.peer_w[crank], 0u), all.w);
-            }
-            cluster_barrier();  // every block's tokens have arrived
-            const unsigned int n = ld_peer_u32(list_n0);  // (the same in every block of the cluster)
-            if (n <= unsigned(kFiltList)) {
-                cluster_arrive();  // this thread has read the first block's count
-                if (crank != 0u) {
-                    cluster_wait();
-                    return;
-                }
-                // A thread per token: its place in the order and the weight in front of it, then its place in token order.
-                const bool have = unsigned(tid) < n;
-                uint4 me = make_uint4(0u, 0u, 0u, 0u);
-                unsigned long long my_w = 0ull;
-                float my_z = 0.f;
-                if (have) {
-                    me = sh.list[tid];
-                    my_z = __uint_as_float(me.x);
-                    my_w = fixed_weight(my_z, M, scale);
-                    me.x = logit_key<DT>(my_z);
-                    sh.list[tid] = make_uint4(me.x, me.y, uint32_t(my_w), uint32_t(my_w >> 32));
-                }
-                __syncthreads();
-                CountMass front{0u, 0ull};
-                const unsigned int last = (top_k > 0 ? min(unsigned(top_k), n) : n) - 1u;
-                if (have) {
-                    for (unsigned int k = 0; k < n; ++k) {
-                        const uint4 o = sh.list[k];
-                        if (o.x > me.x || (o.x == me.x && o.y < me.y))
-                            front += CountMass{1u, (static_cast<unsigned long long>(o.w) << 32) | o.z};
-                    }
-                    if (front.n == last) sh.topk_w = front.w + my_w;
-                }
-                __syncthreads();
-                unsigned long long S = sh.topk_w;
-                if (top_k == 0) {
-                    S = 0ull;
-                    for (uint32_t p = 0; p < n_peers; ++p) S += sh.peer_w[p];
-                }
-                const unsigned long long target = top_p < 1.f ? filt_target(S, top_p) : ~0ull;
-                const bool kept = have && front.n <= last && front.w < target;
-                if (kept && (front.n == last || front.w + my_w >= target)) sh.kept_w = front.w + my_w;
-                if (have && !kept) sh.list[tid] = make_uint4(me.x, me.y, 0u, 0u);
-                __syncthreads();
-                cluster_wait();  // (long since complete: no block may leave while another reads its shared memory)
-                if (!kept) return;
-                const unsigned long long S_kept = sh.kept_w, thr = filt_threshold(S_kept, u);
-                unsigned long long cum = 0ull;
-                for (unsigned int k = 0; k < n; ++k) {
-                    const uint4 o = sh.list[k];
-                    cum += o.y <= me.y ? (static_cast<unsigned long long>(o.w) << 32) | o.z : 0ull;
-                }
-                if (my_w > 0ull && cum - my_w <= thr && thr < cum) write_draw(int(me.y), key_logit<DT>(me.x), S_kept);
-                return;
-            }
-        }
-    }
-
-    // ---- the long way: tau and m
-    // The largest key whose tokens, with those above it, together count (by_weight: weigh) more than thr_of(everything).
-    struct Cut {
-        bool found;
-        uint32_t key;
-        CountMass above, ties, all;
-        unsigned long long thr;
-    };
-    auto search = [&](bool by_weight, auto&& thr_of) {
-        Cut cut{};
-        unsigned long long prefix = 0ull;
-        int hi = bits;
-        bool first = true;
-        do {
-            const int lo = first ? first_lo : max(0, hi - kFiltBits);
-            __syncthreads();
-            hist_clear(sh);
-            __syncthreads();
-            visit(z_zero, [&](int, const float (&e)[8]) {
-#pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    if (e[q] >= z_zero) {
-                        const unsigned long long x = offset_of(e[q]);
-                        if ((x >> hi) == prefix)
-                            hist_add(sh, uint32_t(x >> lo) & ((1u << (hi - lo)) - 1u), fixed_weight(e[q], M, scale));
-                    }
-            });
-            cluster_barrier();
-            if (crank == 0u) {
-                hist_pick(sh, 0u, n_peers, cut.above, by_weight, turn, [&](CountMass all) { return first ? thr_of(all) : cut.thr; });
-                for (int i = tid; i < 8 * int(n_peers - 1u); i += kFiltThreads)
-                    st_peer_u64(peer_shared(&sh.pick[i & 7], 1u + uint32_t(i >> 3)), sh.pick[i & 7]);
-            }
-            cluster_barrier();
-            if (first) {
-                cut.thr = sh.pick[7];
-                cut.all = CountMass{static_cast<unsigned int>(sh.pick[5]), sh.pick[6]};
-                cut.found = sh.pick[0] != ~0ull;
-                if (!cut.found) return cut;
-            }
-            prefix = (prefix << (hi - lo)) | sh.pick[0];
-            cut.above = CountMass{static_cast<unsigned int>(sh.pick[1]), sh.pick[2]};
-            cut.ties = CountMass{static_cast<unsigned int>(sh.pick[3]), sh.pick[4]};
-            hi = lo;
-            first = false;
-        } while (hi > 0);
-        cut.key = key_max - uint32_t(prefix);
-        return cut;
-    };
-    uint32_t tau = 0u;
-    unsigned int m = 0xFFFFFFFFu, n_ties = 0u;
-    unsigned long long w_tie = 0ull, w_above = 0ull, S = 0ull;
-    bool cut = false;
-    auto take = [&](const Cut& c) {
-        tau = c.key;
-        w_tie = fixed_weight(key_logit<DT>(tau), M, scale);
-        w_above = c.above.w;
-        n_ties = c.ties.n;
-        cut = true;
-    };
-    auto ties_for = [&](unsigned long long target, unsigned int most) {  // how many ties reach the target, at least one
-        if (w_tie == 0ull) return most;
-        const unsigned long long q = (target - w_above + w_tie - 1ull) / w_tie;
-        return q < most ? unsigned(q < 1ull ? 1ull : q) : max(most, 1u);
-    };
-    if (top_k > 0) {
-        const Cut c = search(false, [&](CountMass) { return static_cast<unsigned long long>(top_k) - 1ull; });
-        if (c.found) {  // (a top_k beyond everything that carries weight cuts nothing away)
-            take(c);
-            m = unsigned(top_k) - c.above.n;
-            S = w_above + static_cast<unsigned long long>(m) * w_tie;
-        }
-    }
-    if (top_p < 1.f) {
-        const unsigned long long target = cut ? filt_target(S, top_p) : 0ull;
-        if (!cut || w_above >= target) {
-            const Cut c = search(true, [&](CountMass all) { return (cut ? target : filt_target(all.w, top_p)) - 1ull; });
-            if (c.found) {
-                take(c);
-                m = ties_for(c.thr + 1ull, n_ties);
-            }
-        } else {  // the target is reached among the ties at tau itself
-            m = ties_for(target, m);
-        }
-    }
-
-    // ---- the draw, in token order: the weight above tau and the number of ties of every chunk, a warp per chunk
-    {
-        __syncthreads();
-        const uint32_t above0 = peer_shared(sh.chunk.above, 0u), ties0 = peer_shared(sh.chunk.ties, 0u);
-        constexpr int kInFlight = 4;
-        for (int c0 = c_begin + warp; c0 < c_end; c0 += kFiltWarps * kInFlight) {
-            CountMass v[kInFlight];
-#pragma unroll
-            for (int r = 0; r < kInFlight; ++r) v[r] = CountMass{0u, 0ull};
-            for (int piece = 0; piece < pieces; ++piece) {
-                float e[kInFlight][8];
-#pragma unroll
-                for (int r = 0; r < kInFlight; ++r) {
-                    const int c = c0 + r * kFiltWarps;
-                    load_eight<DT>(rowp, c * chunk + piece * 256 + lane * 8 - lead, c < c_end ? a.V : 0, aligned != 0, e[r]);
-                }
-#pragma unroll
-                for (int r = 0; r < kInFlight; ++r)
-                    if (max_eight(e[r]) >= z_zero)
-#pragma unroll
-                        for (int q = 0; q < 8; ++q)
-                            if (e[r][q] >= z_zero) {
-                                const uint32_t key = logit_key<DT>(e[r][q]);
-                                if (key > tau) v[r].w += fixed_weight(e[r][q], M, scale);
-                                else if (key == tau) v[r].n += 1u;
-                            }
-            }
-#pragma unroll
-            for (int r = 0; r < kInFlight; ++r) {
-                const int c = c0 + r * kFiltWarps;
-                v[r].n = __reduce_add_sync(0xFFFFFFFFu, v[r].n);
-#pragma unroll
-                for (int d = 16; d >= 1; d >>= 1) v[r].w += __shfl_xor_sync(0xFFFFFFFFu, v[r].w, d);
-                if (lane == 0 && c < c_end) {
-                    st_peer_u64(above0 + uint32_t(c) * 8u, v[r].w);
-                    st_peer_u32(ties0 + uint32_t(c) * 4u, v[r].n);
-                }
-            }
-        }
-        cluster_barrier();
-    }
-    if (crank != 0u) return;
-    constexpr int kPer = kFiltChunks / kFiltThreads;
-    unsigned int ties[kPer];
-    unsigned long long above[kPer];
-    CountMass mine{0u, 0ull}, total;
-#pragma unroll
-    for (int i = 0; i < kPer; ++i) {
-        const int c = tid * kPer + i;
-        ties[i] = c < n_chunks ? sh.chunk.ties[c] : 0u;
-        above[i] = c < n_chunks ? sh.chunk.above[c] : 0ull;
-        mine.n += ties[i];
-    }
-    auto kept_ties = [&](unsigned int before, unsigned int here) { return min(here, m > before ? m - before : 0u); };
-    unsigned int tie_base = filt_scan(mine, sh, turn, total).n;
-    {
-        unsigned int before = tie_base;
-#pragma unroll
-        for (int i = 0; i < kPer; ++i) {
-            mine.w += above[i] + static_cast<unsigned long long>(kept_ties(before, ties[i])) * w_tie;
-            before += ties[i];
-        }
-    }
-    mine.n = 0u;
-    unsigned long long run = filt_scan(mine, sh, turn, total).w;
-    const unsigned long long S_kept = total.w, thr = filt_threshold(S_kept, u);
-#pragma unroll
-    for (int i = 0; i < kPer; ++i) {
-        const unsigned long long w = above[i] + static_cast<unsigned long long>(kept_ties(tie_base, ties[i])) * w_tie;
-        if (run <= thr && thr < run + w) {  // the one chunk that holds the draw
-            sh.pick[0] = static_cast<unsigned long long>(tid * kPer + i);
-            sh.pick[1] = run;
-            sh.pick[2] = tie_base;
-        }
-        run += w;
-        tie_base += ties[i];
-    }
-    __syncthreads();
-    if (warp != 0) return;
-    run = sh.pick[1];
-    unsigned int tie_run = unsigned(sh.pick[2]);
-    for (int piece = 0; piece < pieces; ++piece) {
-        const int t0 = int(sh.pick[0]) * chunk + piece * 256 + lane * 8 - lead;
-        float e[8];
-        load_eight<DT>(rowp, t0, a.V, aligned != 0, e);
-        unsigned int t_mine = 0u;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) t_mine += e[q] >= z_zero && logit_key<DT>(e[q]) == tau ? 1u : 0u;
-        unsigned int t_inc = t_mine;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const unsigned int up = __shfl_up_sync(0xFFFFFFFFu, t_inc, d);
-            if (lane >= d) t_inc += up;
-        }
-        unsigned int seen = tie_run + t_inc - t_mine;
-        unsigned long long w[8], w_mine = 0ull;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            w[q] = 0ull;
-            if (e[q] >= z_zero) {
-                const uint32_t key = logit_key<DT>(e[q]);
-                if (key > tau || (key == tau && seen++ < m)) w[q] = fixed_weight(e[q], M, scale);
-            }
-            w_mine += w[q];
-        }
-        unsigned long long inc = w_mine;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const unsigned long long up = __shfl_up_sync(0xFFFFFFFFu, inc, d);
-            if (lane >= d) inc += up;
-        }
-        unsigned long long cum = run + inc - w_mine;
-        if (cum <= thr && thr < cum + w_mine)
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                if (cum <= thr && thr < cum + w[q]) write_draw(t0 + q, e[q], S_kept);
-                cum += w[q];
-            }
-        run += __shfl_sync(0xFFFFFFFFu, inc, 31);
-        tie_run += __shfl_sync(0xFFFFFFFFu, t_inc, 31);
-        if (thr < run) return;
-    }
-}
-
-// ---------------------------------------------------------------------------------------
 // Row-split step on caller-provided tables: the per-row kernel above, with each row shared by
 // S blocks that meet through a scratch area of (max, sum-exp, token) states and one ticket
 // per row, exactly as the sparse kernel's blocks do. It touches no context: token->class and
