@@ -669,9 +669,11 @@ int launch_fused(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, in
     }
     if (rc != CFGZIP_OK) return rc;
     if (logp_full) {
-        const dim3 grid(unsigned(std::min(ceil_div(a.V, 256 * 4), 64)), unsigned(std::min<int32_t>(a.B, 65535)));
-        rc = launch(ctx, k_logp_full<DT>, grid, dim3(256), 0, st, (const void*)a.logits, a.row_stride, int(a.B),
-                    int(a.V), (const float*)a.lse, logp_full);
+        const bool quads = a.V % 4 == 0 && (reinterpret_cast<uintptr_t>(logp_full) & 15u) == 0 &&
+                           (reinterpret_cast<uintptr_t>(a.logits) & (DT == kBF16 ? 7u : 15u)) == 0 && a.row_stride % 4 == 0;
+        const dim3 grid(unsigned(ceil_div(a.V, 256 * 4 * (quads ? 4 : 1))), unsigned(std::min<int32_t>(a.B, 65535)));
+        rc = launch(ctx, quads ? k_logp_full<DT, true> : k_logp_full<DT, false>, grid, dim3(256), 0, st, (const void*)a.logits,
+                    a.row_stride, int(a.B), int(a.V), (const float*)a.lse, logp_full);
     }
     return rc;
 }
@@ -1057,19 +1059,10 @@ int cfgzip_mask_logits(cfgzip_ctx* ctx, void* logits, int dtype, int64_t row_str
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return CFGZIP_E_CUDA;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int es = dtype == CFGZIP_BF16 ? 2 : 4;
-    const bool al = aligned16(logits, row_stride_elems, es);
-    const int n_octets = ceil_div(V, 8);
-    const int64_t items = int64_t(B) * ceil_div(n_octets, 256 * 4);
-    const unsigned grid = unsigned(std::min<int64_t>(items, int64_t(ctx->sm_count) * 8));
-    if (dtype == CFGZIP_BF16) {
-        auto kern = al ? k_mask_logits<kBF16, true> : k_mask_logits<kBF16, false>;
-        return launch(ctx, kern, dim3(grid), dim3(256), 0, st, logits, row_stride_elems, int(B), int(V), VW, vocab_mask,
-                      vocab_stride_words, 0);
-    }
-    auto kern = al ? k_mask_logits<kF32, true> : k_mask_logits<kF32, false>;
-    return launch(ctx, kern, dim3(grid), dim3(256), 0, st, logits, row_stride_elems, int(B), int(V), VW, vocab_mask,
-                  vocab_stride_words, aligned32(logits, row_stride_elems, 4) ? 1 : 0);
+    const int chunks = std::max(1, ceil_div(V >> 3, kMaskChunk));
+    const unsigned grid = unsigned(std::min<int64_t>(int64_t(B) * chunks, int64_t(ctx->sm_count) * 8));
+    return launch(ctx, dtype == CFGZIP_BF16 ? k_mask_logits<kBF16> : k_mask_logits<kF32>, dim3(grid), dim3(256), 0, st, logits,
+                  row_stride_elems, int(B), int(V), vocab_mask, vocab_stride_words, chunks);
 }
 
 int cfgzip_masked_logsoftmax_argmax(cfgzip_ctx* ctx, cfgzip_part_id part0, const int32_t* row_part,

@@ -257,18 +257,23 @@ __device__ __forceinline__ void build_class_table_quads(const StepArgs& a, const
     if (warp == 0) T[P.KW * 32 + lane] = 0u;  // the padding class
 }
 
+// From the class words of 8 tokens: byte i of (lo, hi) belongs to row 8*rb + i, bit j of it to token j.
+__device__ __forceinline__ void row_batch_bytes(const uint32_t (&w)[8], int rb, uint32_t& lo, uint32_t& hi) {
+    const uint32_t sel = uint32_t(rb) | (uint32_t(4 + rb) << 4);  // byte rb of both operands
+    lo = __byte_perm(__byte_perm(w[0], w[1], sel), __byte_perm(w[2], w[3], sel), 0x5410);
+    hi = __byte_perm(__byte_perm(w[4], w[5], sel), __byte_perm(w[6], w[7], sel), 0x5410);
+    transpose8x8(lo, hi);
+}
+
 // Allow bits of rows 8*rb .. 8*rb+7 for the 8 tokens whose class ids are packed in cv:
 // byte i of (lo, hi) belongs to row 8*rb + i, bit j of it to token j of the octet.
 __device__ __forceinline__ void octet_allow_bits(const uint4& cv, const uint32_t* T, int rb, bool active, uint32_t& lo,
                                                  uint32_t& hi) {
     lo = hi = 0;
     if (!active) return;
-    const uint32_t w0 = T[cv.x & 0xFFFFu], w1 = T[cv.x >> 16], w2 = T[cv.y & 0xFFFFu], w3 = T[cv.y >> 16];
-    const uint32_t w4 = T[cv.z & 0xFFFFu], w5 = T[cv.z >> 16], w6 = T[cv.w & 0xFFFFu], w7 = T[cv.w >> 16];
-    const uint32_t sel = uint32_t(rb) | (uint32_t(4 + rb) << 4);  // byte rb of both operands
-    lo = __byte_perm(__byte_perm(w0, w1, sel), __byte_perm(w2, w3, sel), 0x5410);
-    hi = __byte_perm(__byte_perm(w4, w5, sel), __byte_perm(w6, w7, sel), 0x5410);
-    transpose8x8(lo, hi);
+    const uint32_t w[8] = {T[cv.x & 0xFFFFu], T[cv.x >> 16], T[cv.y & 0xFFFFu], T[cv.y >> 16],
+                           T[cv.z & 0xFFFFu], T[cv.z >> 16], T[cv.w & 0xFFFFu], T[cv.w >> 16]};
+    row_batch_bytes(w, rb, lo, hi);
 }
 
 // Lowest allowed token of a row, found from the class side: the first member of every allowed
@@ -1264,8 +1269,11 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
 }
 
 // ---------------------------------------------------------------------------------------
-// Dense expansion only: lane <-> token, one ballot per row builds the packed word.
-// Same grid and row groups as the fused kernel; per_split counts 32-token words here.
+// Dense expansion only. Same row groups and class table as the fused kernel; a lane takes the octet of tokens next to its
+// neighbours', looks up its 8 class words once, turns them into one byte per row (four 8x8 bit transposes for the 32 rows)
+// and stores the bytes: 32 bytes side by side per row and warp. per_split counts 32-token words.
+// Bound: the table is built once per block, so few, long blocks; then instruction issue, some 160 instructions per 256 tokens
+// and 32 rows. (A ballot per token word and row took 850: 512 rows of 128256 tokens 37 us, now 14.)
 // ---------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_expand_dense(const __grid_constant__ StepArgs a) {
     extern __shared__ __align__(128) uint32_t smem[];
@@ -1288,27 +1296,24 @@ __global__ void __launch_bounds__(256) k_expand_dense(const __grid_constant__ St
     build_class_table(a, P, s_row, T, stage, warp, lane, n_warps);
     __syncthreads();
 
-    const int w_begin = split * a.per_split, w_end = min(w_begin + a.per_split, a.VW);
-    const int my_row = s_row[lane];
-    uint32_t* out = a.vocab_mask + int64_t(max(my_row, 0)) * a.vm_stride;
-    // a warp takes 8 consecutive words (256 tokens) per iteration; lane r ends up holding row r's words
-    for (int w0 = w_begin + warp * 8; w0 < w_end; w0 += n_warps * 8) {
-        uint32_t mine[8];
+    const int o_begin = 4 * split * a.per_split, o_end = min(o_begin + 4 * a.per_split, 4 * a.VW);  // octets
+    uint8_t* const vm8 = reinterpret_cast<uint8_t*>(a.vocab_mask);
+    for (int o0 = o_begin + warp * 32; o0 < o_end; o0 += n_warps * 32) {
+        const int o = o0 + lane;
+        if (o >= o_end) continue;
+        const uint4 cv = __ldg(reinterpret_cast<const uint4*>(P.c16) + o);  // padded to 32 * VW entries
+        const uint32_t w[8] = {T[cv.x & 0xFFFFu], T[cv.x >> 16], T[cv.y & 0xFFFFu], T[cv.y >> 16],
+                               T[cv.z & 0xFFFFu], T[cv.z >> 16], T[cv.w & 0xFFFFu], T[cv.w >> 16]};
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int w = w0 + q;
-            uint32_t bits = 0;
-            if (w < w_end) bits = T[P.c16[w * 32 + lane]];  // c16 is padded to 32*VW entries
-            mine[q] = 0;
-            for (int r = 0; r < nrow; ++r) {
-                const uint32_t word = __ballot_sync(0xFFFFFFFFu, (bits >> r) & 1u);
-                if (lane == r) mine[q] = word;
+        for (int rb = 0; rb < kGroupRows / kBatchRows; ++rb) {
+            if (rb * kBatchRows >= nrow) break;
+            uint32_t lo, hi;
+            row_batch_bytes(w, rb, lo, hi);
+#pragma unroll
+            for (int i = 0; i < kBatchRows; ++i) {
+                const int r = rb * kBatchRows + i;
+                if (r < nrow) st_global_u8(vm8 + int64_t(s_row[r]) * a.vm_stride * 4 + o, ((i < 4 ? lo : hi) >> (8 * (i & 3))) & 0xFFu);
             }
-        }
-        if (my_row >= 0) {
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-                if (w0 + q < w_end) out[w0 + q] = mine[q];
         }
     }
 }
@@ -1993,50 +1998,69 @@ __global__ void __launch_bounds__(1024) k_plan_rows(const PartDev* parts, int n_
 }
 
 // ---------------------------------------------------------------------------------------
-// mask_logits: apply an existing vocab bitmask in place. Octets whose 8 tokens are all
-// allowed are neither read nor written; octets with none allowed are written without a read.
+// mask_logits: apply an existing vocab bitmask in place. A row's vectors begin at its own first vector boundary, `head` tokens
+// in (0 for rows on the vector grid), so vector o takes its 8 bits from the bytes o and o + 1 of the mask. Vectors whose 8
+// tokens are all allowed are neither read nor written; those with none allowed are written without a read. The tokens left
+// over at both ends go one by one.
+// Bound: HBM (read and write once). The mask bytes of the next piece of work are fetched while the logits of this one are
+// on their way.
 // ---------------------------------------------------------------------------------------
-template <int DT, bool ALIGNED>
-__global__ void __launch_bounds__(256) k_mask_logits(void* logits, int64_t row_stride, int B, int V, int VW,
-                                                     const uint32_t* vocab_mask, int64_t vm_stride, int wide) {
+constexpr int kMaskUnroll = 4, kMaskChunk = 256 * kMaskUnroll;  // vectors per block and piece
+
+template <int DT>
+__global__ void __launch_bounds__(256) k_mask_logits(void* logits, int64_t row_stride, int B, int V, const uint32_t* vocab_mask,
+                                                     int64_t vm_stride, int chunks) {
     pdl_prologue();
     constexpr int ES = DT == kBF16 ? 2 : 4;
-    constexpr int U = 4;
-    const int n_octets = (V + 7) >> 3, n_full = V >> 3;
-    const int chunks = (n_octets + blockDim.x * U - 1) / (blockDim.x * U);
-    const int64_t total = int64_t(B) * chunks;
-    const uint8_t* vm8 = reinterpret_cast<const uint8_t*>(vocab_mask);
-    for (int64_t item = blockIdx.x; item < total; item += gridDim.x) {
-        const int row = int(item / chunks), ch = int(item - int64_t(row) * chunks);
+    const int total = B * chunks, tid = threadIdx.x;
+    struct Piece {
+        char* vec;  // first vector of the row
+        int o;      // this thread's first vector
+        uint32_t byte[kMaskUnroll];
+    };
+    auto fetch = [&](int item) {
+        Piece p;
+        const int row = item / chunks, ch = item - row * chunks;
         char* rowp = reinterpret_cast<char*>(logits) + int64_t(row) * row_stride * ES;
-        const uint8_t* vrow = vm8 + int64_t(row) * vm_stride * 4;
-        const int ob = ch * blockDim.x * U + threadIdx.x;
-        Octet<DT> oc[U];
-        uint32_t byte[U];
+        const uint8_t* bits = reinterpret_cast<const uint8_t*>(vocab_mask) + int64_t(row) * vm_stride * 4;
+        const int head = row_head<DT>(rowp, V), n_vec = (V - head) >> 3;
+        p.vec = rowp + head * ES;
+        p.o = ch * kMaskChunk + tid;
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int o = ob + u * blockDim.x;
-            byte[u] = 0xFFu;
-            if (o < n_octets) {
-                byte[u] = vrow[o];
-                if (8 * o + 8 > V) byte[u] = (byte[u] | (0xFFu << (V - 8 * o))) & 0xFFu;  // past V: leave alone
-                if (ALIGNED && o < n_full && byte[u] != 0xFFu && byte[u] != 0u) oc[u].load(rowp, o);
+        for (int u = 0; u < kMaskUnroll; ++u) {
+            const int o = p.o + u * 256;
+            p.byte[u] = 0xFFu;
+            if (o < n_vec) {
+                p.byte[u] = __ldg(bits + o);
+                if (head) p.byte[u] = ((p.byte[u] | (uint32_t(__ldg(bits + o + 1)) << 8)) >> head) & 0xFFu;
             }
         }
+        if (ch == 0 && tid < 16) {  // the ends of the row
+            const int t = tid < 8 ? tid : head + 8 * n_vec + tid - 8;
+            if ((tid < 8 ? t < head : t < V) && !((__ldg(bits + (t >> 3)) >> (t & 7)) & 1u)) store_neg_inf<DT>(rowp, t);
+        }
+        return p;
+    };
+    int item = blockIdx.x;
+    if (item >= total) return;
+    Piece p = fetch(item);
+    for (;;) {
+        Octet<DT> oc[kMaskUnroll];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int o = ob + u * blockDim.x;
-            if (o >= n_octets || byte[u] == 0xFFu) continue;
+        for (int u = 0; u < kMaskUnroll; ++u)
+            if (p.byte[u] != 0xFFu && p.byte[u] != 0u) oc[u].load(p.vec, p.o + u * 256);
+        const Piece now = p;
+        item += gridDim.x;
+        const bool more = item < total;
+        if (more) p = fetch(item);
+#pragma unroll
+        for (int u = 0; u < kMaskUnroll; ++u) {
+            if (now.byte[u] == 0xFFu) continue;
             float f[8];
-            if (ALIGNED && o < n_full) {
-                if (byte[u] == 0u) oc[u].fill_neg_inf(); else oc[u].mask(byte[u], f);
-                oc[u].store(rowp, o, wide != 0);
-            } else {
-#pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    if (8 * o + j < V && !((byte[u] >> j) & 1u)) store_neg_inf<DT>(rowp, 8 * o + j);
-            }
+            if (now.byte[u] == 0u) oc[u].fill_neg_inf(); else oc[u].mask(now.byte[u], f);
+            oc[u].store(now.vec, now.o + u * 256, true);  // (f32 vectors sit on 32-byte boundaries)
         }
+        if (!more) return;
     }
 }
 
@@ -2073,17 +2097,52 @@ __global__ void __launch_bounds__(256) k_rmw_floor(void* logits, int64_t row_str
     }
 }
 
-// logp_full[b, i] = z'[b, i] - lse[b] from the masked logits (fp32 out, row stride V).
-template <int DT>
+// logp_full[b, i] = z'[b, i] - lse[b] from the masked logits (fp32 out, row stride V). Bound: HBM. QUADS: rows of both sides
+// allow four tokens at a time (16-byte stores, 16- or 8-byte loads); otherwise a token per thread. Four loads per thread
+// are in flight either way (one at a time, token by token, took 42 us for 128 rows of 151936 f32 logits; now 20).
+template <int DT, bool QUADS>
 __global__ void __launch_bounds__(256) k_logp_full(const void* logits, int64_t row_stride, int B, int V, const float* lse,
                                                    float* out) {
     pdl_prologue();
-    // grid: x strides over the tokens of a row, y over the rows
+    constexpr int kPer = QUADS ? 4 : 1, kInFlight = 4;
+    const int units = V / kPer, tid = threadIdx.x;  // (V is a multiple of 4 with QUADS)
+    auto value = [](float z, float l) { return (l == -INFINITY || z == -INFINITY) ? -INFINITY : z - l; };
+    // grid: x strides over the pieces of a row, y over the rows
     for (int row = blockIdx.y; row < B; row += gridDim.y) {
-        const float l = lse[row];
-        for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < V; t += gridDim.x * blockDim.x) {
-            const float z = load_elem<DT>(logits, int64_t(row) * row_stride + t);
-            out[int64_t(row) * V + t] = (l == -INFINITY || z == -INFINITY) ? -INFINITY : z - l;
+        const float l = __ldg(lse + row);
+        const char* zrow = reinterpret_cast<const char*>(logits) + int64_t(row) * row_stride * (DT == kBF16 ? 2 : 4);
+        float* orow = out + int64_t(row) * V;
+        for (int u0 = blockIdx.x * 256 * kInFlight + tid; u0 < units; u0 += gridDim.x * 256 * kInFlight) {
+            if (QUADS) {
+                uint4 v[kInFlight];
+#pragma unroll
+                for (int k = 0; k < kInFlight; ++k) {
+                    const int u = u0 + k * 256;
+                    if (u >= units) break;
+                    if (DT == kF32) {
+                        v[k] = __ldcs(reinterpret_cast<const uint4*>(zrow) + u);
+                    } else {
+                        const uint2 h = __ldcs(reinterpret_cast<const uint2*>(zrow) + u);
+                        v[k] = make_uint4(h.x << 16, h.x & 0xFFFF0000u, h.y << 16, h.y & 0xFFFF0000u);
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < kInFlight; ++k) {
+                    const int u = u0 + k * 256;
+                    if (u >= units) break;
+                    __stcs(reinterpret_cast<float4*>(orow) + u,
+                           make_float4(value(__uint_as_float(v[k].x), l), value(__uint_as_float(v[k].y), l),
+                                       value(__uint_as_float(v[k].z), l), value(__uint_as_float(v[k].w), l)));
+                }
+            } else {
+                float z[kInFlight];
+#pragma unroll
+                for (int k = 0; k < kInFlight; ++k)
+                    if (u0 + k * 256 < units) z[k] = load_elem<DT>(zrow, u0 + k * 256);
+#pragma unroll
+                for (int k = 0; k < kInFlight; ++k)
+                    if (u0 + k * 256 < units) orow[u0 + k * 256] = value(z[k], l);
+            }
         }
     }
 }
