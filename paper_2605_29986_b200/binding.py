@@ -1,4 +1,4 @@
-"""Thin ctypes binding of ``include/cfgzip.h``: same names, argument marshalling only.
+"""Thin binding of ``include/cfgzip.h``: same names, argument marshalling only.
 
 Device buffers are passed as ``torch.Tensor`` (their ``data_ptr()`` is used), host buffers as
 numpy arrays or pinned CPU tensors; raw integer addresses are accepted everywhere. Nothing is
@@ -11,6 +11,9 @@ import ctypes
 from typing import Optional, Tuple
 
 from . import _build
+
+_build.build()
+from . import _calls  # noqa: E402
 
 F32, BF16 = 0, 1
 AUTO, DENSE, SPARSE = 0, 1, 2
@@ -74,6 +77,7 @@ def load_library():
             fn = getattr(lib, name)
             fn.restype = res
             fn.argtypes = args
+        _calls.bind({name: ctypes.cast(getattr(lib, name), _vp).value for name in _SIGNATURES}, _raise)
         _lib = lib
     return _lib
 
@@ -84,9 +88,13 @@ class CfgzipError(RuntimeError):
         super().__init__("%s failed: %s" % (call, cfgzip_status_string(status)))
 
 
+def _raise(status: int, call: str) -> None:
+    raise CfgzipError(status, call)
+
+
 def _check(status: int, call: str) -> None:
     if status != OK:
-        raise CfgzipError(status, call)
+        _raise(status, call)
 
 
 def _ptr(x):
@@ -147,68 +155,19 @@ def cfgzip_free_partition(ctx: int, part: int) -> None:
     _check(load_library().cfgzip_free_partition(ctx, part), "cfgzip_free_partition")
 
 
-def cfgzip_expand_mask(ctx: int, part0: int, row_part, class_mask, class_stride_words: int, vocab_mask,
-                       vocab_stride_words: int, B: int, mode: int = AUTO, stream=None) -> None:
-    _check(load_library().cfgzip_expand_mask(ctx, part0, _ptr(row_part), _ptr(class_mask), class_stride_words,
-                                             _ptr(vocab_mask), vocab_stride_words, B, mode, _stream(stream)),
-           "cfgzip_expand_mask")
-
-
-def cfgzip_mask_logits(ctx: int, logits, dtype: int, row_stride_elems: int, B: int, V: int, vocab_mask,
-                       vocab_stride_words: int, stream=None) -> None:
-    _check(load_library().cfgzip_mask_logits(ctx, _ptr(logits), dtype, row_stride_elems, B, V, _ptr(vocab_mask),
-                                             vocab_stride_words, _stream(stream)), "cfgzip_mask_logits")
-
-
-def cfgzip_masked_logsoftmax_argmax(ctx: int, part0: int, row_part, class_mask, class_stride_words: int, logits,
-                                    dtype: int, row_stride_elems: int, B: int, vocab_mask, vocab_stride_words: int,
-                                    argmax, rep=None, logp_argmax=None, lse=None, logp_full=None, mode: int = AUTO,
-                                    stream=None) -> None:
-    _check(load_library().cfgzip_masked_logsoftmax_argmax(
-        ctx, part0, _ptr(row_part), _ptr(class_mask), class_stride_words, _ptr(logits), dtype, row_stride_elems, B,
-        _ptr(vocab_mask), vocab_stride_words, _ptr(argmax), _ptr(rep), _ptr(logp_argmax), _ptr(lse), _ptr(logp_full),
-        mode, _stream(stream)), "cfgzip_masked_logsoftmax_argmax")
-
-
-def cfgzip_masked_sample(ctx: int, part0: int, row_part, class_mask, class_stride_words: int, logits, dtype: int,
-                         row_stride_elems: int, B: int, vocab_mask, vocab_stride_words: int, u, inv_temperature: float,
-                         token, rep=None, logp_token=None, lse=None, mode: int = AUTO, stream=None) -> None:
-    _check(load_library().cfgzip_masked_sample(
-        ctx, part0, _ptr(row_part), _ptr(class_mask), class_stride_words, _ptr(logits), dtype, row_stride_elems, B,
-        _ptr(vocab_mask), vocab_stride_words, _ptr(u), inv_temperature, _ptr(token), _ptr(rep), _ptr(logp_token),
-        _ptr(lse), mode, _stream(stream)), "cfgzip_masked_sample")
-
-
-def cfgzip_masked_sample_filtered(ctx: int, part0: int, row_part, class_mask, class_stride_words: int, logits, dtype: int,
-                                  row_stride_elems: int, B: int, vocab_mask, vocab_stride_words: int, u,
-                                  inv_temperature: float, top_k: int, top_p: float, token, rep=None, logp_token=None,
-                                  lse=None, mode: int = AUTO, stream=None) -> None:
-    _check(load_library().cfgzip_masked_sample_filtered(
-        ctx, part0, _ptr(row_part), _ptr(class_mask), class_stride_words, _ptr(logits), dtype, row_stride_elems, B,
-        _ptr(vocab_mask), vocab_stride_words, _ptr(u), inv_temperature, top_k, top_p, _ptr(token), _ptr(rep),
-        _ptr(logp_token), _ptr(lse), mode, _stream(stream)), "cfgzip_masked_sample_filtered")
-
-
-def cfgzip_multi_mask_logsoftmax_argmax(ctx: int, part0: int, class_masks, class_stride_words: int, masks_per_row: int,
-                                        logits, dtype: int, row_stride_elems: int, B: int, vocab_masks,
-                                        vocab_stride_words: int, argmax, rep=None, logp_argmax=None, lse=None,
-                                        stream=None) -> None:
-    _check(load_library().cfgzip_multi_mask_logsoftmax_argmax(
-        ctx, part0, _ptr(class_masks), class_stride_words, masks_per_row, _ptr(logits), dtype, row_stride_elems, B,
-        _ptr(vocab_masks), vocab_stride_words, _ptr(argmax), _ptr(rep), _ptr(logp_argmax), _ptr(lse), _stream(stream)),
-        "cfgzip_multi_mask_logsoftmax_argmax")
-
+# The calls a program makes once per decode step are native functions with the arguments of the header, by position or by
+# name (csrc/calls.c); result buffers that are not wanted, the mode (AUTO) and the stream (legacy default) may be left out.
+cfgzip_expand_mask = _calls.cfgzip_expand_mask
+cfgzip_mask_logits = _calls.cfgzip_mask_logits
+cfgzip_masked_logsoftmax_argmax = _calls.cfgzip_masked_logsoftmax_argmax
+cfgzip_masked_sample = _calls.cfgzip_masked_sample
+cfgzip_masked_sample_filtered = _calls.cfgzip_masked_sample_filtered
+cfgzip_multi_mask_logsoftmax_argmax = _calls.cfgzip_multi_mask_logsoftmax_argmax
+cfgzip_plan_rows = _calls.cfgzip_plan_rows
+cfgzip_map_tokens = _calls.cfgzip_map_tokens
+cfgzip_decode_step_host = _calls.cfgzip_decode_step_host
 
 ROWS_AS_PLANNED = 1  # pass as row_part after cfgzip_plan_rows: the kept grouping of that call is reused
-
-
-def cfgzip_plan_rows(ctx: int, part0: int, row_part, B: int, stream=None) -> None:
-    _check(load_library().cfgzip_plan_rows(ctx, part0, _ptr(row_part), B, _stream(stream)), "cfgzip_plan_rows")
-
-
-def cfgzip_map_tokens(ctx: int, part0: int, row_part, tokens, reps, B: int, stream=None) -> None:
-    _check(load_library().cfgzip_map_tokens(ctx, part0, _ptr(row_part), _ptr(tokens), _ptr(reps), B, _stream(stream)),
-           "cfgzip_map_tokens")
 
 
 def cfgzip_choose_mode(ctx: int, part0: int, row_part_host, class_mask_host, class_stride_words: int, B: int,
@@ -219,15 +178,6 @@ def cfgzip_choose_mode(ctx: int, part0: int, row_part_host, class_mask_host, cla
     if mode < 0:
         raise CfgzipError(mode, "cfgzip_choose_mode")
     return mode
-
-
-def cfgzip_decode_step_host(ctx: int, part0: int, row_part_host, class_mask_host, class_stride_words: int,
-                            logits_host, dtype: int, B: int, masked_logits=None, vocab_mask_host=None, argmax=None,
-                            rep=None, logp_argmax=None, lse=None, mode: int = AUTO, stream=None) -> None:
-    _check(load_library().cfgzip_decode_step_host(
-        ctx, part0, _ptr(row_part_host), _ptr(class_mask_host), class_stride_words, _ptr(logits_host), dtype, B,
-        _ptr(masked_logits), _ptr(vocab_mask_host), _ptr(argmax), _ptr(rep), _ptr(logp_argmax), _ptr(lse), mode,
-        _stream(stream)), "cfgzip_decode_step_host")
 
 
 def cfgzip_step_noalloc(token_to_class, V: int, class_to_rep, K: int, class_mask, class_stride_words: int, logits,

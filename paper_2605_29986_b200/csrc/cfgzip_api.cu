@@ -8,6 +8,7 @@
 #include <cstring>
 #include <mutex>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "cfgzip.h"
@@ -73,6 +74,7 @@ struct cfgzip_ctx {
     int32_t st_rows = 0;
     int32_t* st_small_host = nullptr;  // pinned mirror of the four result arrays: they come back in one copy
     int64_t launches = 0;
+    std::vector<std::pair<const void*, size_t>> smem_allowed;  // kernels whose shared-memory limit has been raised, and to what
     // row plan kept by cfgzip_plan_rows (valid until anything overwrites the plan buffers or the partitions change)
     bool plan_valid = false;
     bool plan_in_use = false;  // set for the duration of a call that passed CFGZIP_ROWS_AS_PLANNED
@@ -117,7 +119,8 @@ struct DeviceGuard {
     bool ok = true;
     explicit DeviceGuard(int dev) {
         if (cudaGetDevice(&prev) != cudaSuccess) { ok = false; return; }
-        if (prev != dev && cudaSetDevice(dev) != cudaSuccess) ok = false;
+        if (prev == dev) prev = -1;  // nothing to put back
+        else if (cudaSetDevice(dev) != cudaSuccess) ok = false;
     }
     ~DeviceGuard() { if (prev >= 0) cudaSetDevice(prev); }
 };
@@ -156,13 +159,26 @@ int launch(cfgzip_ctx* ctx, void (*kernel)(KArgs...), dim3 grid, dim3 block, siz
     return CFGZIP_OK;
 }
 
+// More than 48 KB of dynamic shared memory has to be allowed once per kernel; it is allowed up to the device's limit, so that
+// the limit another context may have set is never smaller, and remembered: asking the runtime on every step costs half a
+// microsecond of host time.
 template <typename K>
-int ensure_smem(K kernel, size_t bytes) {
+int ensure_smem(cfgzip_ctx* ctx, K kernel, size_t bytes) {
     if (bytes <= 48 * 1024) return CFGZIP_OK;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes)) != cudaSuccess) {
+    const void* fn = reinterpret_cast<const void*>(kernel);
+    for (const auto& k : ctx->smem_allowed)
+        if (k.first == fn) return bytes <= k.second ? CFGZIP_OK : CFGZIP_E_CUDA;
+    cudaFuncAttributes attr;
+    if (cudaFuncGetAttributes(&attr, fn) != cudaSuccess) {
         cudaGetLastError();
         return CFGZIP_E_CUDA;
     }
+    const size_t most = size_t(ctx->smem_optin) - std::min(size_t(ctx->smem_optin), attr.sharedSizeBytes);
+    if (bytes > most || cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(most)) != cudaSuccess) {
+        cudaGetLastError();
+        return CFGZIP_E_CUDA;
+    }
+    ctx->smem_allowed.emplace_back(fn, most);
     return CFGZIP_OK;
 }
 
@@ -586,7 +602,7 @@ int launch_pipe(cfgzip_ctx* ctx, const StepArgs& a, const DensePlan& d, dim3 gri
         kern = CFGZIP_PIPE_VARIANT(1, 512, 1);
 #undef CFGZIP_PIPE_VARIANT
 #undef CFGZIP_PIPE_SRC
-    if ((rc = ensure_smem(kern, d.smem)) != CFGZIP_OK) return rc;
+    if ((rc = ensure_smem(ctx, kern, d.smem)) != CFGZIP_OK) return rc;
     return launch(ctx, kern, grid, block, d.smem, st, a, tmap);
 }
 
@@ -601,7 +617,7 @@ int launch_fused(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, in
             a.per_split = per_split;
             const size_t smem = size_t(per_split) * 4;
             auto kern = k_step_sparse<DT, true>;
-            if ((rc = ensure_smem(kern, smem)) != CFGZIP_OK) return rc;
+            if ((rc = ensure_smem(ctx, kern, smem)) != CFGZIP_OK) return rc;
             rc = launch(ctx, kern, dim3(unsigned(a.B) * unsigned(S)), dim3(256), smem, st, a);
         } else {
             rc = launch(ctx, k_step_generic<DT, true>, dim3(unsigned(a.B)), dim3(256), 0, st, a);
@@ -637,7 +653,7 @@ int launch_fused(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, in
                 b.per_split = sp_per;
                 const size_t smem = size_t(sp_per) * 4;
                 auto kern = k_step_sparse<DT, true>;
-                if ((rc = ensure_smem(kern, smem)) != CFGZIP_OK) return rc;
+                if ((rc = ensure_smem(ctx, kern, smem)) != CFGZIP_OK) return rc;
                 if ((rc = launch(ctx, kern, dim3(unsigned(d.n_groups_ub) * kGroupRows * unsigned(sp_S)), dim3(256), smem, st, b)) !=
                     CFGZIP_OK)
                     return rc;
@@ -647,7 +663,7 @@ int launch_fused(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, in
                 rc = launch_pipe<DT>(ctx, a, d, grid, block, st);
             } else {
                 auto kern = k_step_dense<DT>;
-                if ((rc = ensure_smem(kern, d.smem)) != CFGZIP_OK) return rc;
+                if ((rc = ensure_smem(ctx, kern, d.smem)) != CFGZIP_OK) return rc;
                 rc = launch(ctx, kern, grid, block, d.smem, st, a);
             }
             // second kernel: one block per row folds the published states and writes the results (unless the
@@ -659,7 +675,7 @@ int launch_fused(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, in
                 {
                     const unsigned rows_grid = unsigned(d.n_groups_ub) * kGroupRows;
                     const size_t pad = row_blocks_pad(ctx, rows_grid, a.B);
-                    if (pad && (rc = ensure_smem(k_finalize_rows<DT>, pad)) != CFGZIP_OK) return rc;
+                    if (pad && (rc = ensure_smem(ctx, k_finalize_rows<DT>, pad)) != CFGZIP_OK) return rc;
                     rc = launch(ctx, k_finalize_rows<DT>, dim3(rows_grid), dim3(kFinalizeThreads), pad, st, a);
                 }
             }
@@ -684,7 +700,7 @@ int launch_fused(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, in
 template <int DT>
 int launch_filtered(cfgzip_ctx* ctx, const StepArgs& a, unsigned rows_grid, int top_k, float top_p, cudaStream_t st) {
     int rc;
-    if ((rc = ensure_smem(k_sample_filtered<DT>, sizeof(FiltShared))) != CFGZIP_OK) return rc;
+    if ((rc = ensure_smem(ctx, k_sample_filtered<DT>, sizeof(FiltShared))) != CFGZIP_OK) return rc;
     const unsigned fit = 2u * unsigned(std::max(ctx->sm_count, 1));
     unsigned per_row = kFiltPeers;
     while (per_row > 1 && unsigned(a.B) * per_row > fit) per_row /= 2;
@@ -724,7 +740,7 @@ int launch_sample(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, b
         const unsigned rows_grid = unsigned(d.n_groups_ub) * kGroupRows;
         if (filtered) return launch_filtered<DT>(ctx, a, rows_grid, top_k, top_p, st);
         const size_t pad = row_blocks_pad(ctx, rows_grid, a.B);
-        if (pad && (rc = ensure_smem(k_sample_rows<DT>, pad)) != CFGZIP_OK) return rc;
+        if (pad && (rc = ensure_smem(ctx, k_sample_rows<DT>, pad)) != CFGZIP_OK) return rc;
         return launch(ctx, k_sample_rows<DT>, dim3(rows_grid), dim3(kSampleThreads), pad, st, a, 1);
     }
     if (size_t(a.B) > kPartialSlots) return CFGZIP_E_NOMEM;
@@ -1037,7 +1053,7 @@ int cfgzip_expand_mask(cfgzip_ctx* ctx, cfgzip_part_id part0, const int32_t* row
             a.per_split = per_split;
             const size_t smem = size_t(per_split) * 4;
             auto kern = k_step_sparse<kF32, false>;
-            if ((rc = ensure_smem(kern, smem)) != CFGZIP_OK) return rc;
+            if ((rc = ensure_smem(ctx, kern, smem)) != CFGZIP_OK) return rc;
             return launch(ctx, kern, dim3(unsigned(B) * unsigned(S)), dim3(256), smem, st, a);
         }
         return launch(ctx, k_step_generic<kF32, false>, dim3(unsigned(B)), dim3(256), 0, st, a);
@@ -1046,7 +1062,7 @@ int cfgzip_expand_mask(cfgzip_ctx* ctx, cfgzip_part_id part0, const int32_t* row
     if (!d.ok) return launch(ctx, k_step_generic<kF32, false>, dim3(unsigned(B)), dim3(256), 0, st, a);
     if (d.use_plan_kernel && (rc = run_plan_kernel(ctx, row_part, B, ps.V, d, st)) != CFGZIP_OK) return rc;
     fill_groups(ctx, a, d);
-    if ((rc = ensure_smem(k_expand_dense, d.smem)) != CFGZIP_OK) return rc;
+    if ((rc = ensure_smem(ctx, k_expand_dense, d.smem)) != CFGZIP_OK) return rc;
     return launch(ctx, k_expand_dense, dim3(unsigned(d.n_groups_ub) * unsigned(d.S)), dim3(256), d.smem, st, a);
 }
 
@@ -1237,7 +1253,7 @@ int cfgzip_multi_mask_logsoftmax_argmax(cfgzip_ctx* ctx, cfgzip_part_id part0, c
     ctx->pdl_now = int64_t(B) * ps.V * es < (int64_t(192) << 20);
     ctx->prefetch_now = int64_t(B) * ps.V * es >= (int64_t(ctx->prefetch_min_mbytes) << 20);
     auto kern = dtype == CFGZIP_BF16 ? k_step_dense<kBF16> : k_step_dense<kF32>;
-    if ((rc = ensure_smem(kern, d.smem)) == CFGZIP_OK)
+    if ((rc = ensure_smem(ctx, kern, d.smem)) == CFGZIP_OK)
         rc = launch(ctx, kern, dim3(unsigned(d.n_groups_ub) * unsigned(d.S)), dim3(unsigned(d.threads)), d.smem, st, a);
     if (rc == CFGZIP_OK) {
         auto fin = dtype == CFGZIP_BF16 ? k_finalize_rows<kBF16> : k_finalize_rows<kF32>;
