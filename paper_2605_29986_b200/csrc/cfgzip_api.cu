@@ -459,6 +459,36 @@ DensePlan plan_pipe(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, i
     return items >= kTwoOctetItemsPerWarp * warps ? two : one;
 }
 
+// Launch shape of the kernel for rows that allow few tokens: three blocks per SM; warps go side by side along the vocabulary
+// as long as a block has enough chunks for them, else they split the row batches. Below kFewRows rows a group of 32 leaves the
+// blocks too little to do between their set-up and the second launch: a block or more per row, one launch, is as fast there
+// (4 rows of 184913 f32: 11.8 against 10.5 us; 32 of 128256: 13.1 against 15.5).
+constexpr int kFewRows = 64;
+DensePlan plan_few(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, int elem_size) {
+    DensePlan d;
+    d.table_words = (ps.maxKW + 1) * 32;
+    d.use_plan_kernel = mixed;
+    d.n_groups_ub = mixed ? ceil_div(B, kGroupRows) + ps.n_live_same_v : ceil_div(B, kGroupRows);
+    if (B < kFewRows || !ps.all_c16 || (mixed && (B > ctx->reserved_rows || d.n_groups_ub > ctx->max_groups))) return d;
+    const size_t fixed = dense_smem_bytes(d.table_words, kFewWarps, 0) + kFewWarps * sizeof(FewWarp);
+    const size_t staging = size_t(ps.maxKW | 1) * kGroupRows * 4;
+    if (fixed > size_t(ctx->smem_optin) - 2048) return d;
+    if (fixed + staging <= 72 * 1024) d.stage_stride = ps.maxKW | 1;  // three blocks per SM still fit
+    d.smem = fixed + (d.stage_stride ? staging : 0);
+    const int n_chunks = std::max(1, ceil_div(ps.V / (32 / elem_size), 32));
+    const int row_batches = ceil_div(std::min<int>(B, kGroupRows), kBatchRows);
+    const int per_sm = std::max(1, std::min(3, int(size_t(ctx->smem_optin) / (d.smem + 1024))));
+    d.S = std::min(std::max(1, per_sm * ctx->sm_count / ceil_div(B, kGroupRows)), n_chunks);
+    while (d.S > 1 && size_t(d.n_groups_ub) * kGroupRows * (size_t(d.S) * kFewWarps + 1) > kPartialSlots) d.S = (d.S + 1) / 2;
+    int WR = 1;
+    while (WR < 4 && WR < row_batches && ceil_div(n_chunks, d.S) * WR * 2 <= kFewWarps) WR <<= 1;
+    d.WT = kFewWarps / WR;
+    d.threads = kFewThreads;
+    d.slots = d.S * d.WT + 1;
+    d.ok = size_t(d.n_groups_ub) * kGroupRows * d.slots <= kPartialSlots;
+    return d;
+}
+
 // A call may pass CFGZIP_ROWS_AS_PLANNED for its row -> partition vector: it then means the vector given to the
 // last cfgzip_plan_rows, whose grouping is still in the plan buffers.
 int resolve_row_part(cfgzip_ctx* ctx, cfgzip_part_id part0, const int32_t** row_part, int32_t B, bool* planned) {
@@ -606,11 +636,33 @@ int launch_pipe(cfgzip_ctx* ctx, const StepArgs& a, const DensePlan& d, dim3 gri
     return launch(ctx, kern, grid, block, d.smem, st, a, tmap);
 }
 
+// Second kernel of a step: folds the states a row's blocks have published and writes the row's results.
+template <int DT>
+int launch_finalize(cfgzip_ctx* ctx, const StepArgs& a, const DensePlan& d, cudaStream_t st) {
+    if (a.slots <= kFinalizeWarpStates)  // few states per row: a warp per row
+        return launch(ctx, k_finalize_rows_warp<DT>, dim3(unsigned(d.n_groups_ub) * (kGroupRows / 8)), dim3(256), 0, st, a);
+    const unsigned rows_grid = unsigned(d.n_groups_ub) * kGroupRows;
+    const size_t pad = row_blocks_pad(ctx, rows_grid, a.B);
+    int rc;
+    if (pad && (rc = ensure_smem(ctx, k_finalize_rows<DT>, pad)) != CFGZIP_OK) return rc;
+    return launch(ctx, k_finalize_rows<DT>, dim3(rows_grid), dim3(kFinalizeThreads), pad, st, a);
+}
+
 template <int DT>
 int launch_fused(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, int mode, bool aligned, float* logp_full,
                  cudaStream_t st) {
     int rc;
-    if (aligned && mode == CFGZIP_SPARSE) {
+    DensePlan few;
+    if (aligned && mode == CFGZIP_SPARSE) few = plan_few(ctx, ps, a.B, mixed, DT == kBF16 ? 2 : 4);
+    if (few.ok) {
+        if (few.use_plan_kernel && (rc = run_plan_kernel(ctx, a.row_part, a.B, a.V, few, st)) != CFGZIP_OK) return rc;
+        fill_groups(ctx, a, few);
+        if ((rc = ensure_smem(ctx, k_step_few<DT>, few.smem)) != CFGZIP_OK) return rc;
+        if ((rc = launch(ctx, k_step_few<DT>, dim3(unsigned(few.n_groups_ub) * unsigned(few.S)), dim3(kFewThreads), few.smem, st, a)) !=
+            CFGZIP_OK)
+            return rc;
+        rc = launch_finalize<DT>(ctx, a, few, st);
+    } else if (aligned && mode == CFGZIP_SPARSE) {
         int S, per_split;
         if (plan_sparse(ctx, ps, a.B, true, &S, &per_split)) {
             a.S = S;
@@ -668,17 +720,7 @@ int launch_fused(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, in
             }
             // second kernel: one block per row folds the published states and writes the results (unless the
             // streaming kernel's last block of each group has done so)
-            if (rc == CFGZIP_OK && !(d.depth && d.fold)) {
-                if (a.slots <= kFinalizeWarpStates)  // few states per row: a warp per row
-                    rc = launch(ctx, k_finalize_rows_warp<DT>, dim3(unsigned(d.n_groups_ub) * (kGroupRows / 8)), dim3(256), 0, st, a);
-                else
-                {
-                    const unsigned rows_grid = unsigned(d.n_groups_ub) * kGroupRows;
-                    const size_t pad = row_blocks_pad(ctx, rows_grid, a.B);
-                    if (pad && (rc = ensure_smem(ctx, k_finalize_rows<DT>, pad)) != CFGZIP_OK) return rc;
-                    rc = launch(ctx, k_finalize_rows<DT>, dim3(rows_grid), dim3(kFinalizeThreads), pad, st, a);
-                }
-            }
+            if (rc == CFGZIP_OK && !(d.depth && d.fold)) rc = launch_finalize<DT>(ctx, a, d, st);
         } else {
             rc = launch(ctx, k_step_generic<DT, true>, dim3(unsigned(a.B)), dim3(256), 0, st, a);
         }

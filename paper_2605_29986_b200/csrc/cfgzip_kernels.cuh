@@ -414,8 +414,9 @@ __device__ __forceinline__ float float_from_order_key(int k) { return __int_as_f
 // rows of the group are dealt over its blocks and their warps, each warp takes its rows one at a time with a lane per
 // token (lanes 0..7 the first octet, lanes 8..23 the 16 tokens from the last whole octet on), allow bits from the class
 // table: two round trips to memory for a row, where one lane walking the tokens took two per token.
-// to_head / to_tail(row slot): where the states go (the same place: one state for both).
-template <int DT, bool SHIFT, typename H, typename T>
+// to_head / to_tail(row slot): where the states go (the same place: one state for both). UNIT: tokens the vectors are taken in
+// (8, or 16 for a kernel that takes them two at a time; rows on the vector grid only).
+template <int DT, bool SHIFT, int UNIT = 8, typename H, typename T>
 __device__ __forceinline__ void publish_edges(const StepArgs& a, const PartDev& P, const uint32_t* table, const int* s_row,
                                               int nrow, int split, int warp, int lane, float scale, bool apart, H&& to_head,
                                               T&& to_tail) {
@@ -438,13 +439,16 @@ __device__ __forceinline__ void publish_edges(const StepArgs& a, const PartDev& 
         const int row = s_row[j];
         char* rowp = reinterpret_cast<char*>(a.logits) + int64_t(row) * a.row_stride * ES;
         const int head = SHIFT ? row_head<DT>(rowp, a.V) : 0;
-        const int tail = head + ((a.V - head) & ~7);  // first token past the last whole vector
+        const int tail = head + ((a.V - head) & ~(UNIT - 1));  // first token past the last whole vector
         const bool mine = have && (in_head ? t < head : t >= tail);
         const bool allowed = (word >> j) & 1u;
         const uint32_t allow = __ballot_sync(0xFFFFFFFFu, allowed && !in_head);
-        if (a.vocab_mask && lane < n_octets - n_full)
-            reinterpret_cast<uint8_t*>(a.vocab_mask)[int64_t(row) * a.vm_stride * 4 + n_full + lane] =
-                lane == 0 ? uint8_t(allow >> 16) : uint8_t(0);
+        const int first = UNIT == 8 ? n_full : n_full & ~1;  // first octet that is not all in whole vectors
+        if (a.vocab_mask && lane < n_octets - first) {
+            const int o = first + lane;
+            reinterpret_cast<uint8_t*>(a.vocab_mask)[int64_t(row) * a.vm_stride * 4 + o] =
+                o == n_full ? uint8_t(allow >> 16) : (o < n_full ? uint8_t(allow >> 8) : uint8_t(0));
+        }
         float z = -INFINITY;
         if (mine) {
             if (allowed) z = load_elem<DT>(rowp, t);
@@ -457,7 +461,7 @@ __device__ __forceinline__ void publish_edges(const StepArgs& a, const PartDev& 
             for (int d = 16; d >= 1; d >>= 1) e += __shfl_xor_sync(0xFFFFFFFFu, e, d);
             return Partial{m, e, m > -INFINITY ? first : kNoPos, 0};
         };
-        const Partial pt = reduce(mine && !in_head, (a.V - head) >> 3);
+        const Partial pt = reduce(mine && !in_head, UNIT == 8 ? (a.V - head) >> 3 : tail >> 3);
         if (!SHIFT) {
             if (lane == 0) *to_tail(j) = pt;
         } else {
@@ -1319,7 +1323,187 @@ __global__ void __launch_bounds__(256) k_expand_dense(const __grid_constant__ St
 }
 
 // ---------------------------------------------------------------------------------------
-// Sparse step: one row per block (S blocks per row). The row's vocab bitmask is built in
+// Step for rows that allow few tokens. Row groups and class table as in the gather kernels. A warp takes 32 vectors of 32
+// bytes (8 f32 or 16 bf16 tokens) of 8 rows at a time; a vector without an allowed token is overwritten with -inf at once,
+// without being read, the others go into a queue of the warp. Whenever 32 have come together they are asked for, a lane each,
+// and the 32 asked for before are masked, written back and folded into the lane's states of the 8 rows (shared memory).
+// Bound: HBM. The -inf stream waits for no load; alone it runs at 5.9 TB/s, and the reads, scattered sectors between the
+// writes, cost a third on top (measured without them: 1024 rows of 128256 f32 logits 134 -> 100 us; more blocks per SM, longer
+// runs per row, asking for the sectors ahead of the stream: no gain). Building every row's mask from the class lists first,
+// a block per row, as the kernel below does, streams nothing meanwhile: 256 to 1024 bf16 rows take 10 to 40 % longer that way
+// (159 rows of 51648 over eight partitions 26.6 -> 17.1 us, 300 of 250000 92 -> 66, 128 of 128256 f32 30 -> 24).
+// Vectors of 32 bytes because a sector whose halves are written at different times costs a read of DRAM.
+// ---------------------------------------------------------------------------------------
+constexpr int kFewThreads = 256, kFewWarps = kFewThreads / 32;
+constexpr int kFewQueue = 64;  // fewer than 32 entries are left when a row adds up to 32
+struct FewWarp {
+    float m[kBatchRows][32], s[kBatchRows][32];
+    int pos[kBatchRows][32];
+    uint2 queue[kFewQueue];  // vector << 3 | row of the batch, allow bits
+};
+
+template <int DT>
+struct FewVec {  // 32 bytes of a row
+    static constexpr int kTokens = DT == kBF16 ? 16 : 8;
+    Octet<DT> o[DT == kBF16 ? 2 : 1];
+    __device__ __forceinline__ void load(const char* p) {
+        o[0].load(p, 0);
+        if (DT == kBF16) o[DT == kBF16].load(p, 1);
+    }
+    __device__ __forceinline__ void store(char* p, bool wide) const {
+        if constexpr (DT == kBF16) {
+            if (wide) {
+                st_stream32(p, o[0].v, o[1].v);
+            } else {
+                o[0].store(p, 0);
+                o[1].store(p, 1);
+            }
+        } else {
+            o[0].store_at(p, wide);
+        }
+    }
+};
+
+template <int DT>
+__global__ void __launch_bounds__(kFewThreads, 3) k_step_few(const __grid_constant__ StepArgs a) {
+    using Vec = FewVec<DT>;
+    constexpr int kOct = Vec::kTokens / 8;  // octets per vector
+    extern __shared__ __align__(128) uint32_t smem[];
+    uint32_t* T = smem;
+    int* s_row = reinterpret_cast<int*>(T + a.table_words);
+    FewWarp* s_warp = reinterpret_cast<FewWarp*>(s_row + kGroupRows);
+    uint32_t* stage = reinterpret_cast<uint32_t*>(s_warp + kFewWarps);
+
+    pdl_prologue();
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int g = blockIdx.x / a.S, split = blockIdx.x - g * a.S;
+    if (a.n_groups && g >= __ldg(a.n_groups)) return;
+    const int part = group_rows_setup(a, g, s_row, tid);
+    __syncthreads();
+    const PartDev P = a.group_part ? a.parts[part] : a.p0;
+    const int nrow = __popc(__ballot_sync(0xFFFFFFFFu, s_row[lane] >= 0));
+    if (a.stage_stride) {
+        stage_class_masks(a, P, s_row, stage, warp, lane, kFewWarps);
+        __syncthreads();
+    }
+    build_class_table(a, P, s_row, T, stage, warp, lane, kFewWarps);
+    __syncthreads();
+
+    constexpr int ES = DT == kBF16 ? 2 : 4;
+    const int wt = warp % a.WT, wr = warp / a.WT, WR = kFewWarps / a.WT;
+    const int n_vec = a.V / Vec::kTokens, n_chunks = (n_vec + 31) >> 5, stride = a.S * a.WT;
+    const bool wide = a.wide != 0;
+    uint8_t* const vm8 = reinterpret_cast<uint8_t*>(a.vocab_mask);
+    publish_edges<DT, false, Vec::kTokens>(
+        a, P, T, s_row, nrow, split, warp, lane, kLog2e, false, [&](int j) { return row_slots(a, g, j); },
+        [&](int j) { return row_slots(a, g, j) + a.slots - 1; });
+    const uint4* const ids = reinterpret_cast<const uint4*>(P.c16);
+    FewWarp& w = s_warp[warp];
+    for (int rb = wr; rb * kBatchRows < nrow; rb += WR) {
+        const int live = min(kBatchRows, nrow - rb * kBatchRows);
+        const int* const rows = s_row + rb * kBatchRows;
+        auto row_base = [&](int i) { return reinterpret_cast<char*>(a.logits) + int64_t(rows[i]) * a.row_stride * ES; };
+#pragma unroll
+        for (int i = 0; i < kBatchRows; ++i) {
+            w.m[i][lane] = -INFINITY;
+            w.s[i][lane] = 0.f;
+            w.pos[i][lane] = kNoPos;
+        }
+        Vec held;         // what this lane has asked for
+        uint2 entry = make_uint2(0u, 0u);  // and its queue entry (no allow bits: nothing)
+        auto consume = [&]() {
+            if (!entry.y) return;
+            const int i = entry.x & 7, v = entry.x >> 3;
+            float f[Vec::kTokens];
+#pragma unroll
+            for (int q = 0; q < kOct; ++q) held.o[q].mask((entry.y >> (8 * q)) & 0xFFu, f + 8 * q);
+            held.store(row_base(i) + size_t(v) * 32, wide);
+            float m = f[0];
+#pragma unroll
+            for (int q = 1; q < Vec::kTokens; ++q) m = fmaxf(m, f[q]);
+            const float ref = fmaxf(m, kRefFloor);
+            float sum = 0.f;
+#pragma unroll
+            for (int q = 0; q < Vec::kTokens; ++q) sum += ex2f((f[q] - ref) * kLog2e);
+            float m0 = w.m[i][lane], s0 = w.s[i][lane];
+            int p0 = w.pos[i][lane];
+            partial_merge(m0, s0, p0, m, sum, m > -INFINITY ? v * kOct : kNoPos);
+            w.m[i][lane] = m0;
+            w.s[i][lane] = s0;
+            w.pos[i][lane] = p0;
+        };
+        int head = 0, count = 0;  // of the queue
+        auto ask = [&]() {        // consume what was asked for, ask for the next 32 (or what is left)
+            consume();
+            entry = make_uint2(0u, 0u);
+            if (lane < count) {
+                entry = w.queue[(head + lane) & (kFewQueue - 1)];
+                held.load(row_base(entry.x & 7) + size_t(entry.x >> 3) * 32);
+            }
+            const int n = min(count, 32);
+            head += n;
+            count -= n;
+            __syncwarp();
+        };
+        int c = (split * a.WT + wt - rb * a.rot_chunks) % stride;  // the deal starts at another warp for every row batch
+        if (c < 0) c += stride;
+        uint4 cv[kOct];
+        auto fetch_ids = [&](int chunk) {
+#pragma unroll
+            for (int q = 0; q < kOct; ++q)
+                if (chunk * 32 + lane < n_vec) cv[q] = __ldg(ids + (chunk * 32 + lane) * kOct + q);
+        };
+        fetch_ids(c);
+        for (; c < n_chunks; c += stride) {
+            const int v = c * 32 + lane;
+            const bool active = v < n_vec;
+            uint32_t lo[kOct], hi[kOct];
+#pragma unroll
+            for (int q = 0; q < kOct; ++q) octet_allow_bits(cv[q], T, rb, active, lo[q], hi[q]);
+            fetch_ids(c + stride);
+#pragma unroll
+            for (int i = 0; i < kBatchRows; ++i) {
+                if (i >= live) break;
+                uint32_t bits = 0u;
+#pragma unroll
+                for (int q = 0; q < kOct; ++q) bits |= (((i < 4 ? lo[q] : hi[q]) >> (8 * (i & 3))) & 0xFFu) << (8 * q);
+                const int row = rows[i];
+                if (active && vm8) {
+                    uint8_t* const vm = vm8 + int64_t(row) * a.vm_stride * 4 + v * kOct;
+                    if (kOct == 1) st_global_u8(vm, bits); else st_global_u16(vm, bits);
+                }
+                const uint32_t some = __ballot_sync(0xFFFFFFFFu, bits != 0u);
+                if (bits) {
+                    w.queue[(head + count + __popc(some & ((1u << lane) - 1u))) & (kFewQueue - 1)] =
+                        make_uint2((unsigned(v) << 3) | unsigned(i), bits);
+                } else if (active) {
+                    Vec none;
+#pragma unroll
+                    for (int q = 0; q < kOct; ++q) none.o[q].fill_neg_inf();
+                    none.store(reinterpret_cast<char*>(a.logits) + int64_t(row) * a.row_stride * ES + size_t(v) * 32, wide);
+                }
+                count += __popc(some);
+                __syncwarp();
+                if (count >= 32) ask();
+            }
+        }
+        ask();
+        ask();
+        consume();
+        RowAcc acc[kBatchRows];
+#pragma unroll
+        for (int i = 0; i < kBatchRows; ++i) {
+            acc[i].m = w.m[i][lane];
+            acc[i].s = w.s[i][lane];
+            acc[i].nrl = -(fmaxf(acc[i].m, kRefFloor) * kLog2e);
+            acc[i].pos = w.pos[i][lane];
+        }
+        warp_rows_publish(a, acc, live, g, split * a.WT + wt, rb, lane);
+    }
+}
+
+// ---------------------------------------------------------------------------------------
+// The same for a few rows (and for class ids beyond 16 bits): one row per block (S blocks per row). The row's vocab bitmask is built in
 // shared memory by scattering the member lists of the allowed classes; then the row is
 // streamed: octets with no allowed token are overwritten with -inf without being read.
 // FUSED = false stops after writing the vocab mask.

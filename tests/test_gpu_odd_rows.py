@@ -95,3 +95,22 @@ def test_filtered_sampling(V, B, inv_t, top_k, top_p, dtype):
     with Ctx([part]) as ctx:
         got = run_filtered(ctx, None, cm, z, V, u, inv_t, top_k, top_p)
         check_filtered(got, [part], None, cm, z, V, u, inv_t, top_k, top_p, "V=%d" % V)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("V,pad,B,parts", [(7, 1, 64, 1), (15, 1, 70, 1), (16, 0, 64, 1), (31, 1, 65, 1), (264, 0, 64, 1), (513, 7, 97, 1),
+                                           (8200, 0, 100, 3), (30000, 0, 64, 1), (70007, 1, 129, 2)])
+def test_rows_that_allow_few_tokens(V, pad, B, parts, dtype):
+    """Vectors of 32 bytes (odd octets left over, rows on a 16-byte but not on a 32-byte grid), queues that never fill and that
+    overflow at once (some rows allow everything, some nothing)."""
+    pad = (-(V + pad)) % 8 + pad
+    K = max(1, min(128, V // 4))
+    ps = [synth.zipf_partition(V, K, seed=40 + i) for i in range(parts)]
+    row_part = None if parts == 1 else (np.arange(B) * 5 % parts).astype(np.int32)
+    cm = synth.class_mask_bernoulli(K, B, 0.03, rng.stream_key(rng.SEED_BASE, 905, V))
+    cm[3], cm[B - 1], cm[B // 2] = 0xFFFFFFFF, 0xFFFFFFFF, 0
+    z = synth.logits_normal(B, V + pad, 2.0, dtype, (906, V))
+    with Ctx(ps) as ctx:
+        got = run_fused(ctx, row_part, cm, z, V, stride=V + pad, mode=cz.SPARSE)
+        compare_step(got, oracle_step(ps, row_part, cm, z, V), V)
+        assert np.array_equal(got["logits"][:, V:].view(np.uint8), z[:, V:].view(np.uint8))
