@@ -321,6 +321,18 @@ __device__ __forceinline__ void write_row_outputs(const StepArgs& a, int row, fl
 template <int DT>
 __device__ __forceinline__ void warp_finalize_row(const StepArgs& a, const PartDev& P, int row, float m, float s,
                                                   int pos, int lane) {
+    if (a.masks_per_row > 0 && s != s) {
+        // the streaming kernel could not sum this mask beside the others (its logits lie too far below the row's largest)
+        const char* rowp = reinterpret_cast<const char*>(a.logits) + logits_row(a, row) * a.row_stride * (DT == kBF16 ? 2 : 4);
+        const uint32_t* cm = a.class_mask + int64_t(row) * a.cm_stride;
+        s = 0.f;
+        for (int t = lane; t < a.V; t += 32) {
+            const int k = __ldg(P.c32 + t);
+            if ((__ldg(cm + (k >> 5)) >> (k & 31)) & 1u) s += ex2f((ldcg_elem<DT>(rowp, t) - m) * kLog2e);
+        }
+#pragma unroll
+        for (int d = 16; d >= 1; d >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, d);
+    }
     unsigned long long cand = ~0ull;
     if (pos == kNoPos) {
         cand = first_allowed_share(a, P, row, lane, 32);

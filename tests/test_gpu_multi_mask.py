@@ -98,3 +98,28 @@ def test_multi_mask_argument_errors():
         assert cz.cfgzip_launch_count(ctx.h) == n0
         assert call() == cz.OK
         torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("V,K,B,M", [(9, 3, 7, 1), (256, 20, 5, 2), (8200, 90, 11, 5), (3000, 40, 3, 12), (2056, 60, 2, 33), (60000, 30000, 2, 9)])
+def test_logits_rows_that_share_a_batch_of_masks(V, K, B, M, dtype):
+    test_multi_mask_shapes(V, K, B, M, dtype)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("gap", [30.0, 90.0, 140.0, 400.0])
+def test_masks_whose_logits_lie_far_below_the_rows_largest(gap, dtype):
+    # class 0 holds the largest logits; the masks without it have to be summed as if it were not there
+    V, K, B, M = 6000, 12, 3, 9
+    part = synth.zipf_partition(V, K, 1.1, seed=5)
+    z = synth.logits_normal(B, V, 1.0, "f32", (94,))
+    z[:, part.c == 0] += np.float32(gap)
+    z[1] -= np.float32(300.0)
+    if dtype == "bf16":
+        z = rng.f32_to_bf16_bits(z.reshape(-1)).reshape(B, V)
+    bits = synth.unpack_bits(synth.class_mask_bernoulli(K, B * M, 0.5, rng.stream_key(95)), K)
+    bits[:, 0] = np.arange(B * M) % 3 == 0
+    bits[:, 1] = True
+    cms = synth.pack_bits(bits)
+    with Ctx([part]) as ctx:
+        _compare(_run(ctx, cms, M, z, V), oracle.multi_mask_step(part, cms, M, z), "gap %g" % gap)
