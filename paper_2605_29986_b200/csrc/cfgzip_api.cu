@@ -61,6 +61,7 @@ struct cfgzip_ctx {
     int32_t* d_group_part = nullptr;
     int32_t* d_group_rows = nullptr;
     int32_t* d_n_groups = nullptr;
+    int32_t* d_group_w = nullptr;       // row batches in front of every group
     int32_t* d_row_mode = nullptr;      // automatic mode: which rows the class-list kernel has finished
     int32_t reserved_rows = 0;
     int32_t max_groups = 0;
@@ -266,6 +267,7 @@ struct DensePlan {
     int fold = 0;        // pipelined kernel: results written by the last block of each group (no finalize launch)
     int fold_off = 0;    // fold: offset of the block's shared (row, warp) states, 0 = warps publish to the scratch directly
     int slots = 0;       // states per row in the global scratch
+    int blocks = 0;      // > 0: pipelined kernel, mixed batch: the blocks are shared out by the groups' sizes, at most S to a group
     size_t smem = 0;
     int n_groups_ub = 1;
     bool use_plan_kernel = false;
@@ -410,7 +412,18 @@ DensePlan plan_pipe_opl(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixe
     d.WT = ctx->token_warps ? ctx->token_warps : n_warps / WR;
     d.WT = std::max(1, std::min(std::min(d.WT, max_warps / WR), chunks));
     d.threads = d.WT * WR * 32;
-    for (;;) {
+    // The groups of a mixed batch may hold 32 rows or one: where there are blocks enough, each group gets its share of them
+    // (one wave of blocks that all have about as much to do; the same number for every group, sized for the fewest groups
+    // the batch can have, took a second wave: 256 rows over eight partitions, V = 256000, 78 us, now %GRAMMARS%).
+    if (mixed && target >= 3 * d.n_groups_ub) {
+        const int batches = ceil_div(B, kBatchRows), most = std::min(batches, kGroupRows / kBatchRows);
+        const int S = std::min(target, ceil_div(int64_t(target) * most, batches) + 2);
+        if (size_t(d.n_groups_ub) * kGroupRows * (size_t(S) * d.WT + 2) <= kPartialSlots) {
+            d.blocks = target;
+            d.S = S;
+        }
+    }
+    while (!d.blocks) {
         d.S = ceil_div(n_oct, per);
         if (size_t(d.n_groups_ub) * kGroupRows * (size_t(d.S) * d.WT + 2) <= kPartialSlots) break;
         if (per >= n_oct) return d;
@@ -554,7 +567,7 @@ int run_plan_kernel(cfgzip_ctx* ctx, const int32_t* row_part, int32_t B, int32_t
     ctx->plan_valid = false;                 // this launch overwrites them
     return launch(ctx, k_plan_rows, dim3(1), dim3(1024), 0, st, (const PartDev*)ctx->d_parts, int(ctx->parts.size()),
                   row_part, int(B), int(V), d.n_groups_ub, ctx->d_group_part, ctx->d_group_rows, ctx->d_n_groups,
-                  ctx->d_status);
+                  ctx->d_group_w, ctx->d_status);
 }
 
 void fill_groups(cfgzip_ctx* ctx, StepArgs& a, const DensePlan& d) {
@@ -567,6 +580,9 @@ void fill_groups(cfgzip_ctx* ctx, StepArgs& a, const DensePlan& d) {
         a.group_rows = nullptr;
         a.n_groups = nullptr;
     }
+    a.group_w = d.blocks ? ctx->d_group_w : nullptr;
+    a.max_groups = d.n_groups_ub;
+    a.blocks = d.blocks;
     a.S = d.S;
     a.per_split = d.per_split;
     a.WT = d.WT;
@@ -742,7 +758,7 @@ int launch_fused(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, in
                     CFGZIP_OK)
                     return rc;
             }
-            const dim3 grid(unsigned(d.n_groups_ub) * unsigned(d.S)), block{unsigned(d.threads)};
+            const dim3 grid(d.blocks ? unsigned(d.blocks) : unsigned(d.n_groups_ub) * unsigned(d.S)), block{unsigned(d.threads)};
             if (d.depth) {
                 rc = launch_pipe<DT>(ctx, a, d, grid, block, st);
             } else {
@@ -809,7 +825,7 @@ int launch_sample(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, b
         const int n_chunks = ceil_div(ps.V >> 3, d.chunk_octets);
         a.run_chunks = std::max(1, ceil_div(n_chunks, d.S * d.WT));
         a.tail_state = 1;
-        const dim3 grid(unsigned(d.n_groups_ub) * unsigned(d.S)), block{unsigned(d.threads)};
+        const dim3 grid(d.blocks ? unsigned(d.blocks) : unsigned(d.n_groups_ub) * unsigned(d.S)), block{unsigned(d.threads)};
         if ((rc = launch_pipe<DT>(ctx, a, d, grid, block, st)) != CFGZIP_OK) return rc;
         const unsigned rows_grid = unsigned(d.n_groups_ub) * kGroupRows;
         if (filtered) return launch_filtered<DT>(ctx, a, rows_grid, top_k, top_p, st);
@@ -885,15 +901,17 @@ int cfgzip_reserve_rows(cfgzip_ctx* ctx, int32_t max_rows) {
     cudaFree(ctx->d_tickets);
     cudaFree(ctx->d_group_part);
     cudaFree(ctx->d_group_rows);
+    cudaFree(ctx->d_group_w);
     cudaFree(ctx->d_row_mode);
     ctx->d_tickets = nullptr;
-    ctx->d_group_part = ctx->d_group_rows = ctx->d_row_mode = nullptr;
+    ctx->d_group_part = ctx->d_group_rows = ctx->d_group_w = ctx->d_row_mode = nullptr;
     ctx->reserved_rows = 0;
     const int32_t groups = ceil_div(max_rows, kGroupRows) + kMaxParts;
     const size_t tickets = size_t(std::max(max_rows, groups));
     if (cudaMalloc(&ctx->d_tickets, tickets * sizeof(unsigned int)) != cudaSuccess ||
         cudaMalloc(&ctx->d_group_part, size_t(groups) * sizeof(int32_t)) != cudaSuccess ||
         cudaMalloc(&ctx->d_group_rows, size_t(groups) * kGroupRows * sizeof(int32_t)) != cudaSuccess ||
+        cudaMalloc(&ctx->d_group_w, size_t(groups + 1) * sizeof(int32_t)) != cudaSuccess ||
         cudaMalloc(&ctx->d_row_mode, size_t(max_rows) * sizeof(int32_t)) != cudaSuccess) {
         cudaGetLastError();
         return CFGZIP_E_NOMEM;
@@ -961,6 +979,7 @@ int cfgzip_destroy(cfgzip_ctx* ctx) {
     cudaFree(ctx->d_status);
     cudaFree(ctx->d_group_part);
     cudaFree(ctx->d_group_rows);
+    cudaFree(ctx->d_group_w);
     cudaFree(ctx->d_row_mode);
     cudaFree(ctx->d_n_groups);
     cudaFree(ctx->st_logits);

@@ -711,6 +711,7 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __gri
     // the run states the streaming kernel published: the row maximum, and the maxima and sums of up to four runs per thread
     // for the bar of the short way (leaving runs out only lowers the bar)
     const Partial* src = row_slots(a, g, j);
+    const int n_states = group_states(a, g);
     const float u = __ldg(a.u + row);  // needed late
     constexpr int kKeep = 4;
     float run_m[kKeep], run_s[kKeep], M = -INFINITY;
@@ -718,13 +719,13 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __gri
     for (int q = 0; q < kKeep; ++q) {
         const int k = tid + q * kFiltThreads;
         float2 r = make_float2(-INFINITY, 0.f);
-        if (k < a.slots) r = __ldcg(reinterpret_cast<const float2*>(src + k));
+        if (k < n_states) r = __ldcg(reinterpret_cast<const float2*>(src + k));
         run_m[q] = r.x;
         run_s[q] = r.y;
         M = fmaxf(M, r.x);
     }
 #pragma unroll 1
-    for (int k = tid + kKeep * kFiltThreads; k < a.slots; k += kFiltThreads) M = fmaxf(M, __ldcg(&src[k].m));
+    for (int k = tid + kKeep * kFiltThreads; k < n_states; k += kFiltThreads) M = fmaxf(M, __ldcg(&src[k].m));
     M = float_from_order_key(__reduce_max_sync(0xFFFFFFFFu, float_order_key(M)));
     if (lane == 0) sh.warp_max[warp] = M;
     __syncthreads();
@@ -773,7 +774,7 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __gri
                 sum += run_s[q] * e;
             }
 #pragma unroll 1
-        for (int k = tid + kKeep * kFiltThreads; k < a.slots; k += kFiltThreads) {  // (their weight counts all the same)
+        for (int k = tid + kKeep * kFiltThreads; k < n_states; k += kFiltThreads) {  // (their weight counts all the same)
             const int4 raw = __ldcg(reinterpret_cast<const int4*>(src + k));
             if (__int_as_float(raw.x) >= w.z_zero) sum += __int_as_float(raw.y) * ex2f((__int_as_float(raw.x) - M) * scale);
         }

@@ -20,6 +20,10 @@ struct StepArgs {
     const int32_t* group_part;  // dev [n_groups]
     const int32_t* group_rows;  // dev [n_groups * 32], -1 = empty slot, valid slots first
     const int32_t* n_groups;    // dev scalar
+    const int32_t* group_w;     // dev [max_groups + 1] or null: row batches in the groups in front of each (the total from n_groups
+                                // on); the blocks of the launch are then shared out by it (group_share), at most S per group
+    int32_t max_groups;
+    int32_t blocks;             // group_w: blocks of the streaming launch
     const uint32_t* class_mask;
     int64_t cm_stride;
     void* logits;
@@ -398,6 +402,48 @@ __device__ __forceinline__ Partial dense_tail_octets(const StepArgs& a, const Pa
     return Partial{m, s, pos, 0};
 }
 
+// The blocks of a streaming launch that work on group g: a.S each, or, where the groups of a mixed batch are of very different
+// size (33 rows of one partition make a group of 32 and one of 1), in proportion to their row batches, at least one.
+struct GroupShare {
+    int first, S;
+};
+__device__ __forceinline__ GroupShare group_share(const StepArgs& a, int g) {
+    if (!a.group_w) return GroupShare{g * a.S, a.S};
+    const int ng = __ldg(a.n_groups), w0 = __ldg(a.group_w + g), w1 = __ldg(a.group_w + g + 1), W = __ldg(a.group_w + a.max_groups);
+    const int spare = a.blocks - ng, first = g + spare * w0 / max(W, 1), next = g + 1 + spare * w1 / max(W, 1);
+    return GroupShare{first, min(next - first, a.S)};
+}
+// ... and the group of this block (false: none). Called by whole warps.
+__device__ __forceinline__ bool block_group(const StepArgs& a, int& g, int& split, int& S) {
+    const int b = blockIdx.x;
+    if (!a.group_w) {
+        g = b / a.S;
+        split = b - g * a.S;
+        S = a.S;
+        return !(a.n_groups && g >= __ldg(a.n_groups));
+    }
+    const int lane = threadIdx.x & 31;
+    for (int g0 = 0; g0 < a.max_groups; g0 += 32) {
+        const bool real = g0 + lane < min(a.max_groups, __ldg(a.n_groups));
+        const GroupShare s = real ? group_share(a, g0 + lane) : GroupShare{0, 0};
+        const uint32_t hit = __ballot_sync(0xFFFFFFFFu, b >= s.first && b < s.first + s.S);
+        if (hit) {
+            const int l = __ffs(int(hit)) - 1;
+            g = g0 + l;
+            split = b - __shfl_sync(0xFFFFFFFFu, s.first, l);
+            S = __shfl_sync(0xFFFFFFFFu, s.S, l);
+            return true;
+        }
+    }
+    return false;
+}
+// States a row of group g has published.
+__device__ __forceinline__ int group_states(const StepArgs& a, int g) {
+    if (!a.group_w) return a.slots;
+    const int S = group_share(a, g).S;
+    return a.fold_off ? S : S * a.WT + 1 + a.head_state;
+}
+
 // Where the (max, sum-exp, position) states of a row go: every warp that streamed a row batch
 // publishes one state per row in its own slot, slot = split * WT + wt, and the block that owns the
 // end of the vocabulary adds the state of the octets past the last whole vector in the last
@@ -430,7 +476,7 @@ __device__ __forceinline__ float float_from_order_key(int k) { return __int_as_f
 // (8, or 16 for a kernel that takes them two at a time; rows on the vector grid only).
 template <int DT, bool SHIFT, int UNIT = 8, typename H, typename T>
 __device__ __forceinline__ void publish_edges(const StepArgs& a, const PartDev& P, const uint32_t* table, const int* s_row,
-                                              int nrow, int split, int warp, int lane, float scale, bool apart, H&& to_head,
+                                              int nrow, int split, int S, int warp, int lane, float scale, bool apart, H&& to_head,
                                               T&& to_tail) {
     constexpr int ES = DT == kBF16 ? 2 : 4;
     const int n_full = a.V >> 3, n_octets = 4 * a.VW;
@@ -439,13 +485,13 @@ __device__ __forceinline__ void publish_edges(const StepArgs& a, const PartDev& 
     const bool have = lane < 24 && t >= 0 && t < a.V;
     const int n_warps = blockDim.x >> 5;
     if (!SHIFT && n_full == n_octets) {  // the vectors cover the vocabulary: nothing is left over
-        for (int j = split + a.S * warp; j < nrow; j += a.S * n_warps)
+        for (int j = split + S * warp; j < nrow; j += S * n_warps)
             if (lane == 0) *to_tail(j) = partial_empty();
         return;
     }
     uint32_t word = 0u;
     bool asked = false;
-    for (int j = split + a.S * warp; j < nrow; j += a.S * n_warps) {
+    for (int j = split + S * warp; j < nrow; j += S * n_warps) {
         if (!asked && have) word = table[P.c16[t]];
         asked = true;
         const int row = s_row[j];
@@ -517,6 +563,7 @@ __global__ void __launch_bounds__(kFinalizeThreads) k_finalize_rows(const __grid
     if (a.row_mode && a.row_mode[row]) return;  // automatic mode: the class-list kernel has finished this row
     const PartDev P = a.group_part ? a.parts[a.group_part[g]] : a.p0;
     const Partial* src = row_slots(a, g, j);
+    const int n_states = group_states(a, g);
     // Two passes over the states, which stay in registers (up to four per thread, all loads in flight together):
     // first the row maximum (shuffles and max only), then every state's sum brought to that maximum with one
     // exponential per state, summed, and the lowest position among the states that hold the maximum. No
@@ -529,13 +576,13 @@ __global__ void __launch_bounds__(kFinalizeThreads) k_finalize_rows(const __grid
         for (int u = 0; u < 4; ++u) {
             const int sp = base + u * kFinalizeThreads + tid;
             v[u] = make_int4(__float_as_int(-INFINITY), 0, kNoPos, 0);
-            if (sp < a.slots) v[u] = __ldcg(reinterpret_cast<const int4*>(src + sp));
+            if (sp < n_states) v[u] = __ldcg(reinterpret_cast<const int4*>(src + sp));
         }
     };
     int4 v0[4];
     fetch(0, v0);
     float M = fmaxf(fmaxf(__int_as_float(v0[0].x), __int_as_float(v0[1].x)), fmaxf(__int_as_float(v0[2].x), __int_as_float(v0[3].x)));
-    for (int base = 4 * kFinalizeThreads; base < a.slots; base += 4 * kFinalizeThreads) {  // more than 1024 states: rare
+    for (int base = 4 * kFinalizeThreads; base < n_states; base += 4 * kFinalizeThreads) {  // more than 1024 states: rare
         int4 w[4];
         fetch(base, w);
         M = fmaxf(M, fmaxf(fmaxf(__int_as_float(w[0].x), __int_as_float(w[1].x)), fmaxf(__int_as_float(w[2].x), __int_as_float(w[3].x))));
@@ -558,7 +605,7 @@ __global__ void __launch_bounds__(kFinalizeThreads) k_finalize_rows(const __grid
         }
     };
     gather(v0);
-    for (int base = 4 * kFinalizeThreads; base < a.slots; base += 4 * kFinalizeThreads) {
+    for (int base = 4 * kFinalizeThreads; base < n_states; base += 4 * kFinalizeThreads) {
         int4 w[4];
         fetch(base, w);
         gather(w);
@@ -606,12 +653,13 @@ __global__ void __launch_bounds__(256) k_finalize_rows_warp(const __grid_constan
     if (a.row_mode && a.row_mode[row]) return;  // automatic mode: the class-list kernel has finished this row
     const PartDev P = a.group_part ? a.parts[a.group_part[g]] : a.p0;
     const Partial* src = row_slots(a, g, j);
+    const int n_states = group_states(a, g);
     int4 v[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
         const int sp = u * 32 + lane;
         v[u] = make_int4(__float_as_int(-INFINITY), 0, kNoPos, 0);
-        if (sp < a.slots) v[u] = __ldcg(reinterpret_cast<const int4*>(src + sp));
+        if (sp < n_states) v[u] = __ldcg(reinterpret_cast<const int4*>(src + sp));
     }
     float m0 = __int_as_float(v[0].x), s0 = __int_as_float(v[0].y), m1 = __int_as_float(v[1].x), s1 = __int_as_float(v[1].y);
     int p0 = v[0].z, p1 = v[1].z;
@@ -940,8 +988,8 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
     if (!implicit) pdl_wait();
     const float scale = TEMPERED ? a.scale : kLog2e;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int g = blockIdx.x / a.S, split = blockIdx.x - g * a.S;
-    if (a.n_groups && g >= __ldg(a.n_groups)) return;
+    int g, split, S;
+    if (!block_group(a, g, split, S)) return;
     const bool early_cm = a.cm_bulk && implicit;
     if (early_cm && tid == 0) {
         mbar_init(&cm_bar, 1);
@@ -979,14 +1027,16 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
     // the others; the deal starts at a different slot for every row batch (rot_chunks further on), which spreads the
     // extra chunks evenly over the warps and the blocks instead of giving the first ones one more in every row batch.
     const int n_chunks = (n_full + kChunkOctets - 1) / kChunkOctets;
-    const int stride_chunks = TEMPERED ? 1 : a.S * a.WT;  // round-robin: warps that share a row batch of the group
+    const int stride_chunks = TEMPERED ? 1 : S * a.WT;  // round-robin: warps that share a row batch of the group
+    const int run_chunks = TEMPERED ? (a.group_w ? max(1, (n_chunks + S * a.WT - 1) / (S * a.WT)) : a.run_chunks) : 0;
+    const int n_slots = a.group_w ? (a.fold_off ? S : S * a.WT + 1 + a.head_state) : a.slots;  // states of a row, the last one for its ends
     auto first_chunk_of = [&](int rb) {  // this warp's first chunk of row batch rb
-        if (TEMPERED) return (split * a.WT + wt) * a.run_chunks;
+        if (TEMPERED) return (split * a.WT + wt) * run_chunks;
         int c = split * a.WT + wt - rb * a.rot_chunks;
         c %= stride_chunks;
         return c < 0 ? c + stride_chunks : c;
     };
-    const int chunk_end = TEMPERED ? min(first_chunk_of(0) + a.run_chunks, n_chunks) : n_chunks;
+    const int chunk_end = TEMPERED ? min(first_chunk_of(0) + run_chunks, n_chunks) : n_chunks;
     int* const slot_info = ring_info + warp * depth; // (rb << 24) | chunk of the item in each slot, -1 = no more items
 
     // automatic mode: bit r = row slot r was finished by the class-list kernel (set after the wait below)
@@ -1158,8 +1208,8 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
     const int my_slot = s_state ? wt : split * a.WT + wt + (SHIFT ? a.head_state : 0);
     // What the vectors leave over, while the first copies are on their way
     publish_edges<DT, SHIFT>(
-        a, P, T, s_row, nrow, split, warp, lane, scale, SHIFT && a.head_state != 0, [&](int j) { return row_slots(a, g, j); },
-        [&](int j) { return pub_base + j * pub_stride + (s_state ? a.WT : a.slots - 1); });
+        a, P, T, s_row, nrow, split, S, warp, lane, scale, SHIFT && a.head_state != 0, [&](int j) { return row_slots(a, g, j); },
+        [&](int j) { return pub_base + j * pub_stride + (s_state ? a.WT : n_slots - 1); });
     // where this lane's octets of a row sit inside a stage: two tiled copies leave two boxes of 8 rows x 32 octets
     // behind one another, anything else whole rows of the chunk
     const uint32_t lane_off = (TMAP && OPL == 2) ? uint32_t(lane >> 4) * G::kBoxBytes + uint32_t(lane & 15) * 2u * G::kOctetBytes
@@ -1255,7 +1305,7 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
         // first the block's own states: one per row and block goes out instead of one per row and warp
         __syncthreads();
         for (int j = warp; j < nrow; j += n_warps) {
-            const int n_mine = a.WT + (j % a.S == split ? 1 : 0);  // the state of what the vectors left over
+            const int n_mine = a.WT + (j % S == split ? 1 : 0);  // the state of what the vectors left over
             float m = -INFINITY, s = 0.f;
             int pos = kNoPos;
             if (lane < n_mine) {
@@ -1271,14 +1321,14 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
     // of the group's rows and writes their results (what k_finalize_rows does in a launch of its own otherwise).
     __threadfence();  // this block's states and masked logits are visible device-wide before its ticket is drawn
     __syncthreads();
-    if (tid == 0) s_last = (atomicAdd(a.tickets + g, 1u) == unsigned(a.S - 1));
+    if (tid == 0) s_last = (atomicAdd(a.tickets + g, 1u) == unsigned(S - 1));
     __syncthreads();
     if (!s_last) return;
     __threadfence();  // the other blocks' states and masked logits, published before their tickets
     for (int j = warp; j < nrow; j += n_warps) {
         float m, s;
         int pos;
-        warp_fold_states(row_slots(a, g, j), a.slots, lane, m, s, pos);
+        warp_fold_states(row_slots(a, g, j), n_slots, lane, m, s, pos);
         warp_finalize_row<DT>(a, P, s_row[j], m, s, pos, lane);
     }
     if (tid == 0) a.tickets[g] = 0u;  // ready for the next launch
@@ -1407,7 +1457,7 @@ __global__ void __launch_bounds__(kFewThreads, 3) k_step_few(const __grid_consta
     const bool wide = a.wide != 0;
     uint8_t* const vm8 = reinterpret_cast<uint8_t*>(a.vocab_mask);
     publish_edges<DT, false, Vec::kTokens>(
-        a, P, T, s_row, nrow, split, warp, lane, kLog2e, false, [&](int j) { return row_slots(a, g, j); },
+        a, P, T, s_row, nrow, split, a.S, warp, lane, kLog2e, false, [&](int j) { return row_slots(a, g, j); },
         [&](int j) { return row_slots(a, g, j) + a.slots - 1; });
     const uint4* const ids = reinterpret_cast<const uint4*>(P.c16);
     FewWarp& w = s_warp[warp];
@@ -1856,7 +1906,7 @@ __global__ void __launch_bounds__(kSampleThreads) k_sample_rows(const __grid_con
     }
     const Partial* src = row_slots(a, g, j);
     const float u = __ldg(a.u + row);  // needed late: in flight together with the states
-    const int n_states = a.slots;
+    const int n_states = group_states(a, g);
     const int per = (n_states + kSampleThreads - 1) / kSampleThreads;  // consecutive states per thread
     const int k0 = tid * per, k1 = min(k0 + per, n_states);
 
@@ -1955,6 +2005,11 @@ __global__ void __launch_bounds__(kSampleThreads) k_sample_rows(const __grid_con
     const char* rowp = reinterpret_cast<const char*>(a.logits) + int64_t(row) * a.row_stride * ES;
     const int head = a.shifted ? row_head<DT>(rowp, a.V) : 0;
     const int vec_end = head + ((a.V - head) & ~7);  // first token past the last whole vector
+    int run_chunks = a.run_chunks;
+    if (a.group_w) {  // (as the streaming kernel's blocks of this group dealt them)
+        const int n_chunks = ((a.V >> 3) + (a.chunk_tokens >> 3) - 1) / (a.chunk_tokens >> 3), warps = group_share(a, g).S * a.WT;
+        run_chunks = max(1, (n_chunks + warps - 1) / warps);
+    }
     int t_lo, t_hi;
     if (a.tail_state && pick == n_states - 1) {
         t_lo = vec_end;
@@ -1963,7 +2018,7 @@ __global__ void __launch_bounds__(kSampleThreads) k_sample_rows(const __grid_con
         t_lo = 0;
         t_hi = head;
     } else {
-        const long long lim = a.tail_state ? vec_end : a.V, run_tokens = static_cast<long long>(a.run_chunks) * a.chunk_tokens;
+        const long long lim = a.tail_state ? vec_end : a.V, run_tokens = static_cast<long long>(run_chunks) * a.chunk_tokens;
         const long long first = head + (pick - a.head_state) * run_tokens;
         t_lo = int(min(first, lim));
         t_hi = int(min(first + run_tokens, lim));
@@ -2159,7 +2214,7 @@ constexpr int kMaxParts = 256;
 
 __global__ void __launch_bounds__(1024) k_plan_rows(const PartDev* parts, int n_parts, const int32_t* row_part, int B,
                                                     int V, int max_groups, int32_t* group_part, int32_t* group_rows,
-                                                    int32_t* n_groups, int32_t* status) {
+                                                    int32_t* n_groups, int32_t* group_w, int32_t* status) {
     __shared__ int cnt[kMaxParts], gbase[kMaxParts + 1], cur[kMaxParts];
     pdl_prologue();
     const int tid = threadIdx.x;
@@ -2176,6 +2231,13 @@ __global__ void __launch_bounds__(1024) k_plan_rows(const PartDev* parts, int n_
         for (int p = 0; p < n_parts; ++p) { gbase[p] = acc; acc += (cnt[p] + kGroupRows - 1) / kGroupRows; }
         gbase[n_parts] = acc;
         *n_groups = acc;
+        int w = 0, gq = 0;  // row batches in front of every group
+        for (int p = 0; p < n_parts; ++p)
+            for (int left = cnt[p]; left > 0; left -= kGroupRows) {
+                group_w[gq++] = w;
+                w += (min(left, kGroupRows) + kBatchRows - 1) / kBatchRows;
+            }
+        for (; gq <= max_groups; ++gq) group_w[gq] = w;
     }
     __syncthreads();
     const int total = gbase[n_parts];

@@ -114,3 +114,25 @@ def test_rows_that_allow_few_tokens(V, pad, B, parts, dtype):
         got = run_fused(ctx, row_part, cm, z, V, stride=V + pad, mode=cz.SPARSE)
         compare_step(got, oracle_step(ps, row_part, cm, z, V), V)
         assert np.array_equal(got["logits"][:, V:].view(np.uint8), z[:, V:].view(np.uint8))
+
+
+@pytest.mark.parametrize("pad", [0, 1])
+@pytest.mark.parametrize("V,counts", [(9000, (33, 1, 64, 2)), (70008, (97, 0, 3, 8)), (20000, (5, 1, 1, 1)), (1000, (31, 33, 40, 200))])
+def test_groups_of_very_different_size(V, counts, pad):
+    """The blocks of a mixed batch are shared out by the sizes of its row groups: greedy (folded in the kernel too), sampling,
+    filtered sampling."""
+    parts = [synth.zipf_partition(V, k, seed=60 + i) for i, k in enumerate((50, 333, 700, 64))]
+    row_part = np.random.RandomState(V).permutation(np.repeat(np.arange(4), counts)).astype(np.int32)
+    B, stride = len(row_part), V + 8 * (1 - pad) + pad
+    cm = synth.class_mask_bernoulli(700, B, 0.2, rng.stream_key(rng.SEED_BASE, 907, V))
+    cm[:, 0] |= 1
+    z = synth.logits_normal(B, stride, 2.0, "bf16", (908, V))
+    u = np.linspace(0, 0.99, B, dtype=np.float32)
+    want = oracle_step(parts, row_part, cm, z, V)
+    with Ctx(parts) as ctx:
+        for fold in (0, 1, 2):
+            cz.cfgzip_set_tuning(ctx.h, "fold", fold)
+            compare_step(run_fused(ctx, row_part, cm, z, V, stride=stride), want, V, "fold %d" % fold)
+        cz.cfgzip_set_tuning(ctx.h, "fold", 0)
+        check_sample(run_sample(ctx, row_part, cm, z, V, u, 1.5, stride=stride), parts, row_part, cm, z, V, u, 1.5)
+        check_filtered(run_filtered(ctx, row_part, cm, z, V, u, 1.5, 30, 0.9, stride=stride), parts, row_part, cm, z, V, u, 1.5, 30, 0.9)
