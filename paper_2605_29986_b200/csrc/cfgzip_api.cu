@@ -414,7 +414,7 @@ DensePlan plan_pipe_opl(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixe
     d.threads = d.WT * WR * 32;
     // The groups of a mixed batch may hold 32 rows or one: where there are blocks enough, each group gets its share of them
     // (one wave of blocks that all have about as much to do; the same number for every group, sized for the fewest groups
-    // the batch can have, took a second wave: 256 rows over eight partitions, V = 256000, 78 us, now %GRAMMARS%).
+    // the batch can have, took a second wave: 256 rows over eight partitions, V = 256000, 78 us, now 65).
     if (mixed && target >= 3 * d.n_groups_ub) {
         const int batches = ceil_div(B, kBatchRows), most = std::min(batches, kGroupRows / kBatchRows);
         const int S = std::min(target, ceil_div(int64_t(target) * most, batches) + 2);
@@ -830,8 +830,9 @@ int launch_sample(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, b
         const unsigned rows_grid = unsigned(d.n_groups_ub) * kGroupRows;
         if (filtered) return launch_filtered<DT>(ctx, a, rows_grid, top_k, top_p, st);
         const size_t pad = row_blocks_pad(ctx, rows_grid, a.B);
-        if (pad && (rc = ensure_smem(ctx, k_sample_rows<DT>, pad)) != CFGZIP_OK) return rc;
-        return launch(ctx, k_sample_rows<DT>, dim3(rows_grid), dim3(kSampleThreads), pad, st, a, 1);
+        auto kern = a.group_w ? k_sample_rows<DT, true> : k_sample_rows<DT, false>;
+        if (pad && (rc = ensure_smem(ctx, kern, pad)) != CFGZIP_OK) return rc;
+        return launch(ctx, kern, dim3(rows_grid), dim3(kSampleThreads), pad, st, a, 1);
     }
     if (size_t(a.B) > kPartialSlots) return CFGZIP_E_NOMEM;
     a.group_part = nullptr;
@@ -845,7 +846,7 @@ int launch_sample(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, b
     if ((rc = launch(ctx, k_step_generic<DT, true>, dim3(unsigned(a.B)), dim3(256), 0, st, a)) != CFGZIP_OK) return rc;
     if (filtered)
         return launch_filtered<DT>(ctx, a, unsigned(ceil_div(a.B, kGroupRows)) * kGroupRows, top_k, top_p, st);
-    return launch(ctx, k_sample_rows<DT>, dim3(unsigned(ceil_div(a.B, kGroupRows)) * kGroupRows), dim3(kSampleThreads), 0, st,
+    return launch(ctx, k_sample_rows<DT, false>, dim3(unsigned(ceil_div(a.B, kGroupRows)) * kGroupRows), dim3(kSampleThreads), 0, st,
                   a, aligned ? 1 : 0);
 }
 

@@ -407,13 +407,16 @@ __device__ __forceinline__ Partial dense_tail_octets(const StepArgs& a, const Pa
 struct GroupShare {
     int first, S;
 };
-__device__ __forceinline__ GroupShare group_share(const StepArgs& a, int g) {
-    if (!a.group_w) return GroupShare{g * a.S, a.S};
-    const int ng = __ldg(a.n_groups), w0 = __ldg(a.group_w + g), w1 = __ldg(a.group_w + g + 1), W = __ldg(a.group_w + a.max_groups);
-    const int spare = a.blocks - ng, first = g + spare * w0 / max(W, 1), next = g + 1 + spare * w1 / max(W, 1);
-    return GroupShare{first, min(next - first, a.S)};
+// (functions of their own: a batch without a row plan, whose steps are the shortest, should not fetch past this code)
+__device__ __noinline__ GroupShare group_share_of(const int32_t* n_groups, const int32_t* group_w, int max_groups, int blocks, int most, int g) {
+    const int ng = __ldg(n_groups), w0 = __ldg(group_w + g), w1 = __ldg(group_w + g + 1), W = __ldg(group_w + max_groups);
+    const int spare = blocks - ng, first = g + spare * w0 / max(W, 1), next = g + 1 + spare * w1 / max(W, 1);
+    return GroupShare{first, min(next - first, most)};
 }
-// ... and the group of this block (false: none). Called by whole warps.
+__device__ __forceinline__ GroupShare group_share(const StepArgs& a, int g) {
+    return group_share_of(a.n_groups, a.group_w, a.max_groups, a.blocks, a.S, g);
+}
+// The group of this block, its place among the group's blocks and their number (false: none). Called by whole warps.
 __device__ __forceinline__ bool block_group(const StepArgs& a, int& g, int& split, int& S) {
     const int b = blockIdx.x;
     if (!a.group_w) {
@@ -436,6 +439,10 @@ __device__ __forceinline__ bool block_group(const StepArgs& a, int& g, int& spli
         }
     }
     return false;
+}
+// Chunks in a run of a sampling step, as the warps of a group of such a batch dealt them.
+__device__ __noinline__ int group_run_chunks(int n_octets, int chunk_octets, int warps) {
+    return max(1, ((n_octets + chunk_octets - 1) / chunk_octets + warps - 1) / warps);
 }
 // States a row of group g has published.
 __device__ __forceinline__ int group_states(const StepArgs& a, int g) {
@@ -989,7 +996,13 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
     const float scale = TEMPERED ? a.scale : kLog2e;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     int g, split, S;
-    if (!block_group(a, g, split, S)) return;
+    if (TMAP) {  // (tiled copies: no row plan)
+        g = blockIdx.x / a.S;
+        split = blockIdx.x - g * a.S;
+        S = a.S;
+    } else if (!block_group(a, g, split, S)) {
+        return;
+    }
     const bool early_cm = a.cm_bulk && implicit;
     if (early_cm && tid == 0) {
         mbar_init(&cm_bar, 1);
@@ -1028,8 +1041,8 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
     // extra chunks evenly over the warps and the blocks instead of giving the first ones one more in every row batch.
     const int n_chunks = (n_full + kChunkOctets - 1) / kChunkOctets;
     const int stride_chunks = TEMPERED ? 1 : S * a.WT;  // round-robin: warps that share a row batch of the group
-    const int run_chunks = TEMPERED ? (a.group_w ? max(1, (n_chunks + S * a.WT - 1) / (S * a.WT)) : a.run_chunks) : 0;
-    const int n_slots = a.group_w ? (a.fold_off ? S : S * a.WT + 1 + a.head_state) : a.slots;  // states of a row, the last one for its ends
+    const int run_chunks = TEMPERED ? (!TMAP && a.group_w ? max(1, (n_chunks + S * a.WT - 1) / (S * a.WT)) : a.run_chunks) : 0;
+    const int n_slots = !TMAP && a.group_w ? (a.fold_off ? S : S * a.WT + 1 + a.head_state) : a.slots;  // states of a row, the last one for its ends
     auto first_chunk_of = [&](int rb) {  // this warp's first chunk of row batch rb
         if (TEMPERED) return (split * a.WT + wt) * run_chunks;
         int c = split * a.WT + wt - rb * a.rot_chunks;
@@ -1046,7 +1059,9 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
         const uint32_t all = n >= 8 ? 0xFFu : (1u << n) - 1u;
         return ((rows_done >> (rb * kBatchRows)) & 0xFFu) == all;
     };
-    // producer cursor (meaningful in lane 0)
+    // Producer cursor: one lane issues the copies of an item when it is a tiled copy; a copy per row is issued side by side, a
+    // lane each, and the whole warp keeps the cursor (256 rows over eight partitions, V = 256000: 65 -> 61 us; 48 rows off the vector grid 13.5 -> 12.8).
+    constexpr bool COOP = !TMAP;
     int p_rb = wr, p_slot = 0, p_issued = 0, p_chunk = 0;
     bool p_first = true, p_done = wr * kBatchRows >= nrow, p_end = false;
     auto issue_next = [&]() {
@@ -1071,11 +1086,11 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
             p_done = p_rb * kBatchRows >= nrow;
         }
         if (chunk < 0) {
-            slot_info[p_slot] = -1;
+            if (!COOP || lane == 0) slot_info[p_slot] = -1;
             p_end = true;
             return;
         }
-        slot_info[p_slot] = (p_rb << 24) | chunk;
+        if (!COOP || lane == 0) slot_info[p_slot] = (p_rb << 24) | chunk;
         const int o0 = chunk * kChunkOctets;
         char* dst = my_ring + size_t(p_slot) * G::kStageBytes;
         const uint32_t nvec = uint32_t(min(n_full - o0, kChunkOctets));  // >= 1: chunk < n_chunks
@@ -1083,16 +1098,13 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
         if (SHIFT) {
             n_ids = uint32_t(min(n_octets - o0, 32));  // one octet more than vectors (the class ids are padded to n_octets)
             const int live = min(kBatchRows, nrow - p_rb * kBatchRows);
-            uint32_t total = n_ids * 16u;
-            for (int i = 0; i < live; ++i)
-                total += uint32_t(max(0, min(s_nvec[p_rb * kBatchRows + i] - o0, kChunkOctets))) * G::kOctetBytes;
-            mbar_expect_tx(bar + p_slot, total);
-            for (int i = 0; i < live; ++i) {
-                const int n = min(s_nvec[p_rb * kBatchRows + i] - o0, kChunkOctets);
-                if (n > 0)
-                    bulk_g2s(dst + i * G::kRowBytes, s_vec[p_rb * kBatchRows + i] + size_t(o0) * G::kOctetBytes,
-                             uint32_t(n) * G::kOctetBytes, bar + p_slot);
-            }
+            uint32_t bytes = 0u;
+            if (lane < live) bytes = uint32_t(max(0, min(s_nvec[p_rb * kBatchRows + lane] - o0, kChunkOctets))) * G::kOctetBytes;
+            const uint32_t total = __reduce_add_sync(0xFFFFFFFFu, bytes);
+            if (lane == 0) mbar_expect_tx(bar + p_slot, total + n_ids * 16u);
+            __syncwarp();
+            if (bytes)
+                bulk_g2s(dst + lane * G::kRowBytes, s_vec[p_rb * kBatchRows + lane] + size_t(o0) * G::kOctetBytes, bytes, bar + p_slot);
         } else if (TMAP) {
             // a box holds 32 octets of the 8 rows; the second box of a two-octet chunk is fetched only if the chunk
             // reaches into it (its lanes are idle otherwise); parts of a box past V or past the last row are filled in
@@ -1103,15 +1115,16 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
         } else {
             const int live = min(kBatchRows, nrow - p_rb * kBatchRows);
             const uint32_t row_bytes = nvec * G::kOctetBytes;
-            mbar_expect_tx(bar + p_slot, uint32_t(live) * row_bytes + nvec * 16u);
-            for (int i = 0; i < live; ++i) {
-                const int row = s_row[p_rb * kBatchRows + i];
-                bulk_g2s(dst + i * G::kRowBytes,
-                         reinterpret_cast<const char*>(a.logits) + (int64_t(row) * a.row_stride * ES + int64_t(o0) * 8 * ES),
+            if (lane == 0) mbar_expect_tx(bar + p_slot, uint32_t(live) * row_bytes + nvec * 16u);
+            __syncwarp();
+            if (lane < live)
+                bulk_g2s(dst + lane * G::kRowBytes,
+                         reinterpret_cast<const char*>(a.logits) +
+                             (int64_t(s_row[p_rb * kBatchRows + lane]) * a.row_stride * ES + int64_t(o0) * 8 * ES),
                          row_bytes, bar + p_slot);
-            }
         }
-        bulk_g2s(dst + kBatchRows * G::kRowBytes, reinterpret_cast<const char*>(P.c16) + size_t(o0) * 16, n_ids * 16u, bar + p_slot);
+        if (!COOP || lane == kBatchRows)
+            bulk_g2s(dst + kBatchRows * G::kRowBytes, reinterpret_cast<const char*>(P.c16) + size_t(o0) * 16, n_ids * 16u, bar + p_slot);
         ++p_issued;
         if (++p_slot == depth) p_slot = 0;
     };
@@ -1175,7 +1188,7 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
                 bulk_g2s(stage + lane * a.stage_stride, a.class_mask + int64_t(row) * a.cm_stride, uint32_t(P.KW) * 4u, &cm_bar);
         }
     }
-    if (lane == 0 && warp >= a.hold_warps)  // hold_warps is 0 unless the staging area lies over the rings
+    if ((COOP || lane == 0) && warp >= a.hold_warps)  // hold_warps is 0 unless the staging area lies over the rings
         for (int d = 0; d < depth && !p_end; ++d) issue_next();  // in flight while the table is built
     bool failed = false;
     if (a.cm_bulk) {
@@ -1191,7 +1204,7 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
     __syncthreads();
     if (__any_sync(0xFFFFFFFFu, failed) && lane == 0) atomicAdd(a.status + 3, 1);  // class masks never arrived
     failed = false;
-    if (lane == 0 && warp < a.hold_warps) {
+    if ((COOP || lane == 0) && warp < a.hold_warps) {
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the staging area was read and written by plain accesses
         for (int d = 0; d < depth && !p_end; ++d) issue_next();
     }
@@ -1281,7 +1294,7 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
         ++consumed;
         if (++slot == depth) { slot = 0; phase ^= 1u; }
         __syncwarp();  // every lane has its data out of the slot before it is refilled
-        if (lane == 0 && !p_end) issue_next();
+        if ((COOP || lane == 0) && !p_end) issue_next();
         __syncwarp();  // slot_info of the refilled slot is visible to the whole warp
     }
     if (!failed) {
@@ -1878,7 +1891,8 @@ __device__ __forceinline__ float block_exclusive_scan(float v, float* s_warp, fl
     return before + inc - v;
 }
 
-template <int DT>
+// SHARED_OUT: a.group_w is set (its code is kept out of the kernel for the short steps without a row plan).
+template <int DT, bool SHARED_OUT>
 __global__ void __launch_bounds__(kSampleThreads) k_sample_rows(const __grid_constant__ StepArgs a, int aligned) {
     __shared__ float s_warp[kSampleThreads / 32], s_scan_states[kSampleThreads / 32], s_scan_tokens[kSampleThreads / 32];
     __shared__ int s_pick, s_last;
@@ -1906,7 +1920,7 @@ __global__ void __launch_bounds__(kSampleThreads) k_sample_rows(const __grid_con
     }
     const Partial* src = row_slots(a, g, j);
     const float u = __ldg(a.u + row);  // needed late: in flight together with the states
-    const int n_states = group_states(a, g);
+    const int n_states = SHARED_OUT ? group_states(a, g) : a.slots;
     const int per = (n_states + kSampleThreads - 1) / kSampleThreads;  // consecutive states per thread
     const int k0 = tid * per, k1 = min(k0 + per, n_states);
 
@@ -2006,10 +2020,7 @@ __global__ void __launch_bounds__(kSampleThreads) k_sample_rows(const __grid_con
     const int head = a.shifted ? row_head<DT>(rowp, a.V) : 0;
     const int vec_end = head + ((a.V - head) & ~7);  // first token past the last whole vector
     int run_chunks = a.run_chunks;
-    if (a.group_w) {  // (as the streaming kernel's blocks of this group dealt them)
-        const int n_chunks = ((a.V >> 3) + (a.chunk_tokens >> 3) - 1) / (a.chunk_tokens >> 3), warps = group_share(a, g).S * a.WT;
-        run_chunks = max(1, (n_chunks + warps - 1) / warps);
-    }
+    if (SHARED_OUT) run_chunks = group_run_chunks(a.V >> 3, a.chunk_tokens >> 3, group_share(a, g).S * a.WT);
     int t_lo, t_hi;
     if (a.tail_state && pick == n_states - 1) {
         t_lo = vec_end;
