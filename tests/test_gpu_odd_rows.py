@@ -136,3 +136,31 @@ def test_groups_of_very_different_size(V, counts, pad):
         cz.cfgzip_set_tuning(ctx.h, "fold", 0)
         check_sample(run_sample(ctx, row_part, cm, z, V, u, 1.5, stride=stride), parts, row_part, cm, z, V, u, 1.5)
         check_filtered(run_filtered(ctx, row_part, cm, z, V, u, 1.5, 30, 0.9, stride=stride), parts, row_part, cm, z, V, u, 1.5, 30, 0.9)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("V,B,parts,p", [(1001, 1, 1, 0.3), (25000, 8, 1, 0.3), (25003, 9, 2, 0.3), (9000, 70, 1, 0.002), (9000, 130, 3, 0.2)])
+def test_host_step_with_pinned_buffers(V, B, parts, p, dtype):
+    """Copies in, expansion, step and copies out on streams of their own: one row chunk, several, a short last one."""
+    ps = [synth.zipf_partition(V, 300, seed=70 + i) for i in range(parts)]
+    row_part = None if parts == 1 else (np.arange(B) * 3 % parts).astype(np.int32)
+    cm = synth.class_mask_bernoulli(300, B, p, rng.stream_key(rng.SEED_BASE, 909, V))
+    VW = (V + 31) // 32
+
+    def pin(a):
+        return torch.from_numpy(a.view(np.int16 if a.dtype == np.uint16 else np.int32 if a.dtype == np.uint32 else a.dtype)).pin_memory()
+
+    with Ctx(ps) as ctx:
+        for step in range(2):
+            z = synth.logits_normal(B, V, 2.0, dtype, (910, V, step))
+            want = oracle_step(ps, row_part, cm, z, V)
+            for want_masked in (False, True):
+                d_z, d_cm, vm = pin(z), pin(cm), torch.zeros((B, VW), dtype=torch.int32).pin_memory()
+                masked = torch.zeros_like(d_z).pin_memory() if want_masked else None
+                am, rep = np.full(B, -7, dtype=np.int32), np.full(B, -7, dtype=np.int32)
+                lse, lpa = np.full(B, 9, dtype=np.float32), np.full(B, 9, dtype=np.float32)
+                cz.cfgzip_decode_step_host(ctx.h, ctx.ids[0], row_part, d_cm, cm.shape[1], d_z, dtype_code(z), B, masked, vm, am,
+                                           rep, lpa, lse)
+                assert np.array_equal(d_z.numpy().view(np.uint8), z.view(np.uint8))
+                compare_step(dict(logits=masked.numpy().view(z.dtype) if want_masked else want["logits"],
+                                  vocab_mask=vm.numpy().view(np.uint32), argmax=am, rep=rep, lse=lse, logp_argmax=lpa), want, V)
