@@ -29,6 +29,7 @@ struct cfgzip_grammar {
     };
     std::vector<Prod> prods;
     std::vector<std::vector<int32_t>> by_term;  // production indices by terminal byte, ascending by head
+    uint8_t byte_class[256] = {};               // bytes with the same productions have the same number
     std::vector<uint8_t> adj;                   // n * n, adj[y * n + z] = 1: z may be popped right after y left nothing
 };
 
@@ -68,6 +69,80 @@ void build_adjacency(cfgzip_grammar& g) {
         }
     }
 }
+
+// Two bytes whose productions have the same heads and right-hand sides can stand for one another in every token.
+void number_bytes(cfgzip_grammar& g) {
+    auto less = [&](int32_t x, int32_t y) {
+        const auto &a = g.prods[size_t(x)], &b = g.prods[size_t(y)];
+        return a.head != b.head ? a.head < b.head : a.rhs < b.rhs;
+    };
+    std::vector<std::vector<int32_t>> known;  // sorted production lists, one per class
+    for (int b = 0; b < 256; ++b) {
+        std::vector<int32_t> list = g.by_term[size_t(b)];
+        std::sort(list.begin(), list.end(), less);
+        size_t k = 0;
+        for (; k < known.size(); ++k)
+            if (known[k].size() == list.size() &&
+                std::equal(list.begin(), list.end(), known[k].begin(), [&](int32_t x, int32_t y) { return !less(x, y) && !less(y, x); }))
+                break;
+        if (k == known.size()) known.push_back(std::move(list));
+        g.byte_class[b] = uint8_t(k);  // (at most 256 classes)
+    }
+}
+
+// Signature rows one worker has already built in this call, by the token's string of byte classes: most tokens of a vocabulary
+// (words, runs of digits) read the same to the grammar as another token. Bounded; what does not fit is built anew.
+class RowCache {
+  public:
+    struct Entry {
+        uint64_t hash;
+        size_t key;      // start in keys_
+        int32_t len, words;  // words: of the signature, -1: too many pairs
+        bool fits;
+    };
+    RowCache(const cfgzip_grammar& g, int32_t row_words, int32_t V)
+        : g_(g), row_words_(size_t(row_words)), most_(std::min({size_t(8192), size_t(V), (size_t(1) << 22) / size_t(row_words)})) {
+        size_t n = 16;
+        while (n < 4 * most_) n *= 2;
+        slots_.assign(n, -1);
+    }
+    // The row of a token, null if it is not known (then `add` takes what is built for it).
+    const int32_t* find(const uint8_t* bytes, int32_t len, const Entry** found) {
+        token_.resize(size_t(len));
+        uint64_t h = 0x9E3779B97F4A7C15ull + uint64_t(len);
+        for (int32_t i = 0; i < len; ++i) {
+            token_[size_t(i)] = g_.byte_class[bytes[i]];
+            h = (h ^ token_[size_t(i)]) * 0x100000001B3ull;
+        }
+        h ^= h >> 29;
+        hash_ = h;
+        for (at_ = size_t(h) & (slots_.size() - 1); slots_[at_] >= 0; at_ = (at_ + 1) & (slots_.size() - 1)) {
+            const Entry& e = entries_[size_t(slots_[at_])];
+            if (e.hash == h && e.len == len && std::memcmp(keys_.data() + e.key, token_.data(), size_t(len)) == 0) {
+                *found = &e;
+                return rows_.data() + size_t(slots_[at_]) * row_words_;
+            }
+        }
+        return nullptr;
+    }
+    void add(const std::vector<int32_t>& row, int32_t words, bool fits) {  // for the token last looked for
+        if (entries_.size() >= most_) return;
+        slots_[at_] = int32_t(entries_.size());
+        entries_.push_back(Entry{hash_, keys_.size(), int32_t(token_.size()), words, fits});
+        keys_.insert(keys_.end(), token_.begin(), token_.end());
+        rows_.insert(rows_.end(), row.begin(), row.end());
+    }
+
+  private:
+    const cfgzip_grammar& g_;
+    const size_t row_words_, most_;
+    std::vector<int32_t> slots_;  // four times as many as entries: an empty one always ends a search
+    std::vector<Entry> entries_;
+    std::vector<uint8_t> keys_, token_;
+    std::vector<int32_t> rows_;
+    uint64_t hash_ = 0;
+    size_t at_ = 0;
+};
 
 // Algorithm 1 as a depth-first enumeration with explicit stacks. `prev` is the symbol popped last (-1: none yet). The
 // pairs found are kept flat in one growing array ([n_in, in .., n_out, out (top first) ..] each) that is reused from
@@ -233,6 +308,7 @@ int cfgzip_grammar_create(int32_t n_nonterminals, int32_t start, const int32_t* 
     }
     for (auto& list : g->by_term)
         std::stable_sort(list.begin(), list.end(), [&](int32_t x, int32_t y) { return g->prods[size_t(x)].head < g->prods[size_t(y)].head; });
+    number_bytes(*g);
     build_adjacency(*g);
     cfgzip::Workspace::hold();
     *out = g;
@@ -263,14 +339,24 @@ int cfgzip_displacement_signatures(const cfgzip_grammar* g, const uint8_t* token
     auto work = [&]() noexcept {
         try {
             Displacer d(*g, max_pairs);
+            RowCache cache(*g, row_words, V);
             std::vector<int32_t> built(static_cast<size_t>(row_words));
             for (;;) {
                 const int32_t first = next.fetch_add(kTokenRun);
                 if (first >= V || first < 0) break;
                 const int32_t last = int32_t(std::min<int64_t>(int64_t(first) + kTokenRun, V));
                 for (int32_t i = first; i < last; ++i) {
-                    d.displace(token_bytes + token_off[i], int32_t(token_off[i + 1] - token_off[i]));
+                    const uint8_t* token = token_bytes + token_off[i];
+                    const int32_t len = int32_t(token_off[i + 1] - token_off[i]);
                     int32_t* row = signatures + int64_t(i) * row_words;
+                    const RowCache::Entry* known = nullptr;
+                    if (const int32_t* same = cache.find(token, len, &known)) {
+                        if (signature_words) signature_words[i] = known->words;
+                        if (!known->fits) rc.store(CFGZIP_E_RANGE);
+                        write_row(row, same, size_t(row_words));
+                        continue;
+                    }
+                    d.displace(token, len);
                     // canonical sequence: the pairs in lexicographic order, each as len(sigma_i), sigma_i, len(sigma_o), sigma_o
                     int64_t n = 0;
                     for (size_t at : d.pairs) n += 2 + d.flat[at] + d.flat[at + 1 + size_t(d.flat[at])];
@@ -288,6 +374,7 @@ int cfgzip_displacement_signatures(const cfgzip_grammar* g, const uint8_t* token
                     }
                     std::fill(out, built.data() + row_words, 0);
                     write_row(row, built.data(), size_t(row_words));
+                    cache.add(built, d.overflow ? -1 : int32_t(n), fits);
                 }
             }
             rows_written();
