@@ -1281,7 +1281,9 @@ int cfgzip_mask_logits(cfgzip_ctx* ctx, void* logits, int dtype, int64_t row_str
     if (!guard.ok) return CFGZIP_E_CUDA;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int chunks = std::max(1, ceil_div(V >> 3, kMaskChunk));
-    const unsigned grid = unsigned(std::min<int64_t>(int64_t(B) * chunks, int64_t(ctx->sm_count) * 8));
+    // (one piece per block until there are some ten waves of them: 512 rows of 128256 bf16 logits 48.2 -> 45.3 us against a
+    // resident set of blocks with twice as long pieces, rows of mixed density 55 -> 46)
+    const unsigned grid = unsigned(std::min<int64_t>(int64_t(B) * chunks, int64_t(ctx->sm_count) * 64));
     return launch(ctx, dtype == CFGZIP_BF16 ? k_mask_logits<kBF16> : k_mask_logits<kF32>, dim3(grid), dim3(256), 0, st, logits,
                   row_stride_elems, int(B), int(V), vocab_mask, vocab_stride_words, chunks);
 }

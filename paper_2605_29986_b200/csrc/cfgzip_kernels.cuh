@@ -2274,7 +2274,7 @@ __global__ void __launch_bounds__(1024) k_plan_rows(const PartDev* parts, int n_
 // Bound: HBM (read and write once). The mask bytes of the next piece of work are fetched while the logits of this one are
 // on their way.
 // ---------------------------------------------------------------------------------------
-constexpr int kMaskUnroll = 4, kMaskChunk = 256 * kMaskUnroll;  // vectors per block and piece
+constexpr int kMaskUnroll = 2, kMaskChunk = 256 * kMaskUnroll;  // vectors per block and piece
 
 template <int DT>
 __global__ void __launch_bounds__(256) k_mask_logits(void* logits, int64_t row_stride, int B, int V, const uint32_t* vocab_mask,
