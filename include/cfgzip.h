@@ -46,7 +46,8 @@ enum {
     CFGZIP_E_ARG = -1,       /* null pointer, negative size, stride too small, unknown enum */
     CFGZIP_E_RANGE = -2,     /* partition id not loaded, V mismatch, size beyond a limit */
     CFGZIP_E_PARTITION = -3, /* c / r do not describe a partition (see cfgzip_check_partition) */
-    CFGZIP_E_ALIGN = -4,     /* reserved; unaligned logits are handled by a slower path */
+    CFGZIP_E_ALIGN = -4,     /* logits rows that must be 16-byte aligned are not (cfgzip_multi_mask_logsoftmax_argmax,
+                                cfgzip_rmw_floor); every other call takes rows that start anywhere */
     CFGZIP_E_CUDA = -5,      /* a CUDA runtime call failed (no device, launch error) */
     CFGZIP_E_NOMEM = -6      /* device allocation failed, or B exceeds the reserved rows */
 };
@@ -84,9 +85,9 @@ int cfgzip_build_class_lists(const int32_t* token_to_class /*host [V]*/, int32_t
 
 /*
  * Load one tokenizer/grammar partition (Section 3.1: vectors c and r, "cached" once per
- * tokenizer/CFG pair). Validates as cfgzip_check_partition does, builds the class->token
- * lists, copies everything to the device on `stream` and waits for the copy. Returns the
- * new id in *out_id. Not a per-step call.
+ * tokenizer/CFG pair). Copies both vectors to the device, validates them there as
+ * cfgzip_check_partition does, builds the class->token lists on the GPU, all on `stream`, and waits for it.
+ * Returns the new id in *out_id. Not a per-step call.
  */
 int cfgzip_load_partition(cfgzip_ctx* ctx, const int32_t* token_to_class /*host [V]*/, int32_t V,
                           const int32_t* class_to_rep /*host [K]*/, int32_t K, void* stream,
@@ -134,8 +135,8 @@ int cfgzip_expand_mask(cfgzip_ctx* ctx, cfgzip_part_id part0, const int32_t* row
  * one keeps its bits (Section 2.2 defines the masking so; Section 3.1 applies it
  * after the gather).
  *   logits : dev [B, row_stride_elems] of `dtype`, row_stride_elems >= V; elements at
- *            index >= V of a row are not touched. 16-byte aligned rows take the
- *            vectorised path, anything else a scalar one.
+ *            index >= V of a row are not touched. Rows may start at any element: each is
+ *            taken by 16-byte vectors from its own first boundary on.
  */
 int cfgzip_mask_logits(cfgzip_ctx* ctx, void* logits, int dtype, int64_t row_stride_elems, int32_t B,
                        int32_t V, const uint32_t* vocab_mask, int64_t vocab_stride_words, void* stream);
@@ -151,9 +152,10 @@ int cfgzip_mask_logits(cfgzip_ctx* ctx, void* logits, int dtype, int64_t row_str
  *   logp_argmax : nullable dev float [B]; z_argmax - lse
  *   logp_full   : nullable dev float [B, V] (row stride V); z_i - lse, -inf where masked
  *   vocab_mask  : nullable; as in cfgzip_expand_mask
- *   mode        : CFGZIP_DENSE streams every row through the gather; CFGZIP_SPARSE builds each row's vocab
- *                 mask from the class->token lists of its allowed classes and never reads a logit that
- *                 is not allowed. CFGZIP_AUTO: the class-list kernel pays off when under 4 % (f32) or 1 %
+ *   mode        : CFGZIP_DENSE streams every row through the gather; CFGZIP_SPARSE is for rows that
+ *                 allow few tokens: it overwrites the 16-byte vectors that hold no allowed token without reading
+ *                 them (batches under 64 rows find them from the class->token lists of a row's allowed classes,
+ *                 larger ones through the gather's class table). CFGZIP_AUTO: the class-list kernel pays off when under 4 % (f32) or 1 %
  *                 (bf16) of the tokens are allowed, the measured break-even. Callers whose class masks are
  *                 still in host memory, where the grammar engine leaves them, get that choice for free
  *                 from cfgzip_choose_mode (cfgzip_decode_step_host with CFGZIP_AUTO uses it). On device
@@ -263,7 +265,10 @@ int cfgzip_choose_mode(cfgzip_ctx* ctx, cfgzip_part_id part0, const int32_t* row
  * The same step for callers whose data lives on the host: copies the class masks and
  * logits (pinned or pageable host memory) to staging buffers owned by the context,
  * runs cfgzip_masked_logsoftmax_argmax, copies the requested results back and waits
- * for `stream`. Staging buffers grow on first use (that call allocates).
+ * for `stream`. Staging buffers grow on first use (that call allocates). With pinned buffers the vocab masks are
+ * expanded and sent back while the logits still come in, the masked logits travel back in chunks of rows beside
+ * the copy in (on two streams of the context, joined before the call returns), and the kernels write the per-row
+ * results to the host's memory themselves. Pageable buffers take the same steps one after the other.
  *   logits_host     : host [B, V] of `dtype`, dense rows; left unmodified
  *   masked_logits   : nullable host [B, V]; receives the masked logits
  *   vocab_mask_host : nullable host uint32 [B, VW]
@@ -381,8 +386,9 @@ int cfgzip_displacement_signatures(const cfgzip_grammar* g, const uint8_t* token
  *   n_classes      : dev int32 [1]
  *   class_off / class_tok : both NULL, or dev int32 [V + 1] / [V]: the class -> token lists in ascending token id
  *                    (entries of class_off past n_classes read V)
- * Runs on the current device; allocates its scratch (about 50 bytes per token), synchronises `stream` before it
- * returns and frees the scratch: an offline call, not a per-step one. No context is needed.
+ * Runs on the current device and synchronises `stream` before it returns: an offline call, not a per-step one. No
+ * context is needed. Its scratch (about 30 bytes per token) is kept for the next call, up to 64 MB per device and while the
+ * process holds a context or a grammar; otherwise it is freed before the call returns.
  */
 int cfgzip_group_tokens(const int32_t* signatures, int32_t row_words, const int32_t* token_len, int32_t V,
                         int32_t* token_to_class, int32_t* class_to_rep, int32_t* n_classes, int32_t* class_off,

@@ -42,6 +42,7 @@ constexpr int kFiltList = 2048;     // tokens of the lists
 constexpr int kFiltBits = 12, kFiltBuckets = 1 << kFiltBits;
 constexpr int kFiltSteps = 8192, kFiltCoarse = kFiltThreads, kFiltFine = kFiltSteps / kFiltCoarse;  // the long way's steps
 constexpr int kFiltWindow = 200;    // tokens the window of the long way aims at
+constexpr unsigned int kFiltWindowMost = 800;  // and holds at most to either side, whole coarse steps
 constexpr int kFiltChunks = 512;    // most chunks of the draw's pass
 constexpr float kFixOne = 1099511627776.f;  // 2^40
 
@@ -103,7 +104,7 @@ struct FiltShared {
     unsigned long long pick[8];  // result of a search, written into every block of the cluster by the first
     unsigned long long scan_w[2][kFiltWarps];
     unsigned int scan_n[2][kFiltWarps];
-    unsigned long long peer_w[kFiltPeers];  // weight of the tokens of a block's share (those below the window's top)
+    unsigned long long peer_w[kFiltPeers];  // weight of the tokens of a block's share
     float warp_max[kFiltWarps], warp_sum[kFiltWarps];
     unsigned int list_n[2];      // of the two lists (they share their space, not their counts)
     uint32_t cut_key;
@@ -419,7 +420,7 @@ __device__ __noinline__ void filt_sort(FiltShared& sh, unsigned int n) {
 #pragma unroll 1
         for (unsigned int d = k / 2; d >= 1; d /= 2) {
             for (unsigned int p = tid; p < size / 2; p += kFiltThreads) {
-                const unsigned int x = 2 * d * (p / d) + p % d, y = x + d;
+                const unsigned int x = p + (p & ~(d - 1u)), y = x + d;  // (d is a power of two)
                 const unsigned long long vx = sh.order[x], vy = sh.order[y];
                 if ((vx > vy) == ((x & k) == 0u)) {
                     sh.order[x] = vy;
@@ -541,8 +542,14 @@ __device__ __noinline__ float2 filt_window(FiltShared& sh, const FiltRow& w, boo
             sh.pick[0] = static_cast<unsigned long long>(tid);
             sh.pick[1] = goal - below;
             sh.pick[2] = n;
+            sh.pick[3] = s.before.n;
         }
         __syncthreads();
+        // Where few tokens lie around the goal, below a peak, their density says little about the steps further down: the window
+        // ends where the coarse steps in front of it hold kFiltWindowMost tokens on either side.
+        const unsigned int through = s.before.n + n, goal_n = unsigned(sh.pick[3]);
+        const int skip = __syncthreads_count(through + kFiltWindowMost <= goal_n),
+                  reach = __syncthreads_count(through <= goal_n + kFiltWindowMost);
         if (tid < 32 && sh.pick[0] != ~0ull) {  // the step inside the coarse step, a lane each
             static_assert(kFiltFine == 32, "a lane per step");
             const int step = int(sh.pick[0]) * kFiltFine + lane;
@@ -560,7 +567,8 @@ __device__ __noinline__ float2 filt_window(FiltShared& sh, const FiltRow& w, boo
             const int in = past ? __ffs(int(past)) - 1 : kFiltFine - 1;
             const int at = int(sh.pick[0]) * kFiltFine + in;
             const float wide = fminf(0.5f * kFiltWindow * kFiltFine / float(unsigned(sh.pick[2])), float(kFiltSteps));
-            const float first = float(at) - wide, beyond = float(at) + 1.f + wide;
+            const float first = fmaxf(float(at) - wide, float(skip * kFiltFine)),
+                        beyond = fminf(float(at) + 1.f + wide, float(max(reach, int(sh.pick[0]) + 1) * kFiltFine));
             if (lane == in) {
                 float hi = first > 0.f ? w.M - first / steps : INFINITY;
                 float lo = beyond < float(kFiltSteps - 1) ? w.M - beyond / steps : w.z_zero;
@@ -859,20 +867,20 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __gri
                                               steps, turn);
             turn ^= 1;
             // (a top_k beyond everything that carries weight cuts nothing away: the window is empty then)
-            unsigned long long low = 0ull;
+            unsigned long long total = 0ull;
             filt_chunks<DT>(w, sh, [&](int t0, const float (&e)[8], CountMass& v) {
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
                     const unsigned long long wt = fixed_weight(e[q], M, scale);
                     const bool above = e[q] >= window.x;
                     v.w += above ? wt : 0ull;
-                    v.n += above ? 1u : 0u;
-                    low += above ? 0ull : wt;
+                    total += wt;
                 }
-                const uint32_t listed = filt_at_least(e, window.y) & ~filt_at_least(e, window.x);
+                const uint32_t above = filt_at_least(e, window.x), listed = filt_at_least(e, window.y) & ~above;
+                v.n += __popc(above);
                 filt_each(e, t0, listed, [&](int t, float z) { filt_push(sh, 1, t, z); });
             });
-            const unsigned long long all = filt_total(CountMass{0u, low}, sh, turn).w;
+            const unsigned long long all = filt_total(CountMass{0u, total}, sh, turn).w;
             turn ^= 1;
             if (tid == 0) st_peer_u64(peer_shared(&sh.peer_w[w.crank], 0u), all);
         }
@@ -895,7 +903,6 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __gri
                 for (unsigned int i = tid; i < n; i += kFiltThreads) listed += fixed_weight(__uint_as_float(sh.list[i].x), M, scale);
             listed = filt_total(CountMass{0u, listed}, sh, turn).w;
             turn ^= 1;
-            S = front.w;
             for (uint32_t p = 0; p < w.n_peers; ++p) S += sh.peer_w[p];
             const unsigned long long target = filt_target(S, top_p);
             const bool ok = n <= unsigned(kFiltList) &&
@@ -939,7 +946,6 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __gri
                 __syncthreads();
                 S = sh.topk_w;
             } else {
-                S = front.w;
                 for (uint32_t p = 0; p < w.n_peers; ++p) S += sh.peer_w[p];
             }
             target = filt_target(S, top_p);
