@@ -43,6 +43,7 @@ constexpr int kFiltBits = 12, kFiltBuckets = 1 << kFiltBits;
 constexpr int kFiltSteps = 8192, kFiltCoarse = kFiltThreads, kFiltFine = kFiltSteps / kFiltCoarse;  // the long way's steps
 constexpr int kFiltWindow = 200;    // tokens the window of the long way aims at
 constexpr unsigned int kFiltWindowMost = 800;  // and holds at most to either side, whole coarse steps
+constexpr int kFiltTries = 3;       // windows before the search
 constexpr int kFiltChunks = 512;    // most chunks of the draw's pass
 constexpr float kFixOne = 1099511627776.f;  // 2^40
 
@@ -106,7 +107,7 @@ struct FiltShared {
     unsigned int scan_n[2][kFiltWarps];
     unsigned long long peer_w[kFiltPeers];  // weight of the tokens of a block's share
     float warp_max[kFiltWarps], warp_sum[kFiltWarps];
-    unsigned int list_n[2];      // of the two lists (they share their space, not their counts)
+    unsigned int list_n[1 + kFiltTries];  // of the short way's list and the windows' (they share their space, not their counts)
     uint32_t cut_key;
     int cut_id;
     unsigned int n_kept;
@@ -528,12 +529,13 @@ __device__ __noinline__ float2 filt_window(FiltShared& sh, const FiltRow& w, boo
     if (w.crank == 0u) {
         unsigned int n = 0u;
         float wt = 0.f;
-#pragma unroll 1
-        for (uint32_t p = 0; p < w.n_peers; ++p) {
-            const uint32_t at = peer_shared(&sh.steps.coarse[tid], p);
-            n += ld_peer_u32(at);
-            wt += __uint_as_float(ld_peer_u32(at + 4u));
-        }
+#pragma unroll
+        for (uint32_t p = 0; p < uint32_t(kFiltPeers); ++p)  // (unrolled: all in flight at once)
+            if (p < w.n_peers) {
+                const uint32_t at = peer_shared(&sh.steps.coarse[tid], p);
+                n += ld_peer_u32(at);
+                wt += __uint_as_float(ld_peer_u32(at + 4u));
+            }
         if (tid == 0) sh.pick[0] = ~0ull;
         const CountMass mine{n, __float2ull_rz(wt * 16777216.f)};
         const FiltScan s = filt_scan(mine, sh, turn);
@@ -554,8 +556,9 @@ __device__ __noinline__ float2 filt_window(FiltShared& sh, const FiltRow& w, boo
             static_assert(kFiltFine == 32, "a lane per step");
             const int step = int(sh.pick[0]) * kFiltFine + lane;
             unsigned int c = 0u;
-#pragma unroll 1
-            for (uint32_t p = 0; p < w.n_peers; ++p) c += ld_peer_u32(peer_shared(&sh.steps.n[step], p));
+#pragma unroll
+            for (uint32_t p = 0; p < uint32_t(kFiltPeers); ++p)
+                if (p < w.n_peers) c += ld_peer_u32(peer_shared(&sh.steps.n[step], p));
             const unsigned long long x = by_count ? c : __float2ull_rz(float(c) * step_weight(step) * 16777216.f);
             unsigned long long inc = x;
 #pragma unroll 1
@@ -577,8 +580,8 @@ __device__ __noinline__ float2 filt_window(FiltShared& sh, const FiltRow& w, boo
                     // an end of the step, the value beyond that end belongs into the window too
                     const uint32_t key = logit_key<DT>(w.M - (float(at) + 0.5f) / steps);
                     const unsigned long long into = sh.pick[1] - min(sh.pick[1], inc - x);
-                    if (4ull * into < x) hi = fmaxf(hi, key_logit<DT>(key + 3u));
-                    if (4ull * into > 3ull * x) lo = fminf(lo, key_logit<DT>(key - 2u));
+                    if (3ull * into < x) hi = fmaxf(hi, key_logit<DT>(key + 3u));
+                    if (3ull * into > 2ull * x) lo = fminf(lo, key_logit<DT>(key - 2u));
                 }
                 sh.pick[6] = (static_cast<unsigned long long>(__float_as_uint(hi)) << 32) | __float_as_uint(fmaxf(lo, w.z_zero));
             }
@@ -669,6 +672,34 @@ __device__ __noinline__ FiltCut filt_search(const FiltRow& w, FiltShared& sh, in
     return cut;
 }
 
+// How many tokens the row's class mask allows, or all ones where `least` (every thread's part of a lower bound) says too many for
+// the list. A lane per class: the masks that get here allow few of them. Called by all threads of the block.
+__device__ __noinline__ unsigned int filt_allowed(const StepArgs& a, const PartDev& P, int row, float least, FiltShared& sh) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __syncthreads();
+#pragma unroll 1
+    for (int d = 16; d >= 1; d >>= 1) least += __shfl_xor_sync(0xFFFFFFFFu, least, d);
+    if (lane == 0) sh.warp_sum[warp] = least;
+    __syncthreads();
+    least = 0.f;
+#pragma unroll
+    for (int i = 0; i < kFiltWarps; ++i) least += sh.warp_sum[i];
+    if (least > 0.4f * kFiltList) return ~0u;  // (it usually says half and less)
+    const uint32_t* cm = a.class_mask + int64_t(row) * a.cm_stride;
+    unsigned int n = 0u;
+#pragma unroll 4
+    for (int k = tid; k < P.K; k += kFiltThreads)
+        if ((__ldg(cm + (k >> 5)) >> (k & 31)) & 1u) n += unsigned(__ldg(P.off + k + 1) - __ldg(P.off + k));
+    n = __reduce_add_sync(0xFFFFFFFFu, n);
+    __syncthreads();
+    if (lane == 0) sh.warp_sum[warp] = __uint_as_float(n);
+    __syncthreads();
+    n = 0u;
+#pragma unroll
+    for (int i = 0; i < kFiltWarps; ++i) n += __float_as_uint(sh.warp_sum[i]);
+    return n;
+}
+
 // One row per cluster of blocks (1 to 8 of them: a short batch has fewer rows than the device has multiprocessors).
 // Every block goes over its share of the row; what they find meets in the shared memory of the cluster's first block.
 template <int DT>
@@ -705,7 +736,7 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __gri
     w.n_chunks = geom.n_chunks;
     w.c_begin = min(int(w.crank) * geom.per_block, w.n_chunks);
     w.c_end = min(w.c_begin + geom.per_block, w.n_chunks);
-    if (tid < 2) sh.list_n[tid] = 0u;
+    if (tid < 1 + kFiltTries) sh.list_n[tid] = 0u;
     sh.bar[tid] = 0u;
     if (!a.group_rows) pdl_wait();
     PartDev P = a.p0;
@@ -767,6 +798,7 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __gri
     // ---- way 0 (short): the bar
     int way = 1;
     float z_bar = w.z_zero;
+    bool guess = false;   // top-p alone: whether the tokens above the bar weigh enough has to be seen
     float run_sum = 1.f;  // top-p alone: the weight of all tokens, relative to the largest, by the run sums
     if (top_k <= kFiltList / 8) {
         // The run maxima by distance from M, in kFiltThreads steps of the range of weights: their number (top-k), or their
@@ -811,9 +843,20 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __gri
         }
         if (lane == 31) sh.scan_n[turn][warp] = inc;
         __syncthreads();
-        uint32_t before = inc - here;
+        uint32_t before = inc - here, all = 0u;
 #pragma unroll
-        for (int i = 0; i < kFiltWarps; ++i) before += i < warp ? sh.scan_n[turn][i] : 0u;
+        for (int i = 0; i < kFiltWarps; ++i) {
+            before += i < warp ? sh.scan_n[turn][i] : 0u;
+            all += sh.scan_n[turn][i];
+        }
+        // The run maxima fall short by little (two heavy tokens in one run, runs of few allowed tokens): a bar that leaves out run
+        // maxima of 4 % of the weight top_p leaves out will do almost always, and the pass over the row says whether it did.
+        // (Where the runs say so, that is: the part of them that reaches the bar tells how many tokens do, the weight of the others
+        // how much lies below it.)
+        if (top_k == 0 && goal >= all && float(all) >= 0.6f * float(goal)) {
+            guess = true;
+            goal = all - 1u - min(all - 1u, uint32_t(0.04f * (1.f - top_p) * run_sum * 1048576.f));
+        }
         turn ^= 1;
         if (before <= goal && goal - before < here) sh.pick[0] = static_cast<unsigned long long>(tid);
         __syncthreads();
@@ -823,6 +866,39 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __gri
         // everything further off, rounded or not)
         if (found && sh.pick[0] + 1ull < kFiltThreads)
             z_bar = fmaxf(w.z_zero, M - (float(sh.pick[0]) + 1.01f) / steps - fabsf(M) * 1e-6f);
+        if (guess) {
+            z_bar = fmaxf(w.z_zero, fminf(z_bar, M + log2f(0.04f * (1.f - top_p) * run_sum) / scale));  // (nor single tokens of that weight)
+            int reach = 0;
+            float below = 0.f;
+#pragma unroll
+            for (int q = 0; q < kKeep; ++q) {
+                reach += __syncthreads_count(run_m[q] >= z_bar);
+                if (run_m[q] >= w.z_zero && run_m[q] < z_bar) below += run_s[q] * ex2f((run_m[q] - M) * scale);
+            }
+#pragma unroll
+            for (int d = 16; d >= 1; d >>= 1) below += __shfl_xor_sync(0xFFFFFFFFu, below, d);
+            if (lane == 0) sh.warp_sum[warp] = below;
+            __syncthreads();
+            below = 0.f;
+#pragma unroll
+            for (int i = 0; i < kFiltWarps; ++i) below += sh.warp_sum[i];
+            const float runs = float(n_states), seen = fminf(runs, float(kKeep * kFiltThreads)), part = float(reach) / seen;
+            if (part >= 1.f || -runs * log1pf(-part) > 0.25f * kFiltList || below * (runs / seen) / (1.f - part) > 0.5f * (1.f - top_p) * run_sum)
+                way = 1, guess = false;
+        }
+        // Rows that allow no more tokens than the list holds (a run's sum, relative to its own maximum, is at most its tokens: most
+        // other rows are told without counting): the tokens that one of them may weigh without all of them together
+        // weighing what top_p leaves out need not be listed. (1 % of 57591 tokens, 308 f32 rows, T = 0.7, top-p 0.95: 110 -> 78 us)
+        if (way == 1 && top_k == 0) {
+            float least = 0.f;
+#pragma unroll
+            for (int q = 0; q < kKeep; ++q) least += run_s[q];
+            const unsigned int allowed = filt_allowed(a, P, row, least, sh);
+            if (allowed <= unsigned(kFiltList)) {
+                way = 0;
+                z_bar = fmaxf(w.z_zero, M - fabsf(M) * 1e-6f + fminf(0.f, log2f(0.9f * (1.f - top_p) * run_sum / float(allowed)) / scale));
+            }
+        }
     }
     cluster_wait();
 
@@ -830,9 +906,11 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __gri
     CountMass front{0u, 0ull};  // what lies above the listed tokens
     FiltCut cut{0u, a.V, 0xFFFFFFFFu, 0ull};
     unsigned int n = 0u;
+    int tries = 0;  // windows looked at
+    float2 window = make_float2(INFINITY, INFINITY);
     if (way == 1 && top_k > 0 && top_p < 1.f) way = 2;
 #pragma unroll 1
-    for (; way < 2; ++way) {
+    while (way < 2) {
         if (way == 0) {
             unsigned long long mine = 0ull;
             auto push = [&](int t, float z) { filt_push(sh, 0, t, z); };
@@ -850,22 +928,25 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __gri
                 if (tid == 0) st_peer_u64(peer_shared(&sh.peer_w[w.crank], 0u), all);
             }
         } else {
-            const bool by_count = top_k > 0;
-            // For top-p the steps need not reach down to weight zero: what lies more than `range` powers of two below M weighs
-            // at most V 2^-range, half of what top_p leaves out.
-            const float range = by_count ? 41.5f : fminf(41.5f, log2f(2.f * float(a.V) / ((1.f - top_p) * run_sum)) + 1.f);
-            const float steps = float(kFiltSteps) * scale / range;
-            const float z_low = fmaxf(w.z_zero, M - range / scale);
-            hist_clear(sh, sizeof(sh.steps.n));
-            filt_visit<DT>(w, [&](int, const float (&e)[8]) {
+            if (tries == 0) {
+                const bool by_count = top_k > 0;
+                // For top-p the steps need not reach down to weight zero: what lies more than `range` powers of two below M weighs
+                // at most V 2^-range, half of what top_p leaves out.
+                const float range = by_count ? 41.5f : fminf(41.5f, log2f(2.f * float(a.V) / ((1.f - top_p) * run_sum)) + 1.f);
+                const float steps = float(kFiltSteps) * scale / range;
+                const float z_low = fmaxf(w.z_zero, M - range / scale);
+                hist_clear(sh, sizeof(sh.steps.n));
+                filt_visit<DT>(w, [&](int, const float (&e)[8]) {
 #pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    if (e[q] >= z_low) atomicAdd(&sh.steps.n[min(int((M - e[q]) * steps), kFiltSteps - 1)], 1u);
-            });
-            const float2 window = filt_window<DT>(sh, w, by_count,
-                                              by_count ? static_cast<unsigned long long>(top_k) - 1ull : __float2ull_rz(run_sum * top_p * 16777216.f),
-                                              steps, turn);
-            turn ^= 1;
+                    for (int q = 0; q < 8; ++q)
+                        if (e[q] >= z_low) atomicAdd(&sh.steps.n[min(int((M - e[q]) * steps), kFiltSteps - 1)], 1u);
+                });
+                window = filt_window<DT>(sh, w, by_count,
+                                         by_count ? static_cast<unsigned long long>(top_k) - 1ull
+                                                  : __float2ull_rz(run_sum * top_p * 16777216.f),
+                                         steps, turn);
+                turn ^= 1;
+            }
             // (a top_k beyond everything that carries weight cuts nothing away: the window is empty then)
             unsigned long long total = 0ull;
             filt_chunks<DT>(w, sh, [&](int t0, const float (&e)[8], CountMass& v) {
@@ -878,26 +959,29 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __gri
                 }
                 const uint32_t above = filt_at_least(e, window.x), listed = filt_at_least(e, window.y) & ~above;
                 v.n += __popc(above);
-                filt_each(e, t0, listed, [&](int t, float z) { filt_push(sh, 1, t, z); });
+                filt_each(e, t0, listed, [&](int t, float z) { filt_push(sh, 1 + tries, t, z); });
             });
             const unsigned long long all = filt_total(CountMass{0u, total}, sh, turn).w;
             turn ^= 1;
             if (tid == 0) st_peer_u64(peer_shared(&sh.peer_w[w.crank], 0u), all);
         }
         cluster_barrier();  // everything has arrived
-        n = ld_peer_u32(peer_shared(&sh.list_n[way], 0u));  // (the same in every block of the cluster)
-        if (way == 0) {
+        n = ld_peer_u32(peer_shared(&sh.list_n[way + tries], 0u));  // (the same in every block of the cluster)
+        if (way == 0 && (!guess || n > unsigned(kFiltList))) {
             if (n <= unsigned(kFiltList)) break;
-            if (top_k > 0 && top_p < 1.f) way = 1;  // both filters: way 1 takes one only
+            way = top_k > 0 && top_p < 1.f ? 2 : 1;  // (both filters: way 1 takes one only)
             continue;
         }
-        // does the cut lie in the window? (or at its end, when nothing is cut away)
+        // does the cut lie among the listed tokens? (or at their end, when nothing is cut away)
         if (w.crank == 0u) {
-            CountMass mine{0u, 0ull};
+            front = CountMass{0u, 0ull};
+            if (way == 1) {
+                CountMass mine{0u, 0ull};
 #pragma unroll 1
-            for (int c = tid; c < w.n_chunks; c += kFiltThreads) mine += CountMass{sh.chunk.ties[c], sh.chunk.above[c]};
-            front = filt_total(mine, sh, turn);
-            turn ^= 1;
+                for (int c = tid; c < w.n_chunks; c += kFiltThreads) mine += CountMass{sh.chunk.ties[c], sh.chunk.above[c]};
+                front = filt_total(mine, sh, turn);
+                turn ^= 1;
+            }
             unsigned long long listed = 0ull, S = 0ull;
             if (n <= unsigned(kFiltList))
                 for (unsigned int i = tid; i < n; i += kFiltThreads) listed += fixed_weight(__uint_as_float(sh.list[i].x), M, scale);
@@ -908,10 +992,37 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __gri
             const bool ok = n <= unsigned(kFiltList) &&
                             (top_k > 0 ? (front.n < unsigned(top_k) && unsigned(top_k) <= front.n + n) || (n == 0u && front.n <= unsigned(top_k))
                                        : front.w < target && target <= front.w + listed);
-            if (tid < int(w.n_peers)) st_peer_u64(peer_shared(&sh.pick[7], uint32_t(tid)), ok ? 1ull : 0ull);
+            // A top-p cut beside the window (1 % of flat bf16 rows, whose next value is a hundred tokens away): the exact sums say
+            // on which side and by how much weight, the window's own density how far. One more pass, the search takes ten.
+            const bool again = !ok && way == 1 && top_k == 0 && n <= unsigned(kFiltList) && tries + 1 < kFiltTries;
+            if (again && tid == 0) {
+                const float per_token = (fminf(window.x, M) - window.y) / float(n + 1u);
+                const bool up = front.w >= target;
+                const float edge = up ? window.x : window.y;
+                const float miss = static_cast<float>(up ? front.w - target : target - front.w - listed) * (1.f / kFixOne);
+                const float wide = (1.25f * miss * ex2f((M - edge) * scale) + 0.5f * kFiltWindow) * per_token;
+                float hi = up ? edge + wide : edge, lo = up ? edge : edge - wide;
+                if (DT == kBF16) {  // (a value or two further on at least)
+                    const uint32_t key = logit_key<DT>(edge);
+                    if (up) hi = fmaxf(hi, key_logit<DT>(key + 2u));
+                    else lo = fminf(lo, key_logit<DT>(key - 2u));
+                }
+                sh.pick[6] = (static_cast<unsigned long long>(__float_as_uint(hi)) << 32) | __float_as_uint(fmaxf(lo, w.z_zero));
+            }
+            __syncthreads();
+            if (tid < int(w.n_peers)) {
+                st_peer_u64(peer_shared(&sh.pick[7], uint32_t(tid)), ok ? 1ull : again ? 2ull : 0ull);
+                if (again && tid > 0) st_peer_u64(peer_shared(&sh.pick[6], uint32_t(tid)), sh.pick[6]);
+            }
         }
         cluster_barrier();
-        if (sh.pick[7] != 0ull) break;
+        if (sh.pick[7] == 1ull) break;
+        if (sh.pick[7] == 2ull) {
+            window = make_float2(__uint_as_float(uint32_t(sh.pick[6] >> 32)), __uint_as_float(uint32_t(sh.pick[6])));
+            ++tries;
+        } else {
+            ++way;
+        }
     }
 
     if (way < 2) {

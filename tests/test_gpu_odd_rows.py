@@ -98,6 +98,43 @@ def test_filtered_sampling(V, B, inv_t, top_k, top_p, dtype):
 
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("V,B", [(9001, 5), (28864, 150)])
+def test_filtered_cut_below_a_peak(V, B, dtype):
+    # a few large logits hold most of the weight and the nucleus ends in the thin top of the bulk below them, row by row a
+    # little further down: the steps around the cut hold few tokens, those below it thousands
+    K = 200
+    part, cm, z = inputs(V, K, B, dtype, 430, p=0.9, sigma=1.0)
+    f = z if dtype == "f32" else (z.astype(np.uint32) << 16).view(np.float32)
+    f = f.copy()
+    f[:, 11 : 11 + 6] = np.linspace(4.0, 9.0, B, dtype=np.float32)[:, None] + np.arange(6, dtype=np.float32) / 8
+    z = f if dtype == "f32" else (f.view(np.uint32) >> 16).astype(np.uint16)
+    u = rng.uniform(rng.stream_key(431, B), B).astype(np.float32)
+    with Ctx([part]) as ctx:
+        for top_p in (0.5, 0.9):
+            got = run_filtered(ctx, None, cm, z, V, u, 1.0, 0, top_p)
+            close, near = check_filtered(got, [part], None, cm, z, V, u, 1.0, 0, top_p, "p=%g" % top_p)
+            assert near <= 1
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("V,B,p,step", [(20000, 150, 0.9, 1 / 16), (20001, 9, 0.9, 1 / 4), (9001, 40, 0.01, 0.0), (57592, 160, 0.01, 0.0)])
+def test_filtered_top_p_alone(V, B, p, step, dtype):
+    # logits on a grid: hundreds of tokens per value, so that the first window holds one of them and the cut may lie in the next;
+    # few allowed tokens: hardly more than one to a run of the row, the run maxima fall short of the weight the nucleus needs
+    part, cm, z = inputs(V, 300, B, dtype, 432, p=p)
+    if step:
+        f = z if dtype == "f32" else (z.astype(np.uint32) << 16).view(np.float32)
+        f = np.round(f / step).astype(np.float32) * np.float32(step)
+        z = f if dtype == "f32" else (f.view(np.uint32) >> 16).astype(np.uint16)
+    u = rng.uniform(rng.stream_key(433, B), B).astype(np.float32)
+    with Ctx([part]) as ctx:
+        for inv_t, top_p in ((1.0, 0.5), (1.0, 0.9), (1.4, 0.95), (5.0, 0.9)):
+            got = run_filtered(ctx, None, cm, z, V, u, inv_t, 0, top_p)
+            close, near = check_filtered(got, [part], None, cm, z, V, u, inv_t, 0, top_p, "1/T=%g p=%g" % (inv_t, top_p))
+            assert near <= 1
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("V,pad,B,parts", [(7, 1, 64, 1), (15, 1, 70, 1), (16, 0, 64, 1), (31, 1, 65, 1), (264, 0, 64, 1), (513, 7, 97, 1),
                                            (8200, 0, 100, 3), (30000, 0, 64, 1), (70007, 1, 129, 2)])
 def test_rows_that_allow_few_tokens(V, pad, B, parts, dtype):
