@@ -17,14 +17,14 @@ namespace cfgzip {
 // Ways through, all exact:
 //   short  The streaming kernel has published the largest logit of every run of tokens. The k-th largest of those is a bar
 //          that at least k tokens reach, and, the runs being many, not many more (k = 50: some 60 to 100 tokens). For top-p
-//          alone the bar is where the run maxima by themselves already weigh enough. One pass over the row collects the
+//          alone the bar is where the run maxima by themselves already weigh enough, or nearly (checked afterwards). One pass over the row collects the
 //          tokens at or above the bar, a thread each, and every thread sums over all of them.
 //   long   Otherwise (a flat distribution, a large k), with one filter: a pass that counts the tokens in 16384 steps of the
 //          distance from the row maximum (one shared-memory addition a token; the weight of a step follows from its count to
 //          better than 0.1 %), which says about where the cut falls; and a pass that sums, exactly and chunk by chunk, what
 //          lies above a window of some 200 tokens around it and lists the tokens of the window. The exact sums then say whether
-//          the cut lies in the window, and where.
-//   search Where it does not (many equal logits), or with both filters, the kept set is { key > tau } plus the first m tokens,
+//          the cut lies in the window, and where; if it does not, they say where to lay the next one.
+//   search Where three do not hold it (many equal logits), or with both filters, the kept set is { key > tau } plus the first m tokens,
 //          in token order, with key == tau, where key is an order-preserving integer image of the logit; tau comes out of a
 //          radix search over the row, twelve bits a pass.
 // Bound: latency of a chain of block-wide steps, most of them executed once or twice, beside one or two passes over a row
