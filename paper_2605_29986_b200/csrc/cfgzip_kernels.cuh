@@ -7,6 +7,7 @@
 #include <cuda.h>
 
 #include "cfgzip_device.cuh"
+#include "ranges.h"
 
 namespace cfgzip {
 
@@ -2281,20 +2282,19 @@ __global__ void __launch_bounds__(256) k_mask_logits(void* logits, int64_t row_s
                                                      int64_t vm_stride, int chunks) {
     pdl_prologue();
     constexpr int ES = DT == kBF16 ? 2 : 4;
-    const int total = B * chunks, tid = threadIdx.x;
+    const int tid = threadIdx.x;
     struct Piece {
         char* vec;  // first vector of the row
         int o;      // this thread's first vector
         uint32_t byte[kMaskUnroll];
     };
-    auto fetch = [&](int item) {
+    auto fetch = [&](const PieceWalk& at) {
         Piece p;
-        const int row = item / chunks, ch = item - row * chunks;
-        char* rowp = reinterpret_cast<char*>(logits) + int64_t(row) * row_stride * ES;
-        const uint8_t* bits = reinterpret_cast<const uint8_t*>(vocab_mask) + int64_t(row) * vm_stride * 4;
+        char* rowp = reinterpret_cast<char*>(logits) + at.row * row_stride * ES;
+        const uint8_t* bits = reinterpret_cast<const uint8_t*>(vocab_mask) + at.row * vm_stride * 4;
         const int head = row_head<DT>(rowp, V), n_vec = (V - head) >> 3;
         p.vec = rowp + head * ES;
-        p.o = ch * kMaskChunk + tid;
+        p.o = at.ch * kMaskChunk + tid;
 #pragma unroll
         for (int u = 0; u < kMaskUnroll; ++u) {
             const int o = p.o + u * 256;
@@ -2304,24 +2304,24 @@ __global__ void __launch_bounds__(256) k_mask_logits(void* logits, int64_t row_s
                 if (head) p.byte[u] = ((p.byte[u] | (uint32_t(__ldg(bits + o + 1)) << 8)) >> head) & 0xFFu;
             }
         }
-        if (ch == 0 && tid < 16) {  // the ends of the row
+        if (at.ch == 0 && tid < 16) {  // the ends of the row
             const int t = tid < 8 ? tid : head + 8 * n_vec + tid - 8;
             if ((tid < 8 ? t < head : t < V) && !((__ldg(bits + (t >> 3)) >> (t & 7)) & 1u)) store_neg_inf<DT>(rowp, t);
         }
         return p;
     };
-    int item = blockIdx.x;
-    if (item >= total) return;
-    Piece p = fetch(item);
+    PieceWalk at(blockIdx.x, gridDim.x, chunks);
+    if (at.row >= B) return;
+    Piece p = fetch(at);
     for (;;) {
         Octet<DT> oc[kMaskUnroll];
 #pragma unroll
         for (int u = 0; u < kMaskUnroll; ++u)
             if (p.byte[u] != 0xFFu && p.byte[u] != 0u) oc[u].load(p.vec, p.o + u * 256);
         const Piece now = p;
-        item += gridDim.x;
-        const bool more = item < total;
-        if (more) p = fetch(item);
+        at.next();
+        const bool more = at.row < B;
+        if (more) p = fetch(at);
 #pragma unroll
         for (int u = 0; u < kMaskUnroll; ++u) {
             if (now.byte[u] == 0xFFu) continue;
