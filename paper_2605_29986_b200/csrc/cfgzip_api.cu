@@ -271,7 +271,9 @@ struct DensePlan {
     int fold = 0;        // pipelined kernel: results written by the last block of each group (no finalize launch)
     int fold_off = 0;    // fold: offset of the block's shared (row, warp) states, 0 = warps publish to the scratch directly
     int slots = 0;       // states per row in the global scratch
-    int blocks = 0;      // > 0: pipelined kernel, mixed batch: the blocks are shared out by the groups' sizes, at most S to a group
+    int blocks = 0;      // > 0: pipelined kernel, mixed batch: S_even blocks to a group where the groups are the fewest they can be,
+                         // else the blocks are shared out by the groups' sizes, at most S to a group
+    int S_even = 0;
     size_t smem = 0;
     int n_groups_ub = 1;
     bool use_plan_kernel = false;
@@ -416,15 +418,17 @@ DensePlan plan_pipe_opl(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixe
     d.WT = ctx->token_warps ? ctx->token_warps : n_warps / WR;
     d.WT = std::max(1, std::min(std::min(d.WT, max_warps / WR), chunks));
     d.threads = d.WT * WR * 32;
-    // The groups of a mixed batch may hold 32 rows or one: where there are blocks enough, each group gets its share of them
-    // (one wave of blocks that all have about as much to do; the same number for every group, sized for the fewest groups
-    // the batch can have, took a second wave: 256 rows over eight partitions, V = 256000, 78 us, now 65).
+    // The groups of a mixed batch may hold 32 rows or one, and only the GPU knows how many there are: where there are blocks
+    // enough it gives every group the same number if the groups are the fewest the batch can have (336 bf16 rows of 128256 in two
+    // partitions: 41.3 us; shares by size 44.1), else its share by size, one wave of blocks that all have about as much to do
+    // (256 rows in eight partitions, V = 256000: 63 us; the same number for every group, in two waves, 78).
     if (mixed && target >= 3 * d.n_groups_ub) {
         const int batches = ceil_div(B, kBatchRows), most = std::min(batches, kGroupRows / kBatchRows);
         const int S = std::min(target, ceil_div(int64_t(target) * most, batches) + 2);
         if (size_t(d.n_groups_ub) * kGroupRows * (size_t(S) * d.WT + 2) <= kPartialSlots) {
             d.blocks = target;
             d.S = S;
+            d.S_even = ceil_div(n_oct, per);
         }
     }
     while (!d.blocks) {
@@ -587,6 +591,7 @@ void fill_groups(cfgzip_ctx* ctx, StepArgs& a, const DensePlan& d) {
     a.group_w = d.blocks ? ctx->d_group_w : nullptr;
     a.max_groups = d.n_groups_ub;
     a.blocks = d.blocks;
+    a.S_even = d.S_even;
     a.S = d.S;
     a.per_split = d.per_split;
     a.WT = d.WT;
@@ -605,7 +610,7 @@ void fill_groups(cfgzip_ctx* ctx, StepArgs& a, const DensePlan& d) {
     // ahead pay (measured: B = 256 -3.6 %, qwen-size -2.3 %, B = 512 -1.6 %; shorter steps lose, B = 32 +7 %: the
     // requests compete with the loads of the kernel in front, whose end the step waits for).
     a.prefetch_items = ((ctx->pdl == 2 || (ctx->pdl && ctx->pdl_now)) && ctx->prefetch_now) ? ctx->prefetch_items : 0;
-    a.rot_chunks = ctx->rotate ? std::max(1, d.S * d.WT / ceil_div(std::min<int>(a.B, kGroupRows), kBatchRows)) : 0;
+    a.rot_chunks = ctx->rotate ? std::max(1, (d.blocks ? d.S_even : d.S) * d.WT / ceil_div(std::min<int>(a.B, kGroupRows), kBatchRows)) : 0;
     a.expire_test = ctx->expire_test;
     a.p0 = ctx->parts[size_t(a.part0)].dev;
 }

@@ -22,9 +22,11 @@ struct StepArgs {
     const int32_t* group_rows;  // dev [n_groups * 32], -1 = empty slot, valid slots first
     const int32_t* n_groups;    // dev scalar
     const int32_t* group_w;     // dev [max_groups + 1] or null: row batches in the groups in front of each (the total from n_groups
-                                // on); the blocks of the launch are then shared out by it (group_share), at most S per group
+                                // on); where the groups are more than the fewest they could be, the blocks of the launch are
+                                // shared out by it (group_share), at most S per group
     int32_t max_groups;
     int32_t blocks;             // group_w: blocks of the streaming launch
+    int32_t S_even;             // group_w: blocks of every group where the groups are the fewest they could be
     const uint32_t* class_mask;
     int64_t cm_stride;
     void* logits;
@@ -403,43 +405,39 @@ __device__ __forceinline__ Partial dense_tail_octets(const StepArgs& a, const Pa
     return Partial{m, s, pos, 0};
 }
 
-// The blocks of a streaming launch that work on group g: a.S each, or, where the groups of a mixed batch are of very different
-// size (33 rows of one partition make a group of 32 and one of 1), in proportion to their row batches, at least one.
+// The blocks of a streaming launch that work on group g: a.S each, or, for a mixed batch with blocks enough, a.S_even each as
+// long as the groups that turn up fit the launch at that number (two partitions of 24 rows: two groups, as 48 rows of one have),
+// else in proportion to the groups' row batches, at least one (33 rows of one partition make a group of 32 and one of 1).
 struct GroupShare {
     int first, S;
 };
-// (functions of their own: a batch without a row plan, whose steps are the shortest, should not fetch past this code)
-__device__ __noinline__ GroupShare group_share_of(const int32_t* n_groups, const int32_t* group_w, int max_groups, int blocks, int most, int g) {
-    const int ng = __ldg(n_groups), w0 = __ldg(group_w + g), w1 = __ldg(group_w + g + 1), W = __ldg(group_w + max_groups);
-    const int spare = blocks - ng, first = g + spare * w0 / max(W, 1), next = g + 1 + spare * w1 / max(W, 1);
-    return GroupShare{first, min(next - first, most)};
-}
 __device__ __forceinline__ GroupShare group_share(const StepArgs& a, int g) {
-    return group_share_of(a.n_groups, a.group_w, a.max_groups, a.blocks, a.S, g);
+    const int n = __ldg(a.n_groups), w0 = __ldg(a.group_w + g), w1 = __ldg(a.group_w + g + 1), W = __ldg(a.group_w + a.max_groups);
+    if (n * a.S_even <= a.blocks) return GroupShare{g * a.S_even, a.S_even};
+    const int spare = a.blocks - n, first = g + spare * w0 / max(W, 1), next = g + 1 + spare * w1 / max(W, 1);
+    return GroupShare{first, min(next - first, a.S)};
 }
-// The group of this block, its place among the group's blocks and their number (false: none). Called by whole warps.
-__device__ __forceinline__ bool block_group(const StepArgs& a, int& g, int& split, int& S) {
-    const int b = blockIdx.x;
-    if (!a.group_w) {
-        g = b / a.S;
-        split = b - g * a.S;
-        S = a.S;
-        return !(a.n_groups && g >= __ldg(a.n_groups));
+// The group of this block of such a launch (-1: none), its place among the group's blocks and their number. Called by one warp (a
+// function of its own: a batch without a row plan, whose steps are the shortest, should not fetch past this code).
+struct BlockPlace {
+    int g, split, S;
+};
+__device__ __noinline__ BlockPlace block_place(const StepArgs& a) {
+    const int b = blockIdx.x, n = __ldg(a.n_groups), even = a.S_even;
+    if (n * even <= a.blocks) {
+        const int g = b / even;
+        return BlockPlace{g < n ? g : -1, b - g * even, even};
     }
     const int lane = threadIdx.x & 31;
-    for (int g0 = 0; g0 < a.max_groups; g0 += 32) {
-        const bool real = g0 + lane < min(a.max_groups, __ldg(a.n_groups));
-        const GroupShare s = real ? group_share(a, g0 + lane) : GroupShare{0, 0};
+    for (int g0 = 0; g0 < n; g0 += 32) {
+        const GroupShare s = g0 + lane < n ? group_share(a, g0 + lane) : GroupShare{0, 0};
         const uint32_t hit = __ballot_sync(0xFFFFFFFFu, b >= s.first && b < s.first + s.S);
         if (hit) {
             const int l = __ffs(int(hit)) - 1;
-            g = g0 + l;
-            split = b - __shfl_sync(0xFFFFFFFFu, s.first, l);
-            S = __shfl_sync(0xFFFFFFFFu, s.S, l);
-            return true;
+            return BlockPlace{g0 + l, b - __shfl_sync(0xFFFFFFFFu, s.first, l), __shfl_sync(0xFFFFFFFFu, s.S, l)};
         }
     }
-    return false;
+    return BlockPlace{-1, 0, 0};
 }
 // Chunks in a run of a sampling step, as the warps of a group of such a batch dealt them.
 __device__ __noinline__ int group_run_chunks(int n_octets, int chunk_octets, int warps) {
@@ -559,6 +557,26 @@ __global__ void __launch_bounds__(kFinalizeThreads) k_finalize_rows(const __grid
     pdl_prologue();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = blockIdx.x / kGroupRows, j = blockIdx.x - g * kGroupRows;
+    // The states are asked for first, as many as a row can have: how many this one has, and whether there is a row, takes loads
+    // in a chain where rows are grouped by a plan.
+    const Partial* src = row_slots(a, g, j);
+    int n_states = a.slots;
+    auto fetch = [&](int base, int4 (&v)[4]) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int sp = base + u * kFinalizeThreads + tid;
+            v[u] = make_int4(__float_as_int(-INFINITY), 0, kNoPos, 0);
+            if (sp < n_states) v[u] = __ldcg(reinterpret_cast<const int4*>(src + sp));
+        }
+    };
+    int4 v0[4];
+    fetch(0, v0);
+    if (a.group_w) {
+        n_states = group_states(a, g);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (u * kFinalizeThreads + tid >= n_states) v0[u] = make_int4(__float_as_int(-INFINITY), 0, kNoPos, 0);
+    }
     if (a.n_groups && g >= __ldg(a.n_groups)) return;
     int row;
     if (a.group_rows) {
@@ -570,8 +588,6 @@ __global__ void __launch_bounds__(kFinalizeThreads) k_finalize_rows(const __grid
     if (row < 0) return;
     if (a.row_mode && a.row_mode[row]) return;  // automatic mode: the class-list kernel has finished this row
     const PartDev P = a.group_part ? a.parts[a.group_part[g]] : a.p0;
-    const Partial* src = row_slots(a, g, j);
-    const int n_states = group_states(a, g);
     // Two passes over the states, which stay in registers (up to four per thread, all loads in flight together):
     // first the row maximum (shuffles and max only), then every state's sum brought to that maximum with one
     // exponential per state, summed, and the lowest position among the states that hold the maximum. No
@@ -579,16 +595,6 @@ __global__ void __launch_bounds__(kFinalizeThreads) k_finalize_rows(const __grid
     constexpr int kWarps = kFinalizeThreads / 32;
     __shared__ float s_max[kWarps], s_sum[kWarps];
     __shared__ int s_pos[kWarps];
-    auto fetch = [&](int base, int4 (&v)[4]) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int sp = base + u * kFinalizeThreads + tid;
-            v[u] = make_int4(__float_as_int(-INFINITY), 0, kNoPos, 0);
-            if (sp < n_states) v[u] = __ldcg(reinterpret_cast<const int4*>(src + sp));
-        }
-    };
-    int4 v0[4];
-    fetch(0, v0);
     float M = fmaxf(fmaxf(__int_as_float(v0[0].x), __int_as_float(v0[1].x)), fmaxf(__int_as_float(v0[2].x), __int_as_float(v0[3].x)));
     for (int base = 4 * kFinalizeThreads; base < n_states; base += 4 * kFinalizeThreads) {  // more than 1024 states: rare
         int4 w[4];
@@ -649,6 +655,20 @@ __global__ void __launch_bounds__(256) k_finalize_rows_warp(const __grid_constan
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int idx = blockIdx.x * 8 + warp;  // (group, row slot)
     const int g = idx / kGroupRows, j = idx - g * kGroupRows;
+    const Partial* src = row_slots(a, g, j);  // (the states first, as above)
+    int4 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int sp = u * 32 + lane;
+        v[u] = make_int4(__float_as_int(-INFINITY), 0, kNoPos, 0);
+        if (sp < a.slots) v[u] = __ldcg(reinterpret_cast<const int4*>(src + sp));
+    }
+    if (a.group_w) {
+        const int n_states = group_states(a, g);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (u * 32 + lane >= n_states) v[u] = make_int4(__float_as_int(-INFINITY), 0, kNoPos, 0);
+    }
     if (a.n_groups && g >= __ldg(a.n_groups)) return;
     int row;
     if (a.group_rows) {
@@ -660,15 +680,6 @@ __global__ void __launch_bounds__(256) k_finalize_rows_warp(const __grid_constan
     if (row < 0) return;
     if (a.row_mode && a.row_mode[row]) return;  // automatic mode: the class-list kernel has finished this row
     const PartDev P = a.group_part ? a.parts[a.group_part[g]] : a.p0;
-    const Partial* src = row_slots(a, g, j);
-    const int n_states = group_states(a, g);
-    int4 v[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const int sp = u * 32 + lane;
-        v[u] = make_int4(__float_as_int(-INFINITY), 0, kNoPos, 0);
-        if (sp < n_states) v[u] = __ldcg(reinterpret_cast<const int4*>(src + sp));
-    }
     float m0 = __int_as_float(v[0].x), s0 = __int_as_float(v[0].y), m1 = __int_as_float(v[1].x), s1 = __int_as_float(v[1].y);
     int p0 = v[0].z, p1 = v[1].z;
     partial_merge(m0, s0, p0, __int_as_float(v[2].x), __int_as_float(v[2].y), v[2].z);
@@ -997,12 +1008,22 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
     const float scale = TEMPERED ? a.scale : kLog2e;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     int g, split, S;
-    if (TMAP) {  // (tiled copies: no row plan)
+    if (TMAP || !a.group_w) {  // (tiled copies: no row plan)
         g = blockIdx.x / a.S;
         split = blockIdx.x - g * a.S;
         S = a.S;
-    } else if (!block_group(a, g, split, S)) {
-        return;
+        if (!TMAP && a.n_groups && g >= __ldg(a.n_groups)) return;
+    } else {  // (one warp looks: sixteen of every block after the same few words wait for one another)
+        __shared__ BlockPlace s_place;
+        if (warp == 0) {
+            const BlockPlace place = block_place(a);
+            if (lane == 0) s_place = place;
+        }
+        __syncthreads();
+        g = s_place.g;
+        split = s_place.split;
+        S = s_place.S;
+        if (g < 0) return;
     }
     const bool early_cm = a.cm_bulk && implicit;
     if (early_cm && tid == 0) {
