@@ -235,30 +235,43 @@ struct FiltOct {
     uint4 a, b;
 };
 template <int DT>
-__device__ __noinline__ FiltOct<DT> filt_edge(FiltOct<DT> o, int t0, int end) {  // rare: some of the eight lie outside
+struct FiltNone {  // -inf in every element of a word
+    static constexpr uint32_t word = DT == kBF16 ? 0xFF80FF80u : 0xFF800000u;
+};
+template <int DT>
+__device__ __noinline__ FiltOct<DT> filt_edge(const char* rowp, int t0, int end) {  // rare: some of the eight lie outside
     constexpr int kPer = DT == kBF16 ? 2 : 1;
-    uint32_t r[8] = {o.a.x, o.a.y, o.a.z, o.a.w, o.b.x, o.b.y, o.b.z, o.b.w};
+    uint32_t r[8];
+#pragma unroll
+    for (int q = 0; q < 8 / kPer; ++q) r[q] = FiltNone<DT>::word;
 #pragma unroll
     for (int q = 0; q < 8; ++q)
-        if (unsigned(t0 + q) >= unsigned(end)) {
-            if (DT == kBF16)
-                r[q / kPer] = (q & 1) ? (r[q / kPer] & 0xFFFFu) | 0xFF800000u : (r[q / kPer] & 0xFFFF0000u) | 0xFF80u;
-            else
-                r[q / kPer] = 0xFF800000u;
+        if (octet_has(t0, q, end)) {
+            if (DT == kBF16) {
+                const uint32_t x = __ldcg(reinterpret_cast<const unsigned short*>(rowp) + (t0 + q));
+                r[q / kPer] = (q & 1) ? (r[q / kPer] & 0xFFFFu) | (x << 16) : (r[q / kPer] & 0xFFFF0000u) | x;
+            } else {
+                r[q] = __ldcg(reinterpret_cast<const unsigned int*>(rowp) + (t0 + q));
+            }
         }
-    return FiltOct<DT>{make_uint4(r[0], r[1], r[2], r[3]), make_uint4(r[4], r[5], r[6], r[7])};
+    FiltOct<DT> o;
+    o.a = make_uint4(r[0], r[1], r[2], r[3]);
+    o.b = DT == kF32 ? make_uint4(r[4], r[5], r[6], r[7]) : o.a;
+    return o;
 }
 template <int DT>
 __device__ __forceinline__ FiltOct<DT> filt_load(const char* rowp, int t0, int end) {
-    constexpr uint32_t kNone = DT == kBF16 ? 0xFF80FF80u : 0xFF800000u;
+    constexpr uint32_t kNone = FiltNone<DT>::word;
     FiltOct<DT> o;
     o.a = o.b = make_uint4(kNone, kNone, kNone, kNone);
-    // (a vector that holds one token of the row lies in memory the row's buffer shares a 16-byte granule with)
-    constexpr int kVec = DT == kBF16 ? 8 : 4;
-    const char* p = rowp + int64_t(t0) * (DT == kBF16 ? 2 : 4);
-    if (t0 < end && t0 > -kVec) o.a = __ldcg(reinterpret_cast<const uint4*>(p));
-    if (DT == kF32 && t0 + 4 < end && t0 > -8) o.b = __ldcg(reinterpret_cast<const uint4*>(p + 16));
-    if (t0 < end && t0 > -8 && (t0 < 0 || t0 + 8 > end)) o = filt_edge<DT>(o, t0, end);
+    octet_loads(
+        t0, end,
+        [&] {
+            const char* p = rowp + int64_t(t0) * (DT == kBF16 ? 2 : 4);
+            o.a = __ldcg(reinterpret_cast<const uint4*>(p));
+            if (DT == kF32) o.b = __ldcg(reinterpret_cast<const uint4*>(p + 16));
+        },
+        [&] { o = filt_edge<DT>(rowp, t0, end); });
     return o;
 }
 template <int DT>

@@ -30,4 +30,16 @@ struct PieceWalk {
     }
 };
 
+// The loads of eight consecutive tokens of a row, t0 .. t0 + 7, of which those from 0 to end - 1 exist: all of them as whole
+// vectors, some of them one by one, or none. Nothing outside the row is asked for: its neighbours need not be readable.
+template <typename Whole, typename One>
+CFGZIP_HD void octet_loads(int t0, int end, Whole&& whole, One&& one) {
+    if (t0 >= 0 && t0 <= end - 8) {
+        whole();
+    } else if (t0 > -8 && t0 < end) {
+        one();
+    }
+}
+CFGZIP_HD bool octet_has(int t0, int q, int end) { return unsigned(t0 + q) < unsigned(end); }  // does its q-th token exist?
+
 }  // namespace cfgzip

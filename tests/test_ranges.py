@@ -14,7 +14,7 @@ def run_cpp(tmp_path_factory):
 
     def run(name, body):
         src = folder / (name + ".cpp")
-        src.write_text('#include "ranges.h"\n#include <cstdio>\n#include <vector>\nusing namespace cfgzip;\n' + body)
+        src.write_text('#include "ranges.h"\n#include <cstdio>\n#include <cstdlib>\n#include <vector>\nusing namespace cfgzip;\n' + body)
         exe = str(folder / name)
         subprocess.check_call([shutil.which("g++") or "c++", "-O2", "-std=c++17", "-Wall", "-Werror", "-ftrapv", "-I", CSRC, "-o", exe, str(src)])
         out = subprocess.run([exe], stdout=subprocess.PIPE, text=True)
@@ -57,6 +57,25 @@ int main() {
             }
             const long long total = (long long)s[0] * s[1];
             if (n != (total - b + blocks - 1) / blocks) { printf("%lld pieces for block %u\n", n, b); return 1; }
+        }
+}
+""")
+
+
+def test_octets_of_a_row_ask_for_its_tokens_and_nothing_else(run_cpp):
+    # rows whose vectors start up to seven tokens in front of them (wherever the row starts in memory), every length around a
+    # vector or two: a vector at either end that reaches past the row is read token by token
+    run_cpp("octets", r"""
+int main() {
+    for (int V = 1; V <= 41; ++V)
+        for (int lead = 0; lead < 8; ++lead) {
+            std::vector<int> seen(size_t(V), 0);
+            for (int t0 = -lead - 16; t0 <= V + 16; t0 += 8) {
+                auto read = [&](int t) { if (t < 0 || t >= V) { printf("V %d lead %d: token %d\n", V, lead, t); exit(1); } ++seen[size_t(t)]; };
+                octet_loads(t0, V, [&] { for (int q = 0; q < 8; ++q) read(t0 + q); },
+                            [&] { for (int q = 0; q < 8; ++q) if (octet_has(t0, q, V)) read(t0 + q); });
+            }
+            for (int n : seen) if (n != 1) { printf("V %d lead %d: a token %d times\n", V, lead, n); return 1; }
         }
 }
 """)
