@@ -481,17 +481,34 @@ DensePlan plan_pipe(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, i
     return items >= kTwoOctetItemsPerWarp * warps ? two : one;
 }
 
+// Whether rows that allow few tokens go through k_step_few (`d`, `per_sm`: its launch shape) or k_step_sparse, the class lists.
+// k_step_few builds a class table per block, 32 rows at a time, and streams all rows at once; the class lists have a block or more
+// per row, most efficient from the row count on at which a block takes a whole row and as long as these fit the device in one wave.
+// Measured, us, class lists / k_step_few, bf16, one to five classes allowed:
+//   under 64 rows    32 of 128256: K = 512 20 / 11, 2000 14.9 / 12.4, 4000 12.8 / 14.2; 48 f32 rows of 256000, K = 2000 20 / 24: by
+//                    classes and row length there, but the class lists are one launch instead of two and are kept for all of them
+//   class table      128 of 128256: K = 4000 25 / 20, 6000 20 / 23, 8192 22 / 33 (from some 4900 classes on the masks are not
+//                    staged); 512 of 256000: K = 6000 106 / 77, 8192 90 / 81 (few blocks per row make up for it), 16000 95 / 93
+//   short rows       450 of 20032 12 / 14, 450 of 32064 15 / 19, 410 of 32064 15.1 / 14.8, 512 of 64064 24 / 27, 800 40 / 39
+//   mixed batches    groups of few rows build tables for little: 64 rows of 128256 in eight partitions, K = 512 19 / 16, 3000
+//                    28 / 17, 4000 13 / 18; 300 rows of 20032 in two of 512 11.2 / 11.7, in eight 11 / 15
+bool few_pays(const cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, int elem_size, const DensePlan& d, int per_sm) {
+    const int wave = ctx->sm_count * ctx->ctas_per_sm;  // rows from half of this on have one block each in the other kernel
+    const int64_t row_kb = int64_t(ps.V) * elem_size >> 10;
+    if (B < 64) return false;
+    if (mixed) return ps.maxK <= 3072 && !(row_kb < 96 && d.n_groups_ub > 16);
+    if (!d.stage_stride && (per_sm < 3 || 4 * int64_t(ps.V) < 3 * int64_t(ps.maxK) * d.S)) return false;
+    return !(row_kb < 96 && B > wave / 2) && !(row_kb < 160 && B > 3 * wave / 4 && B <= wave);
+}
+
 // Launch shape of the kernel for rows that allow few tokens: three blocks per SM; warps go side by side along the vocabulary
-// as long as a block has enough chunks for them, else they split the row batches. Below kFewRows rows a group of 32 leaves the
-// blocks too little to do between their set-up and the second launch: a block or more per row, one launch, is as fast there
-// (4 rows of 184913 f32: 11.8 against 10.5 us; 32 of 128256: 13.1 against 15.5).
-constexpr int kFewRows = 64;
+// as long as a block has enough chunks for them, else they split the row batches.
 DensePlan plan_few(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, int elem_size) {
     DensePlan d;
     d.table_words = (ps.maxKW + 1) * 32;
     d.use_plan_kernel = mixed;
     d.n_groups_ub = mixed ? ceil_div(B, kGroupRows) + ps.n_live_same_v : ceil_div(B, kGroupRows);
-    if (B < kFewRows || !ps.all_c16 || (mixed && (B > ctx->reserved_rows || d.n_groups_ub > ctx->max_groups))) return d;
+    if (!ps.all_c16 || (mixed && (B > ctx->reserved_rows || d.n_groups_ub > ctx->max_groups))) return d;
     const size_t fixed = dense_smem_bytes(d.table_words, kFewWarps, 0) + kFewWarps * sizeof(FewWarp);
     const size_t staging = size_t(ps.maxKW | 1) * kGroupRows * 4;
     if (fixed > size_t(ctx->smem_optin) - 2048) return d;
@@ -507,7 +524,7 @@ DensePlan plan_few(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, in
     d.WT = kFewWarps / WR;
     d.threads = kFewThreads;
     d.slots = d.S * d.WT + 1;
-    d.ok = size_t(d.n_groups_ub) * kGroupRows * d.slots <= kPartialSlots;
+    d.ok = size_t(d.n_groups_ub) * kGroupRows * d.slots <= kPartialSlots && few_pays(ctx, ps, B, mixed, elem_size, d, per_sm);
     return d;
 }
 
