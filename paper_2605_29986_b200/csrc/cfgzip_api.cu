@@ -528,9 +528,29 @@ DensePlan plan_few(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, in
     return d;
 }
 
-// Launch shape of the kernel for several masks per logits row: two blocks per SM of eight warps (four where the class table
-// is large, and where the chunks would not give every SM a block); warps split the row batches of a group first, so that a block builds its table for as many chunks as possible.
-DensePlan plan_multi(cfgzip_ctx* ctx, const PartSet& ps, int32_t rows) {
+// Whether a call with several masks per logits row goes through k_step_multi or, every (row, mask) for itself, k_step_dense.
+// k_step_multi takes the logits rows of a batch of eight (row, mask) pairs one after the other, so with two or three masks a row
+// its chain is the longer one and its sharing small; k_step_dense builds a class table for every few tokens, which costs with K, and
+// takes each exponential once per mask, which costs once the device is full. `items`: (256 tokens, batch) pairs. Measured, us,
+// k_step_dense / k_step_multi, bf16 of 128256, rows x masks:
+//   K = 256    4x2 9.0 / 11.3, 16x2 10.4 / 11.8, 32x2 16 / 15; 4x4 9.3 / 9.9, 16x4 16 / 13; 1x16 9.3 / 8.7, 8x16 22 / 14
+//   K = 2048   4x2 11.3 / 12.1, 16x2 12.6 / 12.7, 32x2 17.5 / 16; 3x3 11.6 / 9.3, 12x3 16 / 15; 2x4 11.0 / 10.0, 8x16 24 / 15
+//   K = 4000   4x2 14.5 / 13.5, 16x2 15.9 / 13.8;  K = 8000  1x2 25 / 13, 4x2 26 / 15
+// f32 of 128256, K = 2048: 4x2 14.8 / 12.6;  f32 of 50048, K = 2048: 4x2 10.1 / 10.8, 24x2 11.7 / 12.6
+bool multi_pays(const PartSet& ps, int32_t B, int masks_per_row, int elem_size, int64_t items) {
+    const int logits_rows = std::min<int>(B, ceil_div(kBatchRows, masks_per_row));  // of a batch
+    if (logits_rows == 1 || ps.maxK > 3072 || int64_t(ps.V) * elem_size >= 400 * 1024) return true;
+    if (ps.maxK < 1024) return items >= (logits_rows == 2 ? 1500 : 2200);
+    return logits_rows == 2 || items >= (logits_rows == 3 ? 1000 : 2200);
+}
+
+// Launch shape of the kernel for several masks per logits row: two blocks per SM of eight warps, four where the class table is
+// large, where eight would get a third of an item each or less (4 rows x 4 masks of 50048 bf16, K = 256: 8.7 against 9.4 us; 4 x 4
+// of 128256, K = 2048: 12.6 with four, 9.3 with eight), and on short calls where only four leave room to stage the class masks
+// (K = 8000, 4 x 2: 14.7 against 18); warps split the row batches of a group first, so that a block builds its table for as many
+// chunks as possible.
+DensePlan plan_multi(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, int masks_per_row, int elem_size) {
+    const int32_t rows = B * masks_per_row;
     DensePlan d;
     d.table_words = (ps.maxKW + 1) * 32;
     d.n_groups_ub = ceil_div(rows, kGroupRows);
@@ -540,7 +560,11 @@ DensePlan plan_multi(cfgzip_ctx* ctx, const PartSet& ps, int32_t rows) {
     auto bytes = [&](int warps) { return dense_smem_bytes(d.table_words, warps, 0) + size_t(warps) * kMultiTable; };
     const int n_chunks = std::max(1, ceil_div(ps.V >> 3, 32));
     const int row_batches = ceil_div(rows, kBatchRows);
-    while (n_warps > 4 && (bytes(n_warps) > cap / 2 || int64_t(n_chunks) * row_batches < int64_t(ctx->sm_count) * n_warps)) n_warps /= 2;
+    const int64_t items = int64_t(n_chunks) * row_batches;
+    if (!multi_pays(ps, B, masks_per_row, elem_size, items)) return d;
+    while (n_warps > 4 && (bytes(n_warps) > cap / 2 || 3 * items <= int64_t(ctx->sm_count) * n_warps ||
+                           (items < int64_t(ctx->sm_count) * n_warps && bytes(n_warps) + staging > cap / 2)))
+        n_warps /= 2;
     d.smem = bytes(n_warps);
     if (d.smem > cap) return d;
     if (d.smem + staging <= cap / 2) {
@@ -1477,9 +1501,9 @@ int cfgzip_multi_mask_logsoftmax_argmax(cfgzip_ctx* ctx, cfgzip_part_id part0, c
     a.inv_t = 1.f;
     a.masks_per_row = masks_per_row;
     DensePlan d;
-    if (masks_per_row > 1) d = plan_multi(ctx, ps, rows);
+    if (masks_per_row > 1) d = plan_multi(ctx, ps, B, masks_per_row, es);
     const bool shared = d.ok;
-    // nothing to share (64 rows with one mask each: 17.3 against 19.2 us), or a class table that leaves no room beside it
+    // nothing to share (64 rows with one mask each: 17.3 against 19.2 us) or too little, or a class table that leaves no room beside it
     if (!shared) d = plan_dense(ctx, ps, rows, false, 4 * ps.VW, 32, true);
     if (!d.ok) return CFGZIP_E_RANGE;  // more than 65535 classes, or a class table beyond shared memory
     fill_groups(ctx, a, d);

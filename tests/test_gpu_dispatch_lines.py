@@ -1,9 +1,10 @@
 """Calls on either side of the lines at which a step takes another kernel, against the CPU oracle: rows that allow few tokens
-(row count, classes, row length, mixed batches)."""
+(row count, classes, row length, mixed batches) and several masks per row (masks, classes, row length)."""
 import numpy as np
 import pytest
 
 import synth
+import test_gpu_multi_mask
 from synth import rng
 from paper_2605_29986_b200 import binding as cz
 from _gpu_util import Ctx, compare_step, oracle_step, run_fused
@@ -25,3 +26,12 @@ def test_rows_that_allow_few_tokens(V, K, B, parts, dtype):
     z = synth.logits_normal(B, V, 2.0, dtype, (912, V, K))
     with Ctx(ps) as ctx:
         compare_step(run_fused(ctx, row_part, cm, z, V, mode=cz.SPARSE), oracle_step(ps, row_part, cm, z, V), V)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("V,K,B,M", [
+    (20008, 200, 1, 3), (20008, 200, 2, 2), (20008, 200, 3, 2), (20008, 2048, 2, 2), (20008, 2048, 3, 2), (20008, 2048, 13, 3),
+    (30000, 3072, 3, 2), (30000, 3073, 3, 2), (30000, 8000, 4, 2), (128256, 300, 5, 5), (102400, 300, 3, 2), (102408, 300, 3, 2), (256000, 300, 2, 2),
+    (40000, 1024, 26, 2), (40000, 1023, 40, 4)])
+def test_several_masks_per_row(V, K, B, M, dtype):
+    test_gpu_multi_mask.test_multi_mask_shapes(V, K, B, M, dtype)
