@@ -57,7 +57,8 @@ struct cfgzip_ctx {
     PartDev* d_parts = nullptr;
     Partial* d_partials = nullptr;
     unsigned int* d_tickets = nullptr;  // reserved_rows entries
-    int32_t* d_status = nullptr;        // 3 counters
+    int32_t* d_status = nullptr;        // 4 counters, and 4 that nobody reads (see uncounted)
+    bool uncounted = false;             // set around a launch that repeats what another launch of the same call counts
     int32_t* d_group_part = nullptr;
     int32_t* d_group_rows = nullptr;
     int32_t* d_n_groups = nullptr;
@@ -132,6 +133,8 @@ struct DeviceGuard {
 };
 
 inline int ceil_div(int64_t a, int64_t b) { return int((a + b - 1) / b); }
+
+int32_t* status_of(const cfgzip_ctx* ctx) { return ctx->d_status + (ctx->uncounted ? 4 : 0); }
 
 template <typename... KArgs, typename... Args>
 int launch(cfgzip_ctx* ctx, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
@@ -616,7 +619,7 @@ int run_plan_kernel(cfgzip_ctx* ctx, const int32_t* row_part, int32_t B, int32_t
     ctx->plan_valid = false;                 // this launch overwrites them
     return launch(ctx, k_plan_rows, dim3(1), dim3(1024), 0, st, (const PartDev*)ctx->d_parts, int(ctx->parts.size()),
                   row_part, int(B), int(V), d.n_groups_ub, ctx->d_group_part, ctx->d_group_rows, ctx->d_n_groups,
-                  ctx->d_group_w, ctx->d_status);
+                  ctx->d_group_w, status_of(ctx));
 }
 
 void fill_groups(cfgzip_ctx* ctx, StepArgs& a, const DensePlan& d) {
@@ -973,7 +976,9 @@ int host_step_pinned(cfgzip_ctx* ctx, const HostStep& h) {
     }
     int rc = CFGZIP_OK, mode = h.mode;
     if (good && h.vocab_mask_host) {
+        ctx->uncounted = true;  // (the step below counts the rows without a partition)
         rc = cfgzip_expand_mask(ctx, h.part0, d_rp, ctx->st_cm, h.class_stride_words, ctx->st_vm, h.VW, h.B, CFGZIP_DENSE, h.stream);
+        ctx->uncounted = false;
         good = rc == CFGZIP_OK && after(out, ctx->st_expanded, h.stream) &&
                ok(cudaMemcpyAsync(h.vocab_mask_host, ctx->st_vm, size_t(h.B) * size_t(h.VW) * 4, cudaMemcpyDeviceToHost, out));
     }
@@ -1101,11 +1106,11 @@ int cfgzip_create(int device, cfgzip_ctx** out) {
     }
     bool ok = cudaMalloc(&ctx->d_parts, kMaxParts * sizeof(PartDev)) == cudaSuccess &&
               cudaMalloc(&ctx->d_partials, kPartialSlots * sizeof(Partial)) == cudaSuccess &&
-              cudaMalloc(&ctx->d_status, 4 * sizeof(int32_t)) == cudaSuccess &&
+              cudaMalloc(&ctx->d_status, 8 * sizeof(int32_t)) == cudaSuccess &&
               cudaMalloc(&ctx->d_n_groups, sizeof(int32_t)) == cudaSuccess;
     if (ok) {
         cudaMemset(ctx->d_parts, 0, kMaxParts * sizeof(PartDev));
-        cudaMemset(ctx->d_status, 0, 4 * sizeof(int32_t));
+        cudaMemset(ctx->d_status, 0, 8 * sizeof(int32_t));
         cudaMemset(ctx->d_n_groups, 0, sizeof(int32_t));
         ok = cfgzip_reserve_rows(ctx, kDefaultRows) == CFGZIP_OK;
     }
@@ -1294,7 +1299,7 @@ int cfgzip_expand_mask(cfgzip_ctx* ctx, cfgzip_part_id part0, const int32_t* row
     a.VW = ps.VW;
     a.partials = ctx->d_partials;
     a.tickets = ctx->d_tickets;
-    a.status = ctx->d_status;
+    a.status = status_of(ctx);
     a.scale = kLog2e;
     a.inv_t = 1.f;
     if (mode == CFGZIP_SPARSE) {
