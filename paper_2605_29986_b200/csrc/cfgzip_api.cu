@@ -949,6 +949,30 @@ struct HostStep {
 };
 constexpr int kHostChunks = 8;  // at most, of at least eight rows
 
+// f(first, n) for every run of rows first .. first + n - 1 in [begin, end) whose partition is loaded and has V tokens: the others
+// are skipped, and what the caller holds for them stays as it is.
+template <typename F>
+void for_row_runs(const cfgzip_ctx* ctx, const int32_t* row_part, int32_t V, int32_t begin, int32_t end, F&& f) {
+    auto known = [&](int32_t b) {
+        const int32_t id = row_part[b];
+        return id >= 0 && size_t(id) < ctx->parts.size() && ctx->parts[size_t(id)].live && ctx->parts[size_t(id)].V == V;
+    };
+    if (!row_part) return f(begin, end - begin);
+    for (int32_t b = begin; b < end;) {
+        int32_t e = b;
+        while (e < end && known(e)) ++e;
+        if (e > b) f(b, e - b);
+        b = e + 1;
+    }
+}
+// The rows of a host array that a call has results for, from a staging copy of it.
+void copy_results(const cfgzip_ctx* ctx, const int32_t* row_part, int32_t V, int32_t B, void* to, const void* from) {
+    if (!to) return;
+    for_row_runs(ctx, row_part, V, 0, B, [&](int32_t first, int32_t n) {
+        std::memcpy(static_cast<char*>(to) + size_t(first) * 4, static_cast<const char*>(from) + size_t(first) * 4, size_t(n) * 4);
+    });
+}
+
 int host_step_pinned(cfgzip_ctx* ctx, const HostStep& h) {
     const size_t es = h.dtype == CFGZIP_BF16 ? 2 : 4, row_bytes = size_t(h.V) * es;
     const int32_t rows = h.masked_logits ? std::max(8, (ceil_div(h.B, kHostChunks) + 7) & ~7) : h.B;
@@ -958,6 +982,15 @@ int host_step_pinned(cfgzip_ctx* ctx, const HostStep& h) {
     const int32_t* d_rp = h.row_part_host ? h.d_rp : nullptr;
     char* d_logits = static_cast<char*>(ctx->st_logits);
     auto ok = [](cudaError_t e) { return e == cudaSuccess; };
+    auto back = [&](void* to, const void* from, size_t bytes_per_row, int32_t first, int32_t n) {  // rows first .. first + n - 1
+        bool good = true;
+        for_row_runs(ctx, h.row_part_host, h.V, first, first + n, [&](int32_t b, int32_t k) {
+            const size_t at = size_t(b) * bytes_per_row;
+            good = good && ok(cudaMemcpyAsync(static_cast<char*>(to) + at, static_cast<const char*>(from) + at, size_t(k) * bytes_per_row,
+                                              cudaMemcpyDeviceToHost, out));
+        });
+        return good;
+    };
     auto after = [&](cudaStream_t waits, cudaEvent_t e, cudaStream_t of) {  // what follows on `waits` comes after what is on `of`
         return ok(cudaEventRecord(e, of)) && ok(cudaStreamWaitEvent(waits, e, 0));
     };
@@ -980,7 +1013,7 @@ int host_step_pinned(cfgzip_ctx* ctx, const HostStep& h) {
         rc = cfgzip_expand_mask(ctx, h.part0, d_rp, ctx->st_cm, h.class_stride_words, ctx->st_vm, h.VW, h.B, CFGZIP_DENSE, h.stream);
         ctx->uncounted = false;
         good = rc == CFGZIP_OK && after(out, ctx->st_expanded, h.stream) &&
-               ok(cudaMemcpyAsync(h.vocab_mask_host, ctx->st_vm, size_t(h.B) * size_t(h.VW) * 4, cudaMemcpyDeviceToHost, out));
+               back(h.vocab_mask_host, ctx->st_vm, size_t(h.VW) * 4, 0, h.B);
     }
     if (mode == CFGZIP_AUTO) {  // (the copies are under way)
         const int chosen = cfgzip_choose_mode(ctx, h.part0, h.row_part_host, h.class_mask_host, h.class_stride_words, h.B, h.dtype);
@@ -995,9 +1028,7 @@ int host_step_pinned(cfgzip_ctx* ctx, const HostStep& h) {
                                              h.rep + first, h.logp + first, h.lse + first, nullptr, mode, h.stream);
         good = rc == CFGZIP_OK;
         if (good && h.masked_logits)
-            good = after(out, ctx->st_chunk_done[size_t(c)], h.stream) &&
-                   ok(cudaMemcpyAsync(static_cast<char*>(h.masked_logits) + size_t(first) * row_bytes,
-                                      d_logits + size_t(first) * row_bytes, size_t(n) * row_bytes, cudaMemcpyDeviceToHost, out));
+            good = after(out, ctx->st_chunk_done[size_t(c)], h.stream) && back(h.masked_logits, d_logits, row_bytes, first, n);
     }
     // Nothing of this call is in flight when it returns, whatever went wrong.
     for (cudaStream_t s : {out, in, h.stream}) good = ok(cudaStreamSynchronize(s)) && good;
@@ -1647,10 +1678,10 @@ int cfgzip_decode_step_host(cfgzip_ctx* ctx, cfgzip_part_id part0, const int32_t
                                             ps.VW, masked_logits, vocab_mask_host, mode, st, d_rp, r, r + step,
                                             reinterpret_cast<float*>(r + 2 * step), reinterpret_cast<float*>(r + 3 * step)});
         if (rc != CFGZIP_OK) return rc;
-        if (argmax) std::memcpy(argmax, r, size_t(B) * 4);
-        if (rep) std::memcpy(rep, r + step, size_t(B) * 4);
-        if (lse) std::memcpy(lse, r + 2 * step, size_t(B) * 4);
-        if (logp_argmax) std::memcpy(logp_argmax, r + 3 * step, size_t(B) * 4);
+        copy_results(ctx, row_part_host, ps.V, B, argmax, r);
+        copy_results(ctx, row_part_host, ps.V, B, rep, r + step);
+        copy_results(ctx, row_part_host, ps.V, B, lse, r + 2 * step);
+        copy_results(ctx, row_part_host, ps.V, B, logp_argmax, r + 3 * step);
         return CFGZIP_OK;
     }
     bool ok = cudaMemcpyAsync(ctx->st_cm, class_mask_host, cm_bytes, cudaMemcpyHostToDevice, st) == cudaSuccess &&
@@ -1669,22 +1700,27 @@ int cfgzip_decode_step_host(cfgzip_ctx* ctx, cfgzip_part_id part0, const int32_t
                                          ctx->st_logits, dtype, ps.V, B, vocab_mask_host ? ctx->st_vm : nullptr, ps.VW,
                                          d_am, d_rep, d_lpa, d_lse, nullptr, mode, stream);
     if (rc != CFGZIP_OK) return rc;
-    auto back = [&](void* dst, const void* src, size_t n) {
-        if (dst && ok) ok = cudaMemcpyAsync(dst, src, n, cudaMemcpyDeviceToHost, st) == cudaSuccess;
+    auto back = [&](void* dst, const void* src, size_t bytes_per_row) {
+        if (!dst) return;
+        for_row_runs(ctx, row_part_host, ps.V, 0, B, [&](int32_t b, int32_t k) {
+            const size_t at = size_t(b) * bytes_per_row;
+            ok = ok && cudaMemcpyAsync(static_cast<char*>(dst) + at, static_cast<const char*>(src) + at, size_t(k) * bytes_per_row,
+                                       cudaMemcpyDeviceToHost, st) == cudaSuccess;
+        });
     };
-    back(masked_logits, ctx->st_logits, logit_bytes);
-    back(vocab_mask_host, ctx->st_vm, vm_bytes);
+    back(masked_logits, ctx->st_logits, size_t(ps.V) * es);
+    back(vocab_mask_host, ctx->st_vm, size_t(ps.VW) * 4);
     // the four small result arrays sit side by side on the device: one copy into a pinned mirror, handed out
     // after the stream has drained (four separate small copies cost more than the kernels of a short step)
     const bool one_copy = ctx->st_small_host != nullptr && (argmax || rep || lse || logp_argmax);
     const size_t span = (size_t(ctx->st_rows) * 3 + size_t(B)) * 4;  // argmax .. logp_argmax, st_rows apart
     if (one_copy) {
-        back(ctx->st_small_host, d_am, span);
+        ok = ok && cudaMemcpyAsync(ctx->st_small_host, d_am, span, cudaMemcpyDeviceToHost, st) == cudaSuccess;
     } else {
-        back(argmax, d_am, size_t(B) * 4);
-        back(rep, d_rep, size_t(B) * 4);
-        back(lse, d_lse, size_t(B) * 4);
-        back(logp_argmax, d_lpa, size_t(B) * 4);
+        back(argmax, d_am, 4);
+        back(rep, d_rep, 4);
+        back(lse, d_lse, 4);
+        back(logp_argmax, d_lpa, 4);
     }
     if (!ok || cudaStreamSynchronize(st) != cudaSuccess) {
         cudaGetLastError();
@@ -1692,11 +1728,11 @@ int cfgzip_decode_step_host(cfgzip_ctx* ctx, cfgzip_part_id part0, const int32_t
     }
     if (one_copy) {
         const int32_t* h = ctx->st_small_host;
-        const size_t n = size_t(B) * 4, step = size_t(ctx->st_rows);
-        if (argmax) std::memcpy(argmax, h, n);
-        if (rep) std::memcpy(rep, h + step, n);
-        if (lse) std::memcpy(lse, h + 2 * step, n);
-        if (logp_argmax) std::memcpy(logp_argmax, h + 3 * step, n);
+        const size_t step = size_t(ctx->st_rows);
+        copy_results(ctx, row_part_host, ps.V, B, argmax, h);
+        copy_results(ctx, row_part_host, ps.V, B, rep, h + step);
+        copy_results(ctx, row_part_host, ps.V, B, lse, h + 2 * step);
+        copy_results(ctx, row_part_host, ps.V, B, logp_argmax, h + 3 * step);
     }
     return CFGZIP_OK;
 }

@@ -36,3 +36,28 @@ def test_rows_without_a_partition_are_counted_once(V, B, dtype, pinned):
         cz.cfgzip_decode_step_host(ctx.h, ctx.ids[0], row_part, pin(cm, pinned), cm.shape[1], pin(z, pinned), dtype_code(z), B, None, vm, am, rep,
                                    lpa, lse, cz.DENSE)
         assert cz.cfgzip_poll_status(ctx.h) == (0, 0, len(row_part[1::4]))
+
+
+@pytest.mark.parametrize("want_masked", [False, True])
+@pytest.mark.parametrize("pinned", [False, True])
+@pytest.mark.parametrize("V,B,dtype", [(3000, 5, "f32"), (9001, 70, "bf16")])
+def test_rows_without_a_partition_are_left_alone(V, B, dtype, pinned, want_masked):
+    # a first call with every row leaves its results in the context's staging memory: none of them may come out of the second
+    ps = [synth.zipf_partition(V, 100, seed=90 + i) for i in range(2)]
+    cm = synth.class_mask_bernoulli(100, B, 0.3, rng.stream_key(rng.SEED_BASE, 922, V))
+    z = synth.logits_normal(B, V, 2.0, dtype, (923, V))
+    row_part = (np.arange(B) % 2).astype(np.int32)
+    with Ctx(ps) as ctx:
+        def call(parts):
+            masked, vm, am, rep, lse, lpa = buffers(B, V, z, pinned)
+            cz.cfgzip_decode_step_host(ctx.h, ctx.ids[0], parts, pin(cm, pinned), cm.shape[1], pin(z, pinned), dtype_code(z), B,
+                                       masked if want_masked else None, vm, am, rep, lpa, lse, cz.DENSE)
+            return [t.numpy().copy() for t in (masked, vm, am, rep, lse, lpa)]
+
+        want, untouched = call(row_part), [t.numpy() for t in buffers(B, V, z, False)]
+        some = row_part.copy()
+        some[[0, 2, B - 1]] = (9, -1, 2)
+        left = np.isin(np.arange(B), [0, 2, B - 1])
+        for got, full, before in zip(call(some), want, untouched):
+            assert np.array_equal(got[left], before[left])
+            assert np.array_equal(got[~left], full[~left]) or np.abs(got[~left] - full[~left]).max() <= 1e-5  # (other row groups: other sums)
