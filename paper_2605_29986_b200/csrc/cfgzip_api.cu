@@ -912,12 +912,14 @@ bool is_pinned(const void* p) {
     return at.type == cudaMemoryTypeHost;
 }
 
-// Streams and events of the host-buffer step, made on its first use with pinned buffers.
-bool host_streams(cfgzip_ctx* ctx, size_t chunks) {
+// Streams and events of the host-buffer step with pinned buffers, made when they are first needed: a stream for what goes back
+// beside the copies in, and another one for these where row chunks come in while the steps of earlier ones run. (The first call of a
+// context, 32 rows of 128256 bf16 logits: 0.80 ms with both and all events, now 0.68, with the vocab masks 0.73.)
+bool host_streams(cfgzip_ctx* ctx, bool back, size_t chunks) {
     auto event = [](cudaEvent_t* e) { return *e || cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess; };
     auto stream = [](cudaStream_t* s) { return *s || cudaStreamCreateWithFlags(s, cudaStreamNonBlocking) == cudaSuccess; };
-    bool ok = stream(&ctx->st_in) && stream(&ctx->st_out) && event(&ctx->st_ready) && event(&ctx->st_masks) &&
-              event(&ctx->st_expanded);
+    bool ok = !back || (stream(&ctx->st_out) && event(&ctx->st_masks) && event(&ctx->st_expanded));
+    if (chunks) ok = ok && stream(&ctx->st_in) && event(&ctx->st_ready) && event(&ctx->st_masks);
     for (auto* list : {&ctx->st_chunk_in, &ctx->st_chunk_done})
         while (ok && list->size() < chunks) {
             cudaEvent_t e = nullptr;
@@ -930,8 +932,9 @@ bool host_streams(cfgzip_ctx* ctx, size_t chunks) {
 // The host-buffer step with pinned logits: the class masks go up first, so that the vocabulary masks are expanded and on their
 // way back while the logits are still coming; the results are written to pinned memory by the kernels. Masked logits, where
 // they are asked for, travel back in row chunks while later rows come in (the bus is full duplex). What is left behind the
-// logits' copy is one step: 32 rows of 128256 bf16 logits 202 -> 189 us, with
-// the masked logits 347 -> 287; the copy in alone, issued and waited for, takes 159.
+// logits' copy is one step: 32 rows of 128256 bf16 logits 194 -> 177 us, with
+// the masked logits 347 -> 287; the copy in alone, issued and waited for, takes 159. Without masked logits the copies in are on the
+// caller's stream, in front of the step that waits for them (182 -> 177 us against a stream of their own).
 struct HostStep {
     cfgzip_part_id part0;
     const int32_t* row_part_host;
@@ -977,8 +980,9 @@ int host_step_pinned(cfgzip_ctx* ctx, const HostStep& h) {
     const size_t es = h.dtype == CFGZIP_BF16 ? 2 : 4, row_bytes = size_t(h.V) * es;
     const int32_t rows = h.masked_logits ? std::max(8, (ceil_div(h.B, kHostChunks) + 7) & ~7) : h.B;
     const int chunks = ceil_div(h.B, rows);
-    if (!host_streams(ctx, size_t(chunks))) return CFGZIP_E_CUDA;
-    const cudaStream_t in = ctx->st_in, out = ctx->st_out;
+    const bool goes_back = h.masked_logits || h.vocab_mask_host;
+    if (!host_streams(ctx, goes_back, h.masked_logits ? size_t(chunks) : 0)) return CFGZIP_E_CUDA;
+    const cudaStream_t in = h.masked_logits ? ctx->st_in : h.stream, out = goes_back ? ctx->st_out : h.stream;
     const int32_t* d_rp = h.row_part_host ? h.d_rp : nullptr;
     char* d_logits = static_cast<char*>(ctx->st_logits);
     auto ok = [](cudaError_t e) { return e == cudaSuccess; };
@@ -992,7 +996,7 @@ int host_step_pinned(cfgzip_ctx* ctx, const HostStep& h) {
         return good;
     };
     auto after = [&](cudaStream_t waits, cudaEvent_t e, cudaStream_t of) {  // what follows on `waits` comes after what is on `of`
-        return ok(cudaEventRecord(e, of)) && ok(cudaStreamWaitEvent(waits, e, 0));
+        return waits == of || (ok(cudaEventRecord(e, of)) && ok(cudaStreamWaitEvent(waits, e, 0)));
     };
     // (class masks in front of the logits on one stream: two streams of copies in were no faster, and slower for small batches)
     bool good = after(in, ctx->st_ready, h.stream) &&
@@ -1000,19 +1004,20 @@ int host_step_pinned(cfgzip_ctx* ctx, const HostStep& h) {
                                    cudaMemcpyHostToDevice, in));
     if (good && h.row_part_host)
         good = ok(cudaMemcpyAsync(h.d_rp, h.row_part_host, size_t(h.B) * 4, cudaMemcpyHostToDevice, in));
-    good = good && after(h.stream, ctx->st_masks, in);
+    if (good && h.vocab_mask_host) good = ok(cudaEventRecord(ctx->st_masks, in)) && ok(cudaStreamWaitEvent(out, ctx->st_masks, 0));
     for (int c = 0; c < chunks && good; ++c) {
         const size_t first = size_t(c) * rows, n = std::min<size_t>(size_t(rows), size_t(h.B) - first);
         good = ok(cudaMemcpyAsync(d_logits + first * row_bytes, static_cast<const char*>(h.logits_host) + first * row_bytes,
                                   n * row_bytes, cudaMemcpyHostToDevice, in)) &&
-               ok(cudaEventRecord(ctx->st_chunk_in[size_t(c)], in));
+               (in == h.stream || ok(cudaEventRecord(ctx->st_chunk_in[size_t(c)], in)));
     }
     int rc = CFGZIP_OK, mode = h.mode;
     if (good && h.vocab_mask_host) {
         ctx->uncounted = true;  // (the step below counts the rows without a partition)
-        rc = cfgzip_expand_mask(ctx, h.part0, d_rp, ctx->st_cm, h.class_stride_words, ctx->st_vm, h.VW, h.B, CFGZIP_DENSE, h.stream);
+        rc = cfgzip_expand_mask(ctx, h.part0, d_rp, ctx->st_cm, h.class_stride_words, ctx->st_vm, h.VW, h.B, CFGZIP_DENSE, out);
         ctx->uncounted = false;
-        good = rc == CFGZIP_OK && after(out, ctx->st_expanded, h.stream) &&
+        // (the step shares the row plan's buffers with the expansion)
+        good = rc == CFGZIP_OK && (!d_rp || after(h.stream, ctx->st_expanded, out)) &&
                back(h.vocab_mask_host, ctx->st_vm, size_t(h.VW) * 4, 0, h.B);
     }
     if (mode == CFGZIP_AUTO) {  // (the copies are under way)
@@ -1021,7 +1026,7 @@ int host_step_pinned(cfgzip_ctx* ctx, const HostStep& h) {
     }
     for (int c = 0; c < chunks && good; ++c) {
         const int32_t first = c * rows, n = std::min(rows, h.B - first);
-        if (!(good = ok(cudaStreamWaitEvent(h.stream, ctx->st_chunk_in[size_t(c)], 0)))) break;
+        if (in != h.stream && !(good = ok(cudaStreamWaitEvent(h.stream, ctx->st_chunk_in[size_t(c)], 0)))) break;
         rc = cfgzip_masked_logsoftmax_argmax(ctx, h.part0, d_rp ? d_rp + first : nullptr,
                                              ctx->st_cm + int64_t(first) * h.class_stride_words, h.class_stride_words,
                                              d_logits + size_t(first) * row_bytes, h.dtype, h.V, n, nullptr, 0, h.argmax + first,
@@ -1031,7 +1036,9 @@ int host_step_pinned(cfgzip_ctx* ctx, const HostStep& h) {
             good = after(out, ctx->st_chunk_done[size_t(c)], h.stream) && back(h.masked_logits, d_logits, row_bytes, first, n);
     }
     // Nothing of this call is in flight when it returns, whatever went wrong.
-    for (cudaStream_t s : {out, in, h.stream}) good = ok(cudaStreamSynchronize(s)) && good;
+    for (cudaStream_t s : {out, in})
+        if (s != h.stream) good = ok(cudaStreamSynchronize(s)) && good;
+    good = ok(cudaStreamSynchronize(h.stream)) && good;
     if (good) return CFGZIP_OK;
     cudaGetLastError();
     return rc != CFGZIP_OK ? rc : CFGZIP_E_CUDA;
