@@ -1374,7 +1374,7 @@ int cfgzip_mask_logits(cfgzip_ctx* ctx, void* logits, int dtype, int64_t row_str
     // resident set of blocks with twice as long pieces, rows of mixed density 55 -> 46)
     const unsigned grid = unsigned(std::min<int64_t>(int64_t(B) * chunks, int64_t(ctx->sm_count) * 64));
     return launch(ctx, dtype == CFGZIP_BF16 ? k_mask_logits<kBF16> : k_mask_logits<kF32>, dim3(grid), dim3(256), 0, st, logits,
-                  row_stride_elems, int(B), int(V), vocab_mask, vocab_stride_words, chunks);
+                  row_stride_elems, int(B), int(V), vocab_mask, vocab_stride_words, chunks, int(grid) / chunks, int(grid) % chunks);
 }
 
 int cfgzip_masked_logsoftmax_argmax(cfgzip_ctx* ctx, cfgzip_part_id part0, const int32_t* row_part,

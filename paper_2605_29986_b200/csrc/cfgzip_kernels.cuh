@@ -2300,7 +2300,7 @@ constexpr int kMaskUnroll = 2, kMaskChunk = 256 * kMaskUnroll;  // vectors per b
 
 template <int DT>
 __global__ void __launch_bounds__(256) k_mask_logits(void* logits, int64_t row_stride, int B, int V, const uint32_t* vocab_mask,
-                                                     int64_t vm_stride, int chunks) {
+                                                     int64_t vm_stride, int chunks, int row_step, int ch_step) {
     pdl_prologue();
     constexpr int ES = DT == kBF16 ? 2 : 4;
     const int tid = threadIdx.x;
@@ -2331,7 +2331,7 @@ __global__ void __launch_bounds__(256) k_mask_logits(void* logits, int64_t row_s
         }
         return p;
     };
-    PieceWalk at(blockIdx.x, gridDim.x, chunks);
+    PieceWalk at(blockIdx.x, chunks, row_step, ch_step);
     if (at.row >= B) return;
     Piece p = fetch(at);
     for (;;) {

@@ -16,10 +16,10 @@ namespace cfgzip {
 struct PieceWalk {
     int64_t row;
     int ch;
-    int row_step, ch_step, chunks;
-    CFGZIP_HD PieceWalk(unsigned block, unsigned blocks, int chunks_)
-        : row(block / unsigned(chunks_)), ch(int(block % unsigned(chunks_))), row_step(int(blocks / unsigned(chunks_))),
-          ch_step(int(blocks % unsigned(chunks_))), chunks(chunks_) {}
+    const int row_step, ch_step, chunks;
+    // row_step, ch_step: the grid's blocks divided by `chunks`, and what is left over
+    CFGZIP_HD PieceWalk(unsigned block, int chunks_, int row_step_, int ch_step_)
+        : row(block / unsigned(chunks_)), ch(int(block - unsigned(row) * unsigned(chunks_))), row_step(row_step_), ch_step(ch_step_), chunks(chunks_) {}
     CFGZIP_HD void next() {
         row += row_step;
         ch += ch_step;

@@ -30,7 +30,7 @@ int main() {
             for (unsigned blocks : {1u, 2u, 5u, 63u, 64u, 700u}) {
                 std::vector<int> seen(size_t(B) * chunks, 0);
                 for (unsigned b = 0; b < blocks; ++b)
-                    for (PieceWalk at(b, blocks, chunks); at.row < B; at.next()) {
+                    for (PieceWalk at(b, chunks, int(blocks) / chunks, int(blocks) % chunks); at.row < B; at.next()) {
                         if (at.row < 0 || at.ch < 0 || at.ch >= chunks) { printf("B %d chunks %d: row %lld piece %d\n", B, chunks, (long long)at.row, at.ch); return 1; }
                         ++seen[size_t(at.row) * chunks + at.ch];
                     }
@@ -50,7 +50,7 @@ int main() {
     for (auto& s : shapes)
         for (unsigned b : {0u, 1u, blocks - 1}) {
             long long last = -1, n = 0;
-            for (PieceWalk at(b, blocks, s[1]); at.row < s[0]; at.next(), ++n) {
+            for (PieceWalk at(b, s[1], int(blocks) / s[1], int(blocks) % s[1]); at.row < s[0]; at.next(), ++n) {
                 const long long piece = (long long)at.row * s[1] + at.ch;
                 if (at.row < 0 || at.ch < 0 || at.ch >= s[1] || piece != (long long)b + n * blocks || piece <= last) { printf("piece %lld after %lld\n", piece, last); return 1; }
                 last = piece;
