@@ -13,7 +13,10 @@ from typing import Optional, Tuple
 from . import _build
 
 _build.build()
-from . import _calls  # noqa: E402
+try:
+    from . import _calls  # noqa: E402
+except ImportError:  # it could not be built here: the same functions through ctypes, a few microseconds slower
+    _calls = None
 
 F32, BF16 = 0, 1
 AUTO, DENSE, SPARSE = 0, 1, 2
@@ -77,7 +80,8 @@ def load_library():
             fn = getattr(lib, name)
             fn.restype = res
             fn.argtypes = args
-        _calls.bind({name: ctypes.cast(getattr(lib, name), _vp).value for name in _SIGNATURES}, _raise)
+        if _calls is not None:
+            _calls.bind({name: ctypes.cast(getattr(lib, name), _vp).value for name in _SIGNATURES}, _raise)
         _lib = lib
     return _lib
 
@@ -155,17 +159,53 @@ def cfgzip_free_partition(ctx: int, part: int) -> None:
     _check(load_library().cfgzip_free_partition(ctx, part), "cfgzip_free_partition")
 
 
-# The calls a program makes once per decode step are native functions with the arguments of the header, by position or by
-# name (csrc/calls.c); result buffers that are not wanted, the mode (AUTO) and the stream (legacy default) may be left out.
-cfgzip_expand_mask = _calls.cfgzip_expand_mask
-cfgzip_mask_logits = _calls.cfgzip_mask_logits
-cfgzip_masked_logsoftmax_argmax = _calls.cfgzip_masked_logsoftmax_argmax
-cfgzip_masked_sample = _calls.cfgzip_masked_sample
-cfgzip_masked_sample_filtered = _calls.cfgzip_masked_sample_filtered
-cfgzip_multi_mask_logsoftmax_argmax = _calls.cfgzip_multi_mask_logsoftmax_argmax
-cfgzip_plan_rows = _calls.cfgzip_plan_rows
-cfgzip_map_tokens = _calls.cfgzip_map_tokens
-cfgzip_decode_step_host = _calls.cfgzip_decode_step_host
+# The calls a program makes once per decode step take the arguments of the header, by position or by name; result buffers that
+# are not wanted, the mode (AUTO) and the stream (legacy default) may be left out. They are native functions (csrc/calls.c) or,
+# where those could not be built, made here from the same table: what every argument is ('p' address, 's' stream, 'i' integer,
+# 'f' number), how many have to be given, and their names.
+_STEP_ARGS = "ctx part0 row_part class_mask class_stride_words logits dtype row_stride_elems B vocab_mask vocab_stride_words "
+_STEP_CALLS = {
+    "cfgzip_expand_mask": ("pippipiiis", 8, "ctx part0 row_part class_mask class_stride_words vocab_mask vocab_stride_words B mode "
+                           "stream"),
+    "cfgzip_mask_logits": ("ppiiiipis", 8, "ctx logits dtype row_stride_elems B V vocab_mask vocab_stride_words stream"),
+    "cfgzip_masked_logsoftmax_argmax": ("pippipiiipipppppis", 12, _STEP_ARGS + "argmax rep logp_argmax lse logp_full mode stream"),
+    "cfgzip_masked_sample": ("pippipiiipipfppppis", 14, _STEP_ARGS + "u inv_temperature token rep logp_token lse mode stream"),
+    "cfgzip_masked_sample_filtered": ("pippipiiipipfifppppis", 16, _STEP_ARGS + "u inv_temperature top_k top_p token rep "
+                                      "logp_token lse mode stream"),
+    "cfgzip_multi_mask_logsoftmax_argmax": ("pipiipiiipipppps", 12, "ctx part0 class_masks class_stride_words masks_per_row logits "
+                                            "dtype row_stride_elems B vocab_masks vocab_stride_words argmax rep logp_argmax lse "
+                                            "stream"),
+    "cfgzip_plan_rows": ("pipis", 4, "ctx part0 row_part B stream"),
+    "cfgzip_map_tokens": ("pipppis", 6, "ctx part0 row_part tokens reps B stream"),
+    "cfgzip_decode_step_host": ("pippipiippppppis", 8, "ctx part0 row_part_host class_mask_host class_stride_words logits_host dtype B "
+                                "masked_logits vocab_mask_host argmax rep logp_argmax lse mode stream"),
+}
+
+
+def _through_ctypes(name: str):
+    kinds, required, names = _STEP_CALLS[name][0], _STEP_CALLS[name][1], _STEP_CALLS[name][2].split()
+    convert = [{"p": _ptr, "s": _stream}.get(k) for k in kinds]
+
+    def call(*args, **given):
+        if len(args) > len(names):
+            raise TypeError("%s() takes %d arguments (%d given)" % (name, len(names), len(args)))
+        values = dict(zip(names, args))
+        for key, value in given.items():
+            if key not in names or key in values:
+                raise TypeError("%s() got an unexpected or repeated argument '%s'" % (name, key))
+            values[key] = value
+        for key in names[:required]:
+            if key not in values:
+                raise TypeError("%s() is missing the argument '%s'" % (name, key))
+        row = [values.get(key, None if c else 0) for key, c in zip(names, convert)]
+        _check(getattr(load_library(), name)(*(c(v) if c else v for c, v in zip(convert, row))), name)
+
+    call.__name__ = call.__qualname__ = name
+    return call
+
+
+for _name in _STEP_CALLS:
+    globals()[_name] = getattr(_calls, _name) if _calls is not None else _through_ctypes(_name)
 
 ROWS_AS_PLANNED = 1  # pass as row_part after cfgzip_plan_rows: the kept grouping of that call is reused
 
@@ -261,3 +301,6 @@ def cfgzip_plan_query(sm_count: int, smem_optin: int, V: int, K: int, B: int, dt
     _check(load_library().cfgzip_plan_query(sm_count, smem_optin, V, K, B, dtype, n_partitions,
                                             1 if aligned_class_masks else 0, out), "cfgzip_plan_query")
     return dict(zip(PLAN_FIELDS, list(out)))
+
+
+load_library()  # (the native functions have their addresses from it)
