@@ -90,11 +90,13 @@ void number_bytes(cfgzip_grammar& g) {
     }
 }
 
+constexpr size_t padded(size_t words) { return (words + 15) & ~size_t(15); }  // to whole lines of 64 bytes
+
 // Signature rows one worker has already built in this call, by the token's string of byte classes: most tokens of a vocabulary
 // (words, runs of digits) read the same to the grammar as another token. Only the words a row uses are kept, as rows may be wide
 // and mostly zeros. Bounded; what does not fit is built anew. (128256 tokens on one core, ms without / with: a JSON grammar without
-// literals and escapes, 99 in 100 tokens known, rows of 64 words 15 / 6.0, of 256 words 21 / 10.5; with them, 6 in 10 known, 29 / 22.5
-// and 34 / 27. Whole rows kept, the wide ones took 42.)
+// literals and escapes, 99 in 100 tokens known, rows of 64 words 15 / 6.1, of 256 words 21 / 12; with them, 6 in 10 known, 29 / 23
+// and 34 / 29. Whole rows kept, the wide ones took 42.)
 class RowCache {
   public:
     struct Entry {
@@ -132,7 +134,7 @@ class RowCache {
         entries_.push_back(Entry{hash_, keys_.size(), rows_.size(), int32_t(token_.size()), words, used, fits});
         keys_.insert(keys_.end(), token_.begin(), token_.end());
         rows_.insert(rows_.end(), row, row + used);
-        rows_.resize((rows_.size() + 3) & ~size_t(3), 0);  // (rows are written four words at a time)
+        rows_.resize(padded(rows_.size()), 0);  // (every row starts a line, as the one before it does)
     }
 
   private:
@@ -256,11 +258,13 @@ constexpr int32_t kRunsPerThread = 8;
 
 // A finished row goes out with stores that pass the caches by, where the row's alignment allows it: rows left dirty in
 // the caches of a dozen cores make the copy to the GPU that usually follows two and a half times slower (33 MB: 1.5 ms
-// against 0.6). `used` words, zeros behind them; `from` has zeros up to the next multiple of four words.
+// against 0.6). `used` words, zeros behind them; `from` has zeros up to the next whole line of 16 words:
+// by lines the loops' lengths differ little from token to token.
 void write_row(int32_t* row, const int32_t* from, size_t used, size_t words) {
 #ifdef __SSE2__
     if (words % 4 == 0 && (reinterpret_cast<uintptr_t>(row) & 15u) == 0) {
         size_t i = 0;
+        used = std::min(padded(used), words);
         for (; i < used; i += 4)
             _mm_stream_si128(reinterpret_cast<__m128i*>(row + i), _mm_loadu_si128(reinterpret_cast<const __m128i*>(from + i)));
         for (; i < words; i += 4) _mm_stream_si128(reinterpret_cast<__m128i*>(row + i), _mm_setzero_si128());
@@ -346,7 +350,7 @@ int cfgzip_displacement_signatures(const cfgzip_grammar* g, const uint8_t* token
         try {
             Displacer d(*g, max_pairs);
             RowCache cache(*g, V);
-            std::vector<int32_t> built(size_t(row_words) + 3);
+            std::vector<int32_t> built(padded(size_t(row_words)));
             for (;;) {
                 const int32_t first = next.fetch_add(kTokenRun);
                 if (first >= V || first < 0) break;
@@ -378,7 +382,7 @@ int cfgzip_displacement_signatures(const cfgzip_grammar* g, const uint8_t* token
                         rc.store(CFGZIP_E_RANGE);
                     }
                     const int32_t used = int32_t(out - built.data());
-                    std::fill(out, out + (-used & 3), 0);
+                    std::fill(out, built.data() + padded(size_t(used)), 0);
                     write_row(row, built.data(), size_t(used), size_t(row_words));
                     cache.add(built.data(), used, d.overflow ? -1 : int32_t(n), fits);
                 }
