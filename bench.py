@@ -52,13 +52,13 @@ LOG_TOL = 1e-4                # absolute, fp32-accumulated log quantities agains
 # DRAM traffic of the dominant (streaming) kernel per launch = per step (dram__bytes_read.sum +
 # dram__bytes_write.sum from one ncu capture, see profiles/), keyed by workload; valid only for the kernel
 # sources whose digest is recorded with it. A workload without a capture of the current sources reports null.
-_CAPTURED = "02183c84a4d7b29e"
+_CAPTURED = "db89a8d6cf402e5f"
 NCU_TRAFFIC = {
-    "cfg2_B32_dense": {"digest": _CAPTURED, "bytes_per_launch": 14954837},      # 8.24 MB read + 6.71 MB written (L2 still filling)
-    "cfg2_B1024_dense": {"digest": _CAPTURED, "bytes_per_launch": 541736960},   # 263.2 MB read + 278.5 MB written
-    "cfg4_B256_dense": {"digest": _CAPTURED, "bytes_per_launch": 269750784},    # 132.4 MB read + 137.4 MB written
-    "cfg5_B1024_dense": {"digest": _CAPTURED, "bytes_per_launch": 1067131051},  # 526.5 MB read + 540.6 MB written
-    "cfg5_B1024_sparse": {"digest": _CAPTURED, "bytes_per_launch": 611983872},  # 65.1 MB read + 546.9 MB written
+    "cfg2_B32_dense": {"digest": _CAPTURED, "bytes_per_launch": 14793983}, # 8.2 MB read + 6.6 MB written (L2 still filling)
+    "cfg2_B1024_dense": {"digest": _CAPTURED, "bytes_per_launch": 541066922}, # 263.1 MB read + 278.0 MB written
+    "cfg4_B256_dense": {"digest": _CAPTURED, "bytes_per_launch": 269499050}, # 132.2 MB read + 137.3 MB written
+    "cfg5_B1024_dense": {"digest": _CAPTURED, "bytes_per_launch": 1066146389}, # 526.3 MB read + 539.9 MB written
+    "cfg5_B1024_sparse": {"digest": _CAPTURED, "bytes_per_launch": 565420799}, # k_step_few: 24.0 MB read + 541.5 MB written
 }
 
 

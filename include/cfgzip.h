@@ -267,8 +267,9 @@ int cfgzip_choose_mode(cfgzip_ctx* ctx, cfgzip_part_id part0, const int32_t* row
  * runs cfgzip_masked_logsoftmax_argmax, copies the requested results back and waits
  * for `stream`. Staging buffers grow on first use (that call allocates). With pinned buffers the vocab masks are
  * expanded and sent back while the logits still come in, the masked logits travel back in chunks of rows beside
- * the copy in (on two streams of the context, joined before the call returns), and the kernels write the per-row
- * results to the host's memory themselves. Pageable buffers take the same steps one after the other.
+ * the copy in (on one or two streams of the context, made when they are first needed and joined before the call
+ * returns), and the kernels write the per-row results to the host's memory themselves. Pageable buffers take the
+ * same steps one after the other. Rows whose partition is not loaded are left alone in all results.
  *   logits_host     : host [B, V] of `dtype`, dense rows; left unmodified
  *   masked_logits   : nullable host [B, V]; receives the masked logits
  *   vocab_mask_host : nullable host uint32 [B, VW]

@@ -423,7 +423,7 @@ DensePlan plan_pipe_opl(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixe
     d.threads = d.WT * WR * 32;
     // The groups of a mixed batch may hold 32 rows or one, and only the GPU knows how many there are: where there are blocks
     // enough it gives every group the same number if the groups are the fewest the batch can have (336 bf16 rows of 128256 in two
-    // partitions: 41.3 us; shares by size 44.1), else its share by size, one wave of blocks that all have about as much to do
+    // partitions: 41 us; shares by size 44), else its share by size, one wave of blocks that all have about as much to do
     // (256 rows in eight partitions, V = 256000: 63 us; the same number for every group, in two waves, 78).
     if (mixed && target >= 3 * d.n_groups_ub) {
         const int batches = ceil_div(B, kBatchRows), most = std::min(batches, kGroupRows / kBatchRows);

@@ -19,7 +19,7 @@ namespace cfgzip {
 //          that at least k tokens reach, and, the runs being many, not many more (k = 50: some 60 to 100 tokens). For top-p
 //          alone the bar is where the run maxima by themselves already weigh enough, or nearly (checked afterwards). One pass over the row collects the
 //          tokens at or above the bar, a thread each, and every thread sums over all of them.
-//   long   Otherwise (a flat distribution, a large k), with one filter: a pass that counts the tokens in 16384 steps of the
+//   long   Otherwise (a flat distribution, a large k), with one filter: a pass that counts the tokens in 8192 steps of the
 //          distance from the row maximum (one shared-memory addition a token; the weight of a step follows from its count to
 //          better than 0.1 %), which says about where the cut falls; and a pass that sums, exactly and chunk by chunk, what
 //          lies above a window of some 200 tokens around it and lists the tokens of the window. The exact sums then say whether
@@ -31,7 +31,21 @@ namespace cfgzip {
 // that is in the L2: loops stay rolled and steps that come up more than once are functions, which keeps the code a third of
 // what it was inlined and unrolled. Collecting every token that carries weight first took 78 us of the step for 64 rows of
 // 151936 bf16 logits at T = 0.7 (15000 such tokens a row), and some 30 passes over the row where they did not fit; this takes
-// 14 of a step of 26. With top-p alone the same rows take 69 us (561), 256 rows that allow nearly everything 186 (1445).
+// 13 of a step of 27 (clock stamps, us from the block's first step: states read 2.3, bar 3.6, pass over the row 8.5, all blocks of
+// the row there 9.6, sort 11, cut 12, draw 12.5). With top-p alone the same rows take 66 us (606), 256 rows that allow nearly
+// everything 174 (1366).
+// Where it is slower than collecting everything was: top-p alone on short rows of which every token that carries weight fitted
+// one list (up to some 12000): 128 bf16 rows of 20032 with 1 % allowed 24 -> 37 us, with 10 % 31 -> 50 (with 90 % 147 -> 47). One
+// row in a hundred that misses its guessed bar sets the time: count, window, list and the sort of some 500 tokens (10 us) one
+// after the other. A lower bar to begin with lost 20 % with 90 % allowed; a second, lower bar for such rows gained 10 to 20 %
+// in four of sixteen cases and lost as much in two.
+//
+// Thresholds (all ways are exact, what they choose is checked; they decide the time only): `0.04` and `0.6` of the guessed bar: with
+// 0.02 or 0.01 256 rows of 151936 take 223 and 229 us instead of 203, 277 rows of 28864 75 instead of 58; kFiltWindow 200 tokens around
+// the cut: 1 % of flat rows need a second window; kFiltWindowMost 800 tokens to a side: without it 277 rows of 28864 163 us instead of
+// 58; `0.4` of the list's length as the lower bound on allowed tokens that skips counting them, `0.9` of what top-p leaves out as
+// the weight that need not be listed, `0.25` of the list as the most tokens a guessed bar may be expected to pass, three tries, and
+// top_k up to an eighth of the list: set once and not varied since.
 // ---------------------------------------------------------------------------------------
 // Threads of a block: much of the work is the same for every warp (scans, set-up) and takes issue slots once per warp; 256
 // threads and two blocks per SM still keep 32 KB of loads in flight per SM and overlap one row's serial steps with another's.

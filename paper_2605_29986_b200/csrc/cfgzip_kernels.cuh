@@ -1425,11 +1425,13 @@ __global__ void __launch_bounds__(256) k_expand_dense(const __grid_constant__ St
 // bytes (8 f32 or 16 bf16 tokens) of 8 rows at a time; a vector without an allowed token is overwritten with -inf at once,
 // without being read, the others go into a queue of the warp. Whenever 32 have come together they are asked for, a lane each,
 // and the 32 asked for before are masked, written back and folded into the lane's states of the 8 rows (shared memory).
-// Bound: HBM. The -inf stream waits for no load; alone it runs at 5.9 TB/s, and the reads, scattered sectors between the
-// writes, cost a third on top (measured without them: 1024 rows of 128256 f32 logits 134 -> 100 us; more blocks per SM, longer
-// runs per row, asking for the sectors ahead of the stream: no gain). Building every row's mask from the class lists first,
-// a block per row, as the kernel below does, streams nothing meanwhile: 256 to 1024 bf16 rows take 10 to 40 % longer that way
-// (159 rows of 51648 over eight partitions 26.6 -> 17.1 us, 300 of 250000 92 -> 66, 128 of 128256 f32 30 -> 24).
+// Bound: HBM and the latency of the reads. The -inf stream waits for no load; alone it runs at 5.9 TB/s, and the reads, scattered
+// sectors between the writes, cost a third on top (measured without them: 1024 rows of 128256 f32 logits 134 -> 100 us; more blocks
+// per SM, longer runs per row, asking for the sectors ahead of the stream: no gain); with them DRAM is busy for 52 % of the time
+// and the L1 for 61, and a warp waits mostly for loads. Building every row's mask from the class lists first, a block per row, as
+// the kernel below does, streams nothing meanwhile: with few classes and long rows that takes 10 to 70 % longer (128 rows of 128256 in
+// 512 classes, bf16 26.9 against 17.3 us, f32 30 against 23; 300 bf16 rows of 256000 in two partitions 80 against 46), at 1024 f32 rows
+// the same (132). Where the table costs more than it saves the kernel below is taken (few_pays, where the launches are planned).
 // Vectors of 32 bytes because a sector whose halves are written at different times costs a read of DRAM.
 // ---------------------------------------------------------------------------------------
 constexpr int kFewThreads = 256, kFewWarps = kFewThreads / 32;
@@ -1601,8 +1603,8 @@ __global__ void __launch_bounds__(kFewThreads, 3) k_step_few(const __grid_consta
 }
 
 // ---------------------------------------------------------------------------------------
-// The same for a few rows (and for class ids beyond 16 bits): one row per block (S blocks per row). The row's vocab bitmask is built in
-// shared memory by scattering the member lists of the allowed classes; then the row is
+// The same for few or short rows, for many classes and for class ids beyond 16 bits: one row per block (S blocks per row).
+// The row's vocab bitmask is built in shared memory by scattering the member lists of the allowed classes; then the row is
 // streamed: octets with no allowed token are overwritten with -inf without being read.
 // FUSED = false stops after writing the vocab mask.
 // ---------------------------------------------------------------------------------------

@@ -10,8 +10,9 @@ namespace cfgzip {
 // row r / masks_per_row. A warp takes 32 octets of 8 virtual rows at a time. What depends on the logits alone is done once per
 // logits row: the octet is loaded and its eight exponentials are taken, and the lane writes down (largest logit, sum of
 // exponentials) of all 16 subsets of either half of the octet. A mask then costs two lookups with the two halves of its byte.
-// Bound: shared-memory bandwidth (8 KB of subsets written per octet and warp, 0.5 KB read per mask) beside instruction issue,
-// some 20 instructions per octet and mask. (Masking and exponentials anew for every mask, a class table per short block:
+// Bound: instruction latency and issue (the schedulers issue in 56 % of the cycles with some four warps each, the shared-memory
+// pipe is busy for 42 %, DRAM for 2; a warp waits mostly for its own last instruction and for shared memory): some 20 instructions
+// per octet and mask, 8 KB of subsets written per octet and warp, 0.5 KB read per mask. (Masking and exponentials anew for every mask, a class table per short block:
 // 8 rows x 16 masks of 128256 bf16 logits 24.3 us, now 14.5; 32 x 32 masks of 151936 f32 logits 134 us, now 65.)
 //
 // The exponentials of a lane share one reference per logits row, whatever a mask allows. It is set 64 powers of two below the
