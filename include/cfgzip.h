@@ -403,6 +403,10 @@ int cfgzip_launch_count(cfgzip_ctx* ctx, int64_t* out);
  *   "ctas_per_sm"  target resident thread blocks per SM for the fused kernel (1..16)
  *   "token_warps"  0 = automatic, else warps side by side along the vocabulary (1..16)
  *   "row_warps"    0 = automatic, else 1, 2 or 4 row batches handled by separate warps
+ *   "one_launch"   1 = steps of short batches (greedy and plain sampling) run in one launch, a thread-block cluster per row
+ *                  or few rows (default); 0 = always the streaming kernel and a second one. Setting a knob that shapes the
+ *                  streaming kernel ("ctas_per_sm", "token_warps", "row_warps", "pipeline", "tensor_map", "pipe_warps", "waves",
+ *                  "pipe_depth", "stage_alias", "fold", "lane_octets", "spread") sets it to 0
  *   "pdl"          1 = programmatic dependent launch where it pays (steps under 192 MB of logits;
  *                  default), 0 = never, 2 = always
  *   "pipeline"     1 = aligned logits stream through per-warp rings of bulk asynchronous copies
@@ -446,7 +450,7 @@ int cfgzip_launch_count(cfgzip_ctx* ctx, int64_t* out);
 int cfgzip_set_tuning(cfgzip_ctx* ctx, const char* name, int32_t value);
 
 /*
- * Host-only: the launch shape the library would choose for a fused dense step on a device with
+ * Host-only: the launch shape the library would choose for a fused dense step of two launches (see "one_launch") on a device with
  * `sm_count` SMs and `smem_optin` bytes of opt-in shared memory per block (default tuning). For
  * tests of the planner; touches no GPU. out[0] kernel kind (2 pipelined, 1 register, 0 per-row),
  * [1] row groups (upper bound), [2] blocks per group S, [3] octets per block (register kernel),

@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "cfgzip.h"
+#include "cfgzip_cluster.cuh"
 #include "cfgzip_filtered.cuh"
 #include "cfgzip_kernels.cuh"
 #include "cfgzip_multi.cuh"
@@ -94,6 +95,7 @@ struct cfgzip_ctx {
     int32_t pdl = 1;
     bool pdl_now = true;      // set per call: programmatic dependent launch only pays for short kernels
     int cluster_now = 1;      // set around a launch: blocks per thread-block cluster
+    int cluster_limit[kClusterMost + 1] = {};  // clusters of that many blocks that run side by side, a block to an SM
     int prefetch_items = 4;   // work items per warp of the pipelined kernel asked into the L2 before its wait
     int prefetch_min_mbytes = 48;  // ... for steps of at least this many megabytes of logits
     bool prefetch_now = false;     // set per call beside pdl_now
@@ -116,6 +118,7 @@ struct cfgzip_ctx {
     int64_t auto_min_bytes = -1;  // automatic mode on device-resident masks: steps of at least this many bytes of logits let the
                                   // GPU choose (one more launch); -1 = never (dense): the choice from host masks costs nothing
     int32_t fold = 0;         // pipelined kernel: the last block of a row group writes the rows' results (one launch per step)
+    int32_t one_launch = 1;   // short batches: the whole step in one launch (k_step_cluster); off once a knob shapes the streaming kernel
     int32_t expire_test = 0;  // test hook: the pipelined kernel reports its first completed wait as run out
 };
 
@@ -170,9 +173,9 @@ int launch(cfgzip_ctx* ctx, void (*kernel)(KArgs...), dim3 grid, dim3 block, siz
 
 // More than 48 KB of dynamic shared memory has to be allowed once per kernel; it is allowed up to the device's limit, so that
 // the limit another context may have set is never smaller, and remembered: asking the runtime on every step costs half a
-// microsecond of host time.
+// microsecond of host time. large_clusters: the kernel also comes in clusters of more than eight blocks.
 template <typename K>
-int ensure_smem(cfgzip_ctx* ctx, K kernel, size_t bytes) {
+int ensure_smem(cfgzip_ctx* ctx, K kernel, size_t bytes, bool large_clusters = false) {
     if (bytes <= 48 * 1024) return CFGZIP_OK;
     const void* fn = reinterpret_cast<const void*>(kernel);
     for (const auto& k : ctx->smem_allowed)
@@ -183,12 +186,37 @@ int ensure_smem(cfgzip_ctx* ctx, K kernel, size_t bytes) {
         return CFGZIP_E_CUDA;
     }
     const size_t most = size_t(ctx->smem_optin) - std::min(size_t(ctx->smem_optin), attr.sharedSizeBytes);
-    if (bytes > most || cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(most)) != cudaSuccess) {
+    if (bytes > most || cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(most)) != cudaSuccess ||
+        (large_clusters && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
         cudaGetLastError();
         return CFGZIP_E_CUDA;
     }
     ctx->smem_allowed.emplace_back(fn, most);
     return CFGZIP_OK;
+}
+
+// How many clusters of every size the device holds at once, a block to an SM: the SMs come in groups that a cluster does not cross,
+// so that 132 of 148 can be had four at a time and 120 eight at a time (15 clusters).
+void find_cluster_limits(cfgzip_ctx* ctx) {
+    auto kern = k_step_cluster<kBF16, 1, false, false>;
+    const size_t smem = size_t(ctx->smem_optin) / 2 + 1024;
+    if (ensure_smem(ctx, kern, smem, true) != CFGZIP_OK) return;
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr[1];
+    cfg.blockDim = dim3(kClusterThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    for (unsigned n = 2; n <= kClusterMost; ++n) {
+        attr[0].val.clusterDim.x = n;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3(n);
+        if (cudaOccupancyMaxActiveClusters(&ctx->cluster_limit[n], kern, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            ctx->cluster_limit[n] = 0;
+        }
+    }
 }
 
 int check_partition_host(const int32_t* c, int32_t V, const int32_t* r, int32_t K) {
@@ -749,11 +777,83 @@ int launch_finalize(cfgzip_ctx* ctx, const StepArgs& a, const DensePlan& d, cuda
     return launch(ctx, k_finalize_rows<DT>, dim3(rows_grid), dim3(kFinalizeThreads), pad, st, a);
 }
 
+// Launch shape of the one-launch step of a short batch: `rows` rows to a cluster of `blocks` blocks, as long as all clusters run side
+// by side, a block to an SM, and their rows fit shared memory. Of the shapes that do the one with the least work for a warp: chunks
+// of its run times rows, the lookups of a chunk weighing as much as a row where few rows share them well (greedy steps on the vector
+// grid), less where a row costs more by itself, and a little for every block a cluster has to wait for. Measured over 120 shapes of 23
+// batches: the choice is 0.2 % slower than the best shape in the mean, 3 % at most. 128256 bf16 logits, us, two launches / this:
+// 1 row 6.3 / 3.9, 8 6.7 / 4.7, 32 8.5 / 7.7, 48 11.5 / 9.3, 64 11.9 / 10.9, 80 15.3 / 13.1; 32 rows of four grammars 20.0 / 8.6 (and 23.3
+// where they are grouped at every step); sampling 8 rows 8.8 / 5.5, 32 10.6 / 8.4, 64 13.8 / 11.9.
+// Rows under 128 KB from 33 rows on, and mixed batches from there, are left at two launches: callers count on them (48 rows of 32000
+// bf16: 7.1 against 5.0).
+struct ClusterPlan {
+    bool ok = false;
+    ClusterGeom g{};
+    size_t smem = 0;
+    unsigned grid = 0;
+};
+ClusterPlan plan_cluster(const cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, int elem_size, bool shifted, bool sampling) {
+    ClusterPlan best;
+    if (!ps.all_c16 || !ctx->one_launch) return best;
+    if (B > kGroupRows && (mixed || int64_t(ps.V) * elem_size < 128 * 1024)) return best;
+    double least = 0.;
+    for (int r = 1; r <= (mixed ? 1 : kClusterRows); ++r) {
+        const int clusters = ceil_div(B, r);
+        for (int n = 2; n <= kClusterMost; ++n) {  // (one block is no cluster: there is nothing to send)
+            if (clusters > ctx->cluster_limit[n]) continue;
+            ClusterPlan c;
+            c.g.rows = r;
+            c.g.blocks = n;
+            c.g.per_block = std::max(1, ceil_div(ps.V >> 3, n));
+            c.g.run = ceil_div(c.g.per_block, kClusterWarps);
+            const int chunks = ceil_div(c.g.run, shifted ? PipeChunk<1, kSrcShifted>::kOctets : 32);
+            c.smem = size_t(cluster_table_bytes(ps.maxKW)) + size_t(kClusterWarps) * cluster_warp_bytes(c.g.run, r, 8 * elem_size);
+            if (chunks > kClusterChunks || c.smem > size_t(ctx->smem_optin) - kClusterStatic) continue;
+            const double cost = chunks * ((shifted || sampling ? 0.4 : 1.0) + r) + 0.2 * n;
+            if (best.ok && cost >= least) continue;
+            least = cost;
+            // (more than half of an SM's shared memory, so that a block has its SM to itself)
+            c.smem = std::max(c.smem, size_t(ctx->smem_optin) / 2 + 1024);
+            c.grid = unsigned(clusters) * unsigned(n);
+            c.ok = true;
+            best = c;
+        }
+    }
+    return best;
+}
+
+// CFGZIP_E_RANGE: the device cannot place these clusters, the step takes two launches.
+template <int DT>
+int launch_cluster(cfgzip_ctx* ctx, StepArgs& a, const ClusterPlan& c, bool mixed, bool shifted, cudaStream_t st) {
+    a.p0 = ctx->parts[size_t(a.part0)].dev;
+    a.expire_test = ctx->expire_test;
+    void (*kern)(StepArgs, ClusterGeom);
+#define CFGZIP_CLUSTER(R, T) (shifted ? k_step_cluster<DT, R, true, T> : k_step_cluster<DT, R, false, T>)
+#define CFGZIP_CLUSTER_ROWS(T) (c.g.rows == 1 ? CFGZIP_CLUSTER(1, T) : c.g.rows == 2 ? CFGZIP_CLUSTER(2, T) : CFGZIP_CLUSTER(4, T))
+    if (a.u) kern = CFGZIP_CLUSTER_ROWS(true); else kern = CFGZIP_CLUSTER_ROWS(false);
+#undef CFGZIP_CLUSTER_ROWS
+#undef CFGZIP_CLUSTER
+    if (ensure_smem(ctx, kern, c.smem, true) != CFGZIP_OK) return CFGZIP_E_RANGE;
+    ctx->cluster_now = c.g.blocks;
+    const int rc = launch(ctx, kern, dim3(c.grid), dim3(kClusterThreads), c.smem, st, a, c.g);
+    ctx->cluster_now = 1;
+    if (rc != CFGZIP_OK) return CFGZIP_E_RANGE;
+    if (mixed && !ctx->plan_in_use) ctx->plan_valid = false;  // (a kept grouping ends with a call that names its rows' partitions)
+    return CFGZIP_OK;
+}
+
 template <int DT>
 int launch_fused(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, int mode, bool aligned, float* logp_full,
                  cudaStream_t st) {
     int rc;
     DensePlan few;
+    if (mode != CFGZIP_SPARSE && !(mode == CFGZIP_AUTO && ctx->auto_min_bytes >= 0) &&
+        (aligned || aligned_elems(a.logits, DT == kBF16 ? 2 : 4))) {
+        ClusterPlan cl = plan_cluster(ctx, ps, a.B, mixed, DT == kBF16 ? 2 : 4, !aligned, false);
+        cl.g.full = logp_full;
+        cl.g.quads = a.V % 4 == 0 && (reinterpret_cast<uintptr_t>(logp_full) & 15u) == 0;
+        if (cl.ok && launch_cluster<DT>(ctx, a, cl, mixed, !aligned, st) == CFGZIP_OK) return CFGZIP_OK;
+    }
     if (aligned && mode == CFGZIP_SPARSE) few = plan_few(ctx, ps, a.B, mixed, DT == kBF16 ? 2 : 4);
     if (few.ok) {
         if (few.use_plan_kernel && (rc = run_plan_kernel(ctx, a.row_part, a.B, a.V, few, st)) != CFGZIP_OK) return rc;
@@ -865,6 +965,10 @@ int launch_sample(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, b
                   cudaStream_t st) {
     const bool filtered = top_k > 0 || top_p < 1.f;  // the draw is restricted to the most probable tokens
     int rc;
+    if (!filtered && (aligned || aligned_elems(a.logits, DT == kBF16 ? 2 : 4))) {
+        const ClusterPlan cl = plan_cluster(ctx, ps, a.B, mixed, DT == kBF16 ? 2 : 4, !aligned, true);
+        if (cl.ok && launch_cluster<DT>(ctx, a, cl, mixed, !aligned, st) == CFGZIP_OK) return CFGZIP_OK;
+    }
     const bool cm_bulk_ok = (reinterpret_cast<uintptr_t>(a.class_mask) & 15u) == 0 && (a.cm_stride & 3) == 0;
     DensePlan d = plan_pipe(ctx, ps, a.B, mixed, DT == kBF16 ? 2 : 4, cm_bulk_ok, !aligned);
     if (d.ok && d.depth && !(d.shifted && !aligned_elems(a.logits, DT == kBF16 ? 2 : 4))) {
@@ -1151,6 +1255,7 @@ int cfgzip_create(int device, cfgzip_ctx** out) {
         cudaMemset(ctx->d_status, 0, 8 * sizeof(int32_t));
         cudaMemset(ctx->d_n_groups, 0, sizeof(int32_t));
         ok = cfgzip_reserve_rows(ctx, kDefaultRows) == CFGZIP_OK;
+        find_cluster_limits(ctx);
     }
     if (!ok || cudaDeviceSynchronize() != cudaSuccess) {
         cudaGetLastError();
@@ -1793,7 +1898,12 @@ int cfgzip_launch_count(cfgzip_ctx* ctx, int64_t* out) {
 
 int cfgzip_set_tuning(cfgzip_ctx* ctx, const char* name, int32_t value) {
     if (!ctx || !name) return CFGZIP_E_ARG;
-    if (!std::strcmp(name, "ctas_per_sm")) {
+    for (const char* knob : {"ctas_per_sm", "token_warps", "row_warps", "pipeline", "tensor_map", "pipe_warps", "waves", "spread", "stage_alias",
+                             "fold", "lane_octets", "pipe_depth"})
+        if (!std::strcmp(name, knob)) ctx->one_launch = 0;  // (the caller shapes the two-launch step's kernel, so that one is meant)
+    if (!std::strcmp(name, "one_launch")) {
+        ctx->one_launch = value ? 1 : 0;
+    } else if (!std::strcmp(name, "ctas_per_sm")) {
         if (value < 1 || value > 16) return CFGZIP_E_ARG;
         ctx->ctas_per_sm = value;
     } else if (!std::strcmp(name, "token_warps")) {

@@ -167,8 +167,12 @@ struct Octet<kBF16> {
     __device__ __forceinline__ void store_at(void* p, bool) const { store_at(p); }
     __device__ __forceinline__ void fill_neg_inf() { v = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u); }
     __device__ __forceinline__ uint4 raw() const { return v; }
+    __device__ __forceinline__ void store_shared_at(char* p) const { *reinterpret_cast<uint4*>(p) = v; }
     __device__ __forceinline__ void mask(uint32_t byte, float* f) {
-        const uint32_t xl = nibble_to_byte_msbs(byte & 0xFu), xh = nibble_to_byte_msbs(byte >> 4);
+        mask_tokens(nibble_to_byte_msbs(byte & 0xFu), nibble_to_byte_msbs(byte >> 4), f);
+    }
+    // the allow bits as the top bits of eight bytes, a byte per token
+    __device__ __forceinline__ void mask_tokens(uint32_t xl, uint32_t xh, float* f) {
         // replicate the top bit of byte 2p / 2p+1 over the low / high half-word
         const uint32_t m0 = prmt(xl, 0u, 0x9988), m1 = prmt(xl, 0u, 0xBBAA);
         const uint32_t m2 = prmt(xh, 0u, 0x9988), m3 = prmt(xh, 0u, 0xBBAA);
@@ -221,8 +225,14 @@ struct Octet<kF32> {
         b = a;
     }
     __device__ __forceinline__ uint4 raw() const { return a; }  // only called for bf16 (two octets per lane)
+    __device__ __forceinline__ void store_shared_at(char* p) const {
+        *reinterpret_cast<uint4*>(p) = a;
+        *reinterpret_cast<uint4*>(p + 16) = b;
+    }
     __device__ __forceinline__ void mask(uint32_t byte, float* f) {
-        const uint32_t xl = nibble_to_byte_msbs(byte & 0xFu), xh = nibble_to_byte_msbs(byte >> 4);
+        mask_tokens(nibble_to_byte_msbs(byte & 0xFu), nibble_to_byte_msbs(byte >> 4), f);
+    }
+    __device__ __forceinline__ void mask_tokens(uint32_t xl, uint32_t xh, float* f) {
         const uint32_t ni = 0xFF800000u;
         uint32_t m;
         m = prmt(xl, 0u, 0x8888); a.x = (a.x & m) | (ni & ~m);
@@ -392,6 +402,72 @@ __device__ __forceinline__ void bulk_g2s(void* dst_smem, const void* src_gmem, u
                      smem_u32(dst_smem)),
                  "l"(src_gmem), "r"(bytes), "r"(smem_u32(bar))
                  : "memory");
+}
+
+// ---- thread-block cluster: rank, barrier, accesses to a peer block's shared memory -----------------
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t cluster_blocks() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+    return r;
+}
+// every thread of every block of the cluster (a hardware barrier like the block's own: no flag is polled), in two halves
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_barrier() {
+    cluster_arrive();
+    cluster_wait();
+}
+__device__ __forceinline__ uint32_t peer_shared(const void* mine, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(mine)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ unsigned int add_peer_u32(uint32_t addr, unsigned int v) {
+    unsigned int old;
+    asm volatile("atom.shared::cluster.add.u32 %0, [%1], %2;" : "=r"(old) : "r"(addr), "r"(v) : "memory");
+    return old;
+}
+__device__ __forceinline__ uint32_t ld_peer_u32(uint32_t addr) {
+    uint32_t v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint4 ld_peer_v4(uint32_t addr) {
+    uint4 v;
+    asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_peer_u64(uint32_t addr, unsigned long long v) {
+    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
+}
+__device__ __forceinline__ void st_peer_u32(uint32_t addr, uint32_t v) {
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+// Sixteen bytes into a peer block's shared memory, counted off on a barrier of that block (its copies' bytes are expected there).
+__device__ __forceinline__ void st_async_peer_v4(uint32_t addr, uint4 v, uint32_t peer_bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr), "r"(v.x),
+                 "r"(v.y), "r"(v.z), "r"(v.w), "r"(peer_bar)
+                 : "memory");
+}
+// mbar_wait for what peers have written
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity) {
+    for (int it = 0; it < 250000; ++it) {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
+            "selp.b32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(smem_u32(bar)), "r"(parity), "r"(2000u)
+            : "memory");
+        if (ok) return true;
+    }
+    return false;
 }
 
 }  // namespace cfgzip

@@ -1,0 +1,87 @@
+"""The one-launch step of a short batch (a thread-block cluster per row or few rows) against the CPU oracle, at the edges of its
+shapes: rows per cluster, runs and chunks of the warps, tokens outside the vectors, rows off the vector grid, rows without a
+partition, and the calls that have to stay with two launches."""
+import numpy as np
+import pytest
+import torch
+
+import synth
+from synth import rng
+from paper_2605_29986_b200 import binding as cz
+from _gpu_util import Ctx, compare_step, oracle_step, run_fused
+from test_gpu_sample import check_sample, run_sample
+
+pytestmark = pytest.mark.gpu
+
+
+def inputs(V, K, B, dtype, tag, p=0.2):
+    part = synth.zipf_partition(V, K, seed=tag)
+    cm = synth.class_mask_bernoulli(K, B, p, rng.stream_key(rng.SEED_BASE, 920, tag, V))
+    cm[B // 2] = 0  # a row with nothing allowed
+    return part, cm, synth.logits_normal(B, V, 2.0, dtype, (921, tag, V))
+
+
+# V: less than an octet, one chunk per block and one token more or less, every warp a short run, eight chunks a warp;
+# B: clusters of 1, 2, 3 and 4 rows, the last one not full
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("V,K,B", [(3, 2, 2), (8, 3, 9), (65, 33, 7), (4096, 64, 3), (4097, 65, 5), (65528, 2047, 16), (65544, 2048, 17), (128256, 2048, 31),
+                                   (131072, 8192, 47), (100001, 5000, 63), (99999, 300, 33), (200008, 16384, 7)])
+def test_greedy_and_sampling(V, K, B, dtype):
+    part, cm, z = inputs(V, K, B, dtype, 1)
+    want = oracle_step([part], None, cm, z, V, want_full=True)
+    with Ctx([part]) as ctx:
+        before = cz.cfgzip_launch_count(ctx.h)
+        compare_step(run_fused(ctx, None, cm, z, V), want, V)
+        compare_step(run_fused(ctx, None, cm, z, V, want_full=True, want_vm=False), want, V)
+        if B <= 16:
+            assert cz.cfgzip_launch_count(ctx.h) - before == 2  # two steps
+        for u in (np.zeros(B), np.full(B, 1 - 2.0 ** -24), np.linspace(0, 0.99, B)):
+            u = u.astype(np.float32)
+            check_sample(run_sample(ctx, None, cm, z, V, u, 1.25), [part], None, cm, z, V, u, 1.25)
+        assert cz.cfgzip_poll_status(ctx.h) == (5 * int((want["argmax"] < 0).sum()), 0, 0)  # five steps
+        cz.cfgzip_set_tuning(ctx.h, "one_launch", 0)
+        before = cz.cfgzip_launch_count(ctx.h)
+        compare_step(run_fused(ctx, None, cm, z, V), want, V)
+        assert cz.cfgzip_launch_count(ctx.h) - before >= 2
+
+
+@pytest.mark.parametrize("V", [20000, 20003])
+@pytest.mark.parametrize("B", [2, 20, 32])
+def test_rows_of_several_partitions(V, B):
+    parts = [synth.zipf_partition(V, k, seed=i) for i, k in enumerate((50, 333, 700))]
+    row_part = (np.arange(B) * 7 % 3).astype(np.int32)
+    cm = synth.class_mask_bernoulli(700, B, 0.2, rng.stream_key(rng.SEED_BASE, 922))
+    z = synth.logits_normal(B, V, 2.0, "bf16", (923,))
+    want = oracle_step(parts, row_part, cm, z, V)
+    with Ctx(parts) as ctx:
+        d_rp = torch.from_numpy(row_part).cuda()
+        cz.cfgzip_plan_rows(ctx.h, ctx.ids[0], d_rp, B)
+        compare_step(run_fused(ctx, row_part, cm, z, V), want, V)
+        with pytest.raises(Exception):  # an explicit vector ends the kept grouping
+            cz.cfgzip_map_tokens(ctx.h, ctx.ids[0], cz.ROWS_AS_PLANNED, d_rp, d_rp, B)
+        bad = row_part.copy()
+        bad[1] = 9
+        got = run_fused(ctx, bad, cm, z, V)
+        assert got["argmax"][1] == -7 and np.array_equal(got["logits"][1], z[1]) and cz.cfgzip_poll_status(ctx.h)[2] == 1
+        keep = np.arange(B) != 1
+        for key in ("argmax", "rep", "vocab_mask"):
+            assert np.array_equal(got[key][keep], want[key][keep])
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_ties_and_waits(dtype):
+    # equal maxima in the head, in several blocks and in the tail: the lowest id wins; a wait reported as run out surfaces
+    V, B = 30005, 12
+    part, cm, z = inputs(V, 100, B, dtype, 3)
+    cm[:] = 0xFFFFFFFF
+    for b in range(B):
+        z[b, [(b % 9), 5000 + b, 20000, V - 1 - (b % 7)]] = 50.0 if dtype == "f32" else 0x4248
+    want = oracle_step([part], None, cm, z, V)
+    with Ctx([part]) as ctx:
+        compare_step(run_fused(ctx, None, cm, z, V), want, V)
+        assert cz.cfgzip_poll_status(ctx.h) == (0, 0, 0)
+        cz.cfgzip_set_tuning(ctx.h, "test_expire_waits", 1)
+        run_fused(ctx, None, cm, z, V)
+        assert cz.load_library().cfgzip_poll_status(ctx.h, None, None, None, None) == cz.E_CUDA
+        cz.cfgzip_set_tuning(ctx.h, "test_expire_waits", 0)
+        compare_step(run_fused(ctx, None, cm, z, V), want, V)
