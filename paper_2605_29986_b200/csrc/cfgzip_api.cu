@@ -34,6 +34,7 @@ struct Part {
 
 constexpr size_t kSpareBytes = size_t(32) << 20;  // most memory of a released partition a context keeps for the next one
 constexpr size_t kPartialSlots = size_t(1) << 18;  // 4 MB of (max, sum, pos) slots
+constexpr size_t kChunkMaxSlots = size_t(1) << 21;  // 8 MB of chunk maxima (rows x chunks of a sampling step with top-k)
 constexpr int kTwoOctetItemsPerWarp = 3;           // bf16: two octets per lane from this many work items per warp on
 constexpr int kDefaultRows = 16384;
 
@@ -57,6 +58,7 @@ struct cfgzip_ctx {
     size_t spare_bytes = 0;
     PartDev* d_parts = nullptr;
     Partial* d_partials = nullptr;
+    float* d_chunk_max = nullptr;
     unsigned int* d_tickets = nullptr;  // reserved_rows entries
     int32_t* d_status = nullptr;        // 4 counters, and 4 that nobody reads (see uncounted)
     bool uncounted = false;             // set around a launch that repeats what another launch of the same call counts
@@ -722,7 +724,7 @@ size_t row_blocks_pad(const cfgzip_ctx* ctx, unsigned rows_grid, int32_t B) {
 
 // The pipelined streaming kernel for a planned step (d.depth > 0; `a` filled by fill_groups).
 template <int DT>
-int launch_pipe(cfgzip_ctx* ctx, const StepArgs& a, const DensePlan& d, dim3 grid, dim3 block, cudaStream_t st) {
+int launch_pipe(cfgzip_ctx* ctx, const StepArgs& a, const DensePlan& d, dim3 grid, dim3 block, int kind, cudaStream_t st) {
     int rc;
     // rows of a batch are consecutive unless the plan kernel regrouped them: then one tiled
     // 2-D copy (box 256 elements x 8 rows) brings a whole batch
@@ -741,10 +743,11 @@ int launch_pipe(cfgzip_ctx* ctx, const StepArgs& a, const DensePlan& d, dim3 gri
                                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     }
     void (*kern)(StepArgs, CUtensorMap);
-    const bool tempered = a.u != nullptr;  // only a sampling step has a temperature
     constexpr int kTwo = DT == kBF16 ? 2 : 1;  // f32 lanes always take one octet (32 bytes)
-#define CFGZIP_PIPE_SRC(OPL, SRC, LBT, MINB) \
-    (tempered ? k_step_dense_pipe<DT, OPL, SRC, LBT, MINB, true> : k_step_dense_pipe<DT, OPL, SRC, LBT, MINB, false>)
+#define CFGZIP_PIPE_SRC(OPL, SRC, LBT, MINB)                                                  \
+    (kind == kStepFiltered ? k_step_dense_pipe<DT, OPL, SRC, LBT, MINB, kStepFiltered>        \
+     : kind == kStepSample ? k_step_dense_pipe<DT, OPL, SRC, LBT, MINB, kStepSample>          \
+                           : k_step_dense_pipe<DT, OPL, SRC, LBT, MINB, kStepGreedy>)
 #define CFGZIP_PIPE_VARIANT(OPL, LBT, MINB) \
     (tiled ? CFGZIP_PIPE_SRC(OPL, kSrcTiled, LBT, MINB) : CFGZIP_PIPE_SRC(OPL, kSrcRows, LBT, MINB))
     if (d.shifted)  // (no variant with more blocks per SM: the rows' own pointers need the registers)
@@ -913,7 +916,7 @@ int launch_fused(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, in
             }
             const dim3 grid(d.blocks ? unsigned(d.blocks) : unsigned(d.n_groups_ub) * unsigned(d.S)), block{unsigned(d.threads)};
             if (d.depth) {
-                rc = launch_pipe<DT>(ctx, a, d, grid, block, st);
+                rc = launch_pipe<DT>(ctx, a, d, grid, block, kStepGreedy, st);
             } else {
                 auto kern = k_step_dense<DT>;
                 if ((rc = ensure_smem(ctx, kern, d.smem)) != CFGZIP_OK) return rc;
@@ -939,20 +942,25 @@ int launch_fused(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, in
 
 // The draw of a sampling step with top-k / top-p. One block per row leaves most of the device idle on a short batch,
 // so 8, 4 or 2 blocks (a thread-block cluster) share a row while that many still fit the device in one wave, two of the
-// kernel's blocks to an SM.
+// kernel's blocks to an SM. With chunk maxima counted in clusters: 32 of 8 blocks do not fit where 256 blocks would (32 f32 rows of
+// 128256 with top-k 23.0 us, by fours 19.2). Without, where the row is gone over several times, more blocks in two waves are as good
+// (top-p alone, 32 bf16 rows of 128256 50 us, by fours 52; 33 rows of 32064 at T = 0.2 20.8 and 16.2).
 template <int DT>
 int launch_filtered(cfgzip_ctx* ctx, const StepArgs& a, unsigned rows_grid, int top_k, float top_p, cudaStream_t st) {
     int rc;
-    if ((rc = ensure_smem(ctx, k_sample_filtered<DT>, sizeof(FiltShared))) != CFGZIP_OK) return rc;
-    const unsigned fit = 2u * unsigned(std::max(ctx->sm_count, 1));
+    auto kern = a.chunk_max ? k_sample_filtered<DT, true> : k_sample_filtered<DT, false>;
+    if ((rc = ensure_smem(ctx, kern, sizeof(FiltShared))) != CFGZIP_OK) return rc;
     unsigned per_row = kFiltPeers;
-    while (per_row > 1 && unsigned(a.B) * per_row > fit) per_row /= 2;
+    auto fits = [&](unsigned n) {
+        return a.chunk_max ? a.B <= 2 * ctx->cluster_limit[n] : unsigned(a.B) * n <= 2u * unsigned(std::max(ctx->sm_count, 1));
+    };
+    while (per_row > 1 && !fits(per_row)) per_row /= 2;
     ctx->cluster_now = int(per_row);
-    rc = launch(ctx, k_sample_filtered<DT>, dim3(rows_grid * per_row), dim3(kFiltThreads), sizeof(FiltShared), st, a,
+    rc = launch(ctx, kern, dim3(rows_grid * per_row), dim3(kFiltThreads), sizeof(FiltShared), st, a,
                 filt_geom(a.V, int(per_row)), top_k, top_p);
     ctx->cluster_now = 1;
     if (rc != CFGZIP_OK && per_row > 1)  // a device that cannot place such a cluster: one block per row
-        rc = launch(ctx, k_sample_filtered<DT>, dim3(rows_grid), dim3(kFiltThreads), sizeof(FiltShared), st, a, filt_geom(a.V, 1),
+        rc = launch(ctx, kern, dim3(rows_grid), dim3(kFiltThreads), sizeof(FiltShared), st, a, filt_geom(a.V, 1),
                     top_k, top_p);
     return rc;
 }
@@ -982,8 +990,16 @@ int launch_sample(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, b
         const int n_chunks = ceil_div(ps.V >> 3, d.chunk_octets);
         a.run_chunks = std::max(1, ceil_div(n_chunks, d.S * d.WT));
         a.tail_state = 1;
+        // With top_k the streaming kernel also leaves the largest logit of every chunk: the draw then reads the chunks that reach its
+        // bar, some fifty, and not the row again (us, top-k 50 and top-p 0.9, bf16: 64 rows of 151936 28.5 -> 23.7, 512 of 128256 95 -> 74,
+        // 100 of 256000 54 -> 39; 200 f32 rows of 100003 off the vector grid 79 -> 52; 8 rows of 32064 15.0 -> 14.9). Its price in the
+        // streaming kernel, a reduction per row and chunk, is not paid by a step without top_k.
+        if (top_k > 0 && n_chunks <= kFiltMaxima && size_t(a.B) * size_t(n_chunks) <= kChunkMaxSlots) {
+            a.chunk_max = ctx->d_chunk_max;
+            a.n_chunks = n_chunks;
+        }
         const dim3 grid(d.blocks ? unsigned(d.blocks) : unsigned(d.n_groups_ub) * unsigned(d.S)), block{unsigned(d.threads)};
-        if ((rc = launch_pipe<DT>(ctx, a, d, grid, block, st)) != CFGZIP_OK) return rc;
+        if ((rc = launch_pipe<DT>(ctx, a, d, grid, block, a.chunk_max ? kStepFiltered : kStepSample, st)) != CFGZIP_OK) return rc;
         const unsigned rows_grid = unsigned(d.n_groups_ub) * kGroupRows;
         if (filtered) return launch_filtered<DT>(ctx, a, rows_grid, top_k, top_p, st);
         const size_t pad = row_blocks_pad(ctx, rows_grid, a.B);
@@ -1248,6 +1264,7 @@ int cfgzip_create(int device, cfgzip_ctx** out) {
     }
     bool ok = cudaMalloc(&ctx->d_parts, kMaxParts * sizeof(PartDev)) == cudaSuccess &&
               cudaMalloc(&ctx->d_partials, kPartialSlots * sizeof(Partial)) == cudaSuccess &&
+              cudaMalloc(&ctx->d_chunk_max, kChunkMaxSlots * sizeof(float)) == cudaSuccess &&
               cudaMalloc(&ctx->d_status, 8 * sizeof(int32_t)) == cudaSuccess &&
               cudaMalloc(&ctx->d_n_groups, sizeof(int32_t)) == cudaSuccess;
     if (ok) {
@@ -1275,6 +1292,7 @@ int cfgzip_destroy(cfgzip_ctx* ctx) {
     cudaFree(ctx->spare_block);
     cudaFree(ctx->d_parts);
     cudaFree(ctx->d_partials);
+    cudaFree(ctx->d_chunk_max);
     cudaFree(ctx->d_tickets);
     cudaFree(ctx->d_status);
     cudaFree(ctx->d_group_part);

@@ -256,6 +256,13 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
     return d;
 }
 
+// The largest value of the lanes in `members`, to all of them.
+__device__ __forceinline__ float redux_max(float v, uint32_t members = 0xFFFFFFFFu) {
+    float m;
+    asm volatile("redux.sync.max.f32 %0, %1, %2;" : "=f"(m) : "f"(v), "r"(members));
+    return m;
+}
+
 // Packed pairs of floats (sm_100 has two-wide fp32 multiply-add and add).
 __device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
     unsigned long long p;
@@ -309,8 +316,9 @@ struct RowAcc {
         pos = kNoPos;
     }
     // N = 8 or 16 consecutive logits of the row (masked ones are -inf), `position` the index of their first octet.
+    // Returns their largest.
     template <int N>
-    __device__ __forceinline__ void add_values(const float* f, int position, float scale = kLog2e) {
+    __device__ __forceinline__ float add_values(const float* f, int position, float scale = kLog2e) {
         float vmax = fmax3(fmax3(f[0], f[1], f[2]), fmax3(f[3], f[4], f[5]), fmaxf(f[6], f[7]));
         if (N == 16)
             vmax = fmaxf(vmax, fmax3(fmax3(f[8], f[9], f[10]), fmax3(f[11], f[12], f[13]), fmaxf(f[14], f[15])));
@@ -336,9 +344,10 @@ struct RowAcc {
         float a0, a1;
         unpack2(e2[0], a0, a1);
         s += a0 + a1;
+        return vmax;
     }
-    __device__ __forceinline__ void add_octet(const float (&f)[8], int position, float scale = kLog2e) {
-        add_values<8>(f, position, scale);
+    __device__ __forceinline__ float add_octet(const float (&f)[8], int position, float scale = kLog2e) {
+        return add_values<8>(f, position, scale);
     }
     // Bring the sum to the convention of Partial: relative to max(m, kRefFloor).
     __device__ __forceinline__ Partial to_partial(float scale = kLog2e) const {

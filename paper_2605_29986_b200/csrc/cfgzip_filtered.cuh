@@ -15,10 +15,11 @@ namespace cfgzip {
 // weight nor the draw.
 //
 // Ways through, all exact:
-//   short  The streaming kernel has published the largest logit of every run of tokens. The k-th largest of those is a bar
-//          that at least k tokens reach, and, the runs being many, not many more (k = 50: some 60 to 100 tokens). For top-p
-//          alone the bar is where the run maxima by themselves already weigh enough, or nearly (checked afterwards). One pass over the row collects the
-//          tokens at or above the bar, a thread each, and every thread sums over all of them.
+//   short  The streaming kernel has published the largest logit of every run of tokens; with top_k of every chunk of 31 to 64
+//          vectors. The k-th largest of those is a bar that at least k tokens reach, and, the chunks being many, not many more
+//          (k = 50: some 60), and only the chunks that reach it are read. For top-p alone the bar is where the run maxima by
+//          themselves already weigh enough, or nearly (checked afterwards), and one pass over the row collects the tokens at or
+//          above it. Up to kFiltThreads tokens get a lane or more each, which sums over all of them: their order needs no sort.
 //   long   Otherwise (a flat distribution, a large k), with one filter: a pass that counts the tokens in 8192 steps of the
 //          distance from the row maximum (one shared-memory addition a token; the weight of a step follows from its count to
 //          better than 0.1 %), which says about where the cut falls; and a pass that sums, exactly and chunk by chunk, what
@@ -30,9 +31,9 @@ namespace cfgzip {
 // Bound: latency of a chain of block-wide steps, most of them executed once or twice, beside one or two passes over a row
 // that is in the L2: loops stay rolled and steps that come up more than once are functions, which keeps the code a third of
 // what it was inlined and unrolled. Collecting every token that carries weight first took 78 us of the step for 64 rows of
-// 151936 bf16 logits at T = 0.7 (15000 such tokens a row), and some 30 passes over the row where they did not fit; this takes
-// 13 of a step of 27 (clock stamps, us from the block's first step: states read 2.3, bar 3.6, pass over the row 8.5, all blocks of
-// the row there 9.6, sort 11, cut 12, draw 12.5). With top-p alone the same rows take 66 us (606), 256 rows that allow nearly
+// 151936 bf16 logits at T = 0.7 (15000 such tokens a row), and some 30 passes over the row where they did not fit. With top_k this
+// takes 9 of a step of 23.4 (a pass over the whole row, a claim on the list for every token and a sort: 13 of 27; the claims alone, one
+// after the other, took 9000 of 19000 cycles). With top-p alone the same rows take 66 us (606), 256 rows that allow nearly
 // everything 174 (1366).
 // Where it is slower than collecting everything was: top-p alone on short rows of which every token that carries weight fitted
 // one list (up to some 12000): 128 bf16 rows of 20032 with 1 % allowed 24 -> 37 us, with 10 % 31 -> 50 (with 90 % 147 -> 47). One
@@ -59,6 +60,7 @@ constexpr int kFiltWindow = 200;    // tokens the window of the long way aims at
 constexpr unsigned int kFiltWindowMost = 800;  // and holds at most to either side, whole coarse steps
 constexpr int kFiltTries = 3;       // windows before the search
 constexpr int kFiltChunks = 512;    // most chunks of the draw's pass
+constexpr int kFiltMaxima = 2048;   // most chunks whose maxima the streaming kernel leaves (of its own chunks)
 constexpr float kFixOne = 1099511627776.f;  // 2^40
 
 // Order-preserving integer image of a logit and its inverse. bf16 logits only use the upper half of the float's
@@ -115,6 +117,8 @@ struct FiltShared {
             } chunk;
         };
     };
+    uint16_t chunks[kFiltMaxima];    // short way with top_k: the chunks whose largest logit reaches the bar
+    unsigned int n_chunks;
     unsigned int bar[kFiltThreads];  // count or weight of the run maxima, by distance from the row maximum
     unsigned long long pick[8];  // result of a search, written into every block of the cluster by the first
     unsigned long long scan_w[2][kFiltWarps];
@@ -684,7 +688,8 @@ __device__ __noinline__ unsigned int filt_allowed(const StepArgs& a, const PartD
 
 // One row per cluster of blocks (1 to 8 of them: a short batch has fewer rows than the device has multiprocessors).
 // Every block goes over its share of the row; what they find meets in the shared memory of the cluster's first block.
-template <int DT>
+// FINE: with top_k, from the maxima of the chunks.
+template <int DT, bool FINE>
 __global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __grid_constant__ StepArgs a, const FiltGeom geom,
                                                                      int top_k, float top_p) {
     extern __shared__ __align__(16) unsigned char filt_smem[];
@@ -720,6 +725,7 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __gri
     w.c_end = min(w.c_begin + geom.per_block, w.n_chunks);
     if (tid < 1 + kFiltTries) sh.list_n[tid] = 0u;
     sh.bar[tid] = 0u;
+    if (tid == 0) sh.n_chunks = 0u;
     if (!a.group_rows) pdl_wait();
     PartDev P = a.p0;
     if (a.group_part) {
@@ -731,22 +737,31 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __gri
     }
     // the run states the streaming kernel published: the row maximum, and the maxima and sums of up to four runs per thread
     // for the bar of the short way (leaving runs out only lowers the bar)
+    // (top_k: the maxima of the chunks, and the few tokens outside the vectors)
     const Partial* src = row_slots(a, g, j);
-    const int n_states = group_states(a, g);
+    const float* const maxima = a.chunk_max + int64_t(row) * a.n_chunks;
+    const int n_states = FINE ? a.n_chunks : group_states(a, g);
+    const int fine_head = FINE && a.shifted ? row_head<DT>(w.rowp, a.V) : 0, fine_end = fine_head + ((a.V - fine_head) & ~7);
+    const int edge_t = tid < 8 ? tid : fine_end + tid - 8;
+    float edge_z = -INFINITY;
+    if (FINE && tid < 16 && (tid < 8 ? edge_t < fine_head : edge_t < a.V)) edge_z = ldcg_elem<DT>(w.rowp, edge_t);
     const float u = __ldg(a.u + row);  // needed late
     constexpr int kKeep = 4;
-    float run_m[kKeep], run_s[kKeep], M = -INFINITY;
+    float run_m[kKeep], run_s[kKeep], M = edge_z;
 #pragma unroll
     for (int q = 0; q < kKeep; ++q) {
         const int k = tid + q * kFiltThreads;
         float2 r = make_float2(-INFINITY, 0.f);
-        if (k < n_states) r = __ldcg(reinterpret_cast<const float2*>(src + k));
+        if (k < n_states) {
+            if (FINE) r.x = __ldcg(maxima + k);
+            else r = __ldcg(reinterpret_cast<const float2*>(src + k));
+        }
         run_m[q] = r.x;
         run_s[q] = r.y;
         M = fmaxf(M, r.x);
     }
 #pragma unroll 1
-    for (int k = tid + kKeep * kFiltThreads; k < n_states; k += kFiltThreads) M = fmaxf(M, __ldcg(&src[k].m));
+    for (int k = tid + kKeep * kFiltThreads; k < n_states; k += kFiltThreads) M = fmaxf(M, __ldcg(FINE ? maxima + k : &src[k].m));
     M = float_from_order_key(__reduce_max_sync(0xFFFFFFFFu, float_order_key(M)));
     if (lane == 0) sh.warp_max[warp] = M;
     __syncthreads();
@@ -769,10 +784,10 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __gri
     // (below M - 40 / scale the fixed-point weight is zero; the extra unit covers the rounding of the threshold itself)
     w.z_zero = fmaxf(key_logit<DT>(logit_key<DT>(M - zero_at)), kRefFloor);
     int turn = 0;
-    auto write_draw = [&](int token, float zt, unsigned long long S_kept) {
+    auto write_draw = [&](int token, float zt, unsigned long long S_kept, int repv) {
         const float l = logf(static_cast<float>(S_kept) * (1.f / kFixOne));
         a.argmax[row] = token;
-        if (a.rep) a.rep[row] = __ldg(P.trep + token);
+        if (a.rep) a.rep[row] = repv;
         if (a.lse) a.lse[row] = fmaf(M, a.inv_t, l);
         if (a.logp_argmax) a.logp_argmax[row] = (zt - M) * a.inv_t - l;
     };
@@ -896,7 +911,71 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __gri
         if (way == 0) {
             unsigned long long mine = 0ull;
             auto push = [&](int t, float z) { filt_push(sh, 0, t, z); };
-            if (top_k > 0)
+            if constexpr (FINE) {
+                // the chunks that reach the bar, dealt to the blocks by their number and there to the warps; 32 vectors at a time,
+                // four loads in flight
+                auto mine_too = [&](int c) { return (uint32_t(c) & (w.n_peers - 1u)) == w.crank; };
+#pragma unroll
+                for (int q = 0; q < kKeep; ++q)
+                    if (run_m[q] >= z_bar && mine_too(tid + q * kFiltThreads)) sh.chunks[atomicAdd(&sh.n_chunks, 1u)] = uint16_t(tid + q * kFiltThreads);
+#pragma unroll 1
+                for (int k = tid + kKeep * kFiltThreads; k < n_states; k += kFiltThreads)
+                    if (mine_too(k) && __ldcg(maxima + k) >= z_bar) sh.chunks[atomicAdd(&sh.n_chunks, 1u)] = uint16_t(k);
+                if (w.crank == 0u && edge_z >= z_bar) push(edge_t, edge_z);
+                __syncthreads();
+                const int vecs = a.chunk_tokens >> 3, halves = (vecs + 31) >> 5, units = int(sh.n_chunks) * halves;
+                constexpr int kFlight = 4;
+#pragma unroll 1
+                for (int i0 = warp; i0 < units; i0 += kFlight * kFiltWarps) {
+                    FiltOct<DT> o[kFlight];
+                    int t0[kFlight];
+#pragma unroll
+                    for (int r = 0; r < kFlight; ++r) {
+                        const int i = i0 + r * kFiltWarps;
+                        const int v = (halves == 2 ? (i & 1) * 32 : 0) + lane;
+                        t0[r] = -1;
+                        o[r].a = o[r].b = make_uint4(FiltNone<DT>::word, FiltNone<DT>::word, FiltNone<DT>::word, FiltNone<DT>::word);
+                        if (i < units && v < vecs) {
+                            const int t = fine_head + int(sh.chunks[halves == 2 ? i >> 1 : i]) * a.chunk_tokens + 8 * v;
+                            if (t < fine_end) {
+                                t0[r] = t;
+                                const char* p = w.rowp + int64_t(t) * (DT == kBF16 ? 2 : 4);
+                                o[r].a = __ldcg(reinterpret_cast<const uint4*>(p));
+                                if (DT == kF32) o[r].b = __ldcg(reinterpret_cast<const uint4*>(p + 16));
+                            }
+                        }
+                    }
+                    // one claim on the list for the warp's tokens
+                    uint32_t over = 0u;
+#pragma unroll
+                    for (int r = 0; r < kFlight; ++r) {
+                        float e[8];
+                        filt_floats<DT>(o[r], e);
+                        over |= filt_at_least(e, z_bar) << (8 * r);
+                    }
+                    const unsigned int here = __popc(over);
+                    unsigned int inc = here;
+#pragma unroll
+                    for (int d = 1; d < 32; d <<= 1) {
+                        const unsigned int up = __shfl_up_sync(0xFFFFFFFFu, inc, d);
+                        if (lane >= d) inc += up;
+                    }
+                    unsigned int at = 0u;
+                    if (lane == 31 && inc) at = add_peer_u32(peer_shared(&sh.list_n[0], 0u), inc);
+                    at = __shfl_sync(0xFFFFFFFFu, at, 31) + inc - here;
+                    const uint32_t list0 = peer_shared(sh.list, 0u);
+#pragma unroll 1
+                    for (int r = 0; over >> (8 * r) && r < kFlight; ++r) {
+                        float e[8];
+                        filt_floats<DT>(r == 0 ? o[0] : r == 1 ? o[1] : r == 2 ? o[2] : o[3], e);
+                        filt_each(e, r == 0 ? t0[0] : r == 1 ? t0[1] : r == 2 ? t0[2] : t0[3], (over >> (8 * r)) & 0xFFu, [&](int t, float z) {
+                            if (at < unsigned(kFiltList))
+                                st_peer_u64(list0 + at * 8u, (static_cast<unsigned long long>(uint32_t(t)) << 32) | __float_as_uint(z));
+                            ++at;
+                        });
+                    }
+                }
+            } else if (top_k > 0)
                 filt_visit<DT>(w, [&](int t0, const float (&e)[8]) { filt_each(e, t0, filt_at_least(e, z_bar), push); });
             else
                 filt_visit<DT>(w, [&](int t0, const float (&e)[8]) {
@@ -1013,6 +1092,65 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __gri
             cluster_wait();
             return;
         }
+        if (way == 0 && n <= unsigned(kFiltThreads)) {
+            // Few tokens, one lane or more each: a token's place in the order and the weight in front of it, then the cut, then the kept
+            // weight up to its place in token order.
+            unsigned long long* const kept_weight = reinterpret_cast<unsigned long long*>(sh.list);  // (read once, by this thread)
+            if (unsigned(tid) < n) {
+                const uint2 e = sh.list[tid];
+                sh.order[tid] = (static_cast<unsigned long long>(~logit_key<DT>(__uint_as_float(e.x))) << 32) | e.y;
+                sh.weight[tid] = fixed_weight(__uint_as_float(e.x), M, scale);
+            }
+            __syncthreads();
+            const int lanes = lanes_per_token(n);
+            const unsigned int i = tid / lanes, sub = tid & (lanes - 1);
+            const bool have = i < n;
+            const unsigned long long me = have ? sh.order[i] : 0ull, mine = have ? sh.weight[i] : 0ull;
+            const uint32_t id = uint32_t(me);
+            const int repv = have ? __ldg(P.trep + id) : -1;  // (asked for early: one of them is the row's)
+            unsigned int rank = 0u;
+            unsigned long long before = 0ull;
+#pragma unroll 4
+            for (unsigned int k = sub; k < n; k += lanes)
+                if (sh.order[k] < me) {
+                    ++rank;
+                    before += sh.weight[k];
+                }
+#pragma unroll 1
+            for (int d = lanes >> 1; d >= 1; d >>= 1) {
+                rank += __shfl_xor_sync(0xFFFFFFFFu, rank, d);
+                before += __shfl_xor_sync(0xFFFFFFFFu, before, d);
+            }
+            const unsigned int end = top_k > 0 ? min(unsigned(top_k), n) : n;
+            unsigned long long target = ~0ull;
+            if (top_p < 1.f) {
+                unsigned long long S = 0ull;
+                if (top_k > 0) {
+                    if (have && sub == 0 && rank + 1 == end) sh.topk_w = before + mine;
+                    __syncthreads();
+                    S = sh.topk_w;
+                } else {
+                    for (uint32_t p = 0; p < w.n_peers; ++p) S += sh.peer_w[p];
+                }
+                target = filt_target(S, top_p);
+            }
+            const bool kept = have && rank < end && before < target;
+            if (have && sub == 0) {
+                kept_weight[i] = kept ? mine : 0ull;
+                if (kept && (rank + 1 == end || before + mine >= target)) sh.kept_w = before + mine;  // the last one that is kept
+            }
+            __syncthreads();
+            const unsigned long long S_kept = sh.kept_w, thr = filt_threshold(S_kept, u);
+            unsigned long long cum = 0ull;
+#pragma unroll 4
+            for (unsigned int k = sub; k < n; k += lanes) cum += uint32_t(sh.order[k]) <= id ? kept_weight[k] : 0ull;
+#pragma unroll 1
+            for (int d = lanes >> 1; d >= 1; d >>= 1) cum += __shfl_xor_sync(0xFFFFFFFFu, cum, d);
+            cluster_wait();  // (long since complete: no block may leave while another reads its shared memory)
+            if (kept && sub == 0 && mine > 0ull && cum - mine <= thr && thr < cum)
+                write_draw(int(id), key_logit<DT>(~uint32_t(me >> 32)), S_kept, repv);
+            return;
+        }
         // the listed tokens in order, with the weight in front of each
         filt_sort<DT>(sh, n);
         const unsigned int per = (n + kFiltThreads - 1) / kFiltThreads, i0 = min(tid * per, n), i1 = min(i0 + per, n);
@@ -1059,26 +1197,7 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __gri
             cut.tau = sh.cut_key;
             cut.id_cut = sh.cut_id;
             const unsigned int n_kept = sh.n_kept;
-            if (way == 0 && n_kept <= unsigned(kFiltThreads)) {
-                // few: every kept token, one lane or more each, sums the kept weight up to its place in token order
-                const unsigned long long S_kept = sh.kept_w, thr = filt_threshold(S_kept, u);
-                const int lanes = lanes_per_token(n_kept);
-                const unsigned int i = tid / lanes, sub = tid & (lanes - 1);
-                const uint32_t id = i < n_kept ? uint32_t(sh.order[i]) : 0u;
-                unsigned long long cum = 0ull;
-#pragma unroll 4
-                for (unsigned int k = sub; k < n_kept; k += lanes) cum += uint32_t(sh.order[k]) <= id ? sh.weight[k] : 0ull;
-#pragma unroll 1
-                for (int d = lanes >> 1; d >= 1; d >>= 1) cum += __shfl_xor_sync(0xFFFFFFFFu, cum, d);
-                cluster_wait();  // (long since complete: no block may leave while another reads its shared memory)
-                if (i < n_kept && sub == 0) {
-                    const unsigned long long mine = sh.weight[i];
-                    if (mine > 0ull && cum - mine <= thr && thr < cum)
-                        write_draw(int(id), key_logit<DT>(~uint32_t(sh.order[i] >> 32)), S_kept);
-                }
-                return;
-            }
-            // many: into the sums of their chunks
+            // into the sums of their chunks
             if (way == 0) {
                 for (int c = tid; c < w.n_chunks; c += kFiltThreads) {
                     sh.chunk.above[c] = 0ull;
@@ -1164,7 +1283,7 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __gri
             seen = tie_run + t_inc - t_mine;
             filt_each(e, t0, filt_at_least(e, w.z_zero), [&](int t, float z) {
                 const unsigned long long wt = weight_of(t, z);
-                if (cum <= thr && thr < cum + wt) write_draw(t, z, S_kept);
+                if (cum <= thr && thr < cum + wt) write_draw(t, z, S_kept, __ldg(P.trep + t));
                 cum += wt;
             });
         }

@@ -77,6 +77,8 @@ struct StepArgs {
     Partial* partials;
     unsigned int* tickets;
     int32_t* status;            // [0] empty rows, [1] bad tokens, [2] bad rows, [3] copies that never arrived
+    float* chunk_max;           // sampling step with top_k: dev [B][n_chunks] largest masked logit of every chunk; else null
+    int32_t n_chunks;
 };
 
 // Tokens in front of the first vector boundary of a row that may start anywhere (16 bytes for bf16, 32 for f32: an
@@ -865,6 +867,7 @@ struct PipeGeom {
 // How the logits of a work item reach shared memory: one bulk copy per row, one tiled 2-D copy for 8 consecutive rows,
 // or one bulk copy per row from that row's own first vector boundary on (rows that start anywhere).
 enum : int { kSrcRows = 0, kSrcTiled = 1, kSrcShifted = 2 };
+enum : int { kStepGreedy = 0, kStepSample = 1, kStepFiltered = 2 };
 
 // Octets of a chunk. Where the rows start anywhere, vector o of a row holds the tokens 8 o + head .. 8 o + head + 7, so
 // its allow bits come from the token octets o and o + 1: a chunk is then the 31 vectors whose bits the 32 octets of
@@ -889,12 +892,13 @@ struct BatchAddr {
 // FULL: all 8 rows live and every lane's octets inside the whole-vector range (no per-row tests).
 // kSrcShifted: n_ids octets of class ids are in the stage; heads: row_head of the 8 rows, four bits each; the vocab-mask
 // byte of token octet o is written by the same lane as vector o of the rows. V: tokens.
-template <int DT, int OPL, bool FULL, int SRC>
+// MAXIMA: chunk_m of lane i becomes the largest masked logit of the chunk in row i.
+template <int DT, int OPL, bool FULL, int SRC, bool MAXIMA>
 __device__ __forceinline__ void pipe_consume_item(const char* src, uint32_t lane_off, uint32_t srow, const uint32_t* T, int rb,
                                                   int live, int n_act, int o, int lane, const BatchAddr& ba,
                                                   char* const (&rowp)[kBatchRows], uint8_t* const (&vmp)[kBatchRows],
                                                   RowAcc (&acc)[kBatchRows], float scale, bool wide, int n_ids, uint32_t heads,
-                                                  int V) {
+                                                  int V, float& chunk_m) {
     using G = PipeGeom<DT, OPL>;
     constexpr bool CONSEC = SRC == kSrcTiled;
     if constexpr (SRC == kSrcShifted) {
@@ -907,6 +911,7 @@ __device__ __forceinline__ void pipe_consume_item(const char* src, uint32_t lane
         if (lane == 31) return;  // its bits served lane 30
 #pragma unroll
         for (int i = 0; i < kBatchRows; ++i) {
+            float top = -INFINITY;
             if (FULL || i < live) {
                 const uint32_t byte = ((i < 4 ? lo : hi) >> (8 * (i & 3))) & 0xFFu;
                 if (vmp[i] && (FULL || 8 * o + 8 <= V)) st_global_u8(vmp[i] + o, byte);
@@ -918,8 +923,12 @@ __device__ __forceinline__ void pipe_consume_item(const char* src, uint32_t lane
                     oc.load_shared_at(src + i * G::kRowBytes + lane_off);
                     oc.mask(((byte | (next << 8)) >> head) & 0xFFu, f);
                     oc.store_at(rowp[i] + size_t(o) * G::kOctetBytes, true);  // f32 vectors sit on 32-byte boundaries here
-                    acc[i].add_octet(f, o, scale);
+                    top = acc[i].add_octet(f, o, scale);
                 }
+            }
+            if constexpr (MAXIMA) {
+                top = redux_max(top, 0x7FFFFFFFu);
+                chunk_m = lane == i ? top : chunk_m;
             }
         }
     } else {
@@ -934,6 +943,7 @@ __device__ __forceinline__ void pipe_consume_item(const char* src, uint32_t lane
         const bool both = FULL || n_act == OPL;
 #pragma unroll
         for (int i = 0; i < kBatchRows; ++i) {
+            float top = -INFINITY;
             if (FULL || (i < live && n_act > 0)) {
                 Octet<DT> oc[OPL];
                 float f[8 * OPL];
@@ -965,7 +975,11 @@ __device__ __forceinline__ void pipe_consume_item(const char* src, uint32_t lane
                         if (both) st_global_u16(vp, bytes); else st_global_u8(vp, bytes & 0xFFu);
                     }
                 }
-                acc[i].template add_values<8 * OPL>(f, o, scale);
+                top = acc[i].template add_values<8 * OPL>(f, o, scale);
+            }
+            if constexpr (MAXIMA) {
+                top = redux_max(top);
+                chunk_m = lane == i ? top : chunk_m;
             }
         }
     }
@@ -977,12 +991,15 @@ __device__ __forceinline__ void pipe_consume_item(const char* src, uint32_t lane
 // vectors start row_head tokens in, the tokens left over on both sides go through publish_edges. (One token per thread
 // and one block per row took 223 us for 48 rows of 100003 bf16 logits.) OPL: octets per lane and row (see PipeGeom).
 // LBT / MINB: launch bounds (threads per block, blocks per SM) the variant is compiled for; they set
-// the register budget: (512, 1) 128 registers, (384, 1) 168, (320, 2) 96, (256, 3) 80. TEMPERED: the sums
-// are of exp(z / T) with the step's temperature (sampling steps); otherwise T = 1 is compiled in.
-template <int DT, int OPL, int SRC, int LBT, int MINB, bool TEMPERED>
+// the register budget: (512, 1) 128 registers, (384, 1) 168, (320, 2) 96, (256, 3) 80.
+// KIND: a greedy step (T = 1 is compiled in), or a sampling step, whose sums are of exp(z / T): kStepSample deals the chunks so that
+// the states of a row follow the token order, kStepFiltered (top-k / top-p follow) deals them as a greedy step does and leaves the
+// largest logit of every chunk of a row in chunk_max.
+template <int DT, int OPL, int SRC, int LBT, int MINB, int KIND>
 __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_constant__ StepArgs a,
                                                          const __grid_constant__ CUtensorMap tmap) {
     using G = PipeGeom<DT, OPL>;
+    constexpr bool TEMPERED = KIND != kStepGreedy, RUNS = KIND == kStepSample, MAXIMA = KIND == kStepFiltered;
     constexpr bool TMAP = SRC == kSrcTiled, SHIFT = SRC == kSrcShifted;
     constexpr int kChunkOctets = PipeChunk<OPL, SRC>::kOctets;
     __shared__ char* s_vec[SHIFT ? kGroupRows : 1];  // first vector of every row of the group
@@ -1057,22 +1074,22 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
     // (warp index among them, then a stride of their number), so that at any moment the group's blocks
     // read neighbouring pieces of the same rows: measured 5 % faster on long steps than one contiguous
     // range per block, and as fast as handing chunks out through global counters.
-    // In a sampling step (TEMPERED) the states of a row must follow the token order: every warp slot then
+    // In a sampling step without filters (RUNS) the states of a row must follow the token order: every warp slot then
     // takes one contiguous run of run_chunks chunks instead.
     // The number of chunks is rarely a multiple of the number of warp slots, so some slots get one chunk more than
     // the others; the deal starts at a different slot for every row batch (rot_chunks further on), which spreads the
     // extra chunks evenly over the warps and the blocks instead of giving the first ones one more in every row batch.
     const int n_chunks = (n_full + kChunkOctets - 1) / kChunkOctets;
-    const int stride_chunks = TEMPERED ? 1 : S * a.WT;  // round-robin: warps that share a row batch of the group
-    const int run_chunks = TEMPERED ? (!TMAP && a.group_w ? max(1, (n_chunks + S * a.WT - 1) / (S * a.WT)) : a.run_chunks) : 0;
+    const int stride_chunks = RUNS ? 1 : S * a.WT;  // round-robin: warps that share a row batch of the group
+    const int run_chunks = RUNS ? (!TMAP && a.group_w ? max(1, (n_chunks + S * a.WT - 1) / (S * a.WT)) : a.run_chunks) : 0;
     const int n_slots = !TMAP && a.group_w ? (a.fold_off ? S : S * a.WT + 1 + a.head_state) : a.slots;  // states of a row, the last one for its ends
     auto first_chunk_of = [&](int rb) {  // this warp's first chunk of row batch rb
-        if (TEMPERED) return (split * a.WT + wt) * run_chunks;
+        if (RUNS) return (split * a.WT + wt) * run_chunks;
         int c = split * a.WT + wt - rb * a.rot_chunks;
         c %= stride_chunks;
         return c < 0 ? c + stride_chunks : c;
     };
-    const int chunk_end = TEMPERED ? min(first_chunk_of(0) + run_chunks, n_chunks) : n_chunks;
+    const int chunk_end = RUNS ? min(first_chunk_of(0) + run_chunks, n_chunks) : n_chunks;
     int* const slot_info = ring_info + warp * depth; // (rb << 24) | chunk of the item in each slot, -1 = no more items
 
     // automatic mode: bit r = row slot r was finished by the class-list kernel (set after the wait below)
@@ -1164,7 +1181,7 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
         const int row0 = g * kGroupRows + wr * kBatchRows;
         const int live0 = min(kBatchRows, nrow - wr * kBatchRows);
         int chunk = first_chunk_of(wr);
-        for (int d = 0; d < a.prefetch_items && chunk < chunk_end; ++d, chunk += TEMPERED ? 1 : stride_chunks) {
+        for (int d = 0; d < a.prefetch_items && chunk < chunk_end; ++d, chunk += stride_chunks) {
             const int o0 = chunk * kChunkOctets;
             const uint32_t nvec = uint32_t(min(n_full - o0, kChunkOctets));
             if (SHIFT) {
@@ -1291,6 +1308,7 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
         const int info = slot_info[slot];
         if (info < 0) break;
         const int rb = info >> 24, o0 = (info & 0xFFFFFF) * kChunkOctets;
+        float chunk_m = -INFINITY;
         while (cur_rb < rb) {  // the previous row batch of this warp is complete (possibly without any chunk)
             warp_rows_publish_to(acc, live, cur_rb, lane, scale, pub_base, pub_stride, my_slot);
             cur_rb += WR;
@@ -1309,11 +1327,12 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
         ba.vm_item = vm0 ? vm0 + o : nullptr;
         // (the vectors of a row that starts anywhere end at most one octet before the last whole octet)
         if (live == kBatchRows && o0 + kChunkOctets <= (SHIFT ? n_full - 1 : n_full))
-            pipe_consume_item<DT, OPL, true, SRC>(src, lane_off, srow, T, rb, live, OPL, o, lane, ba, rowp, vmp, acc, scale,
-                                                  a.wide != 0, 32, heads, a.V);
+            pipe_consume_item<DT, OPL, true, SRC, MAXIMA>(src, lane_off, srow, T, rb, live, OPL, o, lane, ba, rowp, vmp, acc, scale,
+                                                  a.wide != 0, 32, heads, a.V, chunk_m);
         else
-            pipe_consume_item<DT, OPL, false, SRC>(src, lane_off, srow, T, rb, live, max(0, min(OPL, n_full - o)), o, lane, ba,
-                                                   rowp, vmp, acc, scale, a.wide != 0, min(n_octets - o0, 32), heads, a.V);
+            pipe_consume_item<DT, OPL, false, SRC, MAXIMA>(src, lane_off, srow, T, rb, live, max(0, min(OPL, n_full - o)), o, lane, ba,
+                                                   rowp, vmp, acc, scale, a.wide != 0, min(n_octets - o0, 32), heads, a.V, chunk_m);
+        if (MAXIMA && a.chunk_max && lane < live) a.chunk_max[int64_t(s_row[rb * kBatchRows + lane]) * a.n_chunks + (info & 0xFFFFFF)] = chunk_m;
         ++consumed;
         if (++slot == depth) { slot = 0; phase ^= 1u; }
         __syncwarp();  // every lane has its data out of the slot before it is refilled
