@@ -4,8 +4,10 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <cstdint>
 #include <cstring>
+#include <map>
 #include <mutex>
 #include <new>
 #include <utility>
@@ -34,7 +36,7 @@ struct Part {
 
 constexpr size_t kSpareBytes = size_t(32) << 20;  // most memory of a released partition a context keeps for the next one
 constexpr size_t kPartialSlots = size_t(1) << 18;  // 4 MB of (max, sum, pos) slots
-constexpr size_t kChunkMaxSlots = size_t(1) << 21;  // 8 MB of chunk maxima (rows x chunks of a sampling step with top-k)
+constexpr size_t kChunkMaxSlots = size_t(1) << 20;  // 4 MB of chunk maxima (rows x chunks of a sampling step with top-k)
 constexpr int kTwoOctetItemsPerWarp = 3;           // bf16: two octets per lane from this many work items per warp on
 constexpr int kDefaultRows = 16384;
 
@@ -58,7 +60,7 @@ struct cfgzip_ctx {
     size_t spare_bytes = 0;
     PartDev* d_parts = nullptr;
     Partial* d_partials = nullptr;
-    float* d_chunk_max = nullptr;
+    float* d_chunk_max = nullptr;  // behind the states, in the same block
     unsigned int* d_tickets = nullptr;  // reserved_rows entries
     int32_t* d_status = nullptr;        // 4 counters, and 4 that nobody reads (see uncounted)
     bool uncounted = false;             // set around a launch that repeats what another launch of the same call counts
@@ -198,8 +200,17 @@ int ensure_smem(cfgzip_ctx* ctx, K kernel, size_t bytes, bool large_clusters = f
 }
 
 // How many clusters of every size the device holds at once, a block to an SM: the SMs come in groups that a cluster does not cross,
-// so that 132 of 148 can be had four at a time and 120 eight at a time (15 clusters).
+// so that 132 of 148 can be had four at a time and 120 eight at a time (15 clusters). Asked once per device and process: the
+// fifteen questions took as long as the rest of creating a context.
 void find_cluster_limits(cfgzip_ctx* ctx) {
+    static std::mutex mutex;
+    static std::map<int, std::array<int, kClusterMost + 1>> known;
+    std::lock_guard<std::mutex> lock(mutex);
+    const auto found = known.find(ctx->device);
+    if (found != known.end()) {
+        std::copy(found->second.begin(), found->second.end(), ctx->cluster_limit);
+        return;
+    }
     auto kern = k_step_cluster<kBF16, 1, false, false>;
     const size_t smem = size_t(ctx->smem_optin) / 2 + 1024;
     if (ensure_smem(ctx, kern, smem, true) != CFGZIP_OK) return;
@@ -219,6 +230,7 @@ void find_cluster_limits(cfgzip_ctx* ctx) {
             ctx->cluster_limit[n] = 0;
         }
     }
+    std::copy(std::begin(ctx->cluster_limit), std::end(ctx->cluster_limit), known[ctx->device].begin());
 }
 
 int check_partition_host(const int32_t* c, int32_t V, const int32_t* r, int32_t K) {
@@ -1263,11 +1275,11 @@ int cfgzip_create(int device, cfgzip_ctx** out) {
             cudaGetLastError();
     }
     bool ok = cudaMalloc(&ctx->d_parts, kMaxParts * sizeof(PartDev)) == cudaSuccess &&
-              cudaMalloc(&ctx->d_partials, kPartialSlots * sizeof(Partial)) == cudaSuccess &&
-              cudaMalloc(&ctx->d_chunk_max, kChunkMaxSlots * sizeof(float)) == cudaSuccess &&
+              cudaMalloc(&ctx->d_partials, kPartialSlots * sizeof(Partial) + kChunkMaxSlots * sizeof(float)) == cudaSuccess &&
               cudaMalloc(&ctx->d_status, 8 * sizeof(int32_t)) == cudaSuccess &&
               cudaMalloc(&ctx->d_n_groups, sizeof(int32_t)) == cudaSuccess;
     if (ok) {
+        ctx->d_chunk_max = reinterpret_cast<float*>(ctx->d_partials + kPartialSlots);
         cudaMemset(ctx->d_parts, 0, kMaxParts * sizeof(PartDev));
         cudaMemset(ctx->d_status, 0, 8 * sizeof(int32_t));
         cudaMemset(ctx->d_n_groups, 0, sizeof(int32_t));
@@ -1292,7 +1304,6 @@ int cfgzip_destroy(cfgzip_ctx* ctx) {
     cudaFree(ctx->spare_block);
     cudaFree(ctx->d_parts);
     cudaFree(ctx->d_partials);
-    cudaFree(ctx->d_chunk_max);
     cudaFree(ctx->d_tickets);
     cudaFree(ctx->d_status);
     cudaFree(ctx->d_group_part);
