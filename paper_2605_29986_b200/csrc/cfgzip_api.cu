@@ -807,15 +807,20 @@ struct ClusterPlan {
     size_t smem = 0;
     unsigned grid = 0;
 };
-ClusterPlan plan_cluster(const cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, int elem_size, bool shifted, bool sampling) {
+ClusterPlan plan_cluster(const cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, int elem_size, bool shifted, bool sampling,
+                         bool full) {
     ClusterPlan best;
+    // beyond this much work for a warp two launches are as fast (80 rows of 128256 bf16 13.3 and 13.2 us; sampling 64 of 151937 17.0, 16.1)
+    const double most = full ? 1e9 : sampling ? 24. : 30.;
     if (!ps.all_c16 || !ctx->one_launch) return best;
     if (B > kGroupRows && (mixed || int64_t(ps.V) * elem_size < 128 * 1024)) return best;
     double least = 0.;
     for (int r = 1; r <= (mixed ? 1 : kClusterRows); ++r) {
         const int clusters = ceil_div(B, r);
         for (int n = 2; n <= kClusterMost; ++n) {  // (one block is no cluster: there is nothing to send)
-            if (clusters > ctx->cluster_limit[n]) continue;
+            // Clusters of 3 and 5 leave SMs over wherever they are placed; those of the next step, which come while this one runs, take the
+            // room of others up (24 x 5 blocks 7.8 us a step, 23 x 5 4.6; a spin of 4.7 us takes 4.9 in 25 x 5 blocks, 5.9 in 26 x 5 and 45 x 3).
+            if (clusters > ctx->cluster_limit[n] - (n == 3 || n == 5 ? 3 : 0)) continue;
             ClusterPlan c;
             c.g.rows = r;
             c.g.blocks = n;
@@ -825,7 +830,7 @@ ClusterPlan plan_cluster(const cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bo
             c.smem = size_t(cluster_table_bytes(ps.maxKW)) + size_t(kClusterWarps) * cluster_warp_bytes(c.g.run, r, 8 * elem_size);
             if (chunks > kClusterChunks || c.smem > size_t(ctx->smem_optin) - kClusterStatic) continue;
             const double cost = chunks * ((shifted || sampling ? 0.4 : 1.0) + r) + 0.2 * n;
-            if (best.ok && cost >= least) continue;
+            if ((best.ok && cost >= least) || cost > most) continue;
             least = cost;
             // (more than half of an SM's shared memory, so that a block has its SM to itself)
             c.smem = std::max(c.smem, size_t(ctx->smem_optin) / 2 + 1024);
@@ -864,7 +869,7 @@ int launch_fused(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, in
     DensePlan few;
     if (mode != CFGZIP_SPARSE && !(mode == CFGZIP_AUTO && ctx->auto_min_bytes >= 0) &&
         (aligned || aligned_elems(a.logits, DT == kBF16 ? 2 : 4))) {
-        ClusterPlan cl = plan_cluster(ctx, ps, a.B, mixed, DT == kBF16 ? 2 : 4, !aligned, false);
+        ClusterPlan cl = plan_cluster(ctx, ps, a.B, mixed, DT == kBF16 ? 2 : 4, !aligned, false, logp_full != nullptr);
         cl.g.full = logp_full;
         cl.g.quads = a.V % 4 == 0 && (reinterpret_cast<uintptr_t>(logp_full) & 15u) == 0;
         if (cl.ok && launch_cluster<DT>(ctx, a, cl, mixed, !aligned, st) == CFGZIP_OK) return CFGZIP_OK;
@@ -986,7 +991,7 @@ int launch_sample(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, b
     const bool filtered = top_k > 0 || top_p < 1.f;  // the draw is restricted to the most probable tokens
     int rc;
     if (!filtered && (aligned || aligned_elems(a.logits, DT == kBF16 ? 2 : 4))) {
-        const ClusterPlan cl = plan_cluster(ctx, ps, a.B, mixed, DT == kBF16 ? 2 : 4, !aligned, true);
+        const ClusterPlan cl = plan_cluster(ctx, ps, a.B, mixed, DT == kBF16 ? 2 : 4, !aligned, true, false);
         if (cl.ok && launch_cluster<DT>(ctx, a, cl, mixed, !aligned, st) == CFGZIP_OK) return CFGZIP_OK;
     }
     const bool cm_bulk_ok = (reinterpret_cast<uintptr_t>(a.class_mask) & 15u) == 0 && (a.cm_stride & 3) == 0;
