@@ -453,15 +453,36 @@ DensePlan plan_pipe_opl(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixe
     // Warps go side by side along the vocabulary first (long contiguous runs per row are kind to
     // DRAM); only when a block has fewer chunks than warps do warps split the row batches.
     const int chunks = ceil_div(per, chunk_octets);
+    const int batch_rows = std::min<int>(B, kGroupRows), groups = ceil_div(B, kGroupRows);
     int WR = ctx->row_warps;
     if (!WR) {
         WR = 1;
         while (WR < 4 && chunks * WR * 2 <= n_warps) WR <<= 1;
     }
-    while (WR > 1 && (WR - 1) * kBatchRows >= std::min<int>(B, kGroupRows)) WR >>= 1;
+    while (WR > 1 && (WR - 1) * kBatchRows >= batch_rows) WR >>= 1;
     if ((WR != 1 && WR != 2 && WR != 4)) WR = 1;
     d.WT = ctx->token_warps ? ctx->token_warps : n_warps / WR;
     d.WT = std::max(1, std::min(std::min(d.WT, max_warps / WR), chunks));
+    // Where a warp has a handful of work items, what counts is how many the busiest has, how many warps share the schedulers, and
+    // how often a warp opens and publishes a row batch. Time of an item with w warps in the block 0.6 + 0.118 w us (w counted in
+    // fours, a scheduler each), of a row batch 0.48, 0.3 where a row has more states than a warp folds: fitted to 128 bf16 rows of
+    // 128256, it orders the shapes of 18 other batches as measured or within 2 %. Rows by the vocabulary / as chosen, us: bf16 of
+    // 128256 96 rows 16.3 / 14.9, 128 19.0 / 17.2, 256 28.6 / 27.7, 100 rows of 100003 21.7 / 17.9, 80 of 256000 26.3 / 23.6; f32 of 128256
+    // 34 rows 15.3 / 13.4, 150 33.1 / 32.2. Longer steps are bound by DRAM, which likes the long runs better (f32 of 128256, 300 rows 57.0,
+    // split 59.2; 200 rows of 64064 20.8, split 21.5), and a mixed batch may have few row batches in a group.
+    if (!ctx->row_warps && !ctx->token_warps && !mixed && opl == 1 && groups <= (elem_size == 2 ? 8 : 5)) {
+        const int n_chunks = std::max(1, ceil_div(ps.V >> 3, chunk_octets)), S = ceil_div(n_oct, per), batches = ceil_div(batch_rows, kBatchRows);
+        double least = 0.;
+        for (int wr = 1; wr <= 4 && (wr == 1 || (wr - 1) * kBatchRows < batch_rows); wr <<= 1)
+            for (int wt = std::min(n_warps / wr, chunks); wt >= 1; --wt) {
+                const int turns = ceil_div(batches, wr), items = ceil_div(int64_t(turns) * n_chunks, int64_t(S) * wt);
+                const double cost = items * (0.6 + 0.118 * (4 * ceil_div(wt * wr, 4))) + 0.48 * turns + (S * wt + 1 > kFinalizeWarpStates ? 0.3 : 0.);
+                if (least > 0. && cost >= least) continue;
+                least = cost;
+                d.WT = wt;
+                WR = wr;
+            }
+    }
     d.threads = d.WT * WR * 32;
     // The groups of a mixed batch may hold 32 rows or one, and only the GPU knows how many there are: where there are blocks
     // enough it gives every group the same number if the groups are the fewest the batch can have (336 bf16 rows of 128256 in two
