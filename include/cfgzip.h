@@ -56,7 +56,7 @@ enum {
 const char* cfgzip_status_string(int status);
 
 /*
- * Create a context on CUDA device `device`. Allocates the scratch area (some 8 MB)
+ * Create a context on CUDA device `device`. Allocates the scratch area (a few MB)
  * and row-plan buffers for up to 16384 rows per call (see cfgzip_reserve_rows).
  * Fails with CFGZIP_E_CUDA when no usable device exists: there is no CPU fallback.
  */

@@ -36,7 +36,6 @@ struct Part {
 
 constexpr size_t kSpareBytes = size_t(32) << 20;  // most memory of a released partition a context keeps for the next one
 constexpr size_t kPartialSlots = size_t(1) << 18;  // 4 MB of (max, sum, pos) slots
-constexpr size_t kChunkMaxSlots = size_t(1) << 20;  // 4 MB of chunk maxima (rows x chunks of a sampling step with top-k)
 constexpr int kTwoOctetItemsPerWarp = 3;           // bf16: two octets per lane from this many work items per warp on
 constexpr int kDefaultRows = 16384;
 
@@ -60,7 +59,6 @@ struct cfgzip_ctx {
     size_t spare_bytes = 0;
     PartDev* d_parts = nullptr;
     Partial* d_partials = nullptr;
-    float* d_chunk_max = nullptr;  // behind the states, in the same block
     unsigned int* d_tickets = nullptr;  // reserved_rows entries
     int32_t* d_status = nullptr;        // 4 counters, and 4 that nobody reads (see uncounted)
     bool uncounted = false;             // set around a launch that repeats what another launch of the same call counts
@@ -332,10 +330,8 @@ size_t pipe_smem_bytes(int table_words, int n_warps, int depth, int stage_bytes,
            (alias ? std::max(rings, staging) : rings + staging);
 }
 
-// Launch shape of the register-based dense kernels.
-// units: octets (fused) or 32-token words (expand); unit_chunk: units one warp covers per iteration.
-DensePlan plan_dense(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, int units, int unit_chunk,
-                     bool fused) {
+// Launch shape of the register-based dense kernel. units: octets; unit_chunk: units one warp covers per iteration.
+DensePlan plan_dense(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, int units, int unit_chunk) {
     DensePlan d;
     d.table_words = (ps.maxKW + 1) * 32;
     d.use_plan_kernel = mixed;
@@ -351,26 +347,40 @@ DensePlan plan_dense(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, 
     const int n_chunks = ceil_div(units, unit_chunk);
     const int s0 = std::max(1, target / d.n_groups_ub);
     int cps = ceil_div(n_chunks, s0);  // chunks per block
-    int WR = 1;
-    if (fused) {
-        WR = ctx->row_warps ? ctx->row_warps : (cps <= 2 ? 4 : 1);
-        if (WR != 1 && WR != 2 && WR != 4) WR = 1;
-        d.WT = ctx->token_warps ? ctx->token_warps : (WR == 4 ? std::min(cps, 2) : (WR == 2 ? 2 : 4));
-        d.WT = std::max(1, std::min(d.WT, 8 / WR));
-        d.threads = d.WT * WR * 32;
-    } else {
-        d.WT = 8;
-        d.threads = 256;
-    }
+    int WR = ctx->row_warps ? ctx->row_warps : (cps <= 2 ? 4 : 1);
+    if (WR != 1 && WR != 2 && WR != 4) WR = 1;
+    d.WT = ctx->token_warps ? ctx->token_warps : (WR == 4 ? std::min(cps, 2) : (WR == 2 ? 2 : 4));
+    d.WT = std::max(1, std::min(d.WT, 8 / WR));
+    d.threads = d.WT * WR * 32;
     for (;;) {
         d.S = ceil_div(n_chunks, cps);
-        if (!fused || size_t(d.n_groups_ub) * kGroupRows * (size_t(d.S) * d.WT + 1) <= kPartialSlots) break;
+        if (size_t(d.n_groups_ub) * kGroupRows * (size_t(d.S) * d.WT + 1) <= kPartialSlots) break;
         if (cps >= n_chunks) return d;
         cps *= 2;
     }
     d.per_split = cps * unit_chunk;
     d.slots = d.S * d.WT + 1;
-    d.smem = dense_smem_bytes(d.table_words, fused ? d.threads / 32 : 0, d.stage_stride);
+    d.smem = dense_smem_bytes(d.table_words, d.threads / 32, d.stage_stride);
+    d.ok = true;
+    return d;
+}
+
+// Launch shape of the expansion alone: two blocks to an SM, so that a class table serves many tokens.
+DensePlan plan_expand(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, bool cm_quads) {
+    DensePlan d;
+    d.table_words = (ps.maxKW + 1) * 32;
+    d.use_plan_kernel = mixed;
+    d.n_groups_ub = mixed ? ceil_div(B, kGroupRows) + ps.n_live_same_v : ceil_div(B, kGroupRows);
+    const size_t table = dense_smem_bytes(d.table_words, 0, 0);
+    if (!ps.all_c16 || table > size_t(ctx->smem_optin) - 2048) return d;
+    if (mixed && (B > ctx->reserved_rows || d.n_groups_ub > ctx->max_groups)) return d;
+    d.cm_bulk = cm_quads;
+    if (!cm_quads && dense_smem_bytes(d.table_words, 0, ps.maxKW | 1) <= 100 * 1024) d.stage_stride = ps.maxKW | 1;
+    d.smem = dense_smem_bytes(d.table_words, 0, d.stage_stride);
+    const int n_units = ceil_div(ps.VW, 16), per_sm = d.smem > size_t(ctx->smem_optin) / 2 - 2048 ? 1 : 2;
+    d.per_split = ceil_div(n_units, std::max(1, per_sm * ctx->sm_count / d.n_groups_ub));
+    d.S = ceil_div(n_units, d.per_split);
+    d.threads = kExpandThreads;
     d.ok = true;
     return d;
 }
@@ -920,7 +930,7 @@ int launch_fused(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, in
         const bool cm_bulk_ok = (reinterpret_cast<uintptr_t>(a.class_mask) & 15u) == 0 && (a.cm_stride & 3) == 0;
         DensePlan d = plan_pipe(ctx, ps, a.B, mixed, DT == kBF16 ? 2 : 4, cm_bulk_ok, !aligned);
         if (d.shifted && !aligned_elems(a.logits, DT == kBF16 ? 2 : 4)) d.ok = false;
-        if (!d.ok && aligned) d = plan_dense(ctx, ps, a.B, mixed, 4 * ps.VW, 32, true);
+        if (!d.ok && aligned) d = plan_dense(ctx, ps, a.B, mixed, 4 * ps.VW, 32);
         if (d.ok) {
             if (d.use_plan_kernel && (rc = run_plan_kernel(ctx, a.row_part, a.B, a.V, d, st)) != CFGZIP_OK) return rc;
             // Automatic mode on a long step: the class-list kernel runs first, keeps the row batches (the 8 rows the
@@ -1031,9 +1041,10 @@ int launch_sample(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, b
         // With top_k the streaming kernel also leaves the largest logit of every chunk: the draw then reads the chunks that reach its
         // bar, some fifty, and not the row again (us, top-k 50 and top-p 0.9, bf16: 64 rows of 151936 28.5 -> 23.7, 512 of 128256 95 -> 74,
         // 100 of 256000 54 -> 39; 200 f32 rows of 100003 off the vector grid 79 -> 52; 8 rows of 32064 15.0 -> 14.9). Its price in the
-        // streaming kernel, a reduction per row and chunk, is not paid by a step without top_k.
-        if (top_k > 0 && n_chunks <= kFiltMaxima && size_t(a.B) * size_t(n_chunks) <= kChunkMaxSlots) {
-            a.chunk_max = ctx->d_chunk_max;
+        // streaming kernel, a reduction per row and chunk, is not paid by a step without top_k. They lie behind the states.
+        const size_t states = size_t(d.n_groups_ub) * kGroupRows * d.slots;
+        if (top_k > 0 && n_chunks <= kFiltMaxima && states * sizeof(Partial) + size_t(a.B) * size_t(n_chunks) * sizeof(float) <= kPartialSlots * sizeof(Partial)) {
+            a.chunk_max = reinterpret_cast<float*>(ctx->d_partials + states);
             a.n_chunks = n_chunks;
         }
         const dim3 grid(d.blocks ? unsigned(d.blocks) : unsigned(d.n_groups_ub) * unsigned(d.S)), block{unsigned(d.threads)};
@@ -1301,11 +1312,10 @@ int cfgzip_create(int device, cfgzip_ctx** out) {
             cudaGetLastError();
     }
     bool ok = cudaMalloc(&ctx->d_parts, kMaxParts * sizeof(PartDev)) == cudaSuccess &&
-              cudaMalloc(&ctx->d_partials, kPartialSlots * sizeof(Partial) + kChunkMaxSlots * sizeof(float)) == cudaSuccess &&
+              cudaMalloc(&ctx->d_partials, kPartialSlots * sizeof(Partial)) == cudaSuccess &&
               cudaMalloc(&ctx->d_status, 8 * sizeof(int32_t)) == cudaSuccess &&
               cudaMalloc(&ctx->d_n_groups, sizeof(int32_t)) == cudaSuccess;
     if (ok) {
-        ctx->d_chunk_max = reinterpret_cast<float*>(ctx->d_partials + kPartialSlots);
         cudaMemset(ctx->d_parts, 0, kMaxParts * sizeof(PartDev));
         cudaMemset(ctx->d_status, 0, 8 * sizeof(int32_t));
         cudaMemset(ctx->d_n_groups, 0, sizeof(int32_t));
@@ -1512,12 +1522,14 @@ int cfgzip_expand_mask(cfgzip_ctx* ctx, cfgzip_part_id part0, const int32_t* row
         }
         return launch(ctx, k_step_generic<kF32, false>, dim3(unsigned(B)), dim3(256), 0, st, a);
     }
-    const DensePlan d = plan_dense(ctx, ps, B, mixed, ps.VW, 8, false);
-    if (!d.ok) return launch(ctx, k_step_generic<kF32, false>, dim3(unsigned(B)), dim3(256), 0, st, a);
+    const bool cm_quads = (reinterpret_cast<uintptr_t>(class_mask) & 15u) == 0 && (class_stride_words & 3) == 0 && ps.all_kw_mult4;
+    const DensePlan d = plan_expand(ctx, ps, B, mixed, cm_quads);
+    if (!d.ok || vocab_stride_words * 4 >= (int64_t(1) << 32)) return launch(ctx, k_step_generic<kF32, false>, dim3(unsigned(B)), dim3(256), 0, st, a);
     if (d.use_plan_kernel && (rc = run_plan_kernel(ctx, row_part, B, ps.V, d, st)) != CFGZIP_OK) return rc;
     fill_groups(ctx, a, d);
-    if ((rc = ensure_smem(ctx, k_expand_dense, d.smem)) != CFGZIP_OK) return rc;
-    return launch(ctx, k_expand_dense, dim3(unsigned(d.n_groups_ub) * unsigned(d.S)), dim3(256), d.smem, st, a);
+    auto kern = d.use_plan_kernel ? k_expand_dense<true> : k_expand_dense<false>;
+    if ((rc = ensure_smem(ctx, kern, d.smem)) != CFGZIP_OK) return rc;
+    return launch(ctx, kern, dim3(unsigned(d.n_groups_ub) * unsigned(d.S)), dim3(kExpandThreads), d.smem, st, a);
 }
 
 int cfgzip_mask_logits(cfgzip_ctx* ctx, void* logits, int dtype, int64_t row_stride_elems, int32_t B, int32_t V,
@@ -1707,7 +1719,7 @@ int cfgzip_multi_mask_logsoftmax_argmax(cfgzip_ctx* ctx, cfgzip_part_id part0, c
     if (masks_per_row > 1) d = plan_multi(ctx, ps, B, masks_per_row, es);
     const bool shared = d.ok;
     // nothing to share (64 rows with one mask each: 17.3 against 19.2 us) or too little, or a class table that leaves no room beside it
-    if (!shared) d = plan_dense(ctx, ps, rows, false, 4 * ps.VW, 32, true);
+    if (!shared) d = plan_dense(ctx, ps, rows, false, 4 * ps.VW, 32);
     if (!d.ok) return CFGZIP_E_RANGE;  // more than 65535 classes, or a class table beyond shared memory
     fill_groups(ctx, a, d);
     ctx->pdl_now = int64_t(B) * ps.V * es < (int64_t(192) << 20);
@@ -1757,7 +1769,7 @@ int cfgzip_map_tokens(cfgzip_ctx* ctx, cfgzip_part_id part0, const int32_t* row_
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return CFGZIP_E_CUDA;
     return launch(ctx, k_map_tokens, dim3(unsigned(ceil_div(B, 256))), dim3(256), 0, static_cast<cudaStream_t>(stream),
-                  (const PartDev*)ctx->d_parts, int(ctx->parts.size()), int(part0), row_part, tokens, reps, int(B),
+                  (const PartDev*)ctx->d_parts, int(ctx->parts.size()), ctx->parts[size_t(part0)].dev, row_part, tokens, reps, int(B),
                   int(ps.V), ctx->d_status);
 }
 
@@ -2128,7 +2140,7 @@ extern "C" int cfgzip_plan_query(int32_t sm_count, int32_t smem_optin, int32_t V
     DensePlan d = plan_pipe(&fake, ps, B, mixed, es, aligned_class_masks != 0);
     int kind = 2;  // pipelined
     if (!d.ok) {
-        d = plan_dense(&fake, ps, B, mixed, 4 * ps.VW, 32, true);
+        d = plan_dense(&fake, ps, B, mixed, 4 * ps.VW, 32);
         kind = 1;  // register kernel
     }
     if (!d.ok) kind = 0;  // per-row kernel

@@ -1390,50 +1390,112 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
 }
 
 // ---------------------------------------------------------------------------------------
-// Dense expansion only. Same row groups and class table as the fused kernel; a lane takes the octet of tokens next to its
-// neighbours', looks up its 8 class words once, turns them into one byte per row (four 8x8 bit transposes for the 32 rows)
-// and stores the bytes: 32 bytes side by side per row and warp. per_split counts 32-token words.
-// Bound: the table is built once per block, so few, long blocks; then instruction issue, some 160 instructions per 256 tokens
-// and 32 rows. (A ballot per token word and row took 850: 512 rows of 128256 tokens 37 us, now 14.)
+// Dense expansion only. Same row groups and class table as the fused kernel; a lane takes sixteen tokens next to its
+// neighbours', looks up their class words once, turns them into two bytes per row (eight 8x8 bit transposes for the 32 rows)
+// and stores these: 64 bytes side by side per row and warp. per_split counts units of 32 lanes. The class table straight from
+// the masks, four words of a row to a lane, where their alignment allows, else by way of shared memory.
+// Bound: the chain launch - class masks - table - lookups - stores for all but large batches, and for those instruction issue, some
+// 350 instructions per 512 tokens and 32 rows. (Eight tokens a lane, a table for every quarter of an SM and an address from
+// scratch for every row took 1070 with the tables: 512 rows of 128256 tokens 15.1 us, now 7.0; 40 rows of
+// 200064 in 16384 classes with masking and mapping 56, now 21.)
 // ---------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_expand_dense(const __grid_constant__ StepArgs a) {
+constexpr int kExpandThreads = 512, kExpandWarps = kExpandThreads / 32;
+
+__device__ __forceinline__ void build_class_table_direct(const StepArgs& a, const PartDev& P, const int* s_row, uint32_t* T, int warp,
+                                                         int lane, int n_warps) {
+    const uint32_t tail = (P.K & 31) ? (1u << (P.K & 31)) - 1u : 0xFFFFFFFFu;
+    const int row = s_row[lane];
+    const uint4* const cm = reinterpret_cast<const uint4*>(a.class_mask + int64_t(row < 0 ? 0 : row) * a.cm_stride);
+    constexpr int U = 2;
+    for (int q0 = warp; 4 * q0 < P.KW; q0 += U * n_warps) {
+        uint4 x[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int q = q0 + u * n_warps;
+            x[u] = row >= 0 && 4 * q < P.KW ? __ldg(cm + q) : make_uint4(0, 0, 0, 0);
+            if (4 * q + 4 == P.KW) x[u].w &= tail;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int q = q0 + u * n_warps;
+            if (4 * q >= P.KW) break;
+            uint32_t* const dst = T + q * 128 + lane;
+            dst[0] = warp_transpose32(x[u].x, lane);
+            dst[32] = warp_transpose32(x[u].y, lane);
+            dst[64] = warp_transpose32(x[u].z, lane);
+            dst[96] = warp_transpose32(x[u].w, lane);
+        }
+    }
+    if (warp == 0) T[P.KW * 32 + lane] = 0u;  // the padding class
+}
+
+// PLANNED: the row groups come from a row plan; else they are 32 consecutive rows each.
+template <bool PLANNED>
+__global__ void __launch_bounds__(kExpandThreads, 2) k_expand_dense(const __grid_constant__ StepArgs a) {
     extern __shared__ __align__(128) uint32_t smem[];
     uint32_t* T = smem;
     int* s_row = reinterpret_cast<int*>(T + a.table_words);
     uint32_t* stage = reinterpret_cast<uint32_t*>(s_row + kGroupRows);
 
-    pdl_prologue();
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, n_warps = blockDim.x >> 5;
+    pdl_launch_dependents();
+    if (PLANNED) pdl_wait();
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = blockIdx.x / a.S, split = blockIdx.x - g * a.S;
-    if (a.n_groups && g >= __ldg(a.n_groups)) return;
+    if (PLANNED && g >= __ldg(a.n_groups)) return;
     const int part = group_rows_setup(a, g, s_row, tid);
     __syncthreads();
-    const PartDev P = a.group_part ? a.parts[part] : a.p0;
-    const int nrow = __popc(__ballot_sync(0xFFFFFFFFu, s_row[lane] >= 0));
-    if (a.stage_stride) {
-        stage_class_masks(a, P, s_row, stage, warp, lane, n_warps);
-        __syncthreads();
+    const PartDev P = PLANNED ? a.parts[part] : a.p0;
+    const int nrow = PLANNED ? __popc(__ballot_sync(0xFFFFFFFFu, s_row[lane] >= 0)) : min(kGroupRows, a.B - g * kGroupRows);
+    const int n_octets = 4 * a.VW, u_end = min((split + 1) * a.per_split, (n_octets + 63) >> 6);
+    int unit = split * a.per_split + warp;
+    const uint4* const ids = reinterpret_cast<const uint4*>(P.c16);  // padded to 32 * VW entries
+    uint4 c0 = make_uint4(0, 0, 0, 0), c1 = c0;
+    auto fetch = [&](int u) {
+        const int o = u * 64 + lane * 2;
+        if (u < u_end && o < n_octets) {
+            c0 = __ldg(ids + o);
+            c1 = __ldg(ids + o + 1);
+        }
+    };
+    fetch(unit);
+    if (!PLANNED) pdl_wait();
+    if (a.cm_bulk) {
+        build_class_table_direct(a, P, s_row, T, warp, lane, kExpandWarps);
+    } else {
+        if (a.stage_stride) {
+            stage_class_masks(a, P, s_row, stage, warp, lane, kExpandWarps);
+            __syncthreads();
+        }
+        build_class_table(a, P, s_row, T, stage, warp, lane, kExpandWarps);
     }
-    build_class_table(a, P, s_row, T, stage, warp, lane, n_warps);
     __syncthreads();
 
-    const int o_begin = 4 * split * a.per_split, o_end = min(o_begin + 4 * a.per_split, 4 * a.VW);  // octets
     uint8_t* const vm8 = reinterpret_cast<uint8_t*>(a.vocab_mask);
-    for (int o0 = o_begin + warp * 32; o0 < o_end; o0 += n_warps * 32) {
-        const int o = o0 + lane;
-        if (o >= o_end) continue;
-        const uint4 cv = __ldg(reinterpret_cast<const uint4*>(P.c16) + o);  // padded to 32 * VW entries
-        const uint32_t w[8] = {T[cv.x & 0xFFFFu], T[cv.x >> 16], T[cv.y & 0xFFFFu], T[cv.y >> 16],
-                               T[cv.z & 0xFFFFu], T[cv.z >> 16], T[cv.w & 0xFFFFu], T[cv.w >> 16]};
+    const uint32_t vm_bytes = uint32_t(a.vm_stride * 4);
+    for (; unit < u_end; unit += kExpandWarps) {
+        const int o = unit * 64 + lane * 2;
+        const bool active = o < n_octets;
+        const uint4 i0 = c0, i1 = c1;
+        fetch(unit + kExpandWarps);
+        if (!active) continue;
+        const uint32_t w0[8] = {T[i0.x & 0xFFFFu], T[i0.x >> 16], T[i0.y & 0xFFFFu], T[i0.y >> 16],
+                                T[i0.z & 0xFFFFu], T[i0.z >> 16], T[i0.w & 0xFFFFu], T[i0.w >> 16]};
+        const uint32_t w1[8] = {T[i1.x & 0xFFFFu], T[i1.x >> 16], T[i1.y & 0xFFFFu], T[i1.y >> 16],
+                                T[i1.z & 0xFFFFu], T[i1.z >> 16], T[i1.w & 0xFFFFu], T[i1.w >> 16]};
+        char* const first = reinterpret_cast<char*>(vm8 + int64_t(g * kGroupRows) * a.vm_stride * 4 + o);
 #pragma unroll
         for (int rb = 0; rb < kGroupRows / kBatchRows; ++rb) {
             if (rb * kBatchRows >= nrow) break;
-            uint32_t lo, hi;
-            row_batch_bytes(w, rb, lo, hi);
+            uint32_t lo0, hi0, lo1, hi1;
+            row_batch_bytes(w0, rb, lo0, hi0);
+            row_batch_bytes(w1, rb, lo1, hi1);
 #pragma unroll
             for (int i = 0; i < kBatchRows; ++i) {
                 const int r = rb * kBatchRows + i;
-                if (r < nrow) st_global_u8(vm8 + int64_t(s_row[r]) * a.vm_stride * 4 + o, ((i < 4 ? lo : hi) >> (8 * (i & 3))) & 0xFFu);
+                if (r >= nrow) break;
+                const uint32_t two = prmt(i < 4 ? lo0 : hi0, i < 4 ? lo1 : hi1, uint32_t(i & 3) | (uint32_t(4 + (i & 3)) << 4));
+                char* const dst = PLANNED ? reinterpret_cast<char*>(vm8 + int64_t(s_row[r]) * a.vm_stride * 4 + o) : ptr_mad(first, uint32_t(r), vm_bytes);
+                st_global_u16(dst, two);
             }
         }
     }
@@ -2460,20 +2522,25 @@ __global__ void __launch_bounds__(256) k_logp_full(const void* logits, int64_t r
 }
 
 // reps[b] = r[c[tokens[b]]]
-__global__ void __launch_bounds__(256) k_map_tokens(const PartDev* parts, int n_parts, int part0, const int32_t* row_part,
-                                                    const int32_t* tokens, int32_t* reps, int B, int V_expected,
-                                                    int32_t* status) {
+// one: the partition of all rows, as an argument (a look less in the chain: token, representative); else parts[row_part[b]].
+__global__ void __launch_bounds__(256) k_map_tokens(const PartDev* parts, int n_parts, const __grid_constant__ PartDev one,
+                                                    const int32_t* row_part, const int32_t* tokens, int32_t* reps, int B,
+                                                    int V_expected, int32_t* status) {
     pdl_prologue();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= B) return;
-    const int p = row_part ? row_part[b] : part0;
-    if (p < 0 || p >= n_parts || !parts[p].live || parts[p].V != V_expected) {
-        atomicAdd(status + 2, 1);
-        return;
-    }
+    const int32_t* trep = one.trep;
     const int t = tokens[b];
+    if (row_part) {
+        const int p = row_part[b];
+        if (p < 0 || p >= n_parts || !parts[p].live || parts[p].V != V_expected) {
+            atomicAdd(status + 2, 1);
+            return;
+        }
+        trep = parts[p].trep;
+    }
     int rv = -1;
-    if (t >= 0 && t < parts[p].V) rv = parts[p].trep[t];
+    if (t >= 0 && t < V_expected) rv = trep[t];
     else atomicAdd(status + 1, 1);
     reps[b] = rv;
 }
