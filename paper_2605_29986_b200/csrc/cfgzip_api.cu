@@ -330,18 +330,28 @@ size_t pipe_smem_bytes(int table_words, int n_warps, int depth, int stage_bytes,
            (alias ? std::max(rings, staging) : rings + staging);
 }
 
+// Words between the rows of the class masks' staging area where these are not copied or read directly.
+int slice_stride(const PartSet& ps) { return std::min(ps.maxKW, kMaskSlice) | 1; }
+// How a call's class masks can be fetched (kMasks..).
+int masks_kind(const PartSet& ps, const uint32_t* class_mask, int64_t stride, bool mixed, bool block) {
+    if (reinterpret_cast<uintptr_t>(class_mask) & 15u) return kMasksStaged;
+    if ((stride & 3) == 0) return ps.all_kw_mult4 ? kMasksRows : kMasksStaged;
+    return block && !mixed && stride <= ps.maxKW + 64 ? kMasksBlock : kMasksStaged;
+}
+
 // Launch shape of the register-based dense kernel. units: octets; unit_chunk: units one warp covers per iteration.
-DensePlan plan_dense(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, int units, int unit_chunk) {
+DensePlan plan_dense(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, int units, int unit_chunk, int masks) {
     DensePlan d;
     d.table_words = (ps.maxKW + 1) * 32;
     d.use_plan_kernel = mixed;
     d.n_groups_ub = mixed ? ceil_div(B, kGroupRows) + ps.n_live_same_v : ceil_div(B, kGroupRows);
     if (!ps.all_c16) return d;
-    if (dense_smem_bytes(d.table_words, 8, 0) > size_t(ctx->smem_optin) - 2048) return d;
+    if (dense_smem_bytes(d.table_words, 8, masks ? 0 : slice_stride(ps)) > size_t(ctx->smem_optin) - 2048) return d;
     if (mixed && (B > ctx->reserved_rows || d.n_groups_ub > ctx->max_groups)) return d;
     const int ctas_per_sm = ctx->ctas_per_sm;
-    // stage the class masks through shared memory while that keeps a block under 64 KB
-    if (dense_smem_bytes(d.table_words, 8, ps.maxKW | 1) <= 64 * 1024) d.stage_stride = ps.maxKW | 1;
+    // the class masks through shared memory, all at once while that keeps a block under 64 KB
+    d.cm_bulk = masks;
+    if (!masks) d.stage_stride = dense_smem_bytes(d.table_words, 8, ps.maxKW | 1) <= 64 * 1024 ? ps.maxKW | 1 : slice_stride(ps);
     d.ctas_per_sm = ctas_per_sm;
     const int target = ctx->sm_count * ctas_per_sm;
     const int n_chunks = ceil_div(units, unit_chunk);
@@ -366,16 +376,15 @@ DensePlan plan_dense(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, 
 }
 
 // Launch shape of the expansion alone: two blocks to an SM, so that a class table serves many tokens.
-DensePlan plan_expand(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, bool cm_quads) {
+DensePlan plan_expand(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, int masks) {
     DensePlan d;
     d.table_words = (ps.maxKW + 1) * 32;
     d.use_plan_kernel = mixed;
     d.n_groups_ub = mixed ? ceil_div(B, kGroupRows) + ps.n_live_same_v : ceil_div(B, kGroupRows);
-    const size_t table = dense_smem_bytes(d.table_words, 0, 0);
-    if (!ps.all_c16 || table > size_t(ctx->smem_optin) - 2048) return d;
+    if (!ps.all_c16 || dense_smem_bytes(d.table_words, 0, masks ? 0 : slice_stride(ps)) > size_t(ctx->smem_optin) - 2048) return d;
     if (mixed && (B > ctx->reserved_rows || d.n_groups_ub > ctx->max_groups)) return d;
-    d.cm_bulk = cm_quads;
-    if (!cm_quads && dense_smem_bytes(d.table_words, 0, ps.maxKW | 1) <= 100 * 1024) d.stage_stride = ps.maxKW | 1;
+    d.cm_bulk = masks;
+    if (!masks) d.stage_stride = dense_smem_bytes(d.table_words, 0, ps.maxKW | 1) <= 100 * 1024 ? ps.maxKW | 1 : slice_stride(ps);
     d.smem = dense_smem_bytes(d.table_words, 0, d.stage_stride);
     const int n_units = ceil_div(ps.VW, 16), per_sm = d.smem > size_t(ctx->smem_optin) / 2 - 2048 ? 1 : 2;
     d.per_split = ceil_div(n_units, std::max(1, per_sm * ctx->sm_count / d.n_groups_ub));
@@ -387,7 +396,7 @@ DensePlan plan_expand(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed,
 
 // Launch shape of the pipelined fused kernel. A block takes per_split octets (any number, not only
 // whole 32-octet chunks) of one row group, so that the blocks of a step fill the SMs evenly.
-DensePlan plan_pipe_opl(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, int elem_size, bool cm_bulk_ok, int opl,
+DensePlan plan_pipe_opl(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, int elem_size, int masks, int64_t cm_stride, int opl,
                         bool shifted) {
     DensePlan d;
     d.opl = opl;
@@ -405,8 +414,8 @@ DensePlan plan_pipe_opl(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixe
     // more registers per thread)
     int n_warps = opl == 2 ? std::min(ctx->pipe_warps, 12) : ctx->pipe_warps, depth = ctx->pipe_depth;
     const int max_warps = n_warps;
-    d.cm_bulk = cm_bulk_ok && ps.all_kw_mult4;
-    int stride = d.cm_bulk ? ps.maxKW + (ps.maxKW % 8 == 0 ? 4 : 8) : (ps.maxKW | 1);
+    d.cm_bulk = masks;
+    int stride = masks == kMasksRows ? ps.maxKW + (ps.maxKW % 8 == 0 ? 4 : 8) : masks == kMasksBlock ? int(cm_stride) : slice_stride(ps);
     auto fits = [&](int warps, int stages, bool over_rings) {
         return pipe_smem_bytes(d.table_words, warps, stages, stage_bytes, stride, over_rings) <= cap;
     };
@@ -437,11 +446,11 @@ DensePlan plan_pipe_opl(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixe
         }
         if (w >= std::min(8, max_warps)) {
             n_warps = w;
-        } else {  // no staging: every lane reads its row's class-mask words from global memory
+        } else {  // the class masks word by word, a slice at a time
             n_warps = max_warps;
-            stride = 0;
-            d.cm_bulk = 0;
-            alias = false;
+            stride = slice_stride(ps);
+            d.cm_bulk = kMasksStaged;
+            alias = fits(n_warps, 2, true);
         }
     }
     while (depth > 2 && pipe_smem_bytes(d.table_words, n_warps, depth, stage_bytes, stride, alias) > cap) --depth;
@@ -449,7 +458,6 @@ DensePlan plan_pipe_opl(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixe
         n_warps -= opl == 2 ? 1 : 2;
     size_t smem = pipe_smem_bytes(d.table_words, n_warps, depth, stage_bytes, stride, alias);
     if (smem > cap) return d;
-    if (stride == 0) alias = false;
     d.depth = depth;
     d.stage_stride = stride;
     const int fit = std::max(1, int((cap + 1024) / (smem + 1024)));
@@ -543,11 +551,11 @@ DensePlan plan_pipe_opl(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixe
 // Launch shape of the pipelined fused kernel. bf16 rows may be streamed with one octet (16 bytes) or two octets
 // (32 bytes) per lane and row; two octets halve the per-row bookkeeping but double a work item, so they are taken
 // only when every warp of the launch still gets several items.
-DensePlan plan_pipe(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, int elem_size, bool cm_bulk_ok,
+DensePlan plan_pipe(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, int elem_size, int masks, int64_t cm_stride,
                     bool shifted = false) {
-    const DensePlan one = plan_pipe_opl(ctx, ps, B, mixed, elem_size, cm_bulk_ok, 1, shifted);
+    const DensePlan one = plan_pipe_opl(ctx, ps, B, mixed, elem_size, masks, cm_stride, 1, shifted);
     if (elem_size != 2 || ctx->lane_octets == 1 || shifted) return one;
-    const DensePlan two = plan_pipe_opl(ctx, ps, B, mixed, elem_size, cm_bulk_ok, 2, false);
+    const DensePlan two = plan_pipe_opl(ctx, ps, B, mixed, elem_size, masks, cm_stride, 2, false);
     if (!two.ok) return one;
     if (!one.ok || ctx->lane_octets == 2) return two;
     if (ctx->lane_octets == 0) return one;
@@ -573,23 +581,23 @@ bool few_pays(const cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, i
     const int64_t row_kb = int64_t(ps.V) * elem_size >> 10;
     if (B < 64) return false;
     if (mixed) return ps.maxK <= 3072 && !(row_kb < 96 && d.n_groups_ub > 16);
-    if (!d.stage_stride && (per_sm < 3 || 4 * int64_t(ps.V) < 3 * int64_t(ps.maxK) * d.S)) return false;
+    if (ps.maxK > 5344 && (per_sm < 3 || 4 * int64_t(ps.V) < 3 * int64_t(ps.maxK) * d.S)) return false;
     return !(row_kb < 96 && B > wave / 2) && !(row_kb < 160 && B > 3 * wave / 4 && B <= wave);
 }
 
 // Launch shape of the kernel for rows that allow few tokens: three blocks per SM; warps go side by side along the vocabulary
 // as long as a block has enough chunks for them, else they split the row batches.
-DensePlan plan_few(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, int elem_size) {
+DensePlan plan_few(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, int elem_size, int masks) {
     DensePlan d;
     d.table_words = (ps.maxKW + 1) * 32;
     d.use_plan_kernel = mixed;
     d.n_groups_ub = mixed ? ceil_div(B, kGroupRows) + ps.n_live_same_v : ceil_div(B, kGroupRows);
     if (!ps.all_c16 || (mixed && (B > ctx->reserved_rows || d.n_groups_ub > ctx->max_groups))) return d;
     const size_t fixed = dense_smem_bytes(d.table_words, kFewWarps, 0) + kFewWarps * sizeof(FewWarp);
-    const size_t staging = size_t(ps.maxKW | 1) * kGroupRows * 4;
-    if (fixed > size_t(ctx->smem_optin) - 2048) return d;
-    if (fixed + staging <= 72 * 1024) d.stage_stride = ps.maxKW | 1;  // three blocks per SM still fit
-    d.smem = fixed + (d.stage_stride ? staging : 0);
+    d.cm_bulk = masks;
+    if (!masks) d.stage_stride = fixed + size_t(ps.maxKW | 1) * kGroupRows * 4 <= 72 * 1024 ? ps.maxKW | 1 : slice_stride(ps);  // (three blocks per SM still fit)
+    d.smem = fixed + size_t(d.stage_stride) * kGroupRows * 4;
+    if (d.smem > size_t(ctx->smem_optin) - 2048) return d;
     const int n_chunks = std::max(1, ceil_div(ps.V / (32 / elem_size), 32));
     const int row_batches = ceil_div(std::min<int>(B, kGroupRows), kBatchRows);
     const int per_sm = std::max(1, std::min(3, int(size_t(ctx->smem_optin) / (d.smem + 1024))));
@@ -625,28 +633,27 @@ bool multi_pays(const PartSet& ps, int32_t B, int masks_per_row, int elem_size, 
 // of 128256, K = 2048: 12.6 with four, 9.3 with eight), and on short calls where only four leave room to stage the class masks
 // (K = 8000, 4 x 2: 14.7 against 18); warps split the row batches of a group first, so that a block builds its table for as many
 // chunks as possible.
-DensePlan plan_multi(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, int masks_per_row, int elem_size) {
+DensePlan plan_multi(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, int masks_per_row, int elem_size, int masks,
+                      int64_t cm_stride) {
     const int32_t rows = B * masks_per_row;
     DensePlan d;
     d.table_words = (ps.maxKW + 1) * 32;
     d.n_groups_ub = ceil_div(rows, kGroupRows);
     if (!ps.all_c16) return d;
-    const size_t cap = size_t(ctx->smem_optin) - 2048, staging = size_t(ps.maxKW | 1) * kGroupRows * 4;
+    // (the class masks directly, all at once by way of shared memory where they are short, or a slice at a time)
+    const size_t cap = size_t(ctx->smem_optin) - 2048;
+    d.cm_bulk = masks == kMasksBlock && cm_stride > 2 * kMaskSlice ? kMasksStaged : masks;
+    if (d.cm_bulk == kMasksBlock) d.stage_stride = int(cm_stride);
+    if (d.cm_bulk == kMasksStaged) d.stage_stride = ps.maxKW <= 2 * kMaskSlice ? ps.maxKW | 1 : slice_stride(ps);
     int n_warps = kMultiWarps;
-    auto bytes = [&](int warps) { return dense_smem_bytes(d.table_words, warps, 0) + size_t(warps) * kMultiTable; };
+    auto bytes = [&](int warps) { return dense_smem_bytes(d.table_words, warps, d.stage_stride) + size_t(warps) * kMultiTable; };
     const int n_chunks = std::max(1, ceil_div(ps.V >> 3, 32));
     const int row_batches = ceil_div(rows, kBatchRows);
     const int64_t items = int64_t(n_chunks) * row_batches;
     if (!multi_pays(ps, B, masks_per_row, elem_size, items)) return d;
-    while (n_warps > 4 && (bytes(n_warps) > cap / 2 || 3 * items <= int64_t(ctx->sm_count) * n_warps ||
-                           (items < int64_t(ctx->sm_count) * n_warps && bytes(n_warps) + staging > cap / 2)))
-        n_warps /= 2;
+    while (n_warps > 4 && (bytes(n_warps) > cap / 2 || 3 * items <= int64_t(ctx->sm_count) * n_warps)) n_warps /= 2;
     d.smem = bytes(n_warps);
     if (d.smem > cap) return d;
-    if (d.smem + staging <= cap / 2) {
-        d.stage_stride = ps.maxKW | 1;
-        d.smem += staging;
-    }
     int WR = 1;
     while (WR < 4 && WR * kBatchRows < std::min<int>(rows, kGroupRows)) WR <<= 1;
     d.WT = n_warps / WR;
@@ -905,7 +912,7 @@ int launch_fused(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, in
         cl.g.quads = a.V % 4 == 0 && (reinterpret_cast<uintptr_t>(logp_full) & 15u) == 0;
         if (cl.ok && launch_cluster<DT>(ctx, a, cl, mixed, !aligned, st) == CFGZIP_OK) return CFGZIP_OK;
     }
-    if (aligned && mode == CFGZIP_SPARSE) few = plan_few(ctx, ps, a.B, mixed, DT == kBF16 ? 2 : 4);
+    if (aligned && mode == CFGZIP_SPARSE) few = plan_few(ctx, ps, a.B, mixed, DT == kBF16 ? 2 : 4, masks_kind(ps, a.class_mask, a.cm_stride, mixed, false));
     if (few.ok) {
         if (few.use_plan_kernel && (rc = run_plan_kernel(ctx, a.row_part, a.B, a.V, few, st)) != CFGZIP_OK) return rc;
         fill_groups(ctx, a, few);
@@ -927,10 +934,10 @@ int launch_fused(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, in
             rc = launch(ctx, k_step_generic<DT, true>, dim3(unsigned(a.B)), dim3(256), 0, st, a);
         }
     } else {
-        const bool cm_bulk_ok = (reinterpret_cast<uintptr_t>(a.class_mask) & 15u) == 0 && (a.cm_stride & 3) == 0;
-        DensePlan d = plan_pipe(ctx, ps, a.B, mixed, DT == kBF16 ? 2 : 4, cm_bulk_ok, !aligned);
+        const int masks = masks_kind(ps, a.class_mask, a.cm_stride, mixed, true);
+        DensePlan d = plan_pipe(ctx, ps, a.B, mixed, DT == kBF16 ? 2 : 4, masks, a.cm_stride, !aligned);
         if (d.shifted && !aligned_elems(a.logits, DT == kBF16 ? 2 : 4)) d.ok = false;
-        if (!d.ok && aligned) d = plan_dense(ctx, ps, a.B, mixed, 4 * ps.VW, 32);
+        if (!d.ok && aligned) d = plan_dense(ctx, ps, a.B, mixed, 4 * ps.VW, 32, masks == kMasksRows ? kMasksRows : kMasksStaged);
         if (d.ok) {
             if (d.use_plan_kernel && (rc = run_plan_kernel(ctx, a.row_part, a.B, a.V, d, st)) != CFGZIP_OK) return rc;
             // Automatic mode on a long step: the class-list kernel runs first, keeps the row batches (the 8 rows the
@@ -1025,8 +1032,8 @@ int launch_sample(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, b
         const ClusterPlan cl = plan_cluster(ctx, ps, a.B, mixed, DT == kBF16 ? 2 : 4, !aligned, true, false);
         if (cl.ok && launch_cluster<DT>(ctx, a, cl, mixed, !aligned, st) == CFGZIP_OK) return CFGZIP_OK;
     }
-    const bool cm_bulk_ok = (reinterpret_cast<uintptr_t>(a.class_mask) & 15u) == 0 && (a.cm_stride & 3) == 0;
-    DensePlan d = plan_pipe(ctx, ps, a.B, mixed, DT == kBF16 ? 2 : 4, cm_bulk_ok, !aligned);
+    const int masks = masks_kind(ps, a.class_mask, a.cm_stride, mixed, true);
+    DensePlan d = plan_pipe(ctx, ps, a.B, mixed, DT == kBF16 ? 2 : 4, masks, a.cm_stride, !aligned);
     if (d.ok && d.depth && !(d.shifted && !aligned_elems(a.logits, DT == kBF16 ? 2 : 4))) {
         if (d.use_plan_kernel && (rc = run_plan_kernel(ctx, a.row_part, a.B, a.V, d, st)) != CFGZIP_OK) return rc;
         // a sampling step keeps one state per warp slot in token order and a kernel of its own for the draw
@@ -1522,8 +1529,7 @@ int cfgzip_expand_mask(cfgzip_ctx* ctx, cfgzip_part_id part0, const int32_t* row
         }
         return launch(ctx, k_step_generic<kF32, false>, dim3(unsigned(B)), dim3(256), 0, st, a);
     }
-    const bool cm_quads = (reinterpret_cast<uintptr_t>(class_mask) & 15u) == 0 && (class_stride_words & 3) == 0 && ps.all_kw_mult4;
-    const DensePlan d = plan_expand(ctx, ps, B, mixed, cm_quads);
+    const DensePlan d = plan_expand(ctx, ps, B, mixed, masks_kind(ps, class_mask, class_stride_words, mixed, false));
     if (!d.ok || vocab_stride_words * 4 >= (int64_t(1) << 32)) return launch(ctx, k_step_generic<kF32, false>, dim3(unsigned(B)), dim3(256), 0, st, a);
     if (d.use_plan_kernel && (rc = run_plan_kernel(ctx, row_part, B, ps.V, d, st)) != CFGZIP_OK) return rc;
     fill_groups(ctx, a, d);
@@ -1716,10 +1722,11 @@ int cfgzip_multi_mask_logsoftmax_argmax(cfgzip_ctx* ctx, cfgzip_part_id part0, c
     a.inv_t = 1.f;
     a.masks_per_row = masks_per_row;
     DensePlan d;
-    if (masks_per_row > 1) d = plan_multi(ctx, ps, B, masks_per_row, es);
+    const int masks = masks_kind(ps, class_masks, class_stride_words, false, true);
+    if (masks_per_row > 1) d = plan_multi(ctx, ps, B, masks_per_row, es, masks, class_stride_words);
     const bool shared = d.ok;
     // nothing to share (64 rows with one mask each: 17.3 against 19.2 us) or too little, or a class table that leaves no room beside it
-    if (!shared) d = plan_dense(ctx, ps, rows, false, 4 * ps.VW, 32);
+    if (!shared) d = plan_dense(ctx, ps, rows, false, 4 * ps.VW, 32, masks == kMasksRows ? kMasksRows : kMasksStaged);
     if (!d.ok) return CFGZIP_E_RANGE;  // more than 65535 classes, or a class table beyond shared memory
     fill_groups(ctx, a, d);
     ctx->pdl_now = int64_t(B) * ps.V * es < (int64_t(192) << 20);
@@ -2137,10 +2144,11 @@ extern "C" int cfgzip_plan_query(int32_t sm_count, int32_t smem_optin, int32_t V
     ps.all_kw_mult4 = (ps.maxKW % 4) == 0;
     const bool mixed = n_partitions > 1;
     const int es = dtype == CFGZIP_BF16 ? 2 : 4;
-    DensePlan d = plan_pipe(&fake, ps, B, mixed, es, aligned_class_masks != 0);
+    const int masks = aligned_class_masks && ps.all_kw_mult4 ? kMasksRows : kMasksStaged;
+    DensePlan d = plan_pipe(&fake, ps, B, mixed, es, masks, ps.maxKW);
     int kind = 2;  // pipelined
     if (!d.ok) {
-        d = plan_dense(&fake, ps, B, mixed, 4 * ps.VW, 32);
+        d = plan_dense(&fake, ps, B, mixed, 4 * ps.VW, 32, masks);
         kind = 1;  // register kernel
     }
     if (!d.ok) kind = 0;  // per-row kernel

@@ -11,6 +11,14 @@
 
 namespace cfgzip {
 
+// kMasksRows: rows on 16-byte boundaries, KW a multiple of 4 (the pipelined kernel copies every row, the others read four words
+// at a time). kMasksBlock, groups of consecutive rows in the pipelined kernel and under several masks: the rows of a group are one piece
+// of memory on a 16-byte boundary and are copied as such. kMasksStaged: any, word by word. (Three in four class counts leave the rows
+// off these boundaries; us, word by word / the block: 96 bf16 rows of 128256 in 2080 classes 17.1 / 15.2, in 8224 20.1 / 16.6, 64 f32 rows in
+// 16416 28.9 / 22.3.)
+enum : int { kMasksStaged = 0, kMasksRows = 1, kMasksBlock = 2 };
+constexpr uint32_t kMaskPiece = 2048;  // bytes of such a copy
+
 // Arguments of one step (expand / fused), shared by the dense, sparse and generic kernels.
 struct StepArgs {
     const PartDev* parts;
@@ -45,7 +53,7 @@ struct StepArgs {
     int32_t table_words;        // dense: shared-memory words of the bit-sliced class table
     int32_t stage_stride;       // dense: words per row of the class-mask staging area, 0 = no staging
     int32_t depth;              // pipelined dense kernel: stages per warp
-    int32_t cm_bulk;            // pipelined dense kernel: class-mask rows are fetched by bulk copies (16-byte aligned rows)
+    int32_t cm_bulk;            // how the class masks reach the class table: kMasksStaged, kMasksRows or kMasksBlock
     int32_t wide;               // every row of the logits starts on a 32-byte boundary: f32 octets go back as one 32-byte store
     int32_t stage_alias;        // pipelined dense kernel: the class-mask staging area lies over the start of the rings
     int32_t hold_warps;         // stage_alias: warps whose ring it covers; they start their copies after the table is built
@@ -80,6 +88,12 @@ struct StepArgs {
     float* chunk_max;           // sampling step with top_k: dev [B][n_chunks] largest masked logit of every chunk; else null
     int32_t n_chunks;
 };
+
+// kMasksBlock: how much of group g is copied, whole 16 bytes (up to three words of the last row may be left).
+__device__ __forceinline__ uint32_t mask_block_bytes(const StepArgs& a, int g) {
+    const int rows = min(kGroupRows, a.B - g * kGroupRows);
+    return (uint32_t(rows - 1) * uint32_t(a.cm_stride) + uint32_t(a.p0.KW)) * 4u & ~15u;
+}
 
 // Tokens in front of the first vector boundary of a row that may start anywhere (16 bytes for bf16, 32 for f32: an
 // octet is one vector either way), and how many whole vectors follow.
@@ -187,13 +201,13 @@ __device__ __forceinline__ int group_rows_setup(const StepArgs& a, int g, int* s
     return a.group_part ? a.group_part[g] : a.part0;
 }
 
-// Copy the class-mask rows of the group's 32 row slots to shared memory (`stage`, rows
+// Copy words [k0, k1) of the class-mask rows of the group's 32 row slots to shared memory (`stage`, rows
 // stage_stride words apart). A warp takes one row at a time with coalesced loads, four rows
 // and two 32-word spans per pass, so up to eight loads per thread are in flight together.
-__device__ __forceinline__ void stage_class_masks(const StepArgs& a, const PartDev& P, const int* s_row, uint32_t* stage,
-                                                  int warp, int lane, int n_warps) {
+__device__ __forceinline__ void stage_class_masks(const StepArgs& a, const int* s_row, uint32_t* stage, int warp, int lane, int n_warps,
+                                                  int k0, int k1) {
     for (int r0 = warp; r0 < kGroupRows; r0 += 4 * n_warps) {
-        for (int kw0 = lane; kw0 < P.KW; kw0 += 64) {
+        for (int kw0 = k0 + lane; kw0 < k1; kw0 += 64) {
             uint32_t v[4][2];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
@@ -202,7 +216,7 @@ __device__ __forceinline__ void stage_class_masks(const StepArgs& a, const PartD
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
                     const int kw = kw0 + 32 * u;
-                    v[q][u] = (row >= 0 && kw < P.KW) ? __ldg(a.class_mask + int64_t(row) * a.cm_stride + kw) : 0u;
+                    v[q][u] = (row >= 0 && kw < k1) ? __ldg(a.class_mask + int64_t(row) * a.cm_stride + kw) : 0u;
                 }
             }
 #pragma unroll
@@ -211,40 +225,65 @@ __device__ __forceinline__ void stage_class_masks(const StepArgs& a, const PartD
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
                     const int kw = kw0 + 32 * u;
-                    if (r < kGroupRows && kw < P.KW) stage[r * a.stage_stride + kw] = v[q][u];
+                    if (r < kGroupRows && kw < k1) stage[r * a.stage_stride + kw - k0] = v[q][u];
                 }
             }
         }
     }
 }
 
-// Bit-sliced class table of one row group: T[k] bit r = "row slot r allows class k".
-// Entries K .. 32*(KW+1)-1 are zero, so the padding class id K looks up "nobody".
-// With a staging area (filled by stage_class_masks, then a block barrier) the 32x32 bit
-// blocks are read from shared memory; stage_stride is odd, so those column reads hit 32
-// banks. Without one, each lane reads its row's words from global memory, eight at a time.
-__device__ __forceinline__ void build_class_table(const StepArgs& a, const PartDev& P, const int* s_row, uint32_t* T,
-                                                  const uint32_t* stage, int warp, int lane, int n_warps) {
-    const uint32_t tail = (P.K & 31) ? (1u << (P.K & 31)) - 1u : 0xFFFFFFFFu;
+// Bit-sliced class table of one row group: T[k] bit r = "row slot r allows class k", entries 32 k0 .. 32 k1 - 1.
+// Entries K .. 32*(KW+1)-1 are zero, so that the padding class id K looks up "nobody" (k1 = KW + 1 writes them).
+// The 32x32 bit blocks come from a staging area that starts with word k0 of every row; a stage_stride that is odd (or even
+// and no multiple of 4) spreads its column reads over 32 (16) banks. BLOCK: words from `staged` on (counted through the
+// area) are not in it and are read from global memory.
+template <bool BLOCK>
+__device__ __forceinline__ void build_class_table(const StepArgs& a, int K, int KW, const int* s_row, uint32_t* T, const uint32_t* stage,
+                                                  int warp, int lane, int n_warps, int k0, int k1, int staged) {
+    const uint32_t tail = (K & 31) ? (1u << (K & 31)) - 1u : 0xFFFFFFFFu;
     const int row = s_row[lane];
-    const uint32_t* cm = a.class_mask + int64_t(row < 0 ? 0 : row) * a.cm_stride;
     constexpr int U = 4;
-    for (int kw0 = warp; kw0 <= P.KW; kw0 += n_warps * U) {
+    for (int kw0 = k0 + warp; kw0 < k1; kw0 += n_warps * U) {
         uint32_t x[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int kw = kw0 + u * n_warps;
+            const int kw = kw0 + u * n_warps, at = lane * a.stage_stride + kw - k0;
             x[u] = 0u;
-            if (kw < P.KW && row >= 0) x[u] = a.stage_stride ? stage[lane * a.stage_stride + kw] : __ldg(cm + kw);
-            if (kw == P.KW - 1) x[u] &= tail;
+            if (kw < k1 && kw < KW && row >= 0) {
+                if (!BLOCK || at < staged) x[u] = stage[at];
+                else x[u] = __ldg(a.class_mask + int64_t(row) * a.cm_stride + kw);
+            }
+            if (kw == KW - 1) x[u] &= tail;
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int kw = kw0 + u * n_warps;
             const uint32_t t = warp_transpose32(x[u], lane);  // independent chains: their shuffles overlap
-            if (kw <= P.KW) T[kw * 32 + lane] = t;
+            if (kw < k1) T[kw * 32 + lane] = t;
         }
     }
+}
+// The table as many words at a time as the staging area holds: all of them, or kMaskSlice (16416 classes a lane per row, read where
+// they lie, word by word, took 29 of 43 us of a call with 8 x 16 masks). Called by all threads of the block, which meet before the
+// table is read.
+constexpr int kMaskSlice = 128;
+__device__ __forceinline__ void build_class_table_staged(const StepArgs& a, int K, int KW, const int* s_row, uint32_t* T, uint32_t* stage,
+                                                         int warp, int lane, int n_warps) {
+    const int span = a.stage_stride >= KW ? KW + 1 : kMaskSlice;
+    for (int k0 = 0; k0 <= KW; k0 += span) {
+        if (k0) __syncthreads();  // (the words before have been taken)
+        stage_class_masks(a, s_row, stage, warp, lane, n_warps, k0, min(k0 + span, KW));
+        __syncthreads();
+        build_class_table<false>(a, K, KW, s_row, T, stage, warp, lane, n_warps, k0, min(k0 + span, KW + 1), 0);
+    }
+}
+// The same as a function, for the kernel that hardly needs it: inlined there it cost the batches that do not up to 7 % (96 rows of
+// 128256 bf16 in 8192 classes 14.9 -> 16.1 us).
+__device__ __noinline__ void build_class_table_staged_call(const StepArgs& a, int K, int KW, uint32_t rows_at, uint32_t table_at,
+                                                           uint32_t stage_at) {
+    auto words = [](uint32_t at) { return reinterpret_cast<uint32_t*>(__cvta_shared_to_generic(at)); };
+    build_class_table_staged(a, K, KW, reinterpret_cast<const int*>(words(rows_at)), words(table_at), words(stage_at), threadIdx.x >> 5,
+                             threadIdx.x & 31, blockDim.x >> 5);
 }
 
 // The same table from a staging area whose rows are 16-byte aligned and stage_stride (a
@@ -264,6 +303,56 @@ __device__ __forceinline__ void build_class_table_quads(const StepArgs& a, const
         dst[0] = t0; dst[32] = t1; dst[64] = t2; dst[96] = t3;
     }
     if (warp == 0) T[P.KW * 32 + lane] = 0u;  // the padding class
+}
+
+// The same straight from the masks: rows on 16-byte boundaries, KW a multiple of 4, a lane reads four words of its row at once.
+__device__ __forceinline__ void build_class_table_direct(const StepArgs& a, const PartDev& P, const int* s_row, uint32_t* T, int warp,
+                                                         int lane, int n_warps) {
+    const uint32_t tail = (P.K & 31) ? (1u << (P.K & 31)) - 1u : 0xFFFFFFFFu;
+    const int row = s_row[lane];
+    const uint4* const cm = reinterpret_cast<const uint4*>(a.class_mask + int64_t(row < 0 ? 0 : row) * a.cm_stride);
+    constexpr int U = 2;
+    for (int q0 = warp; 4 * q0 < P.KW; q0 += U * n_warps) {
+        uint4 x[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int q = q0 + u * n_warps;
+            x[u] = row >= 0 && 4 * q < P.KW ? __ldg(cm + q) : make_uint4(0, 0, 0, 0);
+            if (4 * q + 4 == P.KW) x[u].w &= tail;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int q = q0 + u * n_warps;
+            if (4 * q >= P.KW) break;
+            uint32_t* const dst = T + q * 128 + lane;
+            dst[0] = warp_transpose32(x[u].x, lane);
+            dst[32] = warp_transpose32(x[u].y, lane);
+            dst[64] = warp_transpose32(x[u].z, lane);
+            dst[96] = warp_transpose32(x[u].w, lane);
+        }
+    }
+    if (warp == 0) T[P.KW * 32 + lane] = 0u;  // the padding class
+}
+__device__ __forceinline__ void make_class_table(const StepArgs& a, const PartDev& P, const int* s_row, uint32_t* T, uint32_t* stage,
+                                                 int warp, int lane, int n_warps) {
+    if (a.cm_bulk) build_class_table_direct(a, P, s_row, T, warp, lane, n_warps);
+    else build_class_table_staged(a, P.K, P.KW, s_row, T, stage, warp, lane, n_warps);
+}
+// For groups of consecutive rows: kMasksBlock too, the group's masks copied as one piece of memory.
+__device__ __forceinline__ void make_class_table_of_group(const StepArgs& a, const PartDev& P, int g, const int* s_row, uint32_t* T,
+                                                          uint32_t* stage, int warp, int lane, int n_warps) {
+    if (a.cm_bulk != kMasksBlock) {
+        make_class_table(a, P, s_row, T, stage, warp, lane, n_warps);
+        return;
+    }
+    const uint32_t* const src = a.class_mask + int64_t(g * kGroupRows) * a.cm_stride;
+    const int quads = int(mask_block_bytes(a, g) / 16u), words = (min(kGroupRows, a.B - g * kGroupRows) - 1) * a.stage_stride + P.KW;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < quads; i += 32 * n_warps)
+        reinterpret_cast<uint4*>(stage)[i] = __ldg(reinterpret_cast<const uint4*>(src) + i);
+    for (int i = 4 * quads + threadIdx.x; i < words; i += 32 * n_warps) stage[i] = __ldg(src + i);
+    __syncthreads();
+    build_class_table<false>(a, P.K, P.KW, s_row, T, stage, warp, lane, n_warps, 0, P.KW + 1, 0);
 }
 
 // From the class words of 8 tokens: byte i of (lo, hi) belongs to row 8*rb + i, bit j of it to token j.
@@ -791,11 +880,7 @@ __global__ void __launch_bounds__(256) k_step_dense(const __grid_constant__ Step
     __syncthreads();
     const PartDev P = a.group_part ? a.parts[part] : a.p0;
     const int nrow = __popc(__ballot_sync(0xFFFFFFFFu, s_row[lane] >= 0));
-    if (a.stage_stride) {
-        stage_class_masks(a, P, s_row, stage, warp, lane, n_warps);
-        __syncthreads();
-    }
-    build_class_table(a, P, s_row, T, stage, warp, lane, n_warps);
+    make_class_table(a, P, s_row, T, stage, warp, lane, n_warps);
     __syncthreads();
 
     const int wt = warp % a.WT, wr = warp / a.WT, WR = n_warps / a.WT;
@@ -1047,7 +1132,7 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
     if (early_cm && tid == 0) {
         mbar_init(&cm_bar, 1);
         mbar_init_fence();
-        mbar_expect_tx(&cm_bar, uint32_t(min(kGroupRows, a.B - g * kGroupRows)) * uint32_t(a.p0.KW) * 4u);
+        mbar_expect_tx(&cm_bar, a.cm_bulk == kMasksBlock ? mask_block_bytes(a, g) : uint32_t(min(kGroupRows, a.B - g * kGroupRows)) * uint32_t(a.p0.KW) * 4u);
         if (TMAP) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap) : "memory");
     }
     const int part = group_rows_setup(a, g, s_row, tid);
@@ -1198,7 +1283,9 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
                                   nvec * G::kOctetBytes);
             }
         }
-        if (warp == 0 && a.cm_bulk)
+        if (warp == 0 && a.cm_bulk == kMasksBlock)
+            bulk_prefetch(a.class_mask + int64_t(g * kGroupRows) * a.cm_stride, mask_block_bytes(a, g));
+        else if (warp == 0 && a.cm_bulk)
             for (int r = 0; r < nrow; ++r)
                 bulk_prefetch(a.class_mask + int64_t(g * kGroupRows + r) * a.cm_stride, uint32_t(a.p0.KW) * 4u);
     }
@@ -1213,7 +1300,11 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
         // the class masks first (everything waits for them): the rows dealt over the warps, so that no warp
         // issues more than a few copies; the barrier was set up by thread 0 before the block met above
         const int r = warp + n_warps * lane;
-        if (r < kGroupRows && g * kGroupRows + r < a.B)
+        if (a.cm_bulk == kMasksBlock) {
+            const char* const src = reinterpret_cast<const char*>(a.class_mask + int64_t(g * kGroupRows) * a.cm_stride);
+            const uint32_t bytes = mask_block_bytes(a, g), at = uint32_t(r) * kMaskPiece;
+            if (at < bytes) bulk_g2s(reinterpret_cast<char*>(stage) + at, src + at, min(bytes - at, kMaskPiece), &cm_bar);
+        } else if (r < kGroupRows && g * kGroupRows + r < a.B)
             bulk_g2s(stage + r * a.stage_stride, a.class_mask + int64_t(g * kGroupRows + r) * a.cm_stride, uint32_t(a.p0.KW) * 4u,
                      &cm_bar);
     }
@@ -1233,13 +1324,12 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
     bool failed = false;
     if (a.cm_bulk) {
         if (!mbar_wait(&cm_bar, 0)) failed = true;
-        build_class_table_quads(a, P, s_row, T, stage, warp, lane, n_warps);
+        if (a.cm_bulk == kMasksBlock)
+            build_class_table<true>(a, P.K, P.KW, s_row, T, stage, warp, lane, n_warps, 0, P.KW + 1, int(mask_block_bytes(a, g) / 4u));
+        else
+            build_class_table_quads(a, P, s_row, T, stage, warp, lane, n_warps);
     } else {
-        if (a.stage_stride) {
-            stage_class_masks(a, P, s_row, stage, warp, lane, n_warps);
-            __syncthreads();
-        }
-        build_class_table(a, P, s_row, T, stage, warp, lane, n_warps);
+        build_class_table_staged_call(a, P.K, P.KW, smem_u32(s_row), smem_u32(T), smem_u32(stage));
     }
     __syncthreads();
     if (__any_sync(0xFFFFFFFFu, failed) && lane == 0) atomicAdd(a.status + 3, 1);  // class masks never arrived
@@ -1401,34 +1491,6 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
 // ---------------------------------------------------------------------------------------
 constexpr int kExpandThreads = 512, kExpandWarps = kExpandThreads / 32;
 
-__device__ __forceinline__ void build_class_table_direct(const StepArgs& a, const PartDev& P, const int* s_row, uint32_t* T, int warp,
-                                                         int lane, int n_warps) {
-    const uint32_t tail = (P.K & 31) ? (1u << (P.K & 31)) - 1u : 0xFFFFFFFFu;
-    const int row = s_row[lane];
-    const uint4* const cm = reinterpret_cast<const uint4*>(a.class_mask + int64_t(row < 0 ? 0 : row) * a.cm_stride);
-    constexpr int U = 2;
-    for (int q0 = warp; 4 * q0 < P.KW; q0 += U * n_warps) {
-        uint4 x[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int q = q0 + u * n_warps;
-            x[u] = row >= 0 && 4 * q < P.KW ? __ldg(cm + q) : make_uint4(0, 0, 0, 0);
-            if (4 * q + 4 == P.KW) x[u].w &= tail;
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int q = q0 + u * n_warps;
-            if (4 * q >= P.KW) break;
-            uint32_t* const dst = T + q * 128 + lane;
-            dst[0] = warp_transpose32(x[u].x, lane);
-            dst[32] = warp_transpose32(x[u].y, lane);
-            dst[64] = warp_transpose32(x[u].z, lane);
-            dst[96] = warp_transpose32(x[u].w, lane);
-        }
-    }
-    if (warp == 0) T[P.KW * 32 + lane] = 0u;  // the padding class
-}
-
 // PLANNED: the row groups come from a row plan; else they are 32 consecutive rows each.
 template <bool PLANNED>
 __global__ void __launch_bounds__(kExpandThreads, 2) k_expand_dense(const __grid_constant__ StepArgs a) {
@@ -1459,15 +1521,7 @@ __global__ void __launch_bounds__(kExpandThreads, 2) k_expand_dense(const __grid
     };
     fetch(unit);
     if (!PLANNED) pdl_wait();
-    if (a.cm_bulk) {
-        build_class_table_direct(a, P, s_row, T, warp, lane, kExpandWarps);
-    } else {
-        if (a.stage_stride) {
-            stage_class_masks(a, P, s_row, stage, warp, lane, kExpandWarps);
-            __syncthreads();
-        }
-        build_class_table(a, P, s_row, T, stage, warp, lane, kExpandWarps);
-    }
+    make_class_table(a, P, s_row, T, stage, warp, lane, kExpandWarps);
     __syncthreads();
 
     uint8_t* const vm8 = reinterpret_cast<uint8_t*>(a.vocab_mask);
@@ -1563,11 +1617,7 @@ __global__ void __launch_bounds__(kFewThreads, 3) k_step_few(const __grid_consta
     __syncthreads();
     const PartDev P = a.group_part ? a.parts[part] : a.p0;
     const int nrow = __popc(__ballot_sync(0xFFFFFFFFu, s_row[lane] >= 0));
-    if (a.stage_stride) {
-        stage_class_masks(a, P, s_row, stage, warp, lane, kFewWarps);
-        __syncthreads();
-    }
-    build_class_table(a, P, s_row, T, stage, warp, lane, kFewWarps);
+    make_class_table(a, P, s_row, T, stage, warp, lane, kFewWarps);
     __syncthreads();
 
     constexpr int ES = DT == kBF16 ? 2 : 4;

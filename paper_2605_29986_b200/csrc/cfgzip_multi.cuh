@@ -78,11 +78,7 @@ __global__ void __launch_bounds__(kMultiWarps * 32, 2) k_step_multi(const __grid
     };
     pdl_wait();
     if (wr * kBatchRows < nrow) open(wr);
-    if (a.stage_stride) {
-        stage_class_masks(a, P, s_row, stage, warp, lane, n_warps);
-        __syncthreads();
-    }
-    build_class_table(a, P, s_row, T, stage, warp, lane, n_warps);
+    make_class_table_of_group(a, P, g, s_row, T, stage, warp, lane, n_warps);
     __syncthreads();
 
     for (int rb = wr; rb * kBatchRows < nrow; rb += WR) {
