@@ -571,17 +571,17 @@ DensePlan plan_pipe(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, i
 // Measured, us, class lists / k_step_few, bf16, one to five classes allowed:
 //   under 64 rows    32 of 128256: K = 512 20 / 11, 2000 14.9 / 12.4, 4000 12.8 / 14.2; 48 f32 rows of 256000, K = 2000 20 / 24: by
 //                    classes and row length there, but the class lists are one launch instead of two and are kept for all of them
-//   class table      128 of 128256: K = 4000 25 / 20, 6000 20 / 23, 8192 22 / 33 (from some 4900 classes on the masks are not
-//                    staged); 512 of 256000: K = 6000 106 / 77, 8192 90 / 81 (few blocks per row make up for it), 16000 95 / 93
+//   class table      128 of 128256: K = 4000 25 / 20, 6000 25 / 21, 8192 23.2 / 24.3, 16000 29 / 24; 512 of 256000: K = 8200 79 / 70, 16000
+//                    108 / 71; f32: 250 of 200064 K = 6001 76 / 54, 100 of 64064 K = 8000 26 / 19; 70 of 90048 K = 11000 19.7 / 20.4 (while the table
+//                    took its masks lane by lane from some 4900 classes on, the lists were better there)
 //   short rows       450 of 20032 12 / 14, 450 of 32064 15 / 19, 410 of 32064 15.1 / 14.8, 512 of 64064 24 / 27, 800 40 / 39
 //   mixed batches    groups of few rows build tables for little: 64 rows of 128256 in eight partitions, K = 512 19 / 16, 3000
 //                    28 / 17, 4000 13 / 18; 300 rows of 20032 in two of 512 11.2 / 11.7, in eight 11 / 15
-bool few_pays(const cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, int elem_size, const DensePlan& d, int per_sm) {
+bool few_pays(const cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, int elem_size, const DensePlan& d) {
     const int wave = ctx->sm_count * ctx->ctas_per_sm;  // rows from half of this on have one block each in the other kernel
     const int64_t row_kb = int64_t(ps.V) * elem_size >> 10;
     if (B < 64) return false;
     if (mixed) return ps.maxK <= 3072 && !(row_kb < 96 && d.n_groups_ub > 16);
-    if (ps.maxK > 5344 && (per_sm < 3 || 4 * int64_t(ps.V) < 3 * int64_t(ps.maxK) * d.S)) return false;
     return !(row_kb < 96 && B > wave / 2) && !(row_kb < 160 && B > 3 * wave / 4 && B <= wave);
 }
 
@@ -608,7 +608,7 @@ DensePlan plan_few(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, in
     d.WT = kFewWarps / WR;
     d.threads = kFewThreads;
     d.slots = d.S * d.WT + 1;
-    d.ok = size_t(d.n_groups_ub) * kGroupRows * d.slots <= kPartialSlots && few_pays(ctx, ps, B, mixed, elem_size, d, per_sm);
+    d.ok = size_t(d.n_groups_ub) * kGroupRows * d.slots <= kPartialSlots && few_pays(ctx, ps, B, mixed, elem_size, d);
     return d;
 }
 
