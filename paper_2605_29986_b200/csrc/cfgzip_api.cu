@@ -905,7 +905,9 @@ int launch_fused(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, in
                  cudaStream_t st) {
     int rc;
     DensePlan few;
-    if (mode != CFGZIP_SPARSE && !(mode == CFGZIP_AUTO && ctx->auto_min_bytes >= 0) &&
+    // (rows that allow few tokens as well while there are fewer than k_step_few takes: class lists / this, us, 32 bf16 rows of 128256 in 512
+    // classes 19.4 / 8.2, 8 f32 rows 14.6 / 5.9, 2 bf16 rows of 50663 in 6332 classes 12.6 / 4.4)
+    if (!(mode == CFGZIP_SPARSE && a.B >= 64) && !(mode == CFGZIP_AUTO && ctx->auto_min_bytes >= 0) &&
         (aligned || aligned_elems(a.logits, DT == kBF16 ? 2 : 4))) {
         ClusterPlan cl = plan_cluster(ctx, ps, a.B, mixed, DT == kBF16 ? 2 : 4, !aligned, false, logp_full != nullptr);
         cl.g.full = logp_full;
@@ -1535,7 +1537,11 @@ int cfgzip_expand_mask(cfgzip_ctx* ctx, cfgzip_part_id part0, const int32_t* row
     fill_groups(ctx, a, d);
     auto kern = d.use_plan_kernel ? k_expand_dense<true> : k_expand_dense<false>;
     if ((rc = ensure_smem(ctx, kern, d.smem)) != CFGZIP_OK) return rc;
-    return launch(ctx, kern, dim3(unsigned(d.n_groups_ub) * unsigned(d.S)), dim3(kExpandThreads), d.smem, st, a);
+    const bool pdl = ctx->pdl_now;
+    if (d.use_plan_kernel) ctx->pdl_now = false;  // (after the whole of the row plan)
+    rc = launch(ctx, kern, dim3(unsigned(d.n_groups_ub) * unsigned(d.S)), dim3(kExpandThreads), d.smem, st, a);
+    ctx->pdl_now = pdl;
+    return rc;
 }
 
 int cfgzip_mask_logits(cfgzip_ctx* ctx, void* logits, int dtype, int64_t row_stride_elems, int32_t B, int32_t V,

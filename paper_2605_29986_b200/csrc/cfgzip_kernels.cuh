@@ -1503,7 +1503,8 @@ __global__ void __launch_bounds__(kExpandThreads, 2) k_expand_dense(const __grid
     if (PLANNED) pdl_wait();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = blockIdx.x / a.S, split = blockIdx.x - g * a.S;
-    if (PLANNED && g >= __ldg(a.n_groups)) return;
+    // (a plain volatile read: a read-only load may be moved in front of the wait, and the plan is written by the kernel in front)
+    if (PLANNED && g >= *const_cast<const volatile int32_t*>(a.n_groups)) return;
     const int part = group_rows_setup(a, g, s_row, tid);
     __syncthreads();
     const PartDev P = PLANNED ? a.parts[part] : a.p0;
