@@ -127,7 +127,7 @@ __device__ __forceinline__ void cluster_draw(const StepArgs& a, const PartDev& P
         return;
     }
     float inc = warp_inclusive_scan(weight, lane);
-    const float total = __shfl_sync(0xFFFFFFFFu, inc, 31), tau = __ldg(a.u + row) * total;
+    const float total = __shfl_sync(0xFFFFFFFFu, inc, 31), tau = ld_after_wait(a.u + row) * total;
     const int block = crossing_lane(weight, inc, tau);
     if (block != rank) return;
     float base = front_of(inc, block);
@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1) k_step_cluster(const __gri
     // The class masks first (everything waits for them), then all logits.
     uint32_t w[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) w[r] = r < live && tid < P.KW ? __ldg(a.class_mask + int64_t(row0 + r) * a.cm_stride + tid) : 0u;
+    for (int r = 0; r < R; ++r) w[r] = r < live && tid < P.KW ? ld_after_wait(a.class_mask + int64_t(row0 + r) * a.cm_stride + tid) : 0u;
     {
         auto vectors = [&](int r, int c) {  // of row r in chunk c
             const int nvec = (a.V - head_of(r)) >> 3;
@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1) k_step_cluster(const __gri
         const uint32_t keep = kw == P.KW ? 0u : (kw == P.KW - 1 && (P.K & 31)) ? (1u << (P.K & 31)) - 1u : 0xFFFFFFFFu;
         if (kw != tid) {
 #pragma unroll
-            for (int r = 0; r < R; ++r) w[r] = r < live && kw < P.KW ? __ldg(a.class_mask + int64_t(row0 + r) * a.cm_stride + kw) : 0u;
+            for (int r = 0; r < R; ++r) w[r] = r < live && kw < P.KW ? ld_after_wait(a.class_mask + int64_t(row0 + r) * a.cm_stride + kw) : 0u;
         }
         uint32_t x[8];
 #pragma unroll

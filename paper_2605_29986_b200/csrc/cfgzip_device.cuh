@@ -118,6 +118,27 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
     return d;
 }
 
+// Reads of what a kernel in front may have written (a row plan, masks, uniform numbers, normalisers), behind griddepcontrol.wait.
+// Not __ldg: that load says its memory does not change while the kernel runs, so nothing keeps it behind the wait, and with a
+// programmatic launch this kernel runs while the one in front is still writing. These stay in order with the wait and cost the same.
+__device__ __forceinline__ uint32_t ld_after_wait(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(__cvta_generic_to_global(p)));
+    return v;
+}
+__device__ __forceinline__ int32_t ld_after_wait(const int32_t* p) { return int32_t(ld_after_wait(reinterpret_cast<const uint32_t*>(p))); }
+__device__ __forceinline__ float ld_after_wait(const float* p) { return __uint_as_float(ld_after_wait(reinterpret_cast<const uint32_t*>(p))); }
+__device__ __forceinline__ uint32_t ld_after_wait(const uint8_t* p) {
+    uint32_t v;
+    asm volatile("ld.global.u8 %0, [%1];" : "=r"(v) : "l"(__cvta_generic_to_global(p)));
+    return v;
+}
+__device__ __forceinline__ uint4 ld_after_wait(const uint4* p) {
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(__cvta_generic_to_global(p)));
+    return v;
+}
+
 // Streaming 16-byte accesses for the logits (read once, written once).
 __device__ __forceinline__ uint4 ld_stream16(const void* p) { return __ldcs(reinterpret_cast<const uint4*>(p)); }
 __device__ __forceinline__ void st_stream16(void* p, uint4 v) { __stcs(reinterpret_cast<uint4*>(p), v); }

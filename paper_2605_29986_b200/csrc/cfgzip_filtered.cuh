@@ -675,7 +675,7 @@ __device__ __noinline__ unsigned int filt_allowed(const StepArgs& a, const PartD
     unsigned int n = 0u;
 #pragma unroll 4
     for (int k = tid; k < P.K; k += kFiltThreads)
-        if ((__ldg(cm + (k >> 5)) >> (k & 31)) & 1u) n += unsigned(__ldg(P.off + k + 1) - __ldg(P.off + k));
+        if ((ld_after_wait(cm + (k >> 5)) >> (k & 31)) & 1u) n += unsigned(__ldg(P.off + k + 1) - __ldg(P.off + k));
     n = __reduce_add_sync(0xFFFFFFFFu, n);
     __syncthreads();
     if (lane == 0) sh.warp_sum[warp] = __uint_as_float(n);
@@ -704,7 +704,7 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __gri
     const int slot = blockIdx.x / w.n_peers;  // the blocks of a cluster are neighbours along x
     const int g = slot / kGroupRows, j = slot - g * kGroupRows;
     // (every way out before the cluster's barriers depends on the row alone, so the blocks of a cluster take it together)
-    if (a.n_groups && g >= __ldg(a.n_groups)) return;
+    if (a.n_groups && g >= ld_after_wait(a.n_groups)) return;
     int row;
     if (a.group_rows) {
         row = a.group_rows[g * kGroupRows + j];
@@ -745,7 +745,7 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __gri
     const int edge_t = tid < 8 ? tid : fine_end + tid - 8;
     float edge_z = -INFINITY;
     if (FINE && tid < 16 && (tid < 8 ? edge_t < fine_head : edge_t < a.V)) edge_z = ldcg_elem<DT>(w.rowp, edge_t);
-    const float u = __ldg(a.u + row);  // needed late
+    const float u = ld_after_wait(a.u + row);  // needed late
     constexpr int kKeep = 4;
     float run_m[kKeep], run_s[kKeep], M = edge_z;
 #pragma unroll

@@ -216,7 +216,7 @@ __device__ __forceinline__ void stage_class_masks(const StepArgs& a, const int* 
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
                     const int kw = kw0 + 32 * u;
-                    v[q][u] = (row >= 0 && kw < k1) ? __ldg(a.class_mask + int64_t(row) * a.cm_stride + kw) : 0u;
+                    v[q][u] = (row >= 0 && kw < k1) ? ld_after_wait(a.class_mask + int64_t(row) * a.cm_stride + kw) : 0u;
                 }
             }
 #pragma unroll
@@ -251,7 +251,7 @@ __device__ __forceinline__ void build_class_table(const StepArgs& a, int K, int 
             x[u] = 0u;
             if (kw < k1 && kw < KW && row >= 0) {
                 if (!BLOCK || at < staged) x[u] = stage[at];
-                else x[u] = __ldg(a.class_mask + int64_t(row) * a.cm_stride + kw);
+                else x[u] = ld_after_wait(a.class_mask + int64_t(row) * a.cm_stride + kw);
             }
             if (kw == KW - 1) x[u] &= tail;
         }
@@ -317,7 +317,7 @@ __device__ __forceinline__ void build_class_table_direct(const StepArgs& a, cons
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int q = q0 + u * n_warps;
-            x[u] = row >= 0 && 4 * q < P.KW ? __ldg(cm + q) : make_uint4(0, 0, 0, 0);
+            x[u] = row >= 0 && 4 * q < P.KW ? ld_after_wait(cm + q) : make_uint4(0, 0, 0, 0);
             if (4 * q + 4 == P.KW) x[u].w &= tail;
         }
 #pragma unroll
@@ -349,8 +349,8 @@ __device__ __forceinline__ void make_class_table_of_group(const StepArgs& a, con
     const int quads = int(mask_block_bytes(a, g) / 16u), words = (min(kGroupRows, a.B - g * kGroupRows) - 1) * a.stage_stride + P.KW;
 #pragma unroll 4
     for (int i = threadIdx.x; i < quads; i += 32 * n_warps)
-        reinterpret_cast<uint4*>(stage)[i] = __ldg(reinterpret_cast<const uint4*>(src) + i);
-    for (int i = 4 * quads + threadIdx.x; i < words; i += 32 * n_warps) stage[i] = __ldg(src + i);
+        reinterpret_cast<uint4*>(stage)[i] = ld_after_wait(reinterpret_cast<const uint4*>(src) + i);
+    for (int i = 4 * quads + threadIdx.x; i < words; i += 32 * n_warps) stage[i] = ld_after_wait(src + i);
     __syncthreads();
     build_class_table<false>(a, P.K, P.KW, s_row, T, stage, warp, lane, n_warps, 0, P.KW + 1, 0);
 }
@@ -426,7 +426,7 @@ __device__ __forceinline__ void warp_finalize_row(const StepArgs& a, const PartD
         s = 0.f;
         for (int t = lane; t < a.V; t += 32) {
             const int k = __ldg(P.c32 + t);
-            if ((__ldg(cm + (k >> 5)) >> (k & 31)) & 1u) s += ex2f((ldcg_elem<DT>(rowp, t) - m) * kLog2e);
+            if ((ld_after_wait(cm + (k >> 5)) >> (k & 31)) & 1u) s += ex2f((ldcg_elem<DT>(rowp, t) - m) * kLog2e);
         }
 #pragma unroll
         for (int d = 16; d >= 1; d >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, d);
@@ -446,7 +446,7 @@ __device__ __forceinline__ void warp_finalize_row(const StepArgs& a, const PartD
             bool ok = z == m;
             if (a.masks_per_row > 0) {  // the logits were left as they are: ask this row's class mask
                 const int k = __ldg(P.c32 + t);
-                ok = ok && ((__ldg(a.class_mask + int64_t(row) * a.cm_stride + (k >> 5)) >> (k & 31)) & 1u);
+                ok = ok && ((ld_after_wait(a.class_mask + int64_t(row) * a.cm_stride + (k >> 5)) >> (k & 31)) & 1u);
             }
             if (ok) cand = (static_cast<unsigned long long>(t) << 32) | static_cast<unsigned int>(repv);
         }
@@ -505,7 +505,7 @@ struct GroupShare {
 // (Functions of their own: a batch without a row plan, whose steps are the shortest, should not fetch past this code. Inlined in the
 // per-row kernels it cost 256 rows that allow few tokens 1.8 of 27 us.)
 __device__ __noinline__ GroupShare group_share(const StepArgs& a, int g) {
-    const int n = __ldg(a.n_groups), w0 = __ldg(a.group_w + g), w1 = __ldg(a.group_w + g + 1), W = __ldg(a.group_w + a.max_groups);
+    const int n = ld_after_wait(a.n_groups), w0 = ld_after_wait(a.group_w + g), w1 = ld_after_wait(a.group_w + g + 1), W = ld_after_wait(a.group_w + a.max_groups);
     if (n * a.S_even <= a.blocks) return GroupShare{g * a.S_even, a.S_even};
     const int spare = a.blocks - n, first = g + spare * w0 / max(W, 1), next = g + 1 + spare * w1 / max(W, 1);
     return GroupShare{first, min(next - first, a.S)};
@@ -515,7 +515,7 @@ struct BlockPlace {
     int g, split, S;
 };
 __device__ __noinline__ BlockPlace block_place(const StepArgs& a) {
-    const int b = blockIdx.x, n = __ldg(a.n_groups), even = a.S_even;
+    const int b = blockIdx.x, n = ld_after_wait(a.n_groups), even = a.S_even;
     if (n * even <= a.blocks) {
         const int g = b / even;
         return BlockPlace{g < n ? g : -1, b - g * even, even};
@@ -669,7 +669,7 @@ __global__ void __launch_bounds__(kFinalizeThreads) k_finalize_rows(const __grid
         for (int u = 0; u < 4; ++u)
             if (u * kFinalizeThreads + tid >= n_states) v0[u] = make_int4(__float_as_int(-INFINITY), 0, kNoPos, 0);
     }
-    if (a.n_groups && g >= __ldg(a.n_groups)) return;
+    if (a.n_groups && g >= ld_after_wait(a.n_groups)) return;
     int row;
     if (a.group_rows) {
         row = a.group_rows[g * kGroupRows + j];
@@ -761,7 +761,7 @@ __global__ void __launch_bounds__(256) k_finalize_rows_warp(const __grid_constan
         for (int u = 0; u < 4; ++u)
             if (u * 32 + lane >= n_states) v[u] = make_int4(__float_as_int(-INFINITY), 0, kNoPos, 0);
     }
-    if (a.n_groups && g >= __ldg(a.n_groups)) return;
+    if (a.n_groups && g >= ld_after_wait(a.n_groups)) return;
     int row;
     if (a.group_rows) {
         row = a.group_rows[g * kGroupRows + j];
@@ -875,7 +875,7 @@ __global__ void __launch_bounds__(256) k_step_dense(const __grid_constant__ Step
     pdl_prologue();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, n_warps = blockDim.x >> 5;
     const int g = blockIdx.x / a.S, split = blockIdx.x - g * a.S;
-    if (a.n_groups && g >= __ldg(a.n_groups)) return;
+    if (a.n_groups && g >= ld_after_wait(a.n_groups)) return;
     const int part = group_rows_setup(a, g, s_row, tid);
     __syncthreads();
     const PartDev P = a.group_part ? a.parts[part] : a.p0;
@@ -1115,7 +1115,7 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
         g = blockIdx.x / a.S;
         split = blockIdx.x - g * a.S;
         S = a.S;
-        if (!TMAP && a.n_groups && g >= __ldg(a.n_groups)) return;
+        if (!TMAP && a.n_groups && g >= ld_after_wait(a.n_groups)) return;
     } else {  // (one warp looks: sixteen of every block after the same few words wait for one another)
         __shared__ BlockPlace s_place;
         if (warp == 0) {
@@ -1503,8 +1503,7 @@ __global__ void __launch_bounds__(kExpandThreads, 2) k_expand_dense(const __grid
     if (PLANNED) pdl_wait();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = blockIdx.x / a.S, split = blockIdx.x - g * a.S;
-    // (a plain volatile read: a read-only load may be moved in front of the wait, and the plan is written by the kernel in front)
-    if (PLANNED && g >= *const_cast<const volatile int32_t*>(a.n_groups)) return;
+    if (PLANNED && g >= ld_after_wait(a.n_groups)) return;
     const int part = group_rows_setup(a, g, s_row, tid);
     __syncthreads();
     const PartDev P = PLANNED ? a.parts[part] : a.p0;
@@ -1613,7 +1612,7 @@ __global__ void __launch_bounds__(kFewThreads, 3) k_step_few(const __grid_consta
     pdl_prologue();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = blockIdx.x / a.S, split = blockIdx.x - g * a.S;
-    if (a.n_groups && g >= __ldg(a.n_groups)) return;
+    if (a.n_groups && g >= ld_after_wait(a.n_groups)) return;
     const int part = group_rows_setup(a, g, s_row, tid);
     __syncthreads();
     const PartDev P = a.group_part ? a.parts[part] : a.p0;
@@ -1769,7 +1768,7 @@ __global__ void __launch_bounds__(256) k_step_sparse(const __grid_constant__ Ste
         // Automatic mode: the grid covers the (group, row slot) pairs of the gather kernel, and the choice is made
         // for the 8 row slots that kernel streams together (its row batch), so that no row is done twice.
         const int g = row / kGroupRows, j = row - g * kGroupRows;
-        if (a.n_groups && g >= __ldg(a.n_groups)) return;
+        if (a.n_groups && g >= ld_after_wait(a.n_groups)) return;
         if (tid < kBatchRows) {
             const int slot = g * kGroupRows + (j & ~(kBatchRows - 1)) + tid;
             int r = a.group_rows ? a.group_rows[slot] : slot;
@@ -1807,7 +1806,7 @@ __global__ void __launch_bounds__(256) k_step_sparse(const __grid_constant__ Ste
 #pragma unroll
             for (int q = 0; q < kBatchRows; ++q) {
                 const int r = s_batch[q];
-                if (r >= 0) cnt += (__ldg(a.class_mask + int64_t(r) * a.cm_stride + (k >> 5)) >> (k & 31)) & 1u;
+                if (r >= 0) cnt += (ld_after_wait(a.class_mask + int64_t(r) * a.cm_stride + (k >> 5)) >> (k & 31)) & 1u;
             }
             if (cnt) mine += static_cast<unsigned long long>(cnt) * static_cast<unsigned>(__ldg(P.off + k + 1) - __ldg(P.off + k));
         }
@@ -1824,7 +1823,7 @@ __global__ void __launch_bounds__(256) k_step_sparse(const __grid_constant__ Ste
     __syncthreads();
 
     for (int kw = warp; kw < P.KW; kw += n_warps) {
-        uint32_t word = __ldg(cm + kw);
+        uint32_t word = ld_after_wait(cm + kw);
         if (kw == P.KW - 1 && (P.K & 31)) word &= (1u << (P.K & 31)) - 1u;
         while (word) {
             const int k = kw * 32 + __ffs(word) - 1;
@@ -1984,7 +1983,7 @@ __global__ void __launch_bounds__(256) k_step_generic(const __grid_constant__ St
         bool allowed = false;
         if (t < a.V) {
             const int k = __ldg(P.c32 + t);
-            allowed = (__ldg(cm + (k >> 5)) >> (k & 31)) & 1u;
+            allowed = (ld_after_wait(cm + (k >> 5)) >> (k & 31)) & 1u;
         }
         const uint32_t word = __ballot_sync(0xFFFFFFFFu, allowed);
         if (out && lane == 0) out[w] = word;
@@ -2058,7 +2057,7 @@ __global__ void __launch_bounds__(kSampleThreads) k_sample_rows(const __grid_con
     pdl_prologue();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = blockIdx.x / kGroupRows, j = blockIdx.x - g * kGroupRows;
-    if (a.n_groups && g >= __ldg(a.n_groups)) return;
+    if (a.n_groups && g >= ld_after_wait(a.n_groups)) return;
     int row;
     if (a.group_rows) {
         row = a.group_rows[g * kGroupRows + j];
@@ -2076,7 +2075,7 @@ __global__ void __launch_bounds__(kSampleThreads) k_sample_rows(const __grid_con
         P = a.parts[part];
     }
     const Partial* src = row_slots(a, g, j);
-    const float u = __ldg(a.u + row);  // needed late: in flight together with the states
+    const float u = ld_after_wait(a.u + row);  // needed late: in flight together with the states
     const int n_states = SHARED_OUT ? group_states(a, g) : a.slots;
     const int per = (n_states + kSampleThreads - 1) / kSampleThreads;  // consecutive states per thread
     const int k0 = tid * per, k1 = min(k0 + per, n_states);
@@ -2456,13 +2455,13 @@ __global__ void __launch_bounds__(256) k_mask_logits(void* logits, int64_t row_s
             const int o = p.o + u * 256;
             p.byte[u] = 0xFFu;
             if (o < n_vec) {
-                p.byte[u] = __ldg(bits + o);
-                if (head) p.byte[u] = ((p.byte[u] | (uint32_t(__ldg(bits + o + 1)) << 8)) >> head) & 0xFFu;
+                p.byte[u] = ld_after_wait(bits + o);
+                if (head) p.byte[u] = ((p.byte[u] | (ld_after_wait(bits + o + 1) << 8)) >> head) & 0xFFu;
             }
         }
         if (at.ch == 0 && tid < 16) {  // the ends of the row
             const int t = tid < 8 ? tid : head + 8 * n_vec + tid - 8;
-            if ((tid < 8 ? t < head : t < V) && !((__ldg(bits + (t >> 3)) >> (t & 7)) & 1u)) store_neg_inf<DT>(rowp, t);
+            if ((tid < 8 ? t < head : t < V) && !((ld_after_wait(bits + (t >> 3)) >> (t & 7)) & 1u)) store_neg_inf<DT>(rowp, t);
         }
         return p;
     };
@@ -2534,7 +2533,7 @@ __global__ void __launch_bounds__(256) k_logp_full(const void* logits, int64_t r
     auto value = [](float z, float l) { return (l == -INFINITY || z == -INFINITY) ? -INFINITY : z - l; };
     // grid: x strides over the pieces of a row, y over the rows
     for (int row = blockIdx.y; row < B; row += gridDim.y) {
-        const float l = __ldg(lse + row);
+        const float l = ld_after_wait(lse + row);
         const char* zrow = reinterpret_cast<const char*>(logits) + int64_t(row) * row_stride * (DT == kBF16 ? 2 : 4);
         float* orow = out + int64_t(row) * V;
         for (int u0 = blockIdx.x * 256 * kInFlight + tid; u0 < units; u0 += gridDim.x * 256 * kInFlight) {
