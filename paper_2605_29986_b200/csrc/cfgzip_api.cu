@@ -1537,11 +1537,7 @@ int cfgzip_expand_mask(cfgzip_ctx* ctx, cfgzip_part_id part0, const int32_t* row
     fill_groups(ctx, a, d);
     auto kern = d.use_plan_kernel ? k_expand_dense<true> : k_expand_dense<false>;
     if ((rc = ensure_smem(ctx, kern, d.smem)) != CFGZIP_OK) return rc;
-    const bool pdl = ctx->pdl_now;
-    if (d.use_plan_kernel) ctx->pdl_now = false;  // (after the whole of the row plan)
-    rc = launch(ctx, kern, dim3(unsigned(d.n_groups_ub) * unsigned(d.S)), dim3(kExpandThreads), d.smem, st, a);
-    ctx->pdl_now = pdl;
-    return rc;
+    return launch(ctx, kern, dim3(unsigned(d.n_groups_ub) * unsigned(d.S)), dim3(kExpandThreads), d.smem, st, a);
 }
 
 int cfgzip_mask_logits(cfgzip_ctx* ctx, void* logits, int dtype, int64_t row_stride_elems, int32_t B, int32_t V,
