@@ -1302,8 +1302,9 @@ __global__ void __launch_bounds__(LBT, MINB) k_step_dense_pipe(const __grid_cons
         const int r = warp + n_warps * lane;
         if (a.cm_bulk == kMasksBlock) {
             const char* const src = reinterpret_cast<const char*>(a.class_mask + int64_t(g * kGroupRows) * a.cm_stride);
-            const uint32_t bytes = mask_block_bytes(a, g), at = uint32_t(r) * kMaskPiece;
-            if (at < bytes) bulk_g2s(reinterpret_cast<char*>(stage) + at, src + at, min(bytes - at, kMaskPiece), &cm_bar);
+            const uint32_t bytes = mask_block_bytes(a, g);
+            for (uint32_t at = uint32_t(r) * kMaskPiece; at < bytes; at += 32u * uint32_t(n_warps) * kMaskPiece)  // (once, but for blocks of one or two warps)
+                bulk_g2s(reinterpret_cast<char*>(stage) + at, src + at, min(bytes - at, kMaskPiece), &cm_bar);
         } else if (r < kGroupRows && g * kGroupRows + r < a.B)
             bulk_g2s(stage + r * a.stage_stride, a.class_mask + int64_t(g * kGroupRows + r) * a.cm_stride, uint32_t(a.p0.KW) * 4u,
                      &cm_bar);

@@ -58,6 +58,19 @@ def test_every_alignment(K, B, pad, offset):
             compare_step(step(ctx, None, d_cm, cm.shape[1] + pad, z, V, mode), want, V)
 
 
+# A block of one or two warps, whose lanes take more than one piece each of a group's masks (20001 classes: 80128 bytes)
+@pytest.mark.parametrize("knob,value", [("token_warps", 1), ("row_warps", 1), ("row_warps", 2), ("pipe_warps", 1)])
+@pytest.mark.parametrize("K,V,B", [(16400, 24000, 448), (20001, 24000, 32)])
+def test_few_warps_fetch_a_whole_block_of_masks(K, V, B, knob, value):
+    part = synth.zipf_partition(V, K, seed=K)
+    cm = synth.class_mask_bernoulli(K, B, 0.2, rng.stream_key(rng.SEED_BASE, 954, K))
+    z = synth.logits_normal(B, V, 2.0, "bf16", (955, K))
+    with Ctx([part]) as ctx:
+        cz.cfgzip_set_tuning(ctx.h, knob, value)
+        compare_step(step(ctx, None, masks_on(cm, 0, 0), cm.shape[1], z, V, cz.DENSE), oracle_step([part], None, cm, z, V), V)
+        assert cz.cfgzip_poll_status(ctx.h) == (0, 0, 0)
+
+
 @pytest.mark.parametrize("K", [50, 1500, 5000, 16420])
 @pytest.mark.parametrize("pad,offset", [(0, 0), (3, 1)])
 def test_several_masks_and_several_partitions(K, pad, offset):
