@@ -129,6 +129,7 @@ __device__ __forceinline__ void cluster_draw(const StepArgs& a, const PartDev& P
     float inc = warp_inclusive_scan(weight, lane);
     const float total = __shfl_sync(0xFFFFFFFFu, inc, 31), tau = ld_after_wait(a.u + row) * total;
     const int block = crossing_lane(weight, inc, tau);
+    if (block < 0 && rank == 0 && lane == 0) write_no_draw(a, row);  // (an allowed +inf makes every weight NaN or zero)
     if (block != rank) return;
     float base = front_of(inc, block);
     const Partial p = lane < kClusterSlots ? sh.state[r][lane] : partial_empty();

@@ -85,3 +85,27 @@ def test_ties_and_waits(dtype):
         assert cz.load_library().cfgzip_poll_status(ctx.h, None, None, None, None) == cz.E_CUDA
         cz.cfgzip_set_tuning(ctx.h, "test_expire_waits", 0)
         compare_step(run_fused(ctx, None, cm, z, V), want, V)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("V", [20000, 20003])
+def test_no_weight_is_no_draw(V, dtype):
+    # values outside the contract: a row without a weight to draw by says so, as it does in two launches, and keeps no earlier token
+    B = 9
+    part, cm, z = inputs(V, 100, B, dtype, 4)
+    cm[:] = 0xFFFFFFFF
+    bad = (1, 4, 8)
+    for b, t in zip(bad, (0, 777, V - 1)):
+        z[b, t] = np.inf if dtype == "f32" else 0x7F80
+    z[4, :] = z[4, 777]
+    u = np.linspace(0, 0.99, B).astype(np.float32)
+    ok = [b for b in range(B) if b not in bad]
+    with Ctx([part]) as ctx:
+        for one_launch in (1, 0):
+            cz.cfgzip_set_tuning(ctx.h, "one_launch", one_launch)
+            before = cz.cfgzip_launch_count(ctx.h)
+            got = run_sample(ctx, None, cm, z, V, u, 1.0)
+            assert cz.cfgzip_launch_count(ctx.h) - before == 2 - one_launch
+            for b in bad:
+                assert got["token"][b] == -1 and got["rep"][b] == -1 and np.isneginf(got["lse"][b]) and np.isneginf(got["logp_token"][b])
+            check_sample({k: v[ok] for k, v in got.items()}, [part], None, cm[ok], z[ok], V, u[ok], 1.0)
