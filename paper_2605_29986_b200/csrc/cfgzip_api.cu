@@ -1974,9 +1974,6 @@ int cfgzip_launch_count(cfgzip_ctx* ctx, int64_t* out) {
 
 int cfgzip_set_tuning(cfgzip_ctx* ctx, const char* name, int32_t value) {
     if (!ctx || !name) return CFGZIP_E_ARG;
-    for (const char* knob : {"ctas_per_sm", "token_warps", "row_warps", "pipeline", "tensor_map", "pipe_warps", "waves", "spread", "stage_alias",
-                             "fold", "lane_octets", "pipe_depth"})
-        if (!std::strcmp(name, knob)) ctx->one_launch = 0;  // (the caller shapes the two-launch step's kernel, so that one is meant)
     if (!std::strcmp(name, "one_launch")) {
         ctx->one_launch = value ? 1 : 0;
     } else if (!std::strcmp(name, "ctas_per_sm")) {
@@ -2034,6 +2031,10 @@ int cfgzip_set_tuning(cfgzip_ctx* ctx, const char* name, int32_t value) {
     } else {
         return CFGZIP_E_ARG;
     }
+    // (an accepted one: what is refused changes nothing)
+    for (const char* knob : {"ctas_per_sm", "token_warps", "row_warps", "pipeline", "tensor_map", "pipe_warps", "waves", "spread", "stage_alias",
+                             "fold", "lane_octets", "pipe_depth"})
+        if (!std::strcmp(name, knob)) ctx->one_launch = 0;  // (the caller shapes the two-launch step's kernel, so that one is meant)
     return CFGZIP_OK;
 }
 

@@ -109,3 +109,20 @@ def test_no_weight_is_no_draw(V, dtype):
             for b in bad:
                 assert got["token"][b] == -1 and got["rep"][b] == -1 and np.isneginf(got["lse"][b]) and np.isneginf(got["logp_token"][b])
             check_sample({k: v[ok] for k, v in got.items()}, [part], None, cm[ok], z[ok], V, u[ok], 1.0)
+
+
+def test_a_refused_knob_changes_nothing():
+    V, B = 20000, 9
+    part, cm, z = inputs(V, 100, B, "bf16", 5)
+    lib = cz.load_library()
+
+    def launches(ctx):
+        before = cz.cfgzip_launch_count(ctx.h)
+        run_fused(ctx, None, cm, z, V)
+        return cz.cfgzip_launch_count(ctx.h) - before
+
+    with Ctx([part]) as ctx:
+        for knob, value in ((b"ctas_per_sm", 0), (b"row_warps", 3), (b"token_warps", 17), (b"pipe_warps", 0), (b"waves", 0), (b"fold", 3),
+                            (b"lane_octets", 3), (b"pipe_depth", 1), (b"nonsense", 1)):
+            assert lib.cfgzip_set_tuning(ctx.h, knob, value) == cz.E_ARG and launches(ctx) == 1, knob
+        assert lib.cfgzip_set_tuning(ctx.h, b"row_warps", 1) == 0 and launches(ctx) == 2
