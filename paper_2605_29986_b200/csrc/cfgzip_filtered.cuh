@@ -965,7 +965,7 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __gri
                     at = __shfl_sync(0xFFFFFFFFu, at, 31) + inc - here;
                     const uint32_t list0 = peer_shared(sh.list, 0u);
 #pragma unroll 1
-                    for (int r = 0; over >> (8 * r) && r < kFlight; ++r) {
+                    for (int r = 0; r < kFlight && over >> (8 * r); ++r) {
                         float e[8];
                         filt_floats<DT>(r == 0 ? o[0] : r == 1 ? o[1] : r == 2 ? o[2] : o[3], e);
                         filt_each(e, r == 0 ? t0[0] : r == 1 ? t0[1] : r == 2 ? t0[2] : t0[3], (over >> (8 * r)) & 0xFFu, [&](int t, float z) {

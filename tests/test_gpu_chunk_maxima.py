@@ -58,3 +58,21 @@ def test_rows_of_several_partitions():
     with Ctx(parts) as ctx:
         got = run_filtered(ctx, row_part, cm, z, V, u, 1.0, 50, 0.9)
         check_filtered(got, parts, row_part, cm, z, V, u, 1.0, 50, 0.9)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_every_vector_of_a_warp_holds_tokens_of_the_list(dtype):
+    # 200 chunks with one token each that reaches the bar: the warps take four loads at a time, tokens in each of the four
+    V, K, B = 65536, 40, 37
+    part = synth.zipf_partition(V, K, seed=6)
+    cm = synth.class_mask_bernoulli(K, B, 1.0, rng.stream_key(rng.SEED_BASE, 938))
+    z = synth.logits_normal(B, V, 1.0, "f32", (939,))
+    for b in range(B):
+        z[b, np.arange(200) * 300 + (b * 7 + np.arange(200)) % 256] = 20.0 + np.arange(200) / 64.0
+    if dtype == "bf16":
+        z = (z.view(np.uint32) >> 16).astype(np.uint16)
+    u = rng.uniform(rng.stream_key(940), B).astype(np.float32)
+    with Ctx([part]) as ctx:
+        for top_k, top_p in ((200, 1.0), (180, 0.9)):
+            got = run_filtered(ctx, None, cm, z, V, u, 0.5, top_k, top_p)
+            check_filtered(got, [part], None, cm, z, V, u, 0.5, top_k, top_p, "k=%d" % top_k)
