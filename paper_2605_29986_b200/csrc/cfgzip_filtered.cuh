@@ -810,10 +810,12 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_sample_filtered(const __gri
                 atomicAdd(&sh.bar[min(int((M - run_m[q]) * steps), kFiltThreads - 1)], top_k > 0 ? 1u : uint32_t(e * 1048576.f));
                 sum += run_s[q] * e;
             }
+        if constexpr (!FINE) {  // (their weight counts all the same; chunk maxima have none, and top_k needs none)
 #pragma unroll 1
-        for (int k = tid + kKeep * kFiltThreads; k < n_states; k += kFiltThreads) {  // (their weight counts all the same)
-            const int4 raw = __ldcg(reinterpret_cast<const int4*>(src + k));
-            if (__int_as_float(raw.x) >= w.z_zero) sum += __int_as_float(raw.y) * ex2f((__int_as_float(raw.x) - M) * scale);
+            for (int k = tid + kKeep * kFiltThreads; k < n_states; k += kFiltThreads) {
+                const int4 raw = __ldcg(reinterpret_cast<const int4*>(src + k));
+                if (__int_as_float(raw.x) >= w.z_zero) sum += __int_as_float(raw.y) * ex2f((__int_as_float(raw.x) - M) * scale);
+            }
         }
         uint32_t goal = uint32_t(top_k) - 1u;
         if (top_k == 0) {

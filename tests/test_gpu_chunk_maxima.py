@@ -76,3 +76,28 @@ def test_every_vector_of_a_warp_holds_tokens_of_the_list(dtype):
         for top_k, top_p in ((200, 1.0), (180, 0.9)):
             got = run_filtered(ctx, None, cm, z, V, u, 0.5, top_k, top_p)
             check_filtered(got, [part], None, cm, z, V, u, 0.5, top_k, top_p, "k=%d" % top_k)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("V,B", [(253952, 3), (253961, 3), (256001, 1), (256001, 36), (262143, 2)])
+def test_more_chunks_than_a_block_keeps(V, B, dtype):
+    # rows off the vector grid have more than 1024 chunks from 253953 tokens on: the maxima past those count for the row's largest logit
+    # and as chunks to read, and not for the bar
+    K = 900
+    part = synth.zipf_partition(V, K, seed=7)
+    cm = synth.class_mask_bernoulli(K, B, 0.5, rng.stream_key(rng.SEED_BASE, 941, V))
+    cm[:, 0] |= 1
+    z = synth.logits_normal(B, V, 2.0, "f32", (942, V))
+    allowed = synth.unpack_bits(cm, K)[:, part.c].astype(bool)
+    for b in range(B):  # the row's keenest tokens among the last: the largest alone, then many
+        last = np.flatnonzero(allowed[b, V - 2000:]) + V - 2000
+        z[b, last[-1 - b % 7]] = 14.0
+        if b % 2:
+            z[b, last] = 12.0 + np.arange(len(last)) % 64 / 32.0
+    if dtype == "bf16":
+        z = (z.view(np.uint32) >> 16).astype(np.uint16)
+    u = rng.uniform(rng.stream_key(943), B).astype(np.float32)
+    with Ctx([part]) as ctx:
+        for top_k, top_p in ((50, 0.9), (200, 1.0)):
+            got = run_filtered(ctx, None, cm, z, V, u, 1.0, top_k, top_p)
+            check_filtered(got, [part], None, cm, z, V, u, 1.0, top_k, top_p, "V=%d k=%d" % (V, top_k))
