@@ -340,18 +340,28 @@ int masks_kind(const PartSet& ps, const uint32_t* class_mask, int64_t stride, bo
 }
 
 // Launch shape of the register-based dense kernel. units: octets; unit_chunk: units one warp covers per iteration.
-DensePlan plan_dense(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, int units, int unit_chunk, int masks) {
+// narrow: also where the class table leaves no room for a whole slice of the masks (some 53400 to 57500 classes off the 16-byte grid), by
+// slices as wide as there is room, or word by word. The per-row kernel is as fast there (64 bf16 rows of 60032 in 53000 classes 167 us by whole
+// slices, 137), but takes one mask per row.
+DensePlan plan_dense(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, int units, int unit_chunk, int masks, bool narrow = false) {
     DensePlan d;
     d.table_words = (ps.maxKW + 1) * 32;
     d.use_plan_kernel = mixed;
     d.n_groups_ub = mixed ? ceil_div(B, kGroupRows) + ps.n_live_same_v : ceil_div(B, kGroupRows);
     if (!ps.all_c16) return d;
-    if (dense_smem_bytes(d.table_words, 8, masks ? 0 : slice_stride(ps)) > size_t(ctx->smem_optin) - 2048) return d;
+    const size_t cap = size_t(ctx->smem_optin) - 2048;
+    narrow = narrow && !masks && dense_smem_bytes(d.table_words, 8, slice_stride(ps)) > cap;
+    const size_t least = dense_smem_bytes(d.table_words, 8, masks || narrow ? 0 : slice_stride(ps));
+    if (least > cap) return d;
     if (mixed && (B > ctx->reserved_rows || d.n_groups_ub > ctx->max_groups)) return d;
     const int ctas_per_sm = ctx->ctas_per_sm;
     // the class masks through shared memory, all at once while that keeps a block under 64 KB
     d.cm_bulk = masks;
-    if (!masks) d.stage_stride = dense_smem_bytes(d.table_words, 8, ps.maxKW | 1) <= 64 * 1024 ? ps.maxKW | 1 : slice_stride(ps);
+    if (narrow) {
+        const int room = int((cap - least) / (kGroupRows * 4));
+        d.stage_stride = room > 16 ? (room - 1) | 1 : 0;
+    }
+    if (!masks && !narrow) d.stage_stride = dense_smem_bytes(d.table_words, 8, ps.maxKW | 1) <= 64 * 1024 ? ps.maxKW | 1 : slice_stride(ps);
     d.ctas_per_sm = ctas_per_sm;
     const int target = ctx->sm_count * ctas_per_sm;
     const int n_chunks = ceil_div(units, unit_chunk);
@@ -1728,7 +1738,7 @@ int cfgzip_multi_mask_logsoftmax_argmax(cfgzip_ctx* ctx, cfgzip_part_id part0, c
     if (masks_per_row > 1) d = plan_multi(ctx, ps, B, masks_per_row, es, masks, class_stride_words);
     const bool shared = d.ok;
     // nothing to share (64 rows with one mask each: 17.3 against 19.2 us) or too little, or a class table that leaves no room beside it
-    if (!shared) d = plan_dense(ctx, ps, rows, false, 4 * ps.VW, 32, masks == kMasksRows ? kMasksRows : kMasksStaged);
+    if (!shared) d = plan_dense(ctx, ps, rows, false, 4 * ps.VW, 32, masks == kMasksRows ? kMasksRows : kMasksStaged, true);
     if (!d.ok) return CFGZIP_E_RANGE;  // more than 65535 classes, or a class table beyond shared memory
     fill_groups(ctx, a, d);
     ctx->pdl_now = int64_t(B) * ps.V * es < (int64_t(192) << 20);

@@ -237,12 +237,11 @@ __device__ __forceinline__ void stage_class_masks(const StepArgs& a, const int* 
 // The 32x32 bit blocks come from a staging area that starts with word k0 of every row; a stage_stride that is odd (or even
 // and no multiple of 4) spreads its column reads over 32 (16) banks. BLOCK: words from `staged` on (counted through the
 // area) are not in it and are read from global memory.
-template <bool BLOCK>
+template <bool BLOCK, int U = 4>
 __device__ __forceinline__ void build_class_table(const StepArgs& a, int K, int KW, const int* s_row, uint32_t* T, const uint32_t* stage,
                                                   int warp, int lane, int n_warps, int k0, int k1, int staged) {
     const uint32_t tail = (K & 31) ? (1u << (K & 31)) - 1u : 0xFFFFFFFFu;
     const int row = s_row[lane];
-    constexpr int U = 4;
     for (int kw0 = k0 + warp; kw0 < k1; kw0 += n_warps * U) {
         uint32_t x[U];
 #pragma unroll
@@ -264,12 +263,14 @@ __device__ __forceinline__ void build_class_table(const StepArgs& a, int K, int 
     }
 }
 // The table as many words at a time as the staging area holds: all of them, or kMaskSlice (16416 classes a lane per row, read where
-// they lie, word by word, took 29 of 43 us of a call with 8 x 16 masks). Called by all threads of the block, which meet before the
-// table is read.
+// they lie, word by word, took 29 of 43 us of a call with 8 x 16 masks). NARROW: where the table leaves no room for that, as many as it does
+// (with a width the compiler does not know all slices are slower, 64 rows in 50000 classes 195 us instead of 160). Called by all threads
+// of the block, which meet before the table is read.
 constexpr int kMaskSlice = 128;
+template <bool NARROW = false>
 __device__ __forceinline__ void build_class_table_staged(const StepArgs& a, int K, int KW, const int* s_row, uint32_t* T, uint32_t* stage,
                                                          int warp, int lane, int n_warps) {
-    const int span = a.stage_stride >= KW ? KW + 1 : kMaskSlice;
+    const int span = NARROW ? a.stage_stride - 1 : a.stage_stride >= KW ? KW + 1 : kMaskSlice;
     for (int k0 = 0; k0 <= KW; k0 += span) {
         if (k0) __syncthreads();  // (the words before have been taken)
         stage_class_masks(a, s_row, stage, warp, lane, n_warps, k0, min(k0 + span, KW));
@@ -880,7 +881,9 @@ __global__ void __launch_bounds__(256) k_step_dense(const __grid_constant__ Step
     __syncthreads();
     const PartDev P = a.group_part ? a.parts[part] : a.p0;
     const int nrow = __popc(__ballot_sync(0xFFFFFFFFu, s_row[lane] >= 0));
-    make_class_table(a, P, s_row, T, stage, warp, lane, n_warps);
+    if (a.cm_bulk || a.stage_stride >= min(P.KW, kMaskSlice)) make_class_table(a, P, s_row, T, stage, warp, lane, n_warps);
+    else if (a.stage_stride) build_class_table_staged<true>(a, P.K, P.KW, s_row, T, stage, warp, lane, n_warps);
+    else build_class_table<true, 8>(a, P.K, P.KW, s_row, T, stage, warp, lane, n_warps, 0, P.KW + 1, 0);  // (no room at all: every word where it lies)
     __syncthreads();
 
     const int wt = warp % a.WT, wr = warp / a.WT, WR = n_warps / a.WT;

@@ -88,3 +88,28 @@ def test_several_masks_and_several_partitions(K, pad, offset):
         assert np.allclose(got["lse"], want["lse"], rtol=0, atol=1e-4)  # as everywhere: f32 sums against f64
         row_part = (np.arange(B * M) % 2).astype(np.int32)
         compare_step(step(ctx, row_part, d_cm, cm.shape[1] + pad, many, V, cz.DENSE), oracle_step(parts, row_part, cm, many, V), V)
+
+
+# Class tables that leave no room for a slice of the masks beside them, and one word of masks more than fits: several masks per row as far as
+# the table goes (57536 classes), one mask per row beyond
+@pytest.mark.parametrize("K", [46500, 48300, 53000, 53600, 57000, 57536, 57537])
+@pytest.mark.parametrize("pad,offset", [(0, 0), (1, 0), (0, 1)])
+def test_tables_that_fill_shared_memory(K, pad, offset):
+    V, B, M = 60032, 3, 3
+    part = synth.zipf_partition(V, K, seed=K)
+    cm = synth.class_mask_bernoulli(K, B * M, 0.2, rng.stream_key(rng.SEED_BASE, 956, K))
+    z = synth.logits_normal(B, V, 2.0, "bf16", (957, K))
+    many = np.repeat(z, M, axis=0)
+    want = oracle_step([part], None, cm, many, V)
+    d_cm = masks_on(cm, pad, offset)
+    with Ctx([part]) as ctx:
+        cz.cfgzip_set_tuning(ctx.h, "one_launch", 0)
+        compare_step(step(ctx, None, d_cm, cm.shape[1] + pad, many, V, cz.DENSE), want, V)
+        if K > 57536:
+            with pytest.raises(cz.CfgzipError):
+                step(ctx, None, d_cm, cm.shape[1] + pad, z, V, cz.DENSE, masks_per_row=M)
+            return
+        got = step(ctx, None, d_cm, cm.shape[1] + pad, z, V, cz.DENSE, masks_per_row=M)
+        for key in ("vocab_mask", "argmax", "rep"):
+            assert np.array_equal(got[key], want[key]), key
+        assert np.allclose(got["lse"], want["lse"], rtol=0, atol=1e-4)  # as everywhere: f32 sums against f64
