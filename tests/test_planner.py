@@ -70,3 +70,12 @@ def test_plan_query_rejects_nonsense():
     assert lib.cfgzip_plan_query(148, 232448, 100, 10, 0, cz.F32, 1, 1, out) == cz.E_ARG
     assert lib.cfgzip_plan_query(148, 232448, 100, 10, 1, 7, 1, 1, out) == cz.E_ARG
     assert lib.cfgzip_plan_query(148, 232448, 100, 10, 1, cz.F32, 1, 1, None) == cz.E_ARG
+
+
+@pytest.mark.parametrize("dtype,most", [(cz.BF16, 48300), (cz.F32, 39900)])
+@pytest.mark.parametrize("aligned", [True, False])
+def test_large_class_tables_keep_the_streaming_kernel(dtype, most, aligned):
+    # four warps' rings of two stages are all that has to fit beside the table: a slice of the class masks lies over them
+    for K in range(30000, most, 1009):
+        for V, B in ((60032, 64), (256000, 64), (256000, 1024)):
+            assert cz.cfgzip_plan_query(SMS, SMEM, V, K, B, dtype, 1, aligned)["kind"] == 2, (K, V, B)
