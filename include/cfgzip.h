@@ -167,7 +167,7 @@ int cfgzip_mask_logits(cfgzip_ctx* ctx, void* logits, int dtype, int64_t row_str
  * A row with no allowed token, or whose allowed logits are all -inf, gets lse =
  * logp_argmax = -inf (the latter still returns the lowest allowed id). +inf and NaN
  * logits are outside the contract for the reductions (the masking itself still copies
- * them bit for bit); logits below -1.7e38 count as -inf in the normaliser.
+ * them bit for bit); logits below -1.4e9 (z / T in a sampling step) count as -inf in the normaliser.
  */
 int cfgzip_masked_logsoftmax_argmax(cfgzip_ctx* ctx, cfgzip_part_id part0, const int32_t* row_part,
                                     const uint32_t* class_mask, int64_t class_stride_words, void* logits,

@@ -119,7 +119,7 @@ template <int R>
 __device__ __forceinline__ void cluster_draw(const StepArgs& a, const PartDev& P, ClusterShared<R>& sh, int row, int r, int lane, int rank,
                                              float M, float weight) {
     if (lane == 0) sh.draw[r].warp = -1;
-    if (!(M > kRefFloor)) {  // nothing allowed, or only -inf allowed: the lowest allowed token (if any) and -inf logs
+    if (!(M * a.scale > kRefLow)) {  // nothing allowed, or nothing that weighs anything: the lowest allowed token (if any) and -inf logs
         if (rank == 0) {
             const unsigned long long pick = first_allowed_warp(a, P, row, lane);
             if (lane == 0) write_row_outputs(a, row, -INFINITY, 0.f, pick);
@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1) k_step_cluster(const __gri
     for (int r = 0; r < R; ++r) {
         if (r >= live) break;
         const float M = float_from_order_key(__reduce_max_sync(0xFFFFFFFFu, float_order_key(acc[r].m)));
-        float s = M > kRefFloor ? acc[r].s * ex2f(-fmaf(M, scale, acc[r].nrl)) : 0.f;
+        float s = acc[r].sum_below(M, scale);
 #pragma unroll
         for (int d = 16; d >= 1; d >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, d);
         const int pos = __reduce_min_sync(0xFFFFFFFFu, acc[r].m == M ? acc[r].pos : kNoPos);

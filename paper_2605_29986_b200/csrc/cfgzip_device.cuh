@@ -13,6 +13,10 @@ constexpr int kBatchRows = 8;         // rows a warp streams together
 constexpr int kNoPos = 0x7FFFFFFF;    // "no allowed token seen"
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kRefFloor = -1.7e38f; // lowest reference used for exp(z - ref)
+// Where the exponent is taken as z * scale - ref * scale (RowAcc): a logit with z * scale below this weighs nothing. The second product is
+// rounded, by up to 64 here, which a sum still holds and the way back undoes; further down it would be infinite or nothing, whatever the
+// logit, and one such run of fill values (-1e10, -1e30) in a lane made the sum of its whole row NaN.
+constexpr float kRefLow = -2147483648.f;
 
 enum : int { kF32 = 0, kBF16 = 1 };
 
@@ -333,7 +337,7 @@ struct RowAcc {
     __device__ __forceinline__ void init() {
         m = -INFINITY;
         s = 0.f;
-        nrl = -(kRefFloor * kLog2e);
+        nrl = -kRefLow;
         pos = kNoPos;
     }
     // N = 8 or 16 consecutive logits of the row (masked ones are -inf), `position` the index of their first octet.
@@ -372,10 +376,10 @@ struct RowAcc {
     }
     // Bring the sum to the convention of Partial: relative to max(m, kRefFloor).
     __device__ __forceinline__ Partial to_partial(float scale = kLog2e) const {
-        // nothing finite seen: the reference never moved off the floor and the sum is empty
-        if (!(m > kRefFloor)) return Partial{m, 0.f, pos, 0};
-        return Partial{m, s * ex2f(-fmaf(m, scale, nrl)), pos, 0};
+        return Partial{m, sum_below(m, scale), pos, 0};
     }
+    // The sum relative to M >= m. (Where nothing above kRefLow was seen the reference has not moved and the sum is empty.)
+    __device__ __forceinline__ float sum_below(float M, float scale) const { return s * ex2f(-fmaxf(fmaf(M, scale, nrl), -126.f)); }
 };
 
 // ---- mbarrier + bulk asynchronous copy (global -> shared) wrappers, CTA scope ----------

@@ -809,7 +809,7 @@ __device__ __forceinline__ void warp_rows_publish_to(RowAcc (&acc)[kBatchRows], 
     for (int i = 0; i < kBatchRows; ++i) M[i] = float_from_order_key(__reduce_max_sync(0xFFFFFFFFu, float_order_key(acc[i].m)));
 #pragma unroll
     for (int i = 0; i < kBatchRows; ++i) {
-        w[i] = M[i] > kRefFloor ? acc[i].s * ex2f(-fmaf(M[i], scale, acc[i].nrl)) : 0.f;
+        w[i] = acc[i].sum_below(M[i], scale);
         pos[i] = __reduce_min_sync(0xFFFFFFFFu, acc[i].m == M[i] ? acc[i].pos : kNoPos);
     }
 #pragma unroll
@@ -1730,7 +1730,11 @@ __global__ void __launch_bounds__(kFewThreads, 3) k_step_few(const __grid_consta
         for (int i = 0; i < kBatchRows; ++i) {
             acc[i].m = w.m[i][lane];
             acc[i].s = w.s[i][lane];
-            acc[i].nrl = -(fmaxf(acc[i].m, kRefFloor) * kLog2e);
+            acc[i].nrl = -(acc[i].m * kLog2e);
+            if (!(acc[i].m * kLog2e > kRefLow)) {
+                acc[i].s = 0.f;
+                acc[i].nrl = -kRefLow;
+            }
             acc[i].pos = w.pos[i][lane];
         }
         warp_rows_publish(a, acc, live, g, split * a.WT + wt, rb, lane);
@@ -2119,8 +2123,8 @@ __global__ void __launch_bounds__(kSampleThreads) k_sample_rows(const __grid_con
     __syncthreads();
 #pragma unroll
     for (int w = 0; w < kSampleThreads / 32; ++w) M = fmaxf(M, s_warp[w]);
-    if (!(M > kRefFloor)) {
-        // nothing allowed, or only -inf allowed: the lowest allowed token (if any) and -inf logs
+    if (!(M * a.scale > kRefLow)) {
+        // nothing allowed, or nothing that weighs anything: the lowest allowed token (if any) and -inf logs
         if (warp == 0) {
             unsigned long long cand = first_allowed_share(a, P, row, lane, 32);
 #pragma unroll

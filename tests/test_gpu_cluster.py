@@ -8,7 +8,7 @@ import torch
 import synth
 from synth import rng
 from paper_2605_29986_b200 import binding as cz
-from _gpu_util import Ctx, compare_step, oracle_step, run_fused
+from _gpu_util import Ctx, assert_close_log, compare_step, dev, oracle_step, run_fused
 from test_gpu_sample import check_sample, run_sample
 
 pytestmark = pytest.mark.gpu
@@ -126,3 +126,78 @@ def test_a_refused_knob_changes_nothing():
                             (b"lane_octets", 3), (b"pipe_depth", 1), (b"nonsense", 1)):
             assert lib.cfgzip_set_tuning(ctx.h, knob, value) == cz.E_ARG and launches(ctx) == 1, knob
         assert lib.cfgzip_set_tuning(ctx.h, b"row_warps", 1) == 0 and launches(ctx) == 2
+
+
+def limit_rows(V, dtype):
+    """Rows whose sums are at the ends of their range: every value close to the one below which a logit weighs nothing, fill values beside one or
+    many others, fill values first, and a climb of 400 nats that moves the sums' reference again and again."""
+    part, cm, z = inputs(V, 50, 6, "f32", 6)
+    cm[:] = 0xFFFFFFFF
+    t = np.arange(V, dtype=np.float32)
+    z[0] = -1.2e9 - 1e4 * t
+    z[0, 5] = -1e9  # (one largest value, also when rounded to bf16: the log of a tie is lost beside 1e9)
+    z[1] = -1e30
+    z[1, V // 3] = 0.0
+    z[2, ::2] = -3e38
+    z[3, 4096:12288] = -1e10
+    z[4] = -200.0 + 400.0 * t / V
+    z[5, :8000] = -1e37
+    return part, cm, rng.f32_to_bf16_bits(z.reshape(-1)).reshape(z.shape) if dtype == "bf16" else z
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("V", [20000, 20003])
+@pytest.mark.parametrize("one_launch", [1, 0])
+def test_sums_at_the_ends_of_their_range(V, dtype, one_launch):
+    part, cm, z = limit_rows(V, dtype)
+    B = len(z)
+    u = np.linspace(0, 0.99, B).astype(np.float32)
+    with Ctx([part]) as ctx:
+        cz.cfgzip_set_tuning(ctx.h, "one_launch", one_launch)
+        compare_step(run_fused(ctx, None, cm, z, V), oracle_step([part], None, cm, z, V), V)
+        check_sample(run_sample(ctx, None, cm, z, V, u, 1.0), [part], None, cm, z, V, u, 1.0)
+        # very low temperatures: logits whose z / T stays where 1e-4 can be told, then ordinary ones, of which the largest is drawn
+        for inv_t, sigma in ((200.0, 0.02), (1e6, 4e-6)):
+            y = synth.logits_normal(B, V, sigma, dtype, (924, V))
+            check_sample(run_sample(ctx, None, cm, y, V, u, inv_t), [part], None, cm, y, V, u, inv_t)
+        y = synth.logits_normal(B, V, 2.0, "f32", (925, V))
+        y[np.arange(B), 1000 * np.arange(B) + 3] = 16.0
+        got = run_sample(ctx, None, cm, y, V, u, 1e6)
+        assert np.array_equal(got["token"], 1000 * np.arange(B) + 3) and np.all(got["lse"] == 16e6) and np.all(got["logp_token"] == 0)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("kind,V,B", [("one launch", 20000, 20), ("streaming", 40000, 96), ("streaming", 40003, 96), ("registers", 20000, 40),
+                                      ("class lists", 20000, 20), ("few tokens", 60000, 96), ("several masks", 20000, 3)])
+def test_fill_values_weigh_nothing(kind, V, B, dtype):
+    # allowed tokens that the program in front has set to a large negative number, whole runs of them
+    K = 60
+    part = synth.zipf_partition(V, K, seed=9)
+    M = 5 if kind == "several masks" else 1
+    cm = synth.class_mask_bernoulli(K, B * M, 0.1 if kind in ("class lists", "few tokens") else 0.7, rng.stream_key(rng.SEED_BASE, 926, V))
+    cm[:, 0] |= 1
+    z = synth.logits_normal(B, V, 2.0, "f32", (927, V))
+    for b in range(B):
+        z[b, 300 * b : 300 * b + V // 2] = (-1e9, -1e10, -1e30, -1e37, -3e38)[b % 5]
+    if dtype == "bf16":
+        z = rng.f32_to_bf16_bits(z.reshape(-1)).reshape(z.shape)
+    many = np.repeat(z, M, axis=0)
+    want = oracle_step([part], None, cm, many, V)
+    with Ctx([part]) as ctx:
+        if kind != "one launch":
+            cz.cfgzip_set_tuning(ctx.h, "one_launch", 0)
+        if kind == "registers":
+            cz.cfgzip_set_tuning(ctx.h, "pipeline", 0)
+        if M > 1:
+            d_z, d_cm = dev(z), dev(cm)
+            tok, rep = (torch.zeros(B * M, dtype=torch.int32, device="cuda") for _ in range(2))
+            lp, lse = (torch.zeros(B * M, device="cuda") for _ in range(2))
+            cz.cfgzip_multi_mask_logsoftmax_argmax(ctx.h, ctx.ids[0], d_cm, cm.shape[1], M, d_z, cz.BF16 if dtype == "bf16" else cz.F32, V, B,
+                                                   None, 0, tok, rep, lp, lse)
+            assert np.array_equal(tok.cpu().numpy(), want["argmax"]) and np.array_equal(rep.cpu().numpy(), want["rep"])
+            assert_close_log(lse.cpu().numpy(), want["lse"], "lse")
+            return
+        compare_step(run_fused(ctx, None, cm, z, V, mode=cz.SPARSE if kind in ("class lists", "few tokens") else cz.DENSE), want, V)
+        if kind in ("one launch", "streaming"):
+            u = rng.uniform(rng.stream_key(928, V), B).astype(np.float32)
+            check_sample(run_sample(ctx, None, cm, z, V, u, 1.3), [part], None, cm, z, V, u, 1.3)
