@@ -529,6 +529,14 @@ def _multi_mask(cz, torch, device: int, B: int = 8, M: int = 16, steps: int = 20
             "what": "V=128256 K=2048 bf16, one logits buffer (L2-resident: a latency figure, not an HBM one)"}
 
 
+def _kernels_of(mode, sampling, launches_per_step):
+    """The kernels of a step, by the launches it took: one for short batches."""
+    per_row = "k_sample_rows" if sampling else "k_finalize_rows"
+    if launches_per_step < 1.5:
+        return "k_step_cluster" if mode != "sparse" else "k_step_cluster or k_step_sparse"
+    return ("k_step_few (+ %s)" if mode == "sparse" else "k_step_dense_pipe (+ %s)") % per_row
+
+
 def _cpu_baseline(runner, budget_s: float = 12.0) -> dict:
     """The CPU oracle timed on steps of the same workload: with one thread per host core (rows split over a thread
     pool) and with a single thread, each for about half of `budget_s`."""
@@ -628,8 +636,7 @@ def run_own(args):
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                      "traffic": traffic, "peak_source": "of " + peak_src, "frac_of_nominal_8TBs": achieved / NOMINAL_HBM_GBS,
                      "algorithmic_bytes_per_step": alg, "launches_per_step": launches / timed_steps,
-                     "kernel": ("k_step_sparse" if args.mode == "sparse" else
-                                "k_step_dense_pipe (+ %s)" % ("k_sample_rows" if sampling else "k_finalize_rows"))},
+                     "kernel": _kernels_of(args.mode, sampling, launches / timed_steps)},
         "clocks": sampler.summary(),
         "paper_context": "paper reports no timing of this path; its speedups (up to two orders of magnitude in grammar-engine "
                          "latency, up to 7.5x end to end) are for 1x H100 + Xeon Gold 6430 x16 threads, precision unstated",

@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("V,K,B,parts", [
     (9000, 300, 63, 1), (9000, 300, 64, 1),
-    (60000, 4800, 64, 1), (60000, 5100, 64, 1), (60000, 16000, 64, 1),       # masks staged or not; two blocks per SM
+    (60000, 4800, 64, 1), (60000, 5100, 64, 1), (60000, 16000, 64, 1),       # masks in slices of 128 words; two blocks per SM, one
     (9000, 200, 296, 1), (9000, 200, 297, 1), (60000, 200, 444, 1), (60000, 200, 445, 1), (60000, 200, 593, 1),
     (20000, 3072, 64, 2), (20000, 3080, 64, 2), (9000, 200, 63, 3), (9000, 200, 420, 3), (9000, 200, 500, 4)])
 def test_rows_that_allow_few_tokens(V, K, B, parts, dtype):
