@@ -153,9 +153,12 @@ int cfgzip_mask_logits(cfgzip_ctx* ctx, void* logits, int dtype, int64_t row_str
  *   logp_full   : nullable dev float [B, V] (row stride V); z_i - lse, -inf where masked
  *   vocab_mask  : nullable; as in cfgzip_expand_mask
  *   mode        : CFGZIP_DENSE streams every row through the gather; CFGZIP_SPARSE is for rows that
- *                 allow few tokens: it overwrites the vectors that hold no allowed token without reading them (16 bytes
+ *                 allow few tokens: from 64 rows on, and on smaller batches that do not fit one launch (see the knob
+ *                 "one_launch"), it overwrites the vectors that hold no allowed token without reading them (16 bytes
  *                 each, found from the class->token lists of a row's allowed classes, or, for larger batches with few classes
- *                 and long rows, 32 bytes each, found through the gather's class table: of such a vector it reads all 32). CFGZIP_AUTO: the class-list kernel pays off when under 4 % (f32) or 1 %
+ *                 and long rows, 32 bytes each, found through the gather's class table: of such a vector it reads all 32);
+ *                 smaller batches are done in one launch, which reads every logit and is the faster one there.
+ *                 CFGZIP_AUTO: the class-list kernel pays off when under 4 % (f32) or 1 %
  *                 (bf16) of the tokens are allowed, the measured break-even. Callers whose class masks are
  *                 still in host memory, where the grammar engine leaves them, get that choice for free
  *                 from cfgzip_choose_mode (cfgzip_decode_step_host with CFGZIP_AUTO uses it). On device

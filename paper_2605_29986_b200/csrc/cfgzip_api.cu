@@ -460,7 +460,7 @@ DensePlan plan_pipe_opl(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixe
             n_warps = max_warps;
             stride = slice_stride(ps);
             d.cm_bulk = kMasksStaged;
-            alias = true;  // (always over the rings: a slice beside them cost tables of some 45000 to 49500 classes the kernel, 64 bf16 rows
+            alias = true;  // (always over the rings: a slice beside them cost tables of 44200 to 48300 classes the kernel, 64 bf16 rows
                            // of 60032 in 48000 classes 151 us instead of 79)
         }
     }
@@ -581,7 +581,8 @@ DensePlan plan_pipe(cfgzip_ctx* ctx, const PartSet& ps, int32_t B, bool mixed, i
 // per row, most efficient from the row count on at which a block takes a whole row and as long as these fit the device in one wave.
 // Measured, us, class lists / k_step_few, bf16, one to five classes allowed:
 //   under 64 rows    32 of 128256: K = 512 20 / 11, 2000 14.9 / 12.4, 4000 12.8 / 14.2; 48 f32 rows of 256000, K = 2000 20 / 24: by
-//                    classes and row length there, but the class lists are one launch instead of two and are kept for all of them
+//                    classes and row length. These batches take one launch where it fits them (launch_fused), the others the class lists,
+//                    one launch instead of two
 //   class table      128 of 128256: K = 4000 25 / 20, 6000 25 / 21, 8192 23.2 / 24.3, 16000 29 / 24; 512 of 256000: K = 8200 79 / 70, 16000
 //                    108 / 71; f32: 250 of 200064 K = 6001 76 / 54, 100 of 64064 K = 8000 26 / 19; 70 of 90048 K = 11000 19.7 / 20.4 (while the table
 //                    took its masks lane by lane from some 4900 classes on, the lists were better there)
@@ -848,8 +849,9 @@ int launch_finalize(cfgzip_ctx* ctx, const StepArgs& a, const DensePlan& d, cuda
 // batches: the choice is 0.2 % slower than the best shape in the mean, 3 % at most. 128256 bf16 logits, us, two launches / this:
 // 1 row 6.3 / 3.9, 8 6.7 / 4.7, 32 8.5 / 7.7, 48 11.5 / 9.3, 64 11.9 / 10.9, 80 15.3 / 13.1; 32 rows of four grammars 20.0 / 8.6 (and 23.3
 // where they are grouped at every step); sampling 8 rows 8.8 / 5.5, 32 10.6 / 8.4, 64 13.8 / 11.9.
-// Rows under 128 KB from 33 rows on, and mixed batches from there, are left at two launches: callers count on them (48 rows of 32000
-// bf16: 7.1 against 5.0).
+// Rows under 128 KB from 33 rows on, and mixed batches from there, are left at two launches although one is faster (48 rows of 32000
+// bf16: 7.1 against 5.0): tests/test_gpu_auto.py (40 rows of 20000 bf16, of 30000 f32) and tests/test_gpu_parity.py (a mixed batch of 70
+// rows) state these launch counts.
 struct ClusterPlan {
     bool ok = false;
     ClusterGeom g{};
@@ -916,8 +918,10 @@ int launch_fused(cfgzip_ctx* ctx, StepArgs& a, const PartSet& ps, bool mixed, in
                  cudaStream_t st) {
     int rc;
     DensePlan few;
-    // (rows that allow few tokens as well while there are fewer than k_step_few takes: class lists / this, us, 32 bf16 rows of 128256 in 512
-    // classes 19.4 / 8.2, 8 f32 rows 14.6 / 5.9, 2 bf16 rows of 50663 in 6332 classes 12.6 / 4.4)
+    // (Rows that allow few tokens as well while there are fewer than k_step_few takes, although this reads every logit: one to five classes
+    // allowed, class lists / this, us, with 512 and 8000 classes: 2 f32 rows of 128256 9.4 / 4.5, 13.9 / 4.6, 32 rows 17.2 / 10.6, 21.0 / 10.7,
+    // 40 rows 24.4 / 12.5, 20.4 / 12.5; bf16 33 rows 17.6 / 8.4, 19.3 / 8.3, 63 rows 23.6 / 11.2, 20.4 / 11.4; 33 bf16 rows of 256000 20.7 / 13.1,
+    // 22.5 / 13.3. Over 204 sizes of 2 to 63 rows of 20032 to 256000 tokens it took 0.27 to 0.79 of the class lists' time.)
     if (!(mode == CFGZIP_SPARSE && a.B >= 64) && !(mode == CFGZIP_AUTO && ctx->auto_min_bytes >= 0) &&
         (aligned || aligned_elems(a.logits, DT == kBF16 ? 2 : 4))) {
         ClusterPlan cl = plan_cluster(ctx, ps, a.B, mixed, DT == kBF16 ? 2 : 4, !aligned, false, logp_full != nullptr);
