@@ -819,7 +819,8 @@ __device__ __forceinline__ void warp_rows_publish_to(RowAcc (&acc)[kBatchRows], 
     for (int i = 0; i < kBatchRows; ++i) M[i] = float_from_order_key(__reduce_max_sync(0xFFFFFFFFu, float_order_key(acc[i].m)));
 #pragma unroll
     for (int i = 0; i < kBatchRows; ++i) {
-        w[i] = acc[i].sum_below(M[i], scale);
+        // (the comparison is not needed, the sum is empty there; without it the streaming kernel spills: 1024 bf16 rows 108.2 -> 112.5 us)
+        w[i] = M[i] > kRefFloor ? acc[i].sum_below(M[i], scale) : 0.f;
         pos[i] = __reduce_min_sync(0xFFFFFFFFu, acc[i].m == M[i] ? acc[i].pos : kNoPos);
     }
 #pragma unroll
